@@ -73,26 +73,49 @@ __device__ __forceinline__ float activate(int act, float v) {
     return 0.5f * v * (1.0f + erff(v * 0.70710678118654752440f));
 }
 
-// The same for kernels whose result is rounded to bf16 right away: erf by the rational-times-exponential
-// formula 7.1.26 of Abramowitz & Stegun (absolute error below 1.5e-7, far inside half a bf16 ulp of the
-// GELU value), one exponential and one division instead of the long polynomial of erff.
+__device__ __forceinline__ float exp2_approx(float v) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {      // NaN if either is
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// GELU for results that are rounded to bf16 right away: v Phi(v) = max(v, 0) - |v| Q(|v|) with the normal tail
+// Q = 1 - Phi evaluated as 2^P(|v|).  log2 Q is so nearly quadratic that a polynomial of degree 6 is enough: its
+// coefficients are a least-squares fit on [0, 6], reweighted until the error of |v| Q is level, which leaves at most
+// 5.1e-8 (7.6e-8 with float32 arithmetic; the formula 7.1.26 of Abramowitz & Stegun that stood here before: 2.1e-7).
+// One exponential and no division.  |v| is cut off at 10, where Q < 2^-74.  kGeluP: coefficients in -|v|.
+constexpr float kGeluCut = -10.0f;
+constexpr float kGeluP0 = -0.9999930609869272f, kGeluP1 = 1.1512017022737409f, kGeluP2 = -0.45877097266965633f,
+                kGeluP3 = 0.05341210482228353f, kGeluP4 = 0.008080716673348184f, kGeluP5 = 0.0007692196373495289f,
+                kGeluP6 = 3.309279284094074e-05f;
+
+// The activations for kernels whose result is rounded to bf16 right away.
 __device__ __forceinline__ float activate_bf16(int act, float v) {
     if (act == kActRelu) return fmaxf(v, 0.0f);
     if (act == kActGeluTanh) {
-        // tanh(u) = 1 - 2 / (1 + e^(2u)), u clamped where tanh is +-1 to float32 anyway (keeps e^(2u) finite)
-        const float u = fminf(fmaxf(0.79788456080286535588f * (v + 0.044715f * v * v * v), -15.0f), 15.0f);
-        const float th = 1.0f - __fdividef(2.0f, 1.0f + __expf(2.0f * u));
-        return 0.5f * v * (1.0f + th);
+        // v / 2 (1 + tanh u) = v / (1 + e^(-2u))
+        const float m = -2.0f * 1.44269504088896340736f * 0.79788456080286535588f;
+        return v * rcp_approx(1.0f + exp2_approx(v * fmaf(m * 0.044715f, v * v, m)));
     }
-    if (act == kActSilu) return v * __fdividef(1.0f, 1.0f + __expf(-fmaxf(v, -80.0f)));      // e^80 is finite; below, the result is -0
-    const float z = fabsf(v) * 0.70710678118654752440f;
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, z, 1.0f));
-    float poly = fmaf(1.061405429f, t, -1.453152027f);
-    poly = fmaf(poly, t, 1.421413741f);
-    poly = fmaf(poly, t, -0.284496736f);
-    poly = fmaf(poly, t, 0.254829592f);
-    const float e = 1.0f - poly * t * __expf(-z * z);          // erf(|v| / sqrt 2)
-    return 0.5f * v * (1.0f + copysignf(e, v));
+    if (act == kActSilu) return v * rcp_approx(1.0f + exp2_approx(-1.44269504088896340736f * fmaxf(v, -80.0f)));
+    const float a = max_nan(-fabsf(v), kGeluCut);
+    float p = fmaf(kGeluP6, a, kGeluP5);
+    p = fmaf(p, a, kGeluP4);
+    p = fmaf(p, a, kGeluP3);
+    p = fmaf(p, a, kGeluP2);
+    p = fmaf(p, a, kGeluP1);
+    p = fmaf(p, a, kGeluP0);
+    return fmaf(a, exp2_approx(p), fmaxf(v, 0.0f));
 }
 
 // Calls f(std::integral_constant<int, act>) with the activation as a compile-time constant.  Code that applies the
