@@ -114,6 +114,10 @@ struct fff_handle_s {
     // FORWARD_T (fff_forward_train): transposed output weights with the output biases appended along K, and the
     // workspace of the three GEMMs (allocated on first use)
     __nv_bfloat16* tr_w2t = nullptr;     // [O][tr_Kp]
+    __nv_bfloat16* tr_w1t = nullptr;     // hidden weights in the order of the GEMM's columns, and their biases
+    float* tr_b1t = nullptr;
+    __nv_bfloat16* tr_wn = nullptr;      // node weights in the order of k_train_nodes' columns (1 <= depth <= 8), and their biases
+    float* tr_bn = nullptr;
     int tr_Kp = 0;                       // 2^d l + 2^d rounded up to 64 (0 = shapes not eligible)
     int64_t tr_cap_B = 0;
     float *tr_c = nullptr, *tr_mix = nullptr, *tr_entpart = nullptr;
@@ -269,7 +273,7 @@ void release(fff_handle_s* h) {
     dfree(h->ws_pos[0]); dfree(h->ws_pos[1]);
     dfree(h->fs_w1g); dfree(h->fs_b1g); dfree(h->fs_w2g); dfree(h->fs_b2f);
     dfree(h->w1codes); dfree(h->w2codes); dfree(h->scale1); dfree(h->scale2);
-    dfree(h->tr_w2t); dfree(h->tr_c); dfree(h->tr_mix); dfree(h->tr_entpart); dfree(h->tr_hp);
+    dfree(h->tr_w2t); dfree(h->tr_w1t); dfree(h->tr_b1t); dfree(h->tr_wn); dfree(h->tr_bn); dfree(h->tr_c); dfree(h->tr_mix); dfree(h->tr_entpart); dfree(h->tr_hp);
     dfree(h->w1img); dfree(h->b1img); dfree(h->w2img); dfree(h->w2uimg); dfree(h->ws_sched); dfree(h->ws_tiles); dfree(h->ws_rank); dfree(h->ws_rank8); dfree(h->ws_counts8); dfree(h->ws_blocksum); dfree(h->ws_matrix); dfree(h->ws_slots); dfree(h->ws_cursor); dfree(h->ws_nslots); dfree(h->ws_ncursor);
     if (h->copy_in) cudaStreamDestroy(h->copy_in);
     if (h->copy_out) cudaStreamDestroy(h->copy_out);
@@ -1125,52 +1129,123 @@ fff_status_t run_fused_small(fff_handle_s* h, const void* x, void* y, int32_t* l
     return launched(h, st, "fused_forward_small");
 }
 
-// FORWARD_T: the transposed output weights (at creation) and the three GEMMs.
+// FORWARD_T: the weight images of the GEMMs (at creation).
+constexpr int kTrainMaxFusedDepth = 8;      // deepest tree whose node logits fit one tile of k_train_nodes
+
 fff_status_t pack_train_images(fff_handle_s* h) {
     if (h->dtype != FFF_DTYPE_BF16 || h->D % fff::kGKB != 0 || !encode_tiled_fn()) return FFF_OK;
-    const int64_t k_used = h->n_leaves * h->l + h->n_leaves;
-    if (k_used > (1 << 24)) return FFF_OK;
-    const int Kp = (int)((k_used + fff::kGKB - 1) / fff::kGKB * fff::kGKB);
+    if (h->n_leaves * (h->l + 1) > (1 << 24)) return FFF_OK;
+    const int hidden = fff::train_hidden_columns((int)h->n_leaves, h->l);
+    const int Kp = (int)((hidden + h->n_leaves + fff::kGKB - 1) / fff::kGKB * fff::kGKB);
+    const int padded = (hidden + 255) / 256 * 256, NP = std::max<int>(32, (int)h->n_leaves);
+    const int blocks = h->sm_count * 8;
+    const __nv_bfloat16 *w1 = (const __nv_bfloat16*)h->w1, *b1 = (const __nv_bfloat16*)h->b1;
     fff_status_t s;
     if ((s = dmalloc((void**)&h->tr_w2t, sizeof(__nv_bfloat16) * (size_t)h->O * Kp)) != FFF_OK) return s;
-    fff::k_pack_w2_transposed<__nv_bfloat16><<<h->sm_count * 8, 256>>>((const __nv_bfloat16*)h->w2, (const __nv_bfloat16*)h->b2,
-                                                                      h->tr_w2t, (int)h->n_leaves, h->l, h->O, Kp);
+    if ((s = dmalloc((void**)&h->tr_w1t, sizeof(__nv_bfloat16) * (size_t)hidden * h->D)) != FFF_OK) return s;
+    if ((s = dmalloc((void**)&h->tr_b1t, sizeof(float) * (size_t)padded)) != FFF_OK) return s;
+    fff::k_pack_w2_transposed<__nv_bfloat16><<<blocks, 256>>>((const __nv_bfloat16*)h->w2, (const __nv_bfloat16*)h->b2, h->tr_w2t,
+                                                             (int)h->n_leaves, h->l, h->O, Kp);
+    fff::k_pack_train_hidden<__nv_bfloat16><<<blocks, 256>>>(w1, b1, h->tr_w1t, h->tr_b1t, (int)h->n_leaves, h->l, h->D, padded);
+    if (h->depth >= 1 && h->depth <= kTrainMaxFusedDepth) {
+        if ((s = dmalloc((void**)&h->tr_wn, sizeof(__nv_bfloat16) * (size_t)NP * h->D)) != FFF_OK) return s;
+        if ((s = dmalloc((void**)&h->tr_bn, sizeof(float) * (size_t)NP)) != FFF_OK) return s;
+        fff::k_pack_train_nodes<__nv_bfloat16><<<blocks, 256>>>((const __nv_bfloat16*)h->node_w, (const __nv_bfloat16*)h->node_b, h->tr_wn,
+                                                               h->tr_bn, h->depth, NP, h->D);
+    }
     if (cudaGetLastError() != cudaSuccess) return FFF_ERR_CUDA;
-    for (auto kern : {(const void*)fff::k_gemm_umma<fff::kGemmNodes>, (const void*)fff::k_gemm_umma<fff::kGemmHidden>,
-                      (const void*)fff::k_gemm_umma<fff::kGemmOutput>})
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, fff::kGSmemBytes) != cudaSuccess)
-            return cudaGetLastError(), FFF_ERR_CUDA;
     h->tr_Kp = Kp;
     return FFF_OK;
 }
 
+// Tensor map of a row-major matrix (element size 2 or 4, `pitch` elements between rows) for boxes of box_cols x box_rows,
+// swizzled in the mode of the box's row width (32, 64 or 128 bytes).
+bool make_matrix_map(CUtensorMap* tm, const void* p, int esize, int64_t rows, int64_t cols, int64_t pitch, int box_cols, int box_rows) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return false;
+    const cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t gstride[1] = {(cuuint64_t)pitch * esize};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    const cuuint32_t estride[2] = {1, 1};
+    const int width = box_cols * esize;
+    return enc(tm, esize == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(p), gdim, gstride,
+               box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               width == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : width == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// C [M, N] = epilogue(A [M, K] . B [N, K]^T) on CTA pairs; lda = row pitch of A; out / out_cols / ld_out: the bf16 matrix that
+// the epilogue stores through a tensor map (nullptr: it stores by itself).
+template <int MODE, int BN>
+fff_status_t launch_gemm_tiles(fff_handle_s* h, const void* a, int64_t M, int lda, const void* b, int64_t N, int64_t K,
+                               fff::GemmEpilogueArgs ep, void* out, cudaStream_t st, const char* name) {
+    using L = fff::GemmLayout<MODE, BN>;
+    static bool limit_raised[kMaxDevices] = {};
+    if (!raise_smem_limit(fff::k_gemm_pair<MODE, BN>, h->device, L::kSmemBytes, limit_raised)) return FFF_ERR_CUDA;
+    CUtensorMap ta, tb, tc, tx;
+    if (!make_matrix_map(&ta, a, 2, M, K, lda, fff::kGKB, fff::kGRows) || !make_matrix_map(&tb, b, 2, N, K, K, fff::kGKB, BN / 2))
+        return FFF_ERR_CUDA;
+    tc = tx = ta;                          // unused ones still have to be valid maps
+    if (out && !make_matrix_map(&tc, out, 2, M, N, ep.ld_out, L::kColsPerWarp, 32)) return FFF_ERR_CUDA;
+    if (MODE == fff::kGemmHidden && ep.n_leaves >= 32 && !make_matrix_map(&tx, ep.mix, 4, M, ep.n_leaves, ep.n_leaves, 32, fff::kGRows)) return FFF_ERR_CUDA;
+    const int64_t tiles = ((M + fff::kGM - 1) / fff::kGM) * ((N + BN - 1) / BN);
+    const int64_t grid = 2 * (MODE == fff::kGemmHidden ? std::min<int64_t>(h->sm_count / 2, tiles) : balanced_grid(h->sm_count / 2, tiles));
+    if (launch_chain(h, fff::k_gemm_pair<MODE, BN>, (unsigned)grid, fff::kGPairThreads, (size_t)L::kSmemBytes, st, 2, ta, tb, tc, tx, (int)M, (int)N,
+                     (int)K, ep, h->d_status) != cudaSuccess)
+        return cudaGetLastError(), FFF_ERR_CUDA;
+    return launched(h, st, name);
+}
+
 template <int MODE>
 fff_status_t launch_gemm(fff_handle_s* h, const void* a, int64_t M, int lda, const void* b, int64_t N, int64_t K,
-                         const fff::GemmEpilogueArgs& ep, cudaStream_t st, const char* name) {
-    CUtensorMap ta, tb;
-    // (row pitch = lda elements; the tensor maps describe K columns of them)
-    EncodeTiledFn enc = encode_tiled_fn();
-    auto encode = [&](CUtensorMap* tm, const void* p, int64_t rows, int64_t pitch, int box_rows) {
-        const cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-        const cuuint64_t gstride[1] = {(cuuint64_t)pitch * 2};
-        const cuuint32_t box[2] = {(cuuint32_t)fff::kGKB, (cuuint32_t)box_rows};
-        const cuuint32_t estride[2] = {1, 1};
-        return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(p), gdim, gstride, box, estride,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    if (!enc || !encode(&ta, a, M, lda, fff::kGM) || !encode(&tb, b, N, K, fff::kGN)) return FFF_ERR_CUDA;
-    const int64_t tiles = ((M + fff::kGM - 1) / fff::kGM) * ((N + fff::kGN - 1) / fff::kGN);
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(h->sm_count, tiles));
-    fff::k_gemm_umma<MODE><<<(unsigned)grid, fff::kGThreads, fff::kGSmemBytes, st>>>(ta, tb, (int)M, (int)N, (int)K, ep, h->d_status);
-    return launched(h, st, name);
+                         const fff::GemmEpilogueArgs& ep, void* out, cudaStream_t st, const char* name) {
+    // 256 columns per tile unless that leaves pairs of SMs without a tile
+    const int64_t tiles = ((M + fff::kGM - 1) / fff::kGM) * ((N + 255) / 256);
+    return tiles >= h->sm_count / 2 ? launch_gemm_tiles<MODE, 256>(h, a, M, lda, b, N, K, ep, out, st, name)
+                                    : launch_gemm_tiles<MODE, 128>(h, a, M, lda, b, N, K, ep, out, st, name);
+}
+
+template <int DEPTH>
+fff_status_t launch_train_nodes(fff_handle_s* h, const void* x, float* mix, float* ent_part, int64_t B, cudaStream_t st, int* ctas) {
+    using L = fff::TrainNodesLayout<DEPTH>;
+    static bool limit_raised[kMaxDevices] = {};
+    if (!raise_smem_limit(fff::k_train_nodes<DEPTH>, h->device, L::kSmemBytes, limit_raised)) return FFF_ERR_CUDA;
+    const int hidden = fff::train_hidden_columns((int)h->n_leaves, h->l);
+    CUtensorMap tx, tw, tm, tt;
+    if (!make_matrix_map(&tx, x, 2, B, h->D, h->D, fff::kGKB, fff::kGRows) || !make_matrix_map(&tw, h->tr_wn, 2, L::NP, h->D, h->D, fff::kGKB, L::NP / 2))
+        return FFF_ERR_CUDA;
+    tm = tt = tx;
+    if (L::kStaged && (!make_matrix_map(&tm, mix, 4, B, h->n_leaves, h->n_leaves, L::kPart, 32) ||
+                       !make_matrix_map(&tt, h->tr_hp + hidden, 2, B, h->n_leaves, h->tr_Kp, L::kPart, 32)))
+        return FFF_ERR_CUDA;
+    const int64_t grid = 2 * balanced_grid(h->sm_count / 2, (B + fff::kGM - 1) / fff::kGM);
+    *ctas = (int)grid;
+    if (launch_chain(h, fff::k_train_nodes<DEPTH>, (unsigned)grid, fff::kGThreads, (size_t)L::kSmemBytes, st, 2, tx, tw, tm, tt, (const float*)h->tr_bn, mix,
+                     h->tr_hp, h->tr_Kp, hidden, ent_part, (int)B, h->D, h->d_status) != cudaSuccess)
+        return cudaGetLastError(), FFF_ERR_CUDA;
+    return launched(h, st, "train_node_choices");
+}
+
+fff_status_t run_train_nodes(fff_handle_s* h, const void* x, float* mix, float* ent_part, int64_t B, cudaStream_t st, int* ctas) {
+    switch (h->depth) {
+        case 1: return launch_train_nodes<1>(h, x, mix, ent_part, B, st, ctas);
+        case 2: return launch_train_nodes<2>(h, x, mix, ent_part, B, st, ctas);
+        case 3: return launch_train_nodes<3>(h, x, mix, ent_part, B, st, ctas);
+        case 4: return launch_train_nodes<4>(h, x, mix, ent_part, B, st, ctas);
+        case 5: return launch_train_nodes<5>(h, x, mix, ent_part, B, st, ctas);
+        case 6: return launch_train_nodes<6>(h, x, mix, ent_part, B, st, ctas);
+        case 7: return launch_train_nodes<7>(h, x, mix, ent_part, B, st, ctas);
+        case 8: return launch_train_nodes<8>(h, x, mix, ent_part, B, st, ctas);
+    }
+    return FFF_ERR_UNSUPPORTED;
 }
 
 fff_status_t run_forward_train(fff_handle_s* h, const void* x, void* y, float* mixture, float* node_entropy, int64_t B,
                                cudaStream_t st) {
-    const int64_t nl = h->n_leaves, nn = h->n_nodes, hidden = nl * h->l;
+    const int64_t nl = h->n_leaves, nn = h->n_nodes, hidden = fff::train_hidden_columns((int)nl, h->l);
+    const bool fused = h->tr_wn != nullptr;
     const int ldc = (int)std::max<int64_t>((nn + 3) & ~(int64_t)3, 4);      // rows of c start on 16-byte boundaries
-    const int64_t n_mt = (B + fff::kGM - 1) / fff::kGM;
+    const int64_t n_mt = (B + fff::kGRows - 1) / fff::kGRows;
     if (B > h->tr_cap_B) {
         if (cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
         dfree(h->tr_c); dfree(h->tr_mix); dfree(h->tr_entpart); dfree(h->tr_hp);
@@ -1178,44 +1253,65 @@ fff_status_t run_forward_train(fff_handle_s* h, const void* x, void* y, float* m
         h->tr_hp = nullptr;
         h->tr_cap_B = 0;
         fff_status_t s;
-        if ((s = dmalloc((void**)&h->tr_c, sizeof(float) * (size_t)B * ldc)) != FFF_OK) return s;
+        if (!fused && (s = dmalloc((void**)&h->tr_c, sizeof(float) * (size_t)B * ldc)) != FFF_OK) return s;
         if ((s = dmalloc((void**)&h->tr_mix, sizeof(float) * (size_t)B * nl)) != FFF_OK) return s;
-        if ((s = dmalloc((void**)&h->tr_entpart, sizeof(float) * (size_t)n_mt * 4 * ldc)) != FFF_OK) return s;
+        if ((s = dmalloc((void**)&h->tr_entpart, sizeof(float) * (fused ? (size_t)h->sm_count * nl : (size_t)n_mt * 4 * ldc))) != FFF_OK) return s;
         if ((s = dmalloc((void**)&h->tr_hp, sizeof(__nv_bfloat16) * (size_t)B * h->tr_Kp)) != FFF_OK) return s;
+        // the columns of h' past the mixture weights stay zero
+        const int pad = h->tr_Kp - (int)(hidden + nl);
+        if (pad > 0 && cudaMemset2D(h->tr_hp + hidden + nl, (size_t)h->tr_Kp * 2, 0, (size_t)pad * 2, (size_t)B) != cudaSuccess)
+            return cudaGetLastError(), FFF_ERR_CUDA;
         h->tr_cap_B = B;
     }
     fff_status_t s = FFF_OK;
     fff::GemmEpilogueArgs ep = {};
-    if (nn > 0) {
-        ep.bias = (const __nv_bfloat16*)h->node_b;
-        ep.out_f32 = h->tr_c;
-        ep.ent_part = node_entropy ? h->tr_entpart : nullptr;
-        ep.ld_out = ldc;
-        if ((s = launch_gemm<fff::kGemmNodes>(h, x, B, h->D, h->node_w, nn, h->D, ep, st, "train_node_choices")) != FFF_OK) return s;
-        if (node_entropy) {
-            fff::k_entropy_reduce<<<(unsigned)((nn + 7) / 8), 256, 0, st>>>(h->tr_entpart, (int)(n_mt * 4), (int)nn, B, node_entropy);
-            if ((s = launched(h, st, "train_node_entropy")) != FFF_OK) return s;
+    float* mix = h->tr_mix;
+    int ent_ctas = 0;
+    if (fused) {
+        // the caller's matrix is the one that the hidden GEMM reads, where its tensor map can take it
+        if (mixture && aligned16(mixture)) mix = mixture;
+        if ((s = run_train_nodes(h, x, mix, node_entropy ? h->tr_entpart : nullptr, B, st, &ent_ctas)) != FFF_OK) return s;
+        if (mixture && mix != mixture &&
+            cudaMemcpyAsync(mixture, mix, sizeof(float) * (size_t)B * nl, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+            return cudaGetLastError(), FFF_ERR_CUDA;
+    } else {
+        if (nn > 0) {
+            ep.bias_bf16 = (const __nv_bfloat16*)h->node_b;
+            ep.out_f32 = h->tr_c;
+            ep.ent_part = node_entropy ? h->tr_entpart : nullptr;
+            ep.ld_out = ldc;
+            if ((s = launch_gemm<fff::kGemmNodes>(h, x, B, h->D, h->node_w, nn, h->D, ep, nullptr, st, "train_node_choices")) != FFF_OK) return s;
+            if (node_entropy) {
+                fff::k_entropy_reduce<<<(unsigned)((nn + 7) / 8), 256, 0, st>>>(h->tr_entpart, (int)((B + 31) / 32), (int)nn, B, node_entropy);
+                if ((s = launched(h, st, "train_node_entropy")) != FFF_OK) return s;
+            }
         }
-    }
-    {
         const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((B + fff::kMixTokens - 1) / fff::kMixTokens, (int64_t)h->sm_count * 16));
         fff::k_mixture_weights<<<(unsigned)blocks, 256, 0, st>>>(h->tr_c, ldc, h->tr_mix, mixture, h->tr_hp, h->tr_Kp, (int)hidden,
                                                                  h->depth, B);
         if ((s = launched(h, st, "train_mixture_weights")) != FFF_OK) return s;
     }
     ep = {};
-    ep.bias = (const __nv_bfloat16*)h->b1;
-    ep.mix = h->tr_mix;
+    ep.bias = h->tr_b1t;
+    ep.mix = mix;
     ep.out_bf16 = h->tr_hp;
     ep.ld_out = h->tr_Kp;
     ep.n_leaves = (int)nl;
     ep.l = h->l;
     ep.act = h->act;
-    if ((s = launch_gemm<fff::kGemmHidden>(h, x, B, h->D, h->w1, hidden, h->D, ep, st, "train_hidden_all_leaves")) != FFF_OK) return s;
+    if (fused && node_entropy) {
+        ep.ent_part = h->tr_entpart;
+        ep.ent_out = node_entropy;
+        ep.ent_rows = ent_ctas;
+        ep.ent_depth = h->depth;
+    }
+    if ((s = launch_gemm<fff::kGemmHidden>(h, x, B, h->D, h->tr_w1t, hidden, h->D, ep, h->tr_hp, st, "train_hidden_all_leaves")) != FFF_OK) return s;
     ep = {};
     ep.out_bf16 = (__nv_bfloat16*)y;
     ep.ld_out = h->O;
-    return launch_gemm<fff::kGemmOutput>(h, h->tr_hp, B, h->tr_Kp, h->tr_w2t, h->O, h->tr_Kp, ep, st, "train_output_mixture");
+    ep.tma_out = h->O % 8 == 0 ? 1 : 0;
+    return launch_gemm<fff::kGemmOutput>(h, h->tr_hp, B, h->tr_Kp, h->tr_w2t, h->O, h->tr_Kp, ep, ep.tma_out ? y : nullptr, st,
+                                         "train_output_mixture");
 }
 
 #define FFF_DISPATCH(h, fn, ...) \

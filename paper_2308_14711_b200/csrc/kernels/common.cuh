@@ -131,6 +131,75 @@ __device__ __forceinline__ void with_activation(int act, F&& f) {
     }
 }
 
+// Two float32 values in one 64-bit register: the packed instructions (add / mul / fma .f32x2) do both in one issue slot,
+// each rounded as its scalar form.
+struct f32x2 { unsigned long long r; };
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d.r) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ f32x2 pack2u(uint32_t lo, uint32_t hi) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d.r) : "r"(lo), "r"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 a, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.r)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.r) : "l"(a.r), "l"(b.r));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.r) : "l"(a.r), "l"(b.r));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.r) : "l"(a.r), "l"(b.r), "l"(c.r));
+    return d;
+}
+__device__ __forceinline__ f32x2 splat2(float v) { return pack2(v, v); }
+__device__ __forceinline__ uint32_t to_bf16x2(f32x2 a) {
+    float lo, hi;
+    unpack2(a, lo, hi);
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// activate_bf16 for two values at once.
+template <int kAct>
+__device__ __forceinline__ f32x2 activate_bf16x2(f32x2 v) {
+    float v0, v1;
+    unpack2(v, v0, v1);
+    if (kAct == kActGelu) {
+        float p0, p1;
+        const f32x2 a = pack2(max_nan(-fabsf(v0), kGeluCut), max_nan(-fabsf(v1), kGeluCut));
+        f32x2 p = fma2(splat2(kGeluP6), a, splat2(kGeluP5));
+        p = fma2(p, a, splat2(kGeluP4));
+        p = fma2(p, a, splat2(kGeluP3));
+        p = fma2(p, a, splat2(kGeluP2));
+        p = fma2(p, a, splat2(kGeluP1));
+        p = fma2(p, a, splat2(kGeluP0));
+        unpack2(p, p0, p1);
+        return fma2(a, pack2(exp2_approx(p0), exp2_approx(p1)), pack2(fmaxf(v0, 0.0f), fmaxf(v1, 0.0f)));
+    }
+    return pack2(activate_bf16(kAct, v0), activate_bf16(kAct, v1));
+}
+
+// One node's choice from its logit: right = sigmoid(z), left = 1 - right (each from the exponential of -|z|, so that the
+// small one keeps its relative accuracy), h = the entropy -right ln right - left ln left = ln(1 + e^-|z|) + |z| min(right, left).
+__device__ __forceinline__ void node_choice(float z, float& right, float& left, float& h) {
+    const float a = fabsf(z);
+    const float e = exp2_approx(a * -1.44269504088896340736f);
+    const float d = 1.0f + e;
+    const float big = rcp_approx(d), small = e * big;
+    right = z >= 0.0f ? big : small;
+    left = z >= 0.0f ? small : big;
+    h = fmaf(fminf(a, 128.0f), small, __logf(d));          // (beyond 128 the small one is 0; keeps 0 x inf out)
+}
+
 // <a, b> over n elements, evaluated by one warp; every lane returns the sum.
 // `vec` says both rows start on 16-byte boundaries and n is a multiple of kVec.
 template <typename T>

@@ -113,12 +113,7 @@ template <int LP, bool kW8 = false, int GL = 1> struct LeafUmmaLayout {
     }
 };
 
-// Swizzle of a byte offset inside an operand tile whose rows are row_bytes (32, 64 or 128) long: the
-// 16-byte unit index inside a row is XORed with bits of the 128-byte line index, as the 32-, 64- and
-// 128-byte swizzle modes of the tensor cores expect.
-__host__ __device__ __forceinline__ uint32_t swz_rows(uint32_t off, int row_bytes) {
-    return off ^ (((off >> 7) & (uint32_t)(row_bytes / 16 - 1)) << 4);
-}
+using ptx::swz_rows;
 
 // W2 image for GEMM2: [leaf][ceil(O/128) pieces]{ [128 rows (output features)][LP columns] swizzled,
 // then the 128 float32 biases of those features }.

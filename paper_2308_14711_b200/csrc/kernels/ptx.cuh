@@ -120,6 +120,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// Swizzle of a byte offset inside an operand tile whose rows are row_bytes (32, 64 or 128) long: the
+// 16-byte unit index inside a row is XORed with bits of the 128-byte line index, as the 32-, 64- and
+// 128-byte swizzle modes of the tensor cores and of tensor-map copies expect.
+__host__ __device__ __forceinline__ uint32_t swz_rows(uint32_t off, int row_bytes) {
+    return off ^ (((off >> 7) & (uint32_t)(row_bytes / 16 - 1)) << 4);
+}
+
 // 128-byte swizzle of a byte offset inside a tile image: the 16-byte unit index within each
 // 128-byte line is XORed with the line index (mod 8).
 __host__ __device__ __forceinline__ uint32_t swz128(uint32_t off) { return off ^ (((off >> 7) & 7u) << 4); }
@@ -150,6 +157,18 @@ __device__ __forceinline__ void tma_gather4(void* dst_smem, const void* tmap, in
         "l"(tmap), "r"(c0), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(smem_addr(bar))
         : "memory");
 }
+
+// Tensor-map store of a box from shared memory (elements outside the tensor are clipped; both coordinates must not be
+// negative), as a bulk group of its own.  The source must have been made visible with fence_proxy_async.
+__device__ __forceinline__ void tma_store_2d(const void* tmap, const void* src_smem, int c0, int c1) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tmap), "r"(c0), "r"(c1),
+                 "r"(smem_addr(src_smem))
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+// Waits until the stores issued so far by this thread have read their sources / have completed.
+__device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // Makes shared-memory writes of this thread visible to the asynchronous proxy (tensor cores, TMA).
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -239,6 +258,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
           "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr)
         : "memory");
+}
+// One column.
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t& v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 

@@ -18,6 +18,15 @@ CASES = [
     C("train_d2_l1", 64, 16, 2, 1, "silu", "bf16", 333, "normal", node_bias_std=0.5),
     C("train_d0", 128, 40, 0, 24, "gelu_tanh", "bf16", 200, "normal"),              # no nodes: one leaf with weight 1
     C("train_d8_l3", 192, 96, 8, 3, "gelu", "bf16", 450, "normal"),                 # 255 nodes, 768 hidden neurons + 256 mixture columns
+    # one case per shape class of the fused node kernel and of the hidden epilogue: trees of 1, 6 and 7 levels, blocks of 32
+    # leaves that end inside a warp's columns (odd l), 256-column tiles, deeper than the node kernel goes, rows of y that a
+    # tensor map cannot describe
+    C("train_d1_l5", 64, 24, 1, 5, "gelu", "bf16", 130, "normal", node_bias_std=0.5),
+    C("train_d4_l16", 128, 136, 4, 16, "silu", "bf16", 257, "normal"),
+    C("train_d6_l23_wide_tiles", 128, 192, 6, 23, "gelu", "bf16", 4100, "normal", node_bias_std=0.2),
+    C("train_d7_l9", 128, 64, 7, 9, "relu", "bf16", 513, "layernorm"),
+    C("train_d9_l2", 64, 64, 9, 2, "gelu", "bf16", 300, "normal"),
+    C("train_d5_l7_odd_output", 128, 44, 5, 7, "gelu_tanh", "bf16", 200, "normal"),
 ]
 
 
