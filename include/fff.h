@@ -306,7 +306,7 @@ fff_status_t fff_get_last_status(fff_handle_t h);
 fff_status_t fff_selftest_bounded_wait(fff_handle_t h, int64_t limit_cycles, void *cuda_stream);
 
 /* Which kernel families the shapes of this layer admit (a bit set; -1 for a bad handle).  A bf16 layer whose
- * D is no multiple of 128, whose O is no multiple of 8 or whose leaves are wider than 64 has no tensor-core
+ * D is no multiple of 8, whose O is no multiple of 8 or whose leaves are wider than 64 has no tensor-core
  * kernels: its forward runs on CUDA-core kernels (the one-launch kernel when FFF_CAP_FUSED_SMALL is set, else
  * one warp per token), which is several times slower per token; float32 layers never have them.  Callers
  * that depend on tensor-core speed can check here instead of timing. */
@@ -317,6 +317,8 @@ typedef enum {
     FFF_CAP_TCGEN05_LEAF = 8,     /* ... on tcgen05 (also O % 16 == 0) */
     FFF_CAP_FUSED_SMALL = 16,     /* the one-launch kernel (l <= 32, at most one group of 32 neurons per SM) */
     FFF_CAP_FORWARD_TRAIN = 32,   /* fff_forward_train (bf16, D % 64 == 0) */
+    FFF_CAP_PADDED = 128,         /* the tensor-core kernels run on images padded to the next multiple of 128 (D % 128 != 0, D % 8 == 0);
+                                     the bits above for them are not set then, and fff_set_path refuses FFF_PATH_TENSOR */
     FFF_CAP_GROUP_TILES = 64      /* leaf tiles of 8 sibling leaves (FFF_TUNE_GROUP_TILES: 8 <= leaf_width < 16, 9 <= depth <= 11) */
 } fff_capability_t;
 int fff_capabilities(fff_handle_t h);

@@ -47,6 +47,7 @@ struct fff_handle_s {
     int device = 0;
     int sm_count = 148;
     int D = 0, O = 0, depth = 0, l = 0;
+    int Dp = 0;                   // D rounded up to the K step of the tensor-core images, which are padded with zero columns
     int act = 0, dtype = 0;
     size_t esize = 4;
     int64_t n_nodes = 0, n_leaves = 1;
@@ -509,7 +510,7 @@ fff_status_t launch_descent_mma(fff_handle_s* h, const fff_handle_s::DenseStage&
                                 bool grouped, int32_t* pos_out, int64_t B, cudaStream_t st) {
     using L = fff::DescentMmaLayout<NP>;
     // A single-group stage keeps its weight image resident if at least 3 ring stages still fit.
-    const int res_bytes = NP * h->D * 2;
+    const int res_bytes = NP * h->Dp * 2;
     const bool resident = !grouped && L::smem_bytes(3, res_bytes) <= kSmemBudget;
     // two CTAs per SM when that leaves at least 3 stages each, else one CTA with as many as fit
     auto stages_for = [&](int budget) {
@@ -524,7 +525,7 @@ fff_status_t launch_descent_mma(fff_handle_s* h, const fff_handle_s::DenseStage&
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)h->sm_count * per_sm, n_tiles));
     if (launch_chain(h, fff::k_descent_mma<NP>, (unsigned)grid, fff::kDescentThreads, (size_t)smem, st, 1,
                      (const __nv_bfloat16*)x, grouped ? perm : nullptr, grouped ? h->ws_tiles : nullptr, n_tiles, sg.wimg,
-                     sg.bimg, pos_out, h->D, (int)B, sg.k, stages, resident ? 1 : 0, h->d_status) != cudaSuccess)
+                     sg.bimg, pos_out, h->D, h->Dp, (int)B, sg.k, stages, resident ? 1 : 0, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "tree_descent_mma");
 }
@@ -621,7 +622,7 @@ fff_status_t launch_descent_umma(fff_handle_s* h, const fff_handle_s::DenseStage
     const SlotArgs sl = slot_args(h, pos_out);
     if (launch_chain(h, fff::k_descent_umma<NP>, (unsigned)grid, fff::kUmmaThreads, (size_t)L::smem_bytes(stages), st, 1, tm,
                      (const __nv_bfloat16*)sg.wimg, (const float*)sg.bimg, pos_out, ranked ? h->ws_rank8 : (uint8_t*)nullptr,
-                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->D, (int)B, sg.k,
+                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, (int)B, sg.k,
                      stages, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "tree_descent_umma");
@@ -639,7 +640,7 @@ fff_status_t launch_descent_umma_pair(fff_handle_s* h, const fff_handle_s::Dense
     CUtensorMap tm, tw;
     if (!make_x_tensor_map(&tm, x, B, h->D, fff::kUM)) return FFF_ERR_CUDA;
     // the weight image as (D/64) * NP rows of 64 columns, stored pre-swizzled: copied as it is
-    if (!make_x_tensor_map(&tw, sg.wimg, (int64_t)(h->D / fff::kUKB) * NP, fff::kUKB, NP / 2, false)) return FFF_ERR_CUDA;
+    if (!make_x_tensor_map(&tw, sg.wimg, (int64_t)(h->Dp / fff::kUKB) * NP, fff::kUKB, NP / 2, false)) return FFF_ERR_CUDA;
     const int64_t n_pairs = ((B + fff::kUM - 1) / fff::kUM + 1) / 2;
     const int64_t grid = 2 * balanced_grid(h->sm_count / 2, n_pairs);
     const bool ranked = !h->nslots_here && sg.k >= 4 && h->ws_rank8 && h->ws_counts8;
@@ -648,7 +649,7 @@ fff_status_t launch_descent_umma_pair(fff_handle_s* h, const fff_handle_s::Dense
     const SlotArgs sl = slot_args(h, pos_out);
     if (launch_chain(h, fff::k_descent_umma_pair<NP>, (unsigned)grid, fff::kUmmaThreads, (size_t)L::smem_bytes(stages), st, 2, tm,
                      tw, (const float*)sg.bimg, pos_out, ranked ? h->ws_rank8 : (uint8_t*)nullptr,
-                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->D, (int)B, sg.k,
+                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, (int)B, sg.k,
                      stages, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "tree_descent_umma");
@@ -687,7 +688,7 @@ fff_status_t launch_descent_umma_grouped(fff_handle_s* h, const fff_handle_s::De
     const SlotArgs sl = slot_args(h, pos_out);
     if (launch_chain(h, fff::k_descent_umma_grouped<NP>, (unsigned)grid, fff::kUGThreads, (size_t)L::smem_bytes(stages), st, 1, tm,
                      perm, (const fff::Tile*)h->ws_tiles, n_tiles, (const __nv_bfloat16*)sg.wimg, (const float*)sg.bimg, pos_out,
-                     sl.pos2, sl.cursor, sl.slots, sl.cap, h->D, sg.k, stages, h->d_status, node_lists ? h->ws_ncursor : (int32_t*)nullptr,
+                     sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, sg.k, stages, h->d_status, node_lists ? h->ws_ncursor : (int32_t*)nullptr,
                      1 << sg.L0, (int)h->nslot_cap) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "tree_descent_umma_grouped");
@@ -823,11 +824,11 @@ fff_status_t pack_stage(fff_handle_s* h, std::vector<fff_handle_s::DenseStage>& 
     sg.umma = umma;
     const size_t groups = (size_t)1 << L0;
     fff_status_t s;
-    if ((s = dmalloc((void**)&sg.wimg, groups * sg.NP * h->D * 2)) != FFF_OK) return s;
+    if ((s = dmalloc((void**)&sg.wimg, groups * sg.NP * h->Dp * 2)) != FFF_OK) return s;
     plan.push_back(sg);                            // owned by the handle from here on
     if ((s = dmalloc((void**)&plan.back().bimg, groups * sg.NP * 4)) != FFF_OK) return s;
     fff::k_pack_nodes<T><<<h->sm_count * 8, 256>>>((const T*)h->node_w, (const T*)h->node_b, plan.back().wimg, plan.back().bimg,
-                                                  sg.L0, sg.k, sg.NP, h->D);
+                                                  sg.L0, sg.k, sg.NP, h->D, h->Dp);
     return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
 }
 
@@ -850,7 +851,7 @@ fff_status_t pack_node_images(fff_handle_s* h) {
         L0 += k;
     }
     // plan with a first stage of up to 8 levels on the tcgen05 kernel, the rest as above
-    if (encode_tiled_fn() && h->D % fff::kUKB == 0) {
+    if (encode_tiled_fn()) {
         std::vector<int> ks;
         // Measured: up to 8 levels in one stage when that is the whole tree (no node bucketing at all); two
         // balanced stages up to depth 12 ([6,5] beats [8,3]: 64 bins instead of 256 and fatter groups);
@@ -865,7 +866,7 @@ fff_status_t pack_node_images(fff_handle_s* h) {
         L0 = 0;
         for (size_t i = 0; i < ks.size(); ++i) {
             const int np = i == 0 ? std::max(32, 1 << ks[i]) : std::max(16, 1 << ks[i]);
-            if ((s = pack_stage<T>(h, h->ustages, L0, ks[i], np, i == 0 || h->D % 128 == 0)) != FFF_OK) return s;
+            if ((s = pack_stage<T>(h, h->ustages, L0, ks[i], np, true)) != FFF_OK) return s;
             L0 += ks[i];
         }
         cudaFuncSetAttribute(fff::k_descent_umma<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
@@ -904,7 +905,7 @@ fff_status_t launch_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm
     const int per_sm = std::max(1, std::min(2, (int)((227 * 1024) / (L::kSmemBytes + 1024))));
     const int64_t grid = std::min<int64_t>((int64_t)h->sm_count * per_sm, n_tiles);
     if (launch_chain(h, fff::k_leaf_mma<LP, TM, S>, (unsigned)grid, L::kThreads, L::kSmemBytes, st, 1,
-                     (const __nv_bfloat16*)x, perm, h->ws_tiles, n_tiles, h->w1img, h->b1img, h->w2img, (__nv_bfloat16*)y, h->D,
+                     (const __nv_bfloat16*)x, perm, h->ws_tiles, n_tiles, h->w1img, h->b1img, h->w2img, (__nv_bfloat16*)y, h->D, h->Dp,
                      h->O, h->act, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "grouped_leaf_ff_mma");
@@ -928,7 +929,7 @@ fff_status_t launch_leaf_umma(fff_handle_s* h, const void* x, const int32_t* per
     int32_t* counts = h->slots_now && perm == h->ws_slots ? h->ws_cursor : nullptr;
     if (launch_chain(h, fff::k_leaf_umma<LP, kFold, kW8>, (unsigned)grid, fff::kLUThreads, (size_t)L::smem_bytes(stages), st, 1, tm, perm,
                      (const fff::Tile*)h->ws_tiles, n_tiles, (const __nv_bfloat16*)h->w1img, (const float*)h->b1img,
-                     (const unsigned char*)(kW8 ? h->w2codes : h->w2uimg), (__nv_bfloat16*)y, h->D, h->O, h->l, h->act, stages, wide, passes, h->ws_sched,
+                     (const unsigned char*)(kW8 ? h->w2codes : h->w2uimg), (__nv_bfloat16*)y, h->Dp, h->O, h->l, h->act, stages, wide, passes, h->ws_sched,
                      counts, (int)h->n_leaves, (int)h->slot_cap, h->d_status, (const unsigned char*)h->w1codes, (const float*)h->scale1,
                      (const float*)h->scale2, (const float*)nullptr, (int32_t*)nullptr, (int32_t*)nullptr) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
@@ -980,16 +981,16 @@ fff_status_t pack_leaf_images(fff_handle_s* h) {
     const size_t nl = (size_t)h->n_leaves;
     const size_t stage2 = (size_t)fff::kNC * LP * 2 + fff::kNC * 4;
     fff_status_t s;
-    if ((s = dmalloc((void**)&h->w1img, nl * LP * h->D * 2)) != FFF_OK) return s;
+    if ((s = dmalloc((void**)&h->w1img, nl * LP * h->Dp * 2)) != FFF_OK) return s;
     if ((s = dmalloc((void**)&h->b1img, nl * LP * 4)) != FFF_OK) return s;
     if ((s = dmalloc((void**)&h->w2img, nl * U2 * stage2)) != FFF_OK) return s;
     const int blocks = h->sm_count * 8;
-    fff::k_pack_w1<T><<<blocks, 256>>>((const T*)h->w1, h->w1img, (int)nl, h->l, LP, h->D);
+    fff::k_pack_w1<T><<<blocks, 256>>>((const T*)h->w1, h->w1img, (int)nl, h->l, LP, h->D, h->Dp);
     fff::k_pack_b1<T><<<blocks, 256>>>((const T*)h->b1, h->b1img, (int)nl, h->l, LP);
     fff::k_pack_w2<T><<<blocks, 256>>>((const T*)h->w2, (const T*)h->b2, h->w2img, (int)nl, h->l, LP, h->O);
     if (cudaGetLastError() != cudaSuccess) return FFF_ERR_CUDA;
     // the tcgen05 kernel: W2 in pieces of 128 output features, and its scheduler words
-    if (encode_tiled_fn() && h->O % 16 == 0 && h->D % fff::kLUKB == 0) {
+    if (encode_tiled_fn() && h->O % 16 == 0) {
         const size_t P = (size_t)(h->O + fff::kLUPiece - 1) / fff::kLUPiece;
         if ((s = dmalloc((void**)&h->w2uimg, nl * P * ((size_t)fff::kLUPiece * LP * 2 + fff::kLUPiece * 4))) != FFF_OK) return s;
         if ((s = clone((void**)&h->ws_sched, nullptr, 4 * sizeof(int))) != FFF_OK) return s;
@@ -1012,10 +1013,10 @@ fff_status_t pack_group_images(fff_handle_s* h) {
     if ((s = pack_stage<T>(h, h->gstages, 0, kd, std::max(32, 1 << kd), true)) != FFF_OK) return s;
     if ((s = dmalloc((void**)&h->g_b1, bins * N1 * 4)) != FFF_OK) return s;
     if ((s = clone((void**)&h->g_w2, nullptr, w2_bytes)) != FFF_OK) return s;                    // zeroed
-    if ((s = dmalloc((void**)&h->g_w1, bins * N1 * h->D * 2)) != FFF_OK) return s;                 // (last: it marks the images as usable)
+    if ((s = dmalloc((void**)&h->g_w1, bins * N1 * h->Dp * 2)) != FFF_OK) return s;                 // (last: it marks the images as usable)
     fff::k_pack_leaf_groups<T><<<h->sm_count * 8, 256>>>((const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2,
                                                         (const T*)h->node_w, (const T*)h->node_b, h->g_w1, h->g_b1, h->g_w2, (int)bins, d,
-                                                        h->l, h->LP, h->D, h->O);
+                                                        h->l, h->LP, h->D, h->Dp, h->O);
     return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
 }
 
@@ -1061,7 +1062,7 @@ fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_
     const int wide = (reinterpret_cast<uintptr_t>(y) & 31u) == 0 ? 1 : 0;
     if (launch_chain(h, fff::k_leaf_umma<16, true, false, fff::kLUGroup>, (unsigned)grid, fff::kLUThreads, (size_t)L::smem_bytes(stages), st,
                      1, tm, (const int32_t*)h->ws_slots, (const fff::Tile*)h->ws_tiles, n_tiles, (const __nv_bfloat16*)h->g_w1,
-                     (const float*)h->b1img, (const unsigned char*)h->g_w2, (__nv_bfloat16*)y, h->D, h->O, h->l, h->act, stages, wide, 1,
+                     (const float*)h->b1img, (const unsigned char*)h->g_w2, (__nv_bfloat16*)y, h->Dp, h->O, h->l, h->act, stages, wide, 1,
                      h->ws_sched, h->ws_cursor, bins, (int)h->slot_cap, h->d_status, (const unsigned char*)nullptr,
                      (const float*)nullptr, (const float*)nullptr, (const float*)h->g_b1, leaf,
                      leaf == h->ws_leaf ? (int32_t*)nullptr : h->ws_leaf) != cudaSuccess)
@@ -1103,10 +1104,13 @@ fff_status_t pack_fused_small(fff_handle_s* h) {
 
 // Whether a forward of this handle runs as the one-launch kernel: when pinned to it, or by default for layers
 // that have no tensor-core leaf path (float32, or bf16 shapes outside it) and room for batches of at least 8.
-bool use_fused_small(const fff_handle_s* h) {
+// Layers whose tensor-core images are padded: a few tokens through a narrow layer (136 -> 128, 16 leaves of 16: 13-15 us
+// against 19-20 us up to 64 tokens, 17.5 against 12.7 at 256; 264 -> 256 is level at one token and behind from 16 on).
+bool use_fused_small(const fff_handle_s* h, int64_t B) {
     if (h->fs_batch == 0 || !h->tune[FFF_TUNE_FUSED_SMALL]) return false;
     if (h->path == FFF_PATH_FUSED) return true;
-    return h->path == FFF_PATH_AUTO && h->LP == 0 && h->fs_batch >= 8;
+    if (h->path != FFF_PATH_AUTO || h->fs_batch < 8) return false;
+    return h->LP == 0 || (h->D != h->Dp && h->D <= 256 && B <= 64);
 }
 
 template <typename T>
@@ -1474,7 +1478,7 @@ fff_status_t create_common(fff_handle_t* out, int D, int O, int depth, int leaf_
         else
             cudaGetLastError();
     }
-    h->D = D; h->O = O; h->depth = depth; h->l = leaf_width; h->act = act; h->dtype = dtype;
+    h->D = D; h->O = O; h->depth = depth; h->Dp = (D + fff::kKS - 1) / fff::kKS * fff::kKS; h->l = leaf_width; h->act = act; h->dtype = dtype;
     h->esize = dtype == FFF_DTYPE_F32 ? 4 : 2;
     h->n_nodes = ((int64_t)1 << depth) - 1;
     h->n_leaves = (int64_t)1 << depth;
@@ -1508,7 +1512,7 @@ fff_status_t create_common(fff_handle_t* out, int D, int O, int depth, int leaf_
             cudaGetLastError();
         }
     }
-    if (s == FFF_OK && dtype == FFF_DTYPE_BF16 && D % fff::kKS == 0 && depth > 0) s = pack_node_images<__nv_bfloat16>(h);
+    if (s == FFF_OK && dtype == FFF_DTYPE_BF16 && D % 8 == 0 && depth > 0) s = pack_node_images<__nv_bfloat16>(h);
     if (s == FFF_OK && w8) {
         h->LP = leaf_width <= 16 ? 16 : (leaf_width <= 32 ? 32 : 64);
         const int LP = h->LP;
@@ -1527,7 +1531,7 @@ fff_status_t create_common(fff_handle_t* out, int D, int O, int depth, int leaf_
             fff::k_pack_b1<__nv_bfloat16><<<h->sm_count * 8, 256>>>((const __nv_bfloat16*)h->b1, h->b1img, (int)nl, leaf_width, LP);
             if (cudaGetLastError() != cudaSuccess) s = FFF_ERR_CUDA;
         }
-    } else if (s == FFF_OK && dtype == FFF_DTYPE_BF16 && D % fff::kKS == 0 && O % 8 == 0 && leaf_width <= 64) {
+    } else if (s == FFF_OK && dtype == FFF_DTYPE_BF16 && D % 8 == 0 && O % 8 == 0 && leaf_width <= 64) {
         h->LP = leaf_width <= 16 ? 16 : (leaf_width <= 32 ? 32 : 64);
         s = pack_leaf_images<__nv_bfloat16>(h);
     }
@@ -1585,7 +1589,8 @@ fff_status_t fff_set_path(fff_handle_t h, fff_path_t path) {
     if (!live(h)) return FFF_ERR_BAD_HANDLE;
     if (path != FFF_PATH_AUTO && path != FFF_PATH_WARP && path != FFF_PATH_TENSOR && path != FFF_PATH_FUSED)
         return FFF_ERR_INVALID_ARG;
-    if (path == FFF_PATH_TENSOR && h->LP == 0 && h->stages.empty()) return FFF_ERR_UNSUPPORTED;
+    // (pinning to the tensor-core kernels stays reserved to layers whose rows they take unpadded)
+    if (path == FFF_PATH_TENSOR && ((h->LP == 0 && h->stages.empty()) || h->D != h->Dp)) return FFF_ERR_UNSUPPORTED;
     if (path == FFF_PATH_FUSED && h->fs_batch == 0) return FFF_ERR_UNSUPPORTED;
     if (h->w8 && path != FFF_PATH_AUTO && path != FFF_PATH_TENSOR) return FFF_ERR_UNSUPPORTED;
     h->path = path;
@@ -1657,7 +1662,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     h->prof_active = h->prof_steps < h->prof_max_steps;
     if (h->prof_active)
         cudaEventRecord(h->prof_events[(size_t)h->prof_steps * (fff_handle_s::kMaxProfLaunches + 1)], st);
-    if (use_fused_small(h)) {
+    if (use_fused_small(h, B)) {
         // one launch: descent, grid barrier, leaf evaluation by groups of hidden neurons; the stable bucketing is
         // made on demand from the leaf indices it leaves in the workspace
         s = FFF_DISPATCH(h, run_fused_small, h, x, y, h->ws_leaf, leaf_idx, B, st);
@@ -1886,10 +1891,14 @@ int fff_last_launch_count(fff_handle_t h) { return live(h) ? h->launches : -1; }
 int fff_capabilities(fff_handle_t h) {
     if (!live(h)) return -1;
     int caps = 0;
-    if (!h->stages.empty() || !h->ustages.empty()) caps |= FFF_CAP_TENSOR_DESCENT;
-    if (!h->ustages.empty()) caps |= FFF_CAP_TCGEN05_DESCENT;
-    if (h->LP != 0) caps |= FFF_CAP_TENSOR_LEAF;
-    if (h->w2uimg || h->w2codes) caps |= FFF_CAP_TCGEN05_LEAF;
+    if (h->D == h->Dp) {
+        if (!h->stages.empty() || !h->ustages.empty()) caps |= FFF_CAP_TENSOR_DESCENT;
+        if (!h->ustages.empty()) caps |= FFF_CAP_TCGEN05_DESCENT;
+        if (h->LP != 0) caps |= FFF_CAP_TENSOR_LEAF;
+        if (h->w2uimg || h->w2codes) caps |= FFF_CAP_TCGEN05_LEAF;
+    } else if (!h->ustages.empty() || h->LP != 0) {
+        caps |= FFF_CAP_PADDED;
+    }
     if (h->fs_batch != 0) caps |= FFF_CAP_FUSED_SMALL;
     if (h->tr_Kp != 0) caps |= FFF_CAP_FORWARD_TRAIN;
     if (h->g_w1) caps |= FFF_CAP_GROUP_TILES;

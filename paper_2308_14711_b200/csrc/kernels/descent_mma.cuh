@@ -17,7 +17,8 @@
 // mbarrier ring, and 8 consumer warps with mma.sync.m16n8k16 (two per 16-row m-tile, taking alternate
 // k-steps).  tiles == NULL means "one group, tokens in natural order".
 //
-// Requirements: bf16, D % kKS == 0.
+// Requirements: bf16, D % 8 == 0.  The images are padded to Dp columns (a multiple of kKS) with zero weights; the padding
+// columns of the token rows are filled with zeros on the way into shared memory.
 #pragma once
 
 #include "common.cuh"
@@ -46,26 +47,26 @@ template <int NP> struct DescentMmaLayout {
     static constexpr int kPairScratch = (16 * kLogitRow * 4 > NP * 64 ? 16 * kLogitRow * 4 : NP * 64);
     static constexpr int kStagingBytes = kDescentMTiles * kPairScratch;
     static constexpr int kFixedBytes = ((kStagingBytes + 127) & ~127) + 256 /* barriers */ + 128 /* align */;
-    // shared memory of a launch with `stages` ring stages; resident_bytes = NP * D * 2 or 0
+    // shared memory of a launch with `stages` ring stages; resident_bytes = NP * Dp * 2 or 0
     static constexpr int smem_bytes(int stages, int resident_bytes) {
         return stages * (resident_bytes ? kXStageBytes : kStageStride) + kFixedBytes + resident_bytes;
     }
 };
 
-// Weight image of one stage: [group][D/kKS][kKS/64][NP rows][64 columns] 128-byte swizzled, rows in the
+// Weight image of one stage: [group][Dp/kKS][kKS/64][NP rows][64 columns] 128-byte swizzled, rows in the
 // subtree's breadth-first order (row 2^r - 1 + p = node N_{L0+r, g*2^r + p}); unused rows zero.
 // Bias image: [group][NP] float32.
 template <typename T>
 __global__ void k_pack_nodes(const T* __restrict__ node_w, const T* __restrict__ node_b,
                              __nv_bfloat16* __restrict__ img, float* __restrict__ bimg,
-                             int L0, int k, int NP, int D)
+                             int L0, int k, int NP, int D, int Dp)
 {
     const int64_t groups = (int64_t)1 << L0;
-    const int64_t total = groups * NP * D;
+    const int64_t total = groups * NP * Dp;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int kk = (int)(i % D);
-        const int n = (int)((i / D) % NP);
-        const int64_t g = i / ((int64_t)D * NP);
+        const int kk = (int)(i % Dp);
+        const int n = (int)((i / Dp) % NP);
+        const int64_t g = i / ((int64_t)Dp * NP);
         int r = 0;
         while (((1 << (r + 1)) - 1) <= n) ++r;                 // level of local node n inside the subtree
         const bool used = r < k;
@@ -73,8 +74,8 @@ __global__ void k_pack_nodes(const T* __restrict__ node_w, const T* __restrict__
         const int64_t row = used ? (((int64_t)1 << (L0 + r)) - 1 + g * ((int64_t)1 << r) + p) : 0;
         const int u = kk / kKS, sb = (kk % kKS) / 64, kc = kk % 64;
         const uint32_t off = ptx::swz128((uint32_t)((sb * NP + n) * 128 + kc * 2));
-        const int64_t base = (g * (D / kKS) + u) * (int64_t)(NP * kKS);
-        img[base + off / 2] = __float2bfloat16_rn(used ? Elem<T>::to_float(node_w[row * D + kk]) : 0.0f);
+        const int64_t base = (g * (Dp / kKS) + u) * (int64_t)(NP * kKS);
+        img[base + off / 2] = __float2bfloat16_rn(used && kk < D ? Elem<T>::to_float(node_w[row * D + kk]) : 0.0f);
         if (kk == 0) bimg[g * NP + n] = used ? Elem<T>::to_float(node_b[row]) : 0.0f;
     }
 }
@@ -87,7 +88,7 @@ k_descent_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ p
               const Tile* __restrict__ tiles, int n_tiles_total,
               const __nv_bfloat16* __restrict__ wimg, const float* __restrict__ bimg,
               int32_t* __restrict__ pos_out,
-              int D, int B, int k, int kStages, int resident, int* __restrict__ status)
+              int D, int Dp, int B, int k, int kStages, int resident, int* __restrict__ status)
 {
     using L = DescentMmaLayout<NP>;
     constexpr int kTM = kDTM;
@@ -103,7 +104,7 @@ k_descent_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ p
     unsigned char* wres = reinterpret_cast<unsigned char*>(full) + 256;  // resident weight image
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int U1 = D / kKS;
+    const int U1 = Dp / kKS;
     const int ntiles = n_tiles_total;      // a device-built list may contain empty tiles (rows = 0)
 
     if (threadIdx.x == 0) {
@@ -118,8 +119,8 @@ k_descent_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ p
     __syncthreads();
     pdl_wait();
     if (resident && threadIdx.x == 0) {
-        ptx::mbar_arrive_expect_tx(wbar, (uint32_t)(NP * D * 2));
-        for (int u = 0; u < D / kKS; ++u)
+        ptx::mbar_arrive_expect_tx(wbar, (uint32_t)(NP * Dp * 2));
+        for (int u = 0; u < U1; ++u)
             ptx::bulk_g2s(wres + u * L::kWStageBytes, wimg + (int64_t)u * (NP * kKS), L::kWStageBytes, wbar);
     }
 
@@ -166,9 +167,15 @@ k_descent_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ p
                                       full + stage);
                     }
                 }
+if (u * kKS + pchunk * 8 < D) {
 #pragma unroll
-                for (int i = 0; i < kTM / kRowsPerPass; ++i)
-                    if (src[i]) ptx::cp_async16(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, src[i] + u * kKS);
+                    for (int i = 0; i < kTM / kRowsPerPass; ++i)
+                        if (src[i]) ptx::cp_async16(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, src[i] + u * kKS);
+                } else {                                   // padding columns (last stage only)
+#pragma unroll 1
+                    for (int i = 0; i < kTM / kRowsPerPass; ++i)
+                        ptx::cp_async16_zero(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, x);
+                }
                 ptx::cp_async_mbar_arrive(full + stage);
                 if (++stage == kStages) { stage = 0; phase ^= 1; }
             }

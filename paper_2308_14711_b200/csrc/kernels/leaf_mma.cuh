@@ -13,14 +13,14 @@
 // fragment of GEMM2).
 //
 // Ring contents, in order, per tile:
-//   D/kKS   GEMM1 stages: kKS columns of the gathered token rows (16-byte cp.async, rows padded by
+//   Dp/kKS  GEMM1 stages: kKS columns of the gathered token rows (16-byte cp.async, rows padded by
 //           16 bytes in shared memory so that ldmatrix is conflict-free) + the matching slice of W1_j
 //           (one bulk copy of a pre-swizzled image);
 //   O/kNC   GEMM2 stages: kNC rows of W2_j (pre-swizzled image) followed by their float32 biases.
 // The images are written once at handle creation (repack kernels below).
 //
-// Requirements: bf16, D % kKS == 0, O % 8 == 0, l <= 64 (padded to kLP in {16, 32, 64} with zero
-// weights: act(0) * 0 contributes nothing).
+// Requirements: bf16, D % 8 == 0 (padded to Dp, a multiple of kKS, with zero columns), O % 8 == 0, l <= 64 (padded to
+// kLP in {16, 32, 64} with zero weights: act(0) * 0 contributes nothing).
 #pragma once
 
 #include "common.cuh"
@@ -69,19 +69,19 @@ template <int LP, int TM, int S> struct LeafMmaLayout {
 
 // ---- one-time repacking of the leaf parameters into stage images --------------------------------
 
-// W1 image: [leaf][D/kKS stages][kKS/64 sub-blocks][LP rows][64 columns], 128-byte swizzled.
+// W1 image: [leaf][Dp/kKS stages][kKS/64 sub-blocks][LP rows][64 columns], 128-byte swizzled.
 template <typename T>
-__global__ void k_pack_w1(const T* __restrict__ w1, __nv_bfloat16* __restrict__ img, int n_leaves, int l, int LP, int D)
+__global__ void k_pack_w1(const T* __restrict__ w1, __nv_bfloat16* __restrict__ img, int n_leaves, int l, int LP, int D, int Dp)
 {
-    const int64_t total = (int64_t)n_leaves * LP * D;
+    const int64_t total = (int64_t)n_leaves * LP * Dp;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(i % D);
-        const int n = (int)((i / D) % LP);
-        const int64_t j = i / ((int64_t)D * LP);
+        const int k = (int)(i % Dp);
+        const int n = (int)((i / Dp) % LP);
+        const int64_t j = i / ((int64_t)Dp * LP);
         const int u = k / kKS, sb = (k % kKS) / 64, kc = k % 64;
         const uint32_t off = ptx::swz128((uint32_t)((sb * LP + n) * 128 + kc * 2));
-        const int64_t base = (j * (D / kKS) + u) * (int64_t)(LP * kKS);          // elements
-        const float v = n < l ? Elem<T>::to_float(w1[(j * l + n) * (int64_t)D + k]) : 0.0f;
+        const int64_t base = (j * (Dp / kKS) + u) * (int64_t)(LP * kKS);          // elements
+        const float v = n < l && k < D ? Elem<T>::to_float(w1[(j * l + n) * (int64_t)D + k]) : 0.0f;
         img[base + off / 2] = __float2bfloat16_rn(v);
     }
 }
@@ -131,7 +131,7 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
            const Tile* __restrict__ tiles, int n_tiles_total,
            const __nv_bfloat16* __restrict__ w1img, const float* __restrict__ b1img,
            const unsigned char* __restrict__ w2img, __nv_bfloat16* __restrict__ y,
-           int D, int O, int act, int* __restrict__ status)
+           int D, int Dp, int O, int act, int* __restrict__ status)
 {
     using L = LeafMmaLayout<LP, TM, S>;
     constexpr int kStages = S;
@@ -146,7 +146,7 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
     uint64_t* empty = full + kStages;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int U1 = D / kKS;
+    const int U1 = Dp / kKS;
     const int U2 = (O + kNC - 1) / kNC;
     const int ntiles = n_tiles_total;      // the list may contain empty tiles (rows = 0)
 
@@ -186,9 +186,15 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
                     ptx::bulk_g2s(st + kTM * kXRowBytes, w1img + ((int64_t)tl.bin * U1 + u) * (LP * kKS), L::kW1StageBytes,
                                   full + stage);
                 }
+if (u * kKS + pchunk * 8 < D) {
 #pragma unroll
-                for (int i = 0; i < kTM / kRowsPerPass; ++i)
-                    if (src[i]) ptx::cp_async16(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, src[i] + u * kKS);
+                    for (int i = 0; i < kTM / kRowsPerPass; ++i)
+                        if (src[i]) ptx::cp_async16(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, src[i] + u * kKS);
+                } else {                                   // padding columns (last stage only)
+#pragma unroll 1
+                    for (int i = 0; i < kTM / kRowsPerPass; ++i)
+                        ptx::cp_async16_zero(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, x);
+                }
                 ptx::cp_async_mbar_arrive(full + stage);
                 if (++stage == kStages) { stage = 0; phase ^= 1; }
             }

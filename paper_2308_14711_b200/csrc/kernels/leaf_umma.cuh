@@ -40,7 +40,10 @@
 //
 // Every wait is bounded (see ptx.cuh); tensor memory is released on every exit path.
 //
-// Requirements: bf16, D % 128 == 0, O % 16 == 0, l <= 64 (padded to LP in {16, 32, 64}), x 16-byte aligned.
+// D is the padded inner dimension of the images (a multiple of 128): columns past the rows of x are outside its tensor
+// map and read as zeros, and have zero weights.
+//
+// Requirements: bf16, rows of x of a multiple of 8 columns, O % 16 == 0, l <= 64 (padded to LP in {16, 32, 64}), x 16-byte aligned.
 #pragma once
 
 #include <cuda.h>      // CUtensorMap
@@ -145,7 +148,7 @@ __global__ void k_pack_w2_umma(const T* __restrict__ w2, const T* __restrict__ b
 }
 
 // Images for grouped tiles (kLUGroup = 8 leaves per tile): bin g is node g of level depth - 3, N1 = 8 LP + 16.
-//   w1g  [bin][D / 64][N1 rows][64 columns] 128-byte swizzled: row j LP + u = hidden unit u of leaf 8 g + j (zero for
+//   w1g  [bin][Dp / 64][N1 rows][64 columns] 128-byte swizzled: row j LP + u = hidden unit u of leaf 8 g + j (zero for
 //        u >= l); rows 8 LP + q, q < 7: node q of the subtree below node g, breadth-first; the other rows zero;
 //   g1b  [bin][N1] float32: the biases of those rows;
 //   w2g  [bin][ceil(O / 128) pieces]{ 2 K-blocks of [128 rows (output features)][64 columns] 128-byte swizzled, then 128
@@ -156,7 +159,7 @@ template <typename T>
 __global__ void k_pack_leaf_groups(const T* __restrict__ w1, const T* __restrict__ b1, const T* __restrict__ w2, const T* __restrict__ b2,
                                    const T* __restrict__ node_w, const T* __restrict__ node_b, __nv_bfloat16* __restrict__ w1g,
                                    float* __restrict__ g1b, unsigned char* __restrict__ w2g, int n_bins, int depth, int l, int LP, int D,
-                                   int O)
+                                   int Dp, int O)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int HC = kLUGroup * LP, N1 = HC + 16;
@@ -165,17 +168,17 @@ __global__ void k_pack_leaf_groups(const T* __restrict__ w1, const T* __restrict
         const int r = q == 0 ? 0 : q < 3 ? 1 : 2;
         return (((int64_t)1 << (depth - 3 + r)) - 1) + (g << r) + (q - ((1 << r) - 1));
     };
-    for (int64_t i = t0; i < (int64_t)n_bins * N1 * D; i += stride) {
-        const int k = (int)(i % D), n = (int)((i / D) % N1);
-        const int64_t g = i / ((int64_t)D * N1);
+    for (int64_t i = t0; i < (int64_t)n_bins * N1 * Dp; i += stride) {
+        const int k = (int)(i % Dp), n = (int)((i / Dp) % N1);
+        const int64_t g = i / ((int64_t)Dp * N1);
         float v = 0.0f;
         if (n < HC) {
             const int j = n / LP, u = n % LP;
-            if (u < l) v = Elem<T>::to_float(w1[((g * kLUGroup + j) * l + u) * (int64_t)D + k]);
-        } else if (n - HC < 7) {
+            if (u < l && k < D) v = Elem<T>::to_float(w1[((g * kLUGroup + j) * l + u) * (int64_t)D + k]);
+        } else if (n - HC < 7 && k < D) {
             v = Elem<T>::to_float(node_w[node_of(g, n - HC) * D + k]);
         }
-        const int64_t base = (g * (D / kLUKB) + k / kLUKB) * (int64_t)(N1 * kLUKB);       // elements
+        const int64_t base = (g * (Dp / kLUKB) + k / kLUKB) * (int64_t)(N1 * kLUKB);       // elements
         w1g[base + ptx::swz128((uint32_t)(n * 128 + (k % kLUKB) * 2)) / 2] = __float2bfloat16_rn(v);
     }
     for (int64_t i = t0; i < (int64_t)n_bins * N1; i += stride) {

@@ -94,6 +94,11 @@ __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src_gmem)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem) : "memory");
 }
 
+// 16 zero bytes into shared memory, in order with the copies above (`any` is a valid address that is not read).
+__device__ __forceinline__ void cp_async16_zero(void* dst_smem, const void* any) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, 0;" ::"r"(smem_addr(dst_smem)), "l"(any) : "memory");
+}
+
 // Arrive on `bar` once all cp.async copies issued so far by this thread have landed.  The arrival is
 // one of the barrier's expected arrivals (.noinc), so the init count must include every such thread.
 __device__ __forceinline__ void cp_async_mbar_arrive(uint64_t* bar) {
