@@ -77,7 +77,7 @@ typedef enum {
     FFF_PATH_AUTO = 0,           /* library picks per stage from shapes and B */
     FFF_PATH_WARP = 1,           /* CUDA-core warp kernels for descent and leaf evaluation */
     FFF_PATH_TENSOR = 2,         /* tensor-core kernels wherever the shapes allow them */
-    FFF_PATH_FUSED = 3           /* the one-launch kernel for small trees with leaves of at most 32 neurons */
+    FFF_PATH_FUSED = 3           /* the one-launch kernel on CUDA cores (small trees with leaves of at most 32 neurons) */
 } fff_path_t;
 
 /*
@@ -198,9 +198,9 @@ typedef enum {
     FFF_TUNE_CTA_PAIRS = 3,       /* first descent stage with 128 or 256 nodes on pairs of CTAs (0: single CTAs) */
     FFF_TUNE_DIRECT_LISTS = 4,    /* descent stages file the tokens under the nodes / leaves they reach, for the kernel
                                      that follows (0: bucketing kernels) */
-    FFF_TUNE_FUSED_SMALL = 5,     /* small trees with thin leaves in one launch: descent, grid barrier, leaf evaluation
-                                     by groups of 32 hidden neurons kept in shared memory (0: descent, bucketing and
-                                     leaf kernels).  Taken by default by layers without a tensor-core leaf path */
+    FFF_TUNE_FUSED_SMALL = 5,     /* one launch on CUDA cores: descent, grid barrier, leaves by tiles of 16 tokens (0: descent,
+                                     bucketing and leaf kernels).  Taken by default by layers without a tensor-core
+                                     leaf path and at most 4096 leaves */
     FFF_TUNE_GROUP_TILES = 6,     /* leaf kernel tiles of tokens that share the node three levels above the leaves: the
                                      first descent stage stops there, the leaf kernel walks the last three levels from
                                      7 extra accumulator columns and evaluates the node's 8 leaves side by side, each
@@ -208,7 +208,10 @@ typedef enum {
                                      layers with 8 <= leaf_width < 16 and 9 <= depth <= 11 (where it replaces the
                                      second descent stage and its node bucketing), when those nodes receive at least
                                      128 tokens each on average */
-    FFF_TUNE_COUNT = 7
+    FFF_TUNE_TOKEN_BLOCKS = 7,    /* a few tokens: one launch in which one CTA takes one token through the tree and its leaf
+                                     (0: the kernels of larger batches).  Taken by default while the weights that the
+                                     tokens fetch one by one stay small */
+    FFF_TUNE_COUNT = 8
 } fff_tuning_t;
 fff_status_t fff_set_tuning(fff_handle_t h, fff_tuning_t key, int value);
 

@@ -22,7 +22,8 @@ STATUS_NAMES = {0: "FFF_OK", 1: "FFF_ERR_INVALID_ARG", 2: "FFF_ERR_UNSUPPORTED",
 ACTIVATIONS = {"relu": 0, "gelu": 1, "gelu_tanh": 2, "silu": 3}
 DTYPES = {"f32": 0, "bf16": 1}
 PATHS = {"auto": 0, "warp": 1, "tensor": 2, "fused": 3}
-TUNING = {"tcgen05_descent": 0, "tcgen05_grouped": 1, "tcgen05_leaf": 2, "cta_pairs": 3, "direct_lists": 4, "fused_small": 5, "group_tiles": 6}
+TUNING = {"tcgen05_descent": 0, "tcgen05_grouped": 1, "tcgen05_leaf": 2, "cta_pairs": 3, "direct_lists": 4, "fused_small": 5, "group_tiles": 6,
+          "token_blocks": 7}
 
 # every symbol include/fff.h declares
 EXPORTS = ["fff_create", "fff_create_w8", "fff_forward_infer", "fff_forward_train", "fff_forward_infer_host", "fff_destroy", "fff_reserve",
@@ -187,10 +188,19 @@ def _torch():
 def _ptr(t, dtype, shape, name):
     if t is None:
         return None
-    if not t.is_cuda or t.dtype != dtype or not t.is_contiguous() or tuple(t.shape) != tuple(shape):
+    if not t.is_cuda or t.dtype != dtype or not t.is_contiguous() or t.shape != shape:
         raise ValueError(f"{name}: expected contiguous CUDA {dtype} tensor of shape {tuple(shape)}, "
                          f"got {t.dtype} {tuple(t.shape)} on {t.device}")
     return t.data_ptr()
+
+
+def _stream_ptr(stream=None):
+    """cudaStream_t of `stream`, by default the current stream of the current device (asked for as a number: making the
+    stream object first costs more than a kernel launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    c = _torch()._C
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
 
 
 class FFFLayer:
@@ -221,6 +231,7 @@ class FFFLayer:
                                  _ptr(node_w, td, (nn, D), "node_w"), _ptr(node_b, td, (nn,), "node_b"),
                                  _ptr(w1, td, (nl, leaf_width, D), "w1"), _ptr(b1, td, (nl, leaf_width), "b1"),
                                  _ptr(w2, td, (nl, O, leaf_width), "w2"), _ptr(b2, td, (nl, O), "b2"))
+        self._forward = lib().fff_forward_infer
         if path != "auto":
             self.set_path(path)
 
@@ -240,8 +251,7 @@ class FFFLayer:
             pass
 
     def _stream(self, stream):
-        s = stream if stream is not None else _torch().cuda.current_stream()
-        return s.cuda_stream
+        return _stream_ptr(stream)
 
     def reserve(self, max_B: int) -> None:
         fff_reserve(self._h, max_B)
@@ -258,14 +268,25 @@ class FFFLayer:
         fff_set_tuning(self._h, TUNING[key], 1 if on else 0)
 
     def forward_infer(self, x, y=None, leaf_idx=None, want_leaf_idx: bool = True, stream=None):
-        torch = _torch()
+        i32 = _torch().int32
+        td = self.tdtype
         B = x.shape[0]
+        xp = _ptr(x, td, (B, self.D), "x")
         if y is None:
-            y = torch.empty((B, self.O), dtype=self.tdtype, device=x.device)
-        if leaf_idx is None and want_leaf_idx:
-            leaf_idx = torch.empty((B,), dtype=torch.int32, device=x.device)
-        fff_forward_infer(self._h, _ptr(x, self.tdtype, (B, self.D), "x"), _ptr(y, self.tdtype, (B, self.O), "y"),
-                          _ptr(leaf_idx, torch.int32, (B,), "leaf_idx"), B, self._stream(stream))
+            y = x.new_empty((B, self.O))
+            yp = y.data_ptr()
+        else:
+            yp = _ptr(y, td, (B, self.O), "y")
+        if leaf_idx is None:
+            lp = None
+            if want_leaf_idx:
+                leaf_idx = x.new_empty((B,), dtype=i32)
+                lp = leaf_idx.data_ptr()
+        else:
+            lp = _ptr(leaf_idx, i32, (B,), "leaf_idx")
+        status = self._forward(self._h, xp, yp, lp, B, _stream_ptr(stream))
+        if status:
+            raise FFFError(status, "fff_forward_infer")
         return y, leaf_idx
 
     def forward_train(self, x, want_mixture: bool = True, want_entropy: bool = True, stream=None):
@@ -383,7 +404,7 @@ class FFFStack:
             y = torch.empty((B, self.D), dtype=self.tdtype, device=x.device)
         if leaf_idx is None and want_leaf_idx:
             leaf_idx = torch.empty((len(self.layers), B), dtype=torch.int32, device=x.device)
-        st = (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
+        st = _stream_ptr(stream)
         _check(lib().fff_stack_forward(self._s, _ptr(x, self.tdtype, (B, self.D), "x"), _ptr(y, self.tdtype, (B, self.D), "y"),
                                        _ptr(leaf_idx, torch.int32, (len(self.layers), B), "leaf_idx"), B, st), "fff_stack_forward")
         return y, leaf_idx

@@ -15,17 +15,18 @@
 #include <set>
 #include <vector>
 
+#include "kernels/block_forward.cuh"
 #include "kernels/bucket.cuh"
 #include "kernels/common.cuh"
 #include "kernels/descent_mma.cuh"
 #include "kernels/descent_umma.cuh"
 #include "kernels/descent_warp.cuh"
-#include "kernels/fused_small.cuh"
 #include "kernels/gemm_umma.cuh"
 #include "kernels/leaf_mma.cuh"
 #include "kernels/leaf_umma.cuh"
 #include "kernels/leaf_warp.cuh"
 #include "kernels/stack.cuh"
+#include "kernels/token_block.cuh"
 
 namespace {
 
@@ -95,7 +96,7 @@ struct fff_handle_s {
     // direct lists (slot_tokens in descent_umma.cuh): when one tcgen05 stage is the whole descent and the tcgen05
     // leaf kernel follows, the descent files every token under its leaf itself and no bucketing kernel runs
     int32_t* ws_slots = nullptr;     // [n_leaves][slot_cap] token numbers
-    int32_t* ws_cursor = nullptr;    // [n_leaves] entries used; zero between calls (the leaf kernel clears it)
+    int32_t* ws_cursor = nullptr;    // [n_leaves] entries used (+ [1] finished CTAs of k_block_forward); zero between calls
     int64_t slot_cap = 0;
     bool cursor_dirty = false;       // a descent has filled the lists and no leaf kernel has cleared the counts since
     bool slots_now = false;          // the call in progress uses the direct lists
@@ -108,9 +109,10 @@ struct fff_handle_s {
     int32_t* ws_perm2 = nullptr;  // second permutation buffer: successive bucketings alternate between the two
     int32_t* ws_offsets2[2] = {nullptr, nullptr};   // offsets of the intermediate (node) bucketings
 
-    // one-launch forward for small trees with thin leaves (fused_small.cuh); fs_batch == 0: shapes not eligible
-    float *fs_w1g = nullptr, *fs_b1g = nullptr, *fs_w2g = nullptr, *fs_b2f = nullptr;
-    int fs_G = 0, fs_lp = 0, fs_Dp = 0, fs_batch = 0;
+    // one-launch forward on CUDA cores (block_forward.cuh): its CTAs per SM (0: shapes not eligible), and whether the layer
+    // may be pinned to it (FFF_PATH_FUSED)
+    int bf_per_sm = 0;
+    bool bf_pinnable = false;
 
     // FORWARD_T (fff_forward_train): transposed output weights with the output biases appended along K, and the
     // workspace of the three GEMMs (allocated on first use)
@@ -119,6 +121,7 @@ struct fff_handle_s {
     float* tr_b1t = nullptr;
     __nv_bfloat16* tr_wn = nullptr;      // node weights in the order of k_train_nodes' columns (1 <= depth <= 8), and their biases
     float* tr_bn = nullptr;
+    bool tr_packed = false;              // the images below exist
     int tr_Kp = 0;                       // 2^d l + 2^d rounded up to 64 (0 = shapes not eligible)
     int64_t tr_cap_B = 0;
     float *tr_c = nullptr, *tr_mix = nullptr, *tr_entpart = nullptr;
@@ -148,7 +151,7 @@ struct fff_handle_s {
     cudaEvent_t ev_in[kMaxHostChunks] = {}, ev_done[kMaxHostChunks] = {}, ev_start = nullptr, ev_end = nullptr;
 
     int path = FFF_PATH_AUTO;
-    bool tune[FFF_TUNE_COUNT] = {true, true, true, true, true, true, true};      // fff_set_tuning; every switch defaults to on
+    bool tune[FFF_TUNE_COUNT] = {true, true, true, true, true, true, true, true};      // fff_set_tuning; every switch defaults to on
     bool pdl = true;              // launch every kernel of a forward but the first as a programmatic dependent
     int launches = 0;
     int64_t last_B = -1;
@@ -272,7 +275,6 @@ void release(fff_handle_s* h) {
     for (auto& sg : h->gstages) { dfree(sg.wimg); dfree(sg.bimg); }
     dfree(h->g_w1); dfree(h->g_b1); dfree(h->g_w2);
     dfree(h->ws_pos[0]); dfree(h->ws_pos[1]);
-    dfree(h->fs_w1g); dfree(h->fs_b1g); dfree(h->fs_w2g); dfree(h->fs_b2f);
     dfree(h->w1codes); dfree(h->w2codes); dfree(h->scale1); dfree(h->scale2);
     dfree(h->tr_w2t); dfree(h->tr_w1t); dfree(h->tr_b1t); dfree(h->tr_wn); dfree(h->tr_bn); dfree(h->tr_c); dfree(h->tr_mix); dfree(h->tr_entpart); dfree(h->tr_hp);
     dfree(h->w1img); dfree(h->b1img); dfree(h->w2img); dfree(h->w2uimg); dfree(h->ws_sched); dfree(h->ws_tiles); dfree(h->ws_rank); dfree(h->ws_rank8); dfree(h->ws_counts8); dfree(h->ws_blocksum); dfree(h->ws_matrix); dfree(h->ws_slots); dfree(h->ws_cursor); dfree(h->ws_nslots); dfree(h->ws_ncursor);
@@ -371,10 +373,12 @@ fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
     if ((s = dmalloc((void**)&h->ws_tiles, sizeof(fff::Tile) * max_tiles(h, B))) != FFF_OK) return s;
     // direct lists: every leaf's list can take the whole batch, so their size grows with n_leaves * B; beyond
     // kMaxSlotBytes the forward keeps the bucketing kernel instead
-    if (!h->ustages.empty() && h->ustages.back().umma && h->ustages.back().L0 + h->ustages.back().k == h->depth && (h->w2uimg || h->w2codes) &&
+    const bool filed_by_descent = !h->ustages.empty() && h->ustages.back().umma &&
+                                  h->ustages.back().L0 + h->ustages.back().k == h->depth && (h->w2uimg || h->w2codes);
+    if ((filed_by_descent || (h->bf_per_sm > 0 && (h->LP == 0 || h->bf_pinnable))) &&
         (size_t)h->n_leaves * (size_t)B * sizeof(int32_t) <= kMaxSlotBytes) {
         if ((s = dmalloc((void**)&h->ws_slots, sizeof(int32_t) * (size_t)h->n_leaves * (size_t)B)) != FFF_OK) return s;
-        if ((s = clone((void**)&h->ws_cursor, nullptr, sizeof(int32_t) * (size_t)h->n_leaves)) != FFF_OK) return s;
+        if ((s = clone((void**)&h->ws_cursor, nullptr, sizeof(int32_t) * (size_t)(h->n_leaves + 1))) != FFF_OK) return s;
         h->slot_cap = B;
         h->cursor_dirty = false;
     }
@@ -726,6 +730,10 @@ int dense_stage_count(const fff_handle_s* h, int64_t B) {
     const auto& plan = stage_plan(h);
     if (plan.empty() || h->path == FFF_PATH_WARP) return 0;
     if (h->path == FFF_PATH_TENSOR) return (int)plan.size();
+    // Thin leaves that are evaluated token by token anyway: up to 8192 tokens the leaf kernel's own walk through all levels
+    // beats two stages, a node bucketing and the walk through the rest (600 columns, 14 levels: 18 against 21 us at 1024
+    // tokens, 21 against 36 at 4096; at 16 384 73 against 56).
+    if (!use_tensor_leaf(h) && B < 4 * h->n_leaves && B <= 8192) return 0;
     int n = 0;
     for (const auto& sg : plan) {
         if ((B >> sg.L0) < 16) break;
@@ -1041,7 +1049,7 @@ bool use_group_tiles(const fff_handle_s* h, int64_t B) {
 fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_t* leaf, int64_t B, cudaStream_t st) {
     using L = fff::LeafUmmaLayout<16, false, fff::kLUGroup>;
     const int bins = (int)(h->n_leaves / fff::kLUGroup);
-    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)h->n_leaves, st) != cudaSuccess)
+    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     h->cursor_dirty = true;
     h->blocksum_wanted = false;
@@ -1072,75 +1080,123 @@ fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_
     return s;
 }
 
-// The one-launch kernel for small trees: eligibility and its weight images (at creation).
+// The one-launch kernel on CUDA cores: eligibility (at creation).
+size_t block_forward_smem(const fff_handle_s* h) {
+    return sizeof(int) * (size_t)((h->n_leaves + 1 + 3) & ~(int64_t)3) + sizeof(float) * (size_t)h->l * fff::kBFTile;
+}
+
 template <typename T>
-fff_status_t pack_fused_small(fff_handle_s* h) {
-    if (h->l > 32 || h->coop_ctas <= 0) return FFF_OK;
+fff_status_t plan_block_forward(fff_handle_s* h) {
+    const size_t smem = block_forward_smem(h);
+    if (h->coop_ctas <= 0 || h->n_leaves > fff::kBFMaxLeaves || smem > 96 * 1024) return FFF_OK;
+    static bool raised[2][kMaxDevices] = {};
+    if (!raise_smem_limit(fff::k_block_forward<T, 1>, h->device, 96 * 1024, raised[0]) ||
+        !raise_smem_limit(fff::k_block_forward<T, 4>, h->device, 96 * 1024, raised[1]))
+        return FFF_ERR_CUDA;
+    int n1 = 0, n4 = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fff::k_block_forward<T, 1>, fff::kBFThreads, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n4, fff::k_block_forward<T, 4>, fff::kBFThreads, smem) != cudaSuccess)
+        return cudaGetLastError(), FFF_OK;
+    h->bf_per_sm = std::min(2, std::min(n1, n4));
+    // layers that can be pinned to it: small trees with thin leaves
     int lp = 1;
     while (lp < h->l) lp <<= 1;
-    const int64_t G = (h->n_leaves * lp + 31) / 32;
-    if (G > h->sm_count) return FFF_OK;
-    const int Dp = (h->D + 3) & ~3;
-    int batch = fff::kFSMaxBatch;
-    while (batch >= 8 && fff::FusedSmallLayout{Dp, h->O, batch}.total() > (size_t)kSmemBudget) batch >>= 1;
-    if (batch < 8) return FFF_OK;
-    fff_status_t s;
-    if ((s = dmalloc((void**)&h->fs_w1g, sizeof(float) * (size_t)G * 32 * Dp)) != FFF_OK) return s;
-    if ((s = dmalloc((void**)&h->fs_b1g, sizeof(float) * (size_t)G * 32)) != FFF_OK) return s;
-    if ((s = dmalloc((void**)&h->fs_w2g, sizeof(float) * (size_t)G * h->O * 32)) != FFF_OK) return s;
-    if ((s = dmalloc((void**)&h->fs_b2f, sizeof(float) * (size_t)h->n_leaves * h->O)) != FFF_OK) return s;
-    fff::k_pack_fused_small<T><<<h->sm_count * 8, 256>>>((const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, h->fs_w1g,
-                                                        h->fs_b1g, h->fs_w2g, h->fs_b2f, (int)h->n_leaves, h->l, lp, h->D, Dp, h->O,
-                                                        (int)G);
-    if (cudaGetLastError() != cudaSuccess) return FFF_ERR_CUDA;
-    if (cudaFuncSetAttribute(fff::k_fused_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) != cudaSuccess)
-        return cudaGetLastError(), FFF_ERR_CUDA;
-    h->fs_G = (int)G;
-    h->fs_lp = lp;
-    h->fs_Dp = Dp;
-    h->fs_batch = batch;
+    const int64_t Dr = (h->D + 3) & ~3, rows = std::max<int64_t>(Dr, 512);
+    h->bf_pinnable = h->bf_per_sm > 0 && h->l <= 32 && (h->n_leaves * lp + 31) / 32 <= h->sm_count &&
+                     128 * Dr + 256 * (int64_t)h->O + 32 * rows + 5432 <= kSmemBudget;
     return FFF_OK;
 }
 
-// Whether a forward of this handle runs as the one-launch kernel: when pinned to it, or by default for layers
-// that have no tensor-core leaf path (float32, or bf16 shapes outside it) and room for batches of at least 8.
-// Layers whose tensor-core images are padded: a few tokens through a narrow layer (136 -> 128, 16 leaves of 16: 13-15 us
-// against 19-20 us up to 64 tokens, 17.5 against 12.7 at 256; 264 -> 256 is level at one token and behind from 16 on).
-bool use_fused_small(const fff_handle_s* h, int64_t B) {
-    if (h->fs_batch == 0 || !h->tune[FFF_TUNE_FUSED_SMALL]) return false;
+// Whether a forward of this handle runs as the one-launch kernel: when pinned to it, or by default for layers that have no
+// tensor-core leaf path (float32, or bf16 shapes outside it); the table of the leaves' token lists must fit.  Measured
+// against what it replaces, one warp per token (three launches) or, for small trees, a kernel that kept 32 hidden neurons
+// per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44 against 110 us; 1000 -> 992, 512 leaves
+// of 32, 8192 tokens 156 against 1148; 512 -> 512, 32 leaves of 16, 8192 tokens 32 against 429; 784 -> 10, 8 leaves of 32,
+// 2048 tokens 18 against 20.  CTAs per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
+bool use_block_forward(const fff_handle_s* h, int64_t B) {
+    if (h->bf_per_sm == 0 || !h->tune[FFF_TUNE_FUSED_SMALL] || !h->ws_slots || B > h->slot_cap) return false;
     if (h->path == FFF_PATH_FUSED) return true;
-    if (h->path != FFF_PATH_AUTO || h->fs_batch < 8) return false;
-    return h->LP == 0 || (h->D != h->Dp && h->D <= 256 && B <= 64);
+    return h->path == FFF_PATH_AUTO && h->LP == 0;
 }
 
 template <typename T>
-fff_status_t run_fused_small(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B,
-                             cudaStream_t st) {
-    const int G = h->fs_G, S = std::max(1, h->sm_count / G);
-    const fff::FusedSmallLayout L{h->fs_Dp, h->O, h->fs_batch};
-    const T* xp = (const T*)x;
-    const T *nw = (const T*)h->node_w, *nb = (const T*)h->node_b;
-    const float *w1g = h->fs_w1g, *b1g = h->fs_b1g, *w2g = h->fs_w2g, *b2f = h->fs_b2f;
-    T* yp = (T*)y;
-    int D = h->D, Dp = h->fs_Dp, O = h->O, depth = h->depth, l = h->l, lp = h->fs_lp, act = h->act, Bi = (int)B, Gi = G,
-        batch = h->fs_batch, vec = h->vec_ok && aligned16(x) ? 1 : 0, nl = (int)h->n_leaves;
-    int* status = h->d_status;
-    void* args[] = {&xp, &nw, &nb, &w1g, &b1g, &w2g, &b2f, &yp, &leaf_out, &leaf_out2, &D, &Dp, &O, &depth, &l, &lp, &act, &Bi,
-                    &Gi, &batch, &vec, &nl, &status};
-    if (cudaLaunchCooperativeKernel((const void*)fff::k_fused_small<T>, dim3((unsigned)(G * S)), dim3(fff::kFSThreads), args,
-                                    L.total(), st) != cudaSuccess)
+fff_status_t run_block_forward(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B,
+                               cudaStream_t st) {
+    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
-    return launched(h, st, "fused_forward_small");
+    h->cursor_dirty = true;
+    // (one: 2048 tokens of 768 columns keep 14 warps per SM busy instead of 3.5; four: a quarter of the node rows' traffic)
+    const bool single = B <= (int64_t)h->sm_count * 2 * fff::kBFWarps * 2;      // one token per warp in the descent
+    const int64_t max_ctas = (int64_t)h->sm_count * h->bf_per_sm;
+    const int64_t grid = std::min(max_ctas, std::max<int64_t>(B, 1));
+    // thinner tiles while full ones would leave CTAs without work, unless the leaves are thin themselves
+    const int tile_rows = B <= 8 * max_ctas && B >= 32 * h->n_leaves ? 8 : fff::kBFTile;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(fff::kBFThreads);
+    cfg.dynamicSmemBytes = block_forward_smem(h);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = h->pdl && !h->prof_active ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, single ? fff::k_block_forward<T, 1> : fff::k_block_forward<T, 4>, (const T*)x, (const T*)h->node_w,
+                           (const T*)h->node_b, (const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, (T*)y, leaf_out, leaf_out2,
+                           h->ws_slots, h->ws_cursor, (int)h->slot_cap, h->D, h->O, h->depth, h->l, h->act, (int)B,
+                           h->vec_ok && aligned16(x), (int)h->n_leaves, tile_rows) != cudaSuccess)
+        return cudaGetLastError(), FFF_ERR_CUDA;
+    const fff_status_t s = launched(h, st, "fused_forward_blocks");
+    if (s == FFF_OK) h->cursor_dirty = false;
+    return s;
 }
 
-// FORWARD_T: the weight images of the GEMMs (at creation).
+// Whether a forward of B tokens runs as one CTA per token.  While the CTAs of all tokens are resident at once (four per SM
+// with bf16) the launch takes one chain of latencies whatever B is, and the other paths take two to five such chains:
+// 768 -> 768, 256 leaves of 12, bf16: 7.4 us at one token, 8.5 at 197, 11.2 at 512 (three launches: 17.6, 19.0, 19.1);
+// float32 7.5 / 9.1 / 16.8 us (18 / 20 / 20).  Past that the weights fetched token by token cost more than the launches:
+// 1024 tokens 19.5 against 19.4 us, 2048 34.6 against 20.6.  Trees that the staged descent cuts in two would run five
+// launches on thin groups: 1024 -> 1024, 2048 leaves of 32: 43 against 68 us at 1024 tokens, 79 against 97 at 2048, 149
+// against 94 at 4096; 512 leaves of 8: 18.6 against 33 at 1024, level at 2048.
+constexpr int64_t kTokenBlockMaxB = 512, kTokenBlockMaxBDeep = 2048, kTokenBlockMaxBytes = (int64_t)96 << 20;
+
+bool use_token_block(const fff_handle_s* h, int64_t B) {
+    if (h->w8 || h->path != FFF_PATH_AUTO || !h->tune[FFF_TUNE_TOKEN_BLOCKS]) return false;
+    if (fff::TokenBlockLayout{h->D, h->l, (int)h->esize}.total() > 100 * 1024) return false;
+    const bool two_stages = use_tensor_leaf(h) && h->ustages.size() >= 2;
+    if (two_stages) return B <= std::max(kTokenBlockMaxB, std::min(kTokenBlockMaxBDeep, 2 * h->n_leaves));
+    const int full = h->depth / fff::kTBLevels, rest = h->depth % fff::kTBLevels;
+    const int64_t nodes = (int64_t)full * ((1 << fff::kTBLevels) - 1) + ((1 << rest) - 1);
+    const int64_t per_token = (nodes * h->D + (int64_t)h->l * (h->D + h->O)) * (int64_t)h->esize;
+    return B <= kTokenBlockMaxB && B * per_token <= kTokenBlockMaxBytes;
+}
+
+template <typename T>
+fff_status_t run_token_block(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B, cudaStream_t st) {
+    const size_t smem = fff::TokenBlockLayout{h->D, h->l, (int)h->esize}.total();
+    static bool limit_raised[kMaxDevices] = {};
+    if (smem > 48 * 1024 && !raise_smem_limit(fff::k_token_block<T>, h->device, 100 * 1024, limit_raised)) return FFF_ERR_CUDA;
+    if (launch_chain(h, fff::k_token_block<T>, (unsigned)B, fff::kTBThreads, smem, st, 1, (const T*)x, (const T*)h->node_w,
+                     (const T*)h->node_b, (const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, (T*)y, leaf_out, leaf_out2, h->D,
+                     h->O, h->depth, h->l, h->act, (int)B, h->vec_ok && aligned16(x)) != cudaSuccess)
+        return cudaGetLastError(), FFF_ERR_CUDA;
+    return launched(h, st, "forward_token_blocks");
+}
+
+// FORWARD_T: the weight images of the GEMMs.  Sizes at creation (tr_Kp; 0: shapes not eligible), the images with the first
+// call, like its workspace: layers that only infer do not pay for them.
 constexpr int kTrainMaxFusedDepth = 8;      // deepest tree whose node logits fit one tile of k_train_nodes
 
-fff_status_t pack_train_images(fff_handle_s* h) {
-    if (h->dtype != FFF_DTYPE_BF16 || h->D % fff::kGKB != 0 || !encode_tiled_fn()) return FFF_OK;
-    if (h->n_leaves * (h->l + 1) > (1 << 24)) return FFF_OK;
+void plan_train(fff_handle_s* h) {
+    if (h->dtype != FFF_DTYPE_BF16 || h->D % fff::kGKB != 0 || !encode_tiled_fn() || h->n_leaves * (h->l + 1) > (1 << 24)) return;
     const int hidden = fff::train_hidden_columns((int)h->n_leaves, h->l);
-    const int Kp = (int)((hidden + h->n_leaves + fff::kGKB - 1) / fff::kGKB * fff::kGKB);
+    h->tr_Kp = (int)((hidden + h->n_leaves + fff::kGKB - 1) / fff::kGKB * fff::kGKB);
+}
+
+fff_status_t pack_train_images(fff_handle_s* h) {
+    const int hidden = fff::train_hidden_columns((int)h->n_leaves, h->l), Kp = h->tr_Kp;
     const int padded = (hidden + 255) / 256 * 256, NP = std::max<int>(32, (int)h->n_leaves);
     const int blocks = h->sm_count * 8;
     const __nv_bfloat16 *w1 = (const __nv_bfloat16*)h->w1, *b1 = (const __nv_bfloat16*)h->b1;
@@ -1157,8 +1213,8 @@ fff_status_t pack_train_images(fff_handle_s* h) {
         fff::k_pack_train_nodes<__nv_bfloat16><<<blocks, 256>>>((const __nv_bfloat16*)h->node_w, (const __nv_bfloat16*)h->node_b, h->tr_wn,
                                                                h->tr_bn, h->depth, NP, h->D);
     }
-    if (cudaGetLastError() != cudaSuccess) return FFF_ERR_CUDA;
-    h->tr_Kp = Kp;
+    if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
+    h->tr_packed = true;
     return FFF_OK;
 }
 
@@ -1247,6 +1303,14 @@ fff_status_t run_train_nodes(fff_handle_s* h, const void* x, float* mix, float* 
 fff_status_t run_forward_train(fff_handle_s* h, const void* x, void* y, float* mixture, float* node_entropy, int64_t B,
                                cudaStream_t st) {
     const int64_t nl = h->n_leaves, nn = h->n_nodes, hidden = fff::train_hidden_columns((int)nl, h->l);
+    if (!h->tr_packed) {
+        // (a packing that failed half-way starts over)
+        dfree(h->tr_w2t); dfree(h->tr_w1t); dfree(h->tr_b1t); dfree(h->tr_wn); dfree(h->tr_bn);
+        h->tr_w2t = h->tr_w1t = h->tr_wn = nullptr;
+        h->tr_b1t = h->tr_bn = nullptr;
+        const fff_status_t ps = pack_train_images(h);
+        if (ps != FFF_OK) return ps;
+    }
     const bool fused = h->tr_wn != nullptr;
     const int ldc = (int)std::max<int64_t>((nn + 3) & ~(int64_t)3, 4);      // rows of c start on 16-byte boundaries
     const int64_t n_mt = (B + fff::kGRows - 1) / fff::kGRows;
@@ -1536,8 +1600,8 @@ fff_status_t create_common(fff_handle_t* out, int D, int O, int depth, int leaf_
         s = pack_leaf_images<__nv_bfloat16>(h);
     }
     if (s == FFF_OK && !w8 && h->w2uimg) s = pack_group_images<__nv_bfloat16>(h);
-    if (s == FFF_OK && !w8) s = FFF_DISPATCH(h, pack_fused_small, h);
-    if (s == FFF_OK && !w8) s = pack_train_images(h);
+    if (s == FFF_OK && !w8) s = FFF_DISPATCH(h, plan_block_forward, h);
+    if (s == FFF_OK && !w8) plan_train(h);
     if (s == FFF_OK && cudaDeviceSynchronize() != cudaSuccess) s = (cudaGetLastError(), FFF_ERR_CUDA);
     if (s != FFF_OK) { release(h); return s; }
     {
@@ -1591,7 +1655,7 @@ fff_status_t fff_set_path(fff_handle_t h, fff_path_t path) {
         return FFF_ERR_INVALID_ARG;
     // (pinning to the tensor-core kernels stays reserved to layers whose rows they take unpadded)
     if (path == FFF_PATH_TENSOR && ((h->LP == 0 && h->stages.empty()) || h->D != h->Dp)) return FFF_ERR_UNSUPPORTED;
-    if (path == FFF_PATH_FUSED && h->fs_batch == 0) return FFF_ERR_UNSUPPORTED;
+    if (path == FFF_PATH_FUSED && !h->bf_pinnable) return FFF_ERR_UNSUPPORTED;
     if (h->w8 && path != FFF_PATH_AUTO && path != FFF_PATH_TENSOR) return FFF_ERR_UNSUPPORTED;
     h->path = path;
     return FFF_OK;
@@ -1662,10 +1726,12 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     h->prof_active = h->prof_steps < h->prof_max_steps;
     if (h->prof_active)
         cudaEventRecord(h->prof_events[(size_t)h->prof_steps * (fff_handle_s::kMaxProfLaunches + 1)], st);
-    if (use_fused_small(h, B)) {
-        // one launch: descent, grid barrier, leaf evaluation by groups of hidden neurons; the stable bucketing is
-        // made on demand from the leaf indices it leaves in the workspace
-        s = FFF_DISPATCH(h, run_fused_small, h, x, y, h->ws_leaf, leaf_idx, B, st);
+    const bool token_blocks = use_token_block(h, B);
+    if (token_blocks || use_block_forward(h, B)) {
+        // one launch: a CTA per token; or descent, grid barrier, leaves.  The stable bucketing is made on demand from the leaf
+        // indices that are left in the workspace
+        s = token_blocks ? FFF_DISPATCH(h, run_token_block, h, x, y, h->ws_leaf, leaf_idx, B, st)
+                         : FFF_DISPATCH(h, run_block_forward, h, x, y, h->ws_leaf, leaf_idx, B, st);
         h->last_perm = h->ws_perm;
         h->bucketing_pending = true;
         if (h->prof_active) {
@@ -1689,7 +1755,8 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     const int tile_rows = plan.tile_rows;
     // The descent ends with a tcgen05 stage and the tcgen05 leaf kernel takes whole 128-row tiles of one leaf:
     // that stage files the tokens under their leaves itself and the leaf kernel follows at once.
-    h->slots_now = h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_DESCENT] && tensor_leaf && plan.umma && tile_rows == fff::kLUM && h->ws_slots &&
+    h->slots_now = h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_DESCENT] && tensor_leaf && plan.umma && tile_rows == fff::kLUM && h->ws_slots && !h->ustages.empty() && h->ustages.back().umma &&
+                   h->ustages.back().L0 + h->ustages.back().k == h->depth &&
                    B <= h->slot_cap && h->n_leaves * h->slot_cap <= INT32_MAX &&
                    dense_stage_count(h, B) == (int)h->ustages.size() &&
                    (h->ustages.size() == 1 || (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> h->ustages.back().L0) >= 64));
@@ -1708,7 +1775,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
         return s;
     }
     if (h->slots_now) {
-        if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)h->n_leaves, st) != cudaSuccess)
+        if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
             return h->slots_now = false, cudaGetLastError(), FFF_ERR_CUDA;
         h->cursor_dirty = true;
         s = run_descent(h, x, leaf, nullptr, B, st);
@@ -1899,7 +1966,7 @@ int fff_capabilities(fff_handle_t h) {
     } else if (!h->ustages.empty() || h->LP != 0) {
         caps |= FFF_CAP_PADDED;
     }
-    if (h->fs_batch != 0) caps |= FFF_CAP_FUSED_SMALL;
+    if (h->bf_pinnable) caps |= FFF_CAP_FUSED_SMALL;
     if (h->tr_Kp != 0) caps |= FFF_CAP_FORWARD_TRAIN;
     if (h->g_w1) caps |= FFF_CAP_GROUP_TILES;
     return caps;

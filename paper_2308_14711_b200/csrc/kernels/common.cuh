@@ -36,6 +36,9 @@ template <> struct Elem<float> {
     static constexpr int kVec = 4;   // elements per 16-byte load
     __device__ __forceinline__ static float to_float(float v) { return v; }
     __device__ __forceinline__ static float from_float(float v) { return v; }
+    __device__ __forceinline__ static void unpack(uint4 v, float (&out)[4]) {
+        out[0] = __uint_as_float(v.x); out[1] = __uint_as_float(v.y); out[2] = __uint_as_float(v.z); out[3] = __uint_as_float(v.w);
+    }
     __device__ __forceinline__ static void load_vec(const float* p, float (&out)[4]) {
         const float4 v = __ldg(reinterpret_cast<const float4*>(p));
         out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
@@ -47,7 +50,9 @@ template <> struct Elem<__nv_bfloat16> {
     __device__ __forceinline__ static float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
     __device__ __forceinline__ static __nv_bfloat16 from_float(float v) { return __float2bfloat16_rn(v); }
     __device__ __forceinline__ static void load_vec(const __nv_bfloat16* p, float (&out)[8]) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+        unpack(__ldg(reinterpret_cast<const uint4*>(p)), out);
+    }
+    __device__ __forceinline__ static void unpack(uint4 v, float (&out)[8]) {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
