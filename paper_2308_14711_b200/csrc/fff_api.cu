@@ -311,6 +311,10 @@ bool raise_smem_limit(K kern, int device, int bytes, bool (&done)[kMaxDevices]) 
 // Length of a tile list: floor(B / tile_rows) + nbins entries, some of them empty (see k_bucket_cluster).
 int tile_list_len(int64_t B, int tile_rows, int nbins) { return (int)(B / tile_rows) + nbins; }
 
+// Leaves whose tiles the mma.sync leaf kernel derives from the lists' counts (more would cost it its second CTA per SM),
+// and the batches for which their number fits 16 bits.
+constexpr int kMaxListedLeaves = 2048;
+constexpr int64_t kMaxListedTokens = 1 << 20;
 constexpr size_t kMaxSlotBytes = (size_t)1 << 30;      // largest table of direct lists a handle allocates
 
 // Capacity of the tile buffer: the longest list any stage can ask for.
@@ -770,7 +774,7 @@ fff_status_t run_descent(fff_handle_s* h, const void* x, int32_t* leaf_out, Coar
     const bool node_lists = n_dense == 2 && &plan == &h->ustages && plan[0].umma && plan[1].umma && h->ws_nslots &&
                             B <= h->nslot_cap && (h->nslot_cap << plan[0].k) <= INT32_MAX &&      // (a tile's start is an int)
                             h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_GROUPED] &&
-                            (B >> plan[1].L0) >= 64 && (coarse == nullptr || defer_tail != nullptr);
+                            (coarse == nullptr || defer_tail != nullptr);
     if (node_lists) {
         if (h->ncursor_dirty &&
             cudaMemsetAsync(h->ws_ncursor, 0, sizeof(int32_t) * (fff::kUGMaxBins + 1), st) != cudaSuccess)
@@ -781,7 +785,8 @@ fff_status_t run_descent(fff_handle_s* h, const void* x, int32_t* leaf_out, Coar
     for (int i = 0; i < n_dense; ++i) {
         const auto& sg = plan[i];
         // later stages: the tcgen05 kernel on 128-row tiles when the groups fill them reasonably, else mma.sync on 64-row tiles
-        const bool grouped_umma = i > 0 && sg.umma && h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> sg.L0) >= 64;
+        // (with node lists there is no bucketing launch that the thinner tiles would have to pay for)
+        const bool grouped_umma = i > 0 && sg.umma && h->tune[FFF_TUNE_TCGEN05_GROUPED] && (node_lists || (B >> sg.L0) >= 64);
         if (i > 0 && !node_lists) {
             // bucket by the node reached so far; buffers alternate so that the previous level stays readable
             int32_t* perm_out = (i & 1) ? h->ws_perm2 : h->ws_perm;
@@ -908,13 +913,16 @@ template <int LP, int TM, int S>
 fff_status_t launch_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, cudaStream_t st) {
     const int n_tiles = tile_list_len(B, TM, (int)h->n_leaves);
     using L = fff::LeafMmaLayout<LP, TM, S>;
+    // direct lists: perm is the table of lists, the tiles come from its counts
+    int32_t* counts = h->slots_now && perm == h->ws_slots ? h->ws_cursor : nullptr;
+    const int smem = L::kSmemBytes + (counts ? L::list_bytes((int)h->n_leaves) : 0);
     static bool limit_raised[kMaxDevices] = {};
-    if (!raise_smem_limit(fff::k_leaf_mma<LP, TM, S>, h->device, L::kSmemBytes, limit_raised)) return FFF_ERR_CUDA;
-    const int per_sm = std::max(1, std::min(2, (int)((227 * 1024) / (L::kSmemBytes + 1024))));
+    if (!raise_smem_limit(fff::k_leaf_mma<LP, TM, S>, h->device, L::kSmemBytes + L::list_bytes(kMaxListedLeaves), limit_raised)) return FFF_ERR_CUDA;
+    const int per_sm = std::max(1, std::min(2, (int)((227 * 1024) / (smem + 1024))));
     const int64_t grid = std::min<int64_t>((int64_t)h->sm_count * per_sm, n_tiles);
-    if (launch_chain(h, fff::k_leaf_mma<LP, TM, S>, (unsigned)grid, L::kThreads, L::kSmemBytes, st, 1,
+    if (launch_chain(h, fff::k_leaf_mma<LP, TM, S>, (unsigned)grid, L::kThreads, (size_t)smem, st, 1,
                      (const __nv_bfloat16*)x, perm, h->ws_tiles, n_tiles, h->w1img, h->b1img, h->w2img, (__nv_bfloat16*)y, h->D, h->Dp,
-                     h->O, h->act, h->d_status) != cudaSuccess)
+                     h->O, h->act, h->d_status, counts, (int)h->n_leaves, (int)h->slot_cap) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "grouped_leaf_ff_mma");
 }
@@ -1753,13 +1761,16 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     DescentTail tail;
     const LeafPlan plan = tensor_leaf ? leaf_plan(h, B) : LeafPlan{};
     const int tile_rows = plan.tile_rows;
-    // The descent ends with a tcgen05 stage and the tcgen05 leaf kernel takes whole 128-row tiles of one leaf:
-    // that stage files the tokens under their leaves itself and the leaf kernel follows at once.
-    h->slots_now = h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_DESCENT] && tensor_leaf && plan.umma && tile_rows == fff::kLUM && h->ws_slots && !h->ustages.empty() && h->ustages.back().umma &&
+    // The descent ends with a tcgen05 stage and a tensor-core leaf kernel follows: that stage files the tokens under their
+    // leaves itself and the leaf kernel follows at once, on tiles it derives from the lists' counts.
+    h->slots_now = h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_DESCENT] && tensor_leaf && h->ws_slots && !h->ustages.empty() &&
+                   (plan.umma ? tile_rows == fff::kLUM : h->n_leaves <= kMaxListedLeaves && B <= kMaxListedTokens) && h->ustages.back().umma &&
                    h->ustages.back().L0 + h->ustages.back().k == h->depth &&
                    B <= h->slot_cap && h->n_leaves * h->slot_cap <= INT32_MAX &&
                    dense_stage_count(h, B) == (int)h->ustages.size() &&
-                   (h->ustages.size() == 1 || (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> h->ustages.back().L0) >= 64));
+                   (h->ustages.size() == 1 || (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> h->ustages.back().L0) >= 64) ||
+                    (h->ustages.size() == 2 && h->tune[FFF_TUNE_TCGEN05_GROUPED] && h->ws_nslots && B <= h->nslot_cap &&
+                     (h->nslot_cap << h->ustages[0].k) <= INT32_MAX));
     if (tensor_leaf && plan.umma && use_group_tiles(h, B)) {
         h->slots_now = false;
         s = run_forward_grouped(h, x, y, leaf, B, st);

@@ -266,29 +266,8 @@ k_block_forward(const T* __restrict__ x, const T* __restrict__ node_w, const T* 
     __threadfence();
     cg::this_grid().sync();
 
-    // ---- tiles of every leaf and their running sum, by every CTA for itself: thread i owns a run of leaves
-    {
-        const int per = (n_leaves + kBFThreads - 1) / kBFThreads;
-        const int j0 = min(tid * per, n_leaves), j1 = min(j0 + per, n_leaves);
-        int mine = 0;
-        for (int j = j0; j < j1; ++j) mine += (__ldcg(cursor + j) + tile_rows - 1) / tile_rows;
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(kFullMask, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) s_wsum[warp] = incl;
-        __syncthreads();
-        int run = incl - mine;
-        for (int w = 0; w < warp; ++w) run += s_wsum[w];
-        for (int j = j0; j < j1; ++j) {
-            s_pre[j] = run;
-            run += (__ldcg(cursor + j) + tile_rows - 1) / tile_rows;
-        }
-        if (tid == kBFThreads - 1) s_pre[n_leaves] = run;
-        __syncthreads();
-    }
+    // ---- tiles of every leaf and their running sum, by every CTA for itself
+    tiles_before_bins([&](int j) { return __ldcg(cursor + j); }, n_leaves, tile_rows, s_pre, s_wsum, kBFThreads);
     const int n_tiles = s_pre[n_leaves];
 
     // ---- phase B
@@ -297,12 +276,7 @@ k_block_forward(const T* __restrict__ x, const T* __restrict__ node_w, const T* 
     while (og < kBFThreads && og < O) og <<= 1;
     const int tpt = kBFTile / min(kBFThreads / og, kBFTile);             // 16, 8, 4 or 2
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        int lo = 0, hi = n_leaves;                          // s_pre[lo] <= tile < s_pre[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (s_pre[mid] <= tile) lo = mid;
-            else hi = mid;
-        }
+        const int lo = bin_of_tile(s_pre, n_leaves, tile);
         const int64_t leaf = lo;
         const int first = (tile - s_pre[lo]) * tile_rows;
         const int rows = min(tile_rows, __ldcg(cursor + lo) - first);

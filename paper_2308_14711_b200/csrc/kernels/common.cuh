@@ -225,4 +225,50 @@ __device__ __forceinline__ float warp_dot(const T* __restrict__ a, const T* __re
     return warp_sum(acc);
 }
 
+// Tiles of up to tile_rows entries of every bin, from the bins' counts: s_pre[b] = tiles before bin b, s_pre[n_bins] = all of
+// them.  By all `n_threads` threads of a CTA (thread i takes a run of bins); s_wsum: one int per warp.  `count(b)` reads a count.
+// Index: int, or uint16_t where the caller knows that there are fewer than 65536 tiles.
+template <class Index, class Count>
+__device__ __forceinline__ void tiles_before_bins(Count&& count, int n_bins, int tile_rows, Index* s_pre, int* s_wsum, int n_threads) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = (n_bins + n_threads - 1) / n_threads;
+    const int b0 = min(tid * per, n_bins), b1 = min(b0 + per, n_bins);
+    int mine = 0;
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) {
+        const int t = (count(b) + tile_rows - 1) / tile_rows;
+        s_pre[b] = (Index)t;
+        mine += t;
+    }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFullMask, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) s_wsum[warp] = incl;
+    __syncthreads();
+    int run = incl - mine;
+    for (int w = 0; w < warp; ++w) run += s_wsum[w];
+    for (int b = b0; b < b1; ++b) {
+        const int t = s_pre[b];
+        s_pre[b] = (Index)run;
+        run += t;
+    }
+    if (tid == n_threads - 1) s_pre[n_bins] = (Index)run;
+    __syncthreads();
+}
+
+// The bin of tile `idx`: s_pre[bin] <= idx < s_pre[bin + 1].
+template <class Index>
+__device__ __forceinline__ int bin_of_tile(const Index* s_pre, int n_bins, int idx) {
+    int lo = 0, hi = n_bins;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (s_pre[mid] <= idx) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
 }  // namespace fff

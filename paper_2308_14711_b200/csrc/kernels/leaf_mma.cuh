@@ -6,7 +6,8 @@
 // and row i of Y is stored at the original position of token T_j[i].
 //
 // Work unit: a tile = up to TM consecutive entries of one bucket.  CTAs are persistent and walk the
-// device-built tile list with a static stride.  Inside a CTA the producer warps stream operands into a
+// device-built tile list with a static stride, or derive the tiles themselves from the counts of the leaves' token lists
+// that the descent has filled (slot_counts).  Inside a CTA the producer warps stream operands into a
 // ring of shared-memory stages (cp.async for the gathered token rows, 1-D bulk (TMA) copies for the
 // weight images) whose stages complete on mbarriers; 8 consumer warps run both GEMMs with
 // mma.sync.m16n8k16, keeping H in registers between them (the accumulator fragment of GEMM1 is the A
@@ -63,6 +64,9 @@ template <int LP, int TM, int S> struct LeafMmaLayout {
     static constexpr int kWarpScratch = (16 * kOutRowBytes > LP * 64 ? 16 * kOutRowBytes : LP * 64);
     static constexpr int kStagingBytes = kLeafConsumers * kWarpScratch;
     static constexpr int kSmemBytes = S * kStageStride + kStagingBytes + 128 /* barriers */ + 128 /* align */;
+    // with the tiles derived from counts: + tiles before each of n_bins leaves, the warps' sums, rows of each leaf's last tile
+    // (16-bit indices and 8-bit rows: with 2048 leaves of 32 neurons two CTAs still fit an SM, and one CTA per SM is 20 % slower)
+    static constexpr int list_bytes(int n_bins) { return 64 + (((n_bins + 1) * 2 + 3) & ~3) + ((n_bins + 3) & ~3); }
     static_assert(S <= kMaxStages, "barrier area holds 2 * kMaxStages mbarriers");
     static_assert((kKS / 16) % kNSplit == 0 && (kNC / kOutBlock) % kNSplit == 0, "split must divide the stage");
 };
@@ -131,7 +135,7 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
            const Tile* __restrict__ tiles, int n_tiles_total,
            const __nv_bfloat16* __restrict__ w1img, const float* __restrict__ b1img,
            const unsigned char* __restrict__ w2img, __nv_bfloat16* __restrict__ y,
-           int D, int Dp, int O, int act, int* __restrict__ status)
+           int D, int Dp, int O, int act, int* __restrict__ status, int32_t* __restrict__ slot_counts, int n_bins, int cap)
 {
     using L = LeafMmaLayout<LP, TM, S>;
     constexpr int kStages = S;
@@ -148,7 +152,9 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int U1 = Dp / kKS;
     const int U2 = (O + kNC - 1) / kNC;
-    const int ntiles = n_tiles_total;      // the list may contain empty tiles (rows = 0)
+    // (only with slot_counts)
+    int* s_wsum = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(full) + 128);    // [16]
+    uint16_t* s_pre = reinterpret_cast<uint16_t*>(s_wsum + 16);                            // [n_bins + 1]
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -160,6 +166,24 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
     pdl_trigger();
     __syncthreads();
     pdl_wait();
+    uint8_t* s_rest = reinterpret_cast<uint8_t*>(s_pre) + (((n_bins + 1) * 2 + 3) & ~3);   // [n_bins] rows of the last tile
+    if (slot_counts)
+        tiles_before_bins([&](int b) {
+            const int c = __ldcg(slot_counts + b);
+            s_rest[b] = (uint8_t)((c + kTM - 1) % kTM + 1);
+            return c;
+        }, n_bins, kTM, s_pre, s_wsum, L::kThreads);
+    const int ntiles = slot_counts ? s_pre[n_bins] : n_tiles_total;      // a list may contain empty tiles (rows = 0)
+    auto tile_at = [&](int idx) {
+        if (!slot_counts) return tiles[idx];
+        Tile tl;
+        tl.bin = bin_of_tile(s_pre, n_bins, idx);
+        const int local = idx - s_pre[tl.bin];
+        tl.start = tl.bin * cap + local * kTM;
+        tl.rows = idx + 1 < s_pre[tl.bin + 1] ? kTM : s_rest[tl.bin];
+        tl.pad = 0;
+        return tl;
+    };
 
     int stage = 0;
     uint32_t phase = 0;
@@ -170,7 +194,7 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
         const int ptid = threadIdx.x - kLeafConsumers * 32;
         const int prow = ptid >> 4, pchunk = ptid & 15;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-            const Tile tl = tiles[tile];
+            const Tile tl = tile_at(tile);
             if (tl.rows == 0) continue;
             const __nv_bfloat16* src[kTM / kRowsPerPass];
 #pragma unroll
@@ -218,7 +242,7 @@ if (u * kKS + pchunk * 8 < D) {
         const int bn = (lane & 7) + ((lane >> 4) << 3);
         const int bk = ((lane >> 3) & 1) * 8;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-            const Tile tl = tiles[tile];
+            const Tile tl = tile_at(tile);
             if (tl.rows == 0) continue;
             const bool active = m0 < tl.rows;          // m-tiles without valid rows only keep the ring moving
 
@@ -354,6 +378,18 @@ if (u * kKS + pchunk * 8 < D) {
     if (timed_out) {
         if (lane == 0) atomicExch(status, kDevTimeout);
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);     // let bulk copies still in flight land before exit
+    }
+    // the last CTA to finish clears the counts (and the word behind them that counts the CTAs) for the next call
+    if (slot_counts) {
+        __shared__ int s_last;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(slot_counts + n_bins, 1) == (int)gridDim.x - 1 ? 1 : 0;
+        }
+        __syncthreads();
+        if (s_last)
+            for (int b = threadIdx.x; b <= n_bins; b += L::kThreads) slot_counts[b] = 0;
     }
 }
 
