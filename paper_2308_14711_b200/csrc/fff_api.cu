@@ -943,7 +943,7 @@ fff_status_t launch_leaf_umma(fff_handle_s* h, const void* x, const int32_t* per
     const int passes = 1;      // two passes (full tiles first) measured slightly slower
     // direct lists: perm is the table of lists, the tiles come from its counts
     int32_t* counts = h->slots_now && perm == h->ws_slots ? h->ws_cursor : nullptr;
-    if (launch_chain(h, fff::k_leaf_umma<LP, kFold, kW8>, (unsigned)grid, fff::kLUThreads, (size_t)L::smem_bytes(stages), st, 1, tm, perm,
+    if (launch_chain(h, fff::k_leaf_umma<LP, kFold, kW8>, (unsigned)grid, fff::LeafUmmaWarps<kW8>::kThreads, (size_t)L::smem_bytes(stages), st, 1, tm, perm,
                      (const fff::Tile*)h->ws_tiles, n_tiles, (const __nv_bfloat16*)h->w1img, (const float*)h->b1img,
                      (const unsigned char*)(kW8 ? h->w2codes : h->w2uimg), (__nv_bfloat16*)y, h->Dp, h->O, h->l, h->act, stages, wide, passes, h->ws_sched,
                      counts, (int)h->n_leaves, (int)h->slot_cap, h->d_status, (const unsigned char*)h->w1codes, (const float*)h->scale1,

@@ -69,13 +69,21 @@ constexpr int kLUThreads = kLUWarps * 32;
 constexpr int kLUMaxStages = 8;
 constexpr int kLUMaxW2Slots = 12;
 constexpr int kLUQueue = 4;                // tiles published ahead by the scheduler
-constexpr int kLUConsumerWarps = kLUWarps - 1;     // every warp but the scheduler reads the tile queue
+constexpr int kLUExpandWarps = 2;          // 8-bit weights: further warps, this many for W1 stages and as many for W2 pieces
+template <bool kW8> struct LeafUmmaWarps {
+    static constexpr int kWarps = kLUWarps + (kW8 ? 2 * kLUExpandWarps : 0);
+    static constexpr int kThreads = kWarps * 32;
+    static constexpr int kConsumers = kWarps - 1;          // every warp but the scheduler reads the tile queue
+};
 constexpr int kLUTmemCols = 512;
 
 // kW8: the leaf weights are stored as 8-bit floats (e4m3 codes, one float32 scale per leaf and matrix).  The MMA wants
-// both operands as bf16, so the codes land in a staging part of their ring slot and the warp that issues the MMAs
-// expands them (every code is exactly a bf16 value) into the operand layout first; the scales multiply the
-// accumulators in the epilogue.
+// both operands as bf16, so the codes land in a staging part of their ring slot and are expanded (every code is exactly a
+// bf16 value) into the operand layout first; the scales multiply the accumulators in the epilogue.  Four warps do nothing
+// else, two for W1 stages and two for W2 pieces, each starting as soon as the codes of a stage have landed, whether or not
+// its token rows have.  (When the two warps that issue the MMAs expanded the codes themselves, at the 0.25 instructions per
+// cycle of a lone warp, every stage waited 0.8 us for them: 2048 leaves of 32, 65 536 tokens, 189 us; now 148.  Three or four warps each cost the
+// epilogue its registers: 204-212.)
 // GL: leaves per tile.  1: a tile holds tokens of one leaf.  8: a tile holds tokens of one node three levels above the
 // leaves; GEMM1 then runs against the hidden units of that node's 8 leaves side by side plus the 7 nodes of its
 // subtree (N = 8 LP + 16 columns, the last 9 zero), the epilogue walks the three levels from the node logits, keeps
@@ -110,7 +118,7 @@ template <int LP, bool kW8 = false, int GL = 1> struct LeafUmmaLayout {
     // W2 ring: a whole tile's pieces (O <= 1024) when they are small, so that no copy waits for an MMA just issued
     static constexpr int kW2Slots = GL > 1 ? 3 : LP <= 16 ? 8 : LP <= 32 ? (kW8 ? 6 : 8) : 4;
     static constexpr int kAcc2Col = GL > 1 ? 256 : 64;                       // first tensor-memory column of the two GEMM2 accumulators
-    static constexpr int kBarrierBytes = 640;
+    static constexpr int kBarrierBytes = kW8 ? 896 : 640;
     static constexpr int smem_bytes(int stages) {
         return 1024 + stages * kStageBytes + kW2Slots * kW2SlotStride + kHBytes + kBarrierBytes;
     }
@@ -246,15 +254,15 @@ __device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t pair) {
     return out;
 }
 
-// A tile of e4m3 codes, [rows][COLS] row-major, expanded by one warp into the K-major bf16 operand layout with rows of
+// A tile of e4m3 codes, [rows][COLS] row-major, expanded by `part` of kLUExpandWarps warps into the K-major bf16 operand layout with rows of
 // 2 COLS bytes, swizzled in the mode of that width.  Units of 16 codes (16 bytes in, two 16-byte units out).
 template <int COLS>
 __device__ __forceinline__ void expand_e4m3_tile(const unsigned char* __restrict__ src, unsigned char* __restrict__ dst, int rows,
-                                                 int lane)
+                                                 int lane, int part)
 {
     const int n_units = rows * COLS / 16;
 #pragma unroll 4
-    for (int u = lane; u < n_units; u += 32) {
+    for (int u = part * 32 + lane; u < n_units; u += kLUExpandWarps * 32) {
         const uint4 raw = *reinterpret_cast<const uint4*>(src + u * 16);
         const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
         uint32_t o[8];
@@ -283,7 +291,7 @@ __device__ __forceinline__ void expand_e4m3_tile(const unsigned char* __restrict
 // [bin][8 LP + 16] the matching biases, w2img per bin and piece the 128 x 8 LP output weights in two K-blocks (kFold:
 // every leaf's spare column carries its output bias); leaf_out / leaf_out2 (optional) receive every token's leaf.
 template <int LP, bool kFold, bool kW8 = false, int GL = 1>
-__global__ void __launch_bounds__(kLUThreads, 1)
+__global__ void __launch_bounds__(LeafUmmaWarps<kW8>::kThreads, 1)
 k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restrict__ perm,
             const Tile* __restrict__ tiles, int n_tiles_total,
             const __nv_bfloat16* __restrict__ w1img, const float* __restrict__ b1img,
@@ -314,6 +322,8 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
     Tile* queue = reinterpret_cast<Tile*>(y_empty + 2);                      // [kLUQueue]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(queue + kLUQueue);
     uint64_t* want = reinterpret_cast<uint64_t*>(tmem_slot + 2);             // the gathers have started another tile
+    uint64_t* code_full = want + 1;                                          // [kLUMaxStages] the W1 codes of a stage have landed (kW8)
+    uint64_t* w2code_full = code_full + kLUMaxStages;                        // [kLUMaxW2Slots] likewise the codes of a W2 piece
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KB = D / (kLUKB * L::kSub);                   // ring stages per tile
@@ -321,16 +331,18 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            ptx::mbar_init(full + s, kLUGatherWarps);           // one arrival per gather warp
+            ptx::mbar_init(full + s, kLUGatherWarps + (kW8 ? kLUExpandWarps : 0));      // one arrival per gather (and expanding) warp
             ptx::mbar_init(empty + s, 1);
+            if (kW8) ptx::mbar_init(code_full + s, 1);
         }
         for (int s = 0; s < L::kW2Slots; ++s) {
-            ptx::mbar_init(w2_full + s, 1);
+            ptx::mbar_init(w2_full + s, kW8 ? kLUExpandWarps : 1);
+            if (kW8) ptx::mbar_init(w2code_full + s, 1);
             ptx::mbar_init(w2_empty + s, 1 + kLUEpiWarps);      // the MMAs that read the weights + every reader of the biases
         }
         for (int s = 0; s < kLUQueue; ++s) {
             ptx::mbar_init(q_full + s, 1);
-            ptx::mbar_init(q_empty + s, kLUConsumerWarps);
+            ptx::mbar_init(q_empty + s, LeafUmmaWarps<kW8>::kConsumers);
         }
         ptx::mbar_init(want, 1);
         ptx::mbar_init(acc1_full, 1);
@@ -466,6 +478,42 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             __syncwarp();
             if (++q_slot == kLUQueue) { q_slot = 0; q_phase ^= 1; }
         }
+    } else if (kW8 && warp >= kLUWarps) {
+        // ------------------------------------------------------------------ expansion of 8-bit weights
+        const int part = (warp - kLUWarps) % kLUExpandWarps;
+        if (warp < kLUWarps + kLUExpandWarps) {
+            // W1: kSub tiles of LP rows x 64 columns per stage, stacked
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int it = 0; it < max_iters; ++it) {
+                if (next_tile().rows <= 0) break;
+                for (int kb = 0; kb < KB; ++kb) {
+                    if (!timed_out && !ptx::mbar_wait(code_full + stage, phase)) timed_out = true;
+                    unsigned char* w1s = ring + stage * L::kStageBytes + L::kXStageBytes;
+                    expand_e4m3_tile<kLUKB>(w1s + L::kW1StageBytes, w1s, L::kSub * LP, lane, part);
+                    ptx::fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(full + stage);
+                    if (++stage == kStages) { stage = 0; phase ^= 1; }
+                }
+            }
+        } else {
+            // W2: 128 output features x LP columns per piece
+            int slot = 0;
+            uint32_t phase = 0;
+            for (int it = 0; it < max_iters; ++it) {
+                if (next_tile().rows <= 0) break;
+                for (int p = 0; p < P; ++p) {
+                    if (!timed_out && !ptx::mbar_wait(w2code_full + slot, phase)) timed_out = true;
+                    unsigned char* piece = w2ring + slot * L::kW2SlotStride;
+                    expand_e4m3_tile<LP>(piece + L::kW2CopyOff, piece, kLUPiece, lane, part);
+                    ptx::fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(w2_full + slot);
+                    if (++slot == L::kW2Slots) { slot = 0; phase ^= 1; }
+                }
+            }
+        }
     } else if (warp >= kLUFirstGatherWarp) {
         // ------------------------------------------------------------------ row gathers
         const int gw = warp - kLUFirstGatherWarp;
@@ -487,14 +535,15 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             for (int kb = 0; kb < KB; ++kb) {
                 if (!timed_out && !ptx::mbar_wait_relaxed(empty + stage, phase ^ 1)) timed_out = true;
                 if (lane == 0) {
-                    const uint32_t bytes = (uint32_t)groups * (512u * L::kSub) + (gw == 0 ? (uint32_t)L::kW1CopyBytes : 0u);
+                    const uint32_t bytes = (uint32_t)groups * (512u * L::kSub) + (!kW8 && gw == 0 ? (uint32_t)L::kW1CopyBytes : 0u);
                     if (bytes > 0) ptx::mbar_arrive_expect_tx(full + stage, bytes);
                     else ptx::mbar_arrive(full + stage);
                     if (gw == 0) {
-                        if constexpr (kW8)
+                        if constexpr (kW8) {
+                            ptx::mbar_arrive_expect_tx(code_full + stage, (uint32_t)L::kW1CodeBytes);
                             ptx::bulk_g2s(ring + stage * L::kStageBytes + L::kXStageBytes + L::kW1StageBytes,
-                                          w1codes + ((int64_t)tl.bin * KB + kb) * L::kW1CodeBytes, L::kW1CodeBytes, full + stage);
-                        else
+                                          w1codes + ((int64_t)tl.bin * KB + kb) * L::kW1CodeBytes, L::kW1CodeBytes, code_full + stage);
+                        } else
                             ptx::bulk_g2s(ring + stage * L::kStageBytes + L::kXStageBytes,
                                           w1img + ((int64_t)tl.bin * KB + kb) * (L::kW1StageBytes / 2), L::kW1StageBytes, full + stage);
                     }
@@ -522,13 +571,6 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             for (int kb = 0; kb < KB; ++kb) {
                 if (!timed_out && !ptx::mbar_wait(full + stage, phase)) timed_out = true;
                 ptx::tc_fence_after_sync();
-                if constexpr (kW8) {
-                    // the stage's W1 codes -> bf16 operand tiles (kSub tiles of LP rows x 64 columns, stacked)
-                    unsigned char* w1s = ring + stage * L::kStageBytes + L::kXStageBytes;
-                    expand_e4m3_tile<kLUKB>(w1s + L::kW1StageBytes, w1s, L::kSub * LP, lane);
-                    ptx::fence_proxy_async();
-                    __syncwarp();
-                }
                 if (lane == 0) {
                     const uint32_t xs = ptx::smem_addr(ring + stage * L::kStageBytes);
 #pragma unroll
@@ -565,9 +607,10 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                     return false;
                 }
                 if (lane == 0) {
-                    ptx::mbar_arrive_expect_tx(w2_full + ld_slot, (uint32_t)L::kW2PieceBytes);
+                    uint64_t* landed = (kW8 ? w2code_full : w2_full) + ld_slot;
+                    ptx::mbar_arrive_expect_tx(landed, (uint32_t)L::kW2PieceBytes);
                     ptx::bulk_g2s(w2ring + ld_slot * L::kW2SlotStride + L::kW2CopyOff, w2j + (int64_t)loaded * L::kW2PieceBytes,
-                                  L::kW2PieceBytes, w2_full + ld_slot);
+                                  L::kW2PieceBytes, landed);
                 }
                 __syncwarp();
                 ++loaded;
@@ -587,13 +630,6 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                 const int b = pc & 1;
                 load_ahead(p);
                 if (!timed_out && !ptx::mbar_wait(w2_full + mm_slot, mm_phase)) timed_out = true;
-                if constexpr (kW8) {
-                    // the piece's codes -> bf16 operand tile (128 output features x LP columns)
-                    unsigned char* slot = w2ring + mm_slot * L::kW2SlotStride;
-                    expand_e4m3_tile<LP>(slot + L::kW2CopyOff, slot, kLUPiece, lane);
-                    ptx::fence_proxy_async();
-                    __syncwarp();
-                }
                 if (!timed_out && !ptx::mbar_wait(y_empty + b, ((pc >> 1) & 1) ^ 1)) timed_out = true;
                 ptx::tc_fence_after_sync();
                 if (lane == 0) {
