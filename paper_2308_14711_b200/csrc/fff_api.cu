@@ -2050,9 +2050,15 @@ fff_status_t stack_glue(fff_stack_s* s, const void* x_prev, const void* y_prev, 
                         cudaStream_t st) {
     const int64_t blocks = std::min<int64_t>((B + fff::kStackWarps - 1) / fff::kStackWarps, (int64_t)s->sm_count * 8);
     const bool vec = s->D % (int)(16 / s->esize) == 0 && aligned16(x_prev) && aligned16(y_prev) && aligned16(x_out) && aligned16(z);
-    fff::k_stack_glue<T><<<(unsigned)blocks, fff::kStackWarps * 32, 0, st>>>(
-        (const T*)x_prev, (const T*)y_prev, (T*)x_out, (T*)z, z ? (const T*)s->gamma[layer] : nullptr,
-        z ? (const T*)s->beta[layer] : nullptr, s->eps, s->D, B, vec);
+    const T *g = z ? (const T*)s->gamma[layer] : nullptr, *b = z ? (const T*)s->beta[layer] : nullptr;
+    cudaError_t e;
+    if (vec && s->D <= 32 * 32)          // (in registers: 32 values per lane)
+        e = launch_chain(s->layers[0], fff::k_stack_glue_rows<T>, (unsigned)blocks, fff::kStackWarps * 32, 0, st, 1, (const T*)x_prev,
+                         (const T*)y_prev, (T*)x_out, (T*)z, g, b, s->eps, s->D, B);
+    else
+        e = launch_chain(s->layers[0], fff::k_stack_glue<T>, (unsigned)blocks, fff::kStackWarps * 32, 0, st, 1, (const T*)x_prev,
+                         (const T*)y_prev, (T*)x_out, (T*)z, g, b, s->eps, s->D, B, vec);
+    if (e != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
     ++s->launches;
     return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
 }
