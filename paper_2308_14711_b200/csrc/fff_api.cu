@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
@@ -155,6 +156,7 @@ struct fff_handle_s {
     bool pdl = true;              // launch every kernel of a forward but the first as a programmatic dependent
     int launches = 0;
     int64_t last_B = -1;
+    int64_t plan_B = 0;           // chunk of a larger batch: the leaf kernel is chosen as for that many tokens (0: the call's own)
 
     // optional per-launch timing of forwards (fff_profile_*)
     static constexpr int kMaxProfLaunches = 16;
@@ -326,8 +328,36 @@ struct LeafPlan {
     bool umma = false;
 };
 
+// Tiles of tile_rows rows that B tokens spread over the leaves fill, on average (a leaf's count is about Poisson).
+double expected_tiles(const fff_handle_s* h, int64_t B, int tile_rows) {
+    const double mean = (double)B / (double)h->n_leaves, sd2 = std::sqrt(2.0 * mean);
+    double per_leaf = 1.0 - std::exp(-mean);
+    for (int k = 1; k < 64 && (k * tile_rows - mean) / sd2 < 4.5; ++k) per_leaf += 0.5 * std::erfc((k * tile_rows + 0.5 - mean) / sd2);
+    return per_leaf * (double)h->n_leaves;
+}
+
+template <int LP, int TM, int S> int leaf_mma_slots(const fff_handle_s* h) {
+    using L = fff::LeafMmaLayout<LP, TM, S>;
+    const int smem = L::kSmemBytes + L::list_bytes((int)std::min<int64_t>(h->n_leaves, kMaxListedLeaves));
+    return h->sm_count * std::max(1, std::min(2, (227 * 1024) / (smem + 1024)));
+}
+// CTAs of the mma.sync leaf kernel that are resident at once (ring depths as in run_leaf_mma).
+int leaf_mma_slots(const fff_handle_s* h, int tile_rows) {
+    switch (h->LP) {
+        case 16: return tile_rows == 32 ? leaf_mma_slots<16, 32, 6>(h) : leaf_mma_slots<16, 64, 4>(h);
+        case 32: return tile_rows == 32 ? leaf_mma_slots<32, 32, 5>(h) : leaf_mma_slots<32, 64, 3>(h);
+        default: return tile_rows == 32 ? leaf_mma_slots<64, 32, 4>(h) : leaf_mma_slots<64, 64, 4>(h);
+    }
+}
+
 LeafPlan leaf_plan(const fff_handle_s* h, int64_t B) {
     if (h->w8) return LeafPlan{fff::kLUM, true};
+    // While the tiles of all leaves are resident at once, the mma.sync kernel (two CTAs per SM for leaves of up to 32 neurons,
+    // no tensor memory to set up) is ahead: 768 -> 768, 256 leaves of 12, with the descent: 19.3 against 24.1 us at 4096 tokens
+    // and 19.6 against 24.6 at 6144 (32-row tiles), 22.7 against 25.8 at 8192 and 25.0 against 30.1 at 12 608 (64-row tiles);
+    // a second round of tiles costs more than it saves: 38.3 against 34.0 at 16 384.
+    for (int rows : {32, 64})
+        if (expected_tiles(h, B, rows) <= 0.98 * leaf_mma_slots(h, rows)) return LeafPlan{rows, false};
     // The tcgen05 kernel works on 128-row tiles.  Measured against the mma.sync kernel it is far ahead when
     // some buckets are large (skewed routing), about level with uniformly thin buckets of 32 tokens, and is
     // left out only when buckets are thinner still (tiles of at most 64 rows are stacked in the MMA rows, so the
@@ -1759,7 +1789,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     if (lazy_bucketing) leaf = h->ws_leaf;
     Coarse coarse;
     DescentTail tail;
-    const LeafPlan plan = tensor_leaf ? leaf_plan(h, B) : LeafPlan{};
+    const LeafPlan plan = tensor_leaf ? leaf_plan(h, std::max(B, h->plan_B)) : LeafPlan{};
     const int tile_rows = plan.tile_rows;
     // The descent ends with a tcgen05 stage and a tensor-core leaf kernel follows: that stage files the tokens under their
     // leaves itself and the leaf kernel follows at once, on tiles it derives from the lists' counts.
@@ -1902,8 +1932,10 @@ fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_
         if (n <= 0) break;
         ok = cudaStreamWaitEvent(st, h->ev_in[c], 0) == cudaSuccess;
         if (!ok) break;
-        if ((s = fff_forward_infer(h, (char*)h->st_x + b0 * xrow, (char*)h->st_y + b0 * yrow, h->st_leaf + b0, n, cuda_stream)) != FFF_OK)
-            return s;
+        h->plan_B = B;           // results do not depend on the chunking
+        s = fff_forward_infer(h, (char*)h->st_x + b0 * xrow, (char*)h->st_y + b0 * yrow, h->st_leaf + b0, n, cuda_stream);
+        h->plan_B = 0;
+        if (s != FFF_OK) return s;
         ok = cudaEventRecord(h->ev_done[c], st) == cudaSuccess && cudaStreamWaitEvent(h->copy_out, h->ev_done[c], 0) == cudaSuccess &&
              cudaMemcpyAsync((char*)y_host + b0 * yrow, (char*)h->st_y + b0 * yrow, (size_t)n * yrow, cudaMemcpyDeviceToHost,
                              h->copy_out) == cudaSuccess &&
