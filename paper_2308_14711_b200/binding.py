@@ -90,6 +90,26 @@ def lib():
     return L
 
 
+_call = None
+
+
+def torch_call():
+    """The CPython module behind FFFLayer.forward_infer (csrc/torch_call.cpp), told where fff_forward_infer is (once)."""
+    global _call
+    if _call is None:
+        import importlib.util
+        _torch()                                   # its libraries first: the module links against them
+        path = os.path.join(HERE, "torch_call.so")
+        if not os.path.exists(path):
+            raise ImportError(f"{path} not found: build it with `python -m paper_2308_14711_b200.build`")
+        spec = importlib.util.spec_from_file_location("torch_call", path)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.set_address(C.cast(lib().fff_forward_infer, C.c_void_p).value)
+        _call = mod
+    return _call
+
+
 def status_string(status: int) -> str:
     return lib().fff_status_string(int(status)).decode()
 
@@ -231,7 +251,8 @@ class FFFLayer:
                                  _ptr(node_w, td, (nn, D), "node_w"), _ptr(node_b, td, (nn,), "node_b"),
                                  _ptr(w1, td, (nl, leaf_width, D), "w1"), _ptr(b1, td, (nl, leaf_width), "b1"),
                                  _ptr(w2, td, (nl, O, leaf_width), "w2"), _ptr(b2, td, (nl, O), "b2"))
-        self._forward = lib().fff_forward_infer
+        self._bf16 = self.tdtype == torch.bfloat16
+        self._forward = torch_call().forward
         if path != "auto":
             self.set_path(path)
 
@@ -268,26 +289,21 @@ class FFFLayer:
         fff_set_tuning(self._h, TUNING[key], 1 if on else 0)
 
     def forward_infer(self, x, y=None, leaf_idx=None, want_leaf_idx: bool = True, stream=None):
-        i32 = _torch().int32
-        td = self.tdtype
+        got = self._forward(self._h, self.D, self.O, self._bf16, x, y, leaf_idx, want_leaf_idx,
+                            None if stream is None else stream.cuda_stream)
+        if got is None:
+            self._explain(x, y, leaf_idx)
+        if got[0]:
+            raise FFFError(got[0], "fff_forward_infer")
+        return got[1], got[2]
+
+    def _explain(self, x, y, leaf_idx):
+        """Raises the error of the argument that forward_infer could not take."""
         B = x.shape[0]
-        xp = _ptr(x, td, (B, self.D), "x")
-        if y is None:
-            y = x.new_empty((B, self.O))
-            yp = y.data_ptr()
-        else:
-            yp = _ptr(y, td, (B, self.O), "y")
-        if leaf_idx is None:
-            lp = None
-            if want_leaf_idx:
-                leaf_idx = x.new_empty((B,), dtype=i32)
-                lp = leaf_idx.data_ptr()
-        else:
-            lp = _ptr(leaf_idx, i32, (B,), "leaf_idx")
-        status = self._forward(self._h, xp, yp, lp, B, _stream_ptr(stream))
-        if status:
-            raise FFFError(status, "fff_forward_infer")
-        return y, leaf_idx
+        _ptr(x, self.tdtype, (B, self.D), "x")
+        _ptr(y, self.tdtype, (B, self.O), "y")
+        _ptr(leaf_idx, _torch().int32, (B,), "leaf_idx")
+        raise ValueError("forward_infer: arguments not understood")
 
     def forward_train(self, x, want_mixture: bool = True, want_entropy: bool = True, stream=None):
         """FORWARD_T: returns (y, mixture weights float32 [B, 2^d] or None, node entropies float32 [2^d - 1] or None)."""

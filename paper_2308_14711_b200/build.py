@@ -1,4 +1,5 @@
-"""Compile the CUDA library in-tree: paper_2308_14711_b200/libfff.so (sm_100a only)."""
+"""Compile in-tree: the CUDA library paper_2308_14711_b200/libfff.so (sm_100a only) and the CPython module torch_call that
+makes its tensor-level call."""
 from __future__ import annotations
 
 import glob
@@ -9,6 +10,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfff.so")
+CALL_SRC = os.path.join(CSRC, "torch_call.cpp")
+CALL_LIB = os.path.join(HERE, "torch_call.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -29,6 +32,7 @@ def up_to_date() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_call(force)
     if not force and up_to_date():
         return LIB
     tmp = LIB + f".{os.getpid()}.tmp"
@@ -38,5 +42,26 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_call(force: bool = False) -> str:
+    """The CPython module (needs torch's headers, not a GPU)."""
+    if not force and os.path.exists(CALL_LIB) and os.path.getmtime(CALL_LIB) >= os.path.getmtime(CALL_SRC):
+        return CALL_LIB
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(NVCC))
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    tmp = CALL_LIB + f".{os.getpid()}.tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [f"-isystem{d}" for d in inc] + ["-o", tmp, CALL_SRC, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu",
+                                           "-lc10_cuda", "-lc10"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, CALL_LIB)
+    return CALL_LIB
+
+
 if __name__ == "__main__":
     print(build(force=True, verbose="-v" in sys.argv))
+    print(build_call(force=True))
