@@ -56,7 +56,8 @@ typedef enum {
 typedef enum {
     FFF_ACT_RELU = 0,            /* max(v, 0) */
     FFF_ACT_GELU = 1,            /* v * Phi(v), erf form (not the tanh approximation); the bf16 tensor-core
-                                    kernels evaluate erf to 1.5e-7 absolute, below bf16 resolution */
+                                    kernels evaluate the normal distribution's tail to 7.6e-8, far below bf16
+                                    resolution */
     FFF_ACT_GELU_TANH = 2,       /* v/2 * (1 + tanh(sqrt(2/pi) * (v + 0.044715 v^3))): a different function from
                                     FFF_ACT_GELU (up to 5e-4 apart), not a cheaper evaluation of it */
     FFF_ACT_SILU = 3             /* v * sigmoid(v) */
@@ -77,7 +78,7 @@ typedef enum {
     FFF_PATH_AUTO = 0,           /* library picks per stage from shapes and B */
     FFF_PATH_WARP = 1,           /* CUDA-core warp kernels for descent and leaf evaluation */
     FFF_PATH_TENSOR = 2,         /* tensor-core kernels wherever the shapes allow them */
-    FFF_PATH_FUSED = 3           /* the one-launch kernel on CUDA cores (small trees with leaves of at most 32 neurons) */
+    FFF_PATH_FUSED = 3           /* the one-launch kernel on CUDA cores (the layers of FFF_CAP_FUSED_SMALL) */
 } fff_path_t;
 
 /*

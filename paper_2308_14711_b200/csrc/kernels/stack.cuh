@@ -6,7 +6,7 @@
 // and z_k is what the block's FFF layer reads.  Both are stored in the stack's element type; the statistics are
 // taken in float32 from the stored x_k (two passes: mean, then squared deviations).
 // One warp per token.  Rows of up to kStackVecs 16-byte vectors per lane (1024 columns in bf16) stay in registers between the
-// sum, the statistics and the normalised row, with all loads of a row issued at once (12 608 rows of 768: 20 -> 13 us;
+// sum, the statistics and the normalised row, with all loads of a row issued at once (12 608 rows of 768: 20 -> 14 us;
 // read again from L1 / L2 for each of them, as longer and unaligned rows still are, a row was a chain of four round trips).
 // These are plain element-wise passes bound by HBM bandwidth: 1-2 reads and 1-2 writes of a [B, D] matrix.
 #pragma once
