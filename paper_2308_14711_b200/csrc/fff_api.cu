@@ -105,6 +105,7 @@ struct fff_handle_s {
     int max_bucket_clusters = 8;
     int32_t* last_perm = nullptr; // where the most recent forward left its leaf permutation
     bool bucketing_pending = false;   // the last forward skipped the leaf bucketing; ws_leaf holds its leaf indices
+    bool pending_in_staging = false;  // ... or, after a host-buffer forward in chunks, st_leaf
     int* ws_matrix = nullptr;     // per-CTA bin totals of the grid-wide bucketing kernel
     int coop_ctas = 0;            // CTAs of that kernel that are resident at once (0 = cooperative launch unavailable)
     int32_t* ws_perm2 = nullptr;  // second permutation buffer: successive bucketings alternate between the two
@@ -156,7 +157,7 @@ struct fff_handle_s {
     bool pdl = true;              // launch every kernel of a forward but the first as a programmatic dependent
     int launches = 0;
     int64_t last_B = -1;
-    int64_t plan_B = 0;           // chunk of a larger batch: the leaf kernel is chosen as for that many tokens (0: the call's own)
+    int64_t plan_B = 0;           // chunk of a larger batch: kernels that round differently are chosen as for that many tokens (0: the call's own)
 
     // optional per-launch timing of forwards (fff_profile_*)
     static constexpr int kMaxProfLaunches = 16;
@@ -1072,14 +1073,14 @@ fff_status_t pack_group_images(fff_handle_s* h) {
 // per tile), which costs more than it saves unless it also replaces a second descent stage and its node bucketing:
 // so only trees that the staged descent would cut in two.  The nodes three levels above the leaves must receive
 // whole tiles on average, and the lists must fit.
-bool use_group_tiles(const fff_handle_s* h, int64_t B) {
+bool use_group_tiles(const fff_handle_s* h, int64_t B, int64_t plan_B) {
     if (!h->g_w1 || !h->ws_slots || h->path == FFF_PATH_WARP || h->path == FFF_PATH_FUSED) return false;
     if (h->ustages.size() < 2) return false;
     if (!h->tune[FFF_TUNE_GROUP_TILES] || !h->tune[FFF_TUNE_TCGEN05_DESCENT] || !h->tune[FFF_TUNE_TCGEN05_LEAF] ||
         !h->tune[FFF_TUNE_DIRECT_LISTS])
         return false;
     const int64_t bins = h->n_leaves / fff::kLUGroup;
-    return B <= h->slot_cap && bins * h->slot_cap <= INT32_MAX && B >= fff::kLUM * bins;
+    return B <= h->slot_cap && bins * h->slot_cap <= INT32_MAX && plan_B >= fff::kLUM * bins;
 }
 
 // First stage (depth - 3 levels, files the tokens under the nodes it reaches), then the leaf kernel on grouped tiles,
@@ -1761,10 +1762,12 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     int32_t* leaf = leaf_idx ? leaf_idx : h->ws_leaf;
     h->launches = 0;
     h->last_B = B;
+    h->pending_in_staging = false;
     h->prof_active = h->prof_steps < h->prof_max_steps;
     if (h->prof_active)
         cudaEventRecord(h->prof_events[(size_t)h->prof_steps * (fff_handle_s::kMaxProfLaunches + 1)], st);
-    const bool token_blocks = use_token_block(h, B);
+    const int64_t plan_B = std::max(B, h->plan_B);
+    const bool token_blocks = use_token_block(h, plan_B);
     if (token_blocks || use_block_forward(h, B)) {
         // one launch: a CTA per token; or descent, grid barrier, leaves.  The stable bucketing is made on demand from the leaf
         // indices that are left in the workspace
@@ -1789,7 +1792,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     if (lazy_bucketing) leaf = h->ws_leaf;
     Coarse coarse;
     DescentTail tail;
-    const LeafPlan plan = tensor_leaf ? leaf_plan(h, std::max(B, h->plan_B)) : LeafPlan{};
+    const LeafPlan plan = tensor_leaf ? leaf_plan(h, plan_B) : LeafPlan{};
     const int tile_rows = plan.tile_rows;
     // The descent ends with a tcgen05 stage and a tensor-core leaf kernel follows: that stage files the tokens under their
     // leaves itself and the leaf kernel follows at once, on tiles it derives from the lists' counts.
@@ -1801,7 +1804,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
                    (h->ustages.size() == 1 || (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> h->ustages.back().L0) >= 64) ||
                     (h->ustages.size() == 2 && h->tune[FFF_TUNE_TCGEN05_GROUPED] && h->ws_nslots && B <= h->nslot_cap &&
                      (h->nslot_cap << h->ustages[0].k) <= INT32_MAX));
-    if (tensor_leaf && plan.umma && use_group_tiles(h, B)) {
+    if (tensor_leaf && plan.umma && use_group_tiles(h, B, plan_B)) {
         h->slots_now = false;
         s = run_forward_grouped(h, x, y, leaf, B, st);
         h->last_perm = h->ws_perm;
@@ -1873,6 +1876,19 @@ fff_status_t fff_forward_train(fff_handle_t h, const void* x, void* y, float* mi
     return run_forward_train(h, x, y, mixture, node_entropy, B, (cudaStream_t)cuda_stream);
 }
 
+// Chunks of a host-buffer forward: of 8192 tokens, or two for a smaller batch of at least 4 MB of x and y (less, and the
+// second chunk's submission and launches cost what the overlap saves), as long as the weights that a chunk fetches again cost
+// less than a quarter of its copies (16 times its bytes: memory is about 120 times as fast as the link).  One chunk against
+// two, us, 768 -> 768, bf16, 256 leaves of 12: 3 MB 104 and 104, 4 MB 128 and 115, 8 MB 193 and 174, 12 MB 272 and 242, 24 MB
+// 484 and 412; three or four are level with two or behind.  A smaller first or last chunk gains nothing: a copy that runs
+// while another one goes the other way costs about 7 us more than its bytes.
+static int host_chunks(const fff_handle_s* h, int64_t B) {
+    const int64_t per_token = (int64_t)(h->D + h->O) * (int64_t)h->esize, half = (B + 1) / 2;
+    const bool profiled = h->prof_steps < h->prof_max_steps;      // a profiled step is a whole forward
+    const bool halves = !profiled && B * per_token >= 4000000 && std::min<int64_t>(h->n_leaves, half) * h->l <= 16 * half;
+    return (int)std::max<int64_t>(halves ? 2 : 1, std::min<int64_t>(fff_handle_s::kMaxHostChunks, B / 8192));
+}
+
 fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_host, int32_t* leaf_idx_host,
                                     int64_t B, void* cuda_stream) {
     fff_status_t s = check_forward_args(h, B);
@@ -1890,9 +1906,9 @@ fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_
         h->cap_host_B = B;
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // Large batches go through in chunks so that the copy of chunk i+1 to the device, the kernels of chunk i
+    // Batches go through in chunks so that the copy of chunk i+1 to the device, the kernels of chunk i
     // and the copy of chunk i-1 back overlap (tokens are independent, so chunking does not change any result).
-    const int n_chunks = (int)std::max<int64_t>(1, std::min<int64_t>(fff_handle_s::kMaxHostChunks, B / 8192));
+    const int n_chunks = host_chunks(h, B);
     if (n_chunks == 1) {
         if (cudaMemcpyAsync(h->st_x, x_host, (size_t)B * h->D * h->esize, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return cudaGetLastError(), FFF_ERR_CUDA;
@@ -1916,20 +1932,23 @@ fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_
         if (!ok) return cudaGetLastError(), FFF_ERR_CUDA;
     }
     const int64_t chunk = (((B + n_chunks - 1) / n_chunks) + 127) & ~int64_t(127);
+    const int n_full = (int)((B + chunk - 1) / chunk);
     const size_t xrow = (size_t)h->D * h->esize, yrow = (size_t)h->O * h->esize;
+    auto copy_leaves = [&](int64_t from, int64_t to) {
+        return !leaf_idx_host || cudaMemcpyAsync(leaf_idx_host + from, h->st_leaf + from, (size_t)(to - from) * sizeof(int32_t),
+                                                 cudaMemcpyDeviceToHost, h->copy_out) == cudaSuccess;
+    };
     bool ok = cudaEventRecord(h->ev_start, st) == cudaSuccess &&              // the copies come after what the caller enqueued
               cudaStreamWaitEvent(h->copy_in, h->ev_start, 0) == cudaSuccess &&
               cudaStreamWaitEvent(h->copy_out, h->ev_start, 0) == cudaSuccess;
-    for (int c = 0; ok && c < n_chunks; ++c) {
+    for (int c = 0; ok && c < n_full; ++c) {
         const int64_t b0 = c * chunk, n = std::min(chunk, B - b0);
-        if (n <= 0) break;
         ok = cudaMemcpyAsync((char*)h->st_x + b0 * xrow, (const char*)x_host + b0 * xrow, (size_t)n * xrow, cudaMemcpyHostToDevice,
                              h->copy_in) == cudaSuccess &&
              cudaEventRecord(h->ev_in[c], h->copy_in) == cudaSuccess;
     }
-    for (int c = 0; ok && c < n_chunks; ++c) {
+    for (int c = 0; ok && c < n_full; ++c) {
         const int64_t b0 = c * chunk, n = std::min(chunk, B - b0);
-        if (n <= 0) break;
         ok = cudaStreamWaitEvent(st, h->ev_in[c], 0) == cudaSuccess;
         if (!ok) break;
         h->plan_B = B;           // results do not depend on the chunking
@@ -1939,12 +1958,15 @@ fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_
         ok = cudaEventRecord(h->ev_done[c], st) == cudaSuccess && cudaStreamWaitEvent(h->copy_out, h->ev_done[c], 0) == cudaSuccess &&
              cudaMemcpyAsync((char*)y_host + b0 * yrow, (char*)h->st_y + b0 * yrow, (size_t)n * yrow, cudaMemcpyDeviceToHost,
                              h->copy_out) == cudaSuccess &&
-             (!leaf_idx_host || cudaMemcpyAsync(leaf_idx_host + b0, h->st_leaf + b0, (size_t)n * sizeof(int32_t),
-                                                cudaMemcpyDeviceToHost, h->copy_out) == cudaSuccess);
+             (c != n_full - 2 || copy_leaves(0, b0 + n)) &&            // the leaves of all chunks but the last in one copy
+             (c != n_full - 1 || copy_leaves(n_full > 1 ? b0 : 0, b0 + n));
     }
     ok = ok && cudaEventRecord(h->ev_end, h->copy_out) == cudaSuccess && cudaStreamWaitEvent(st, h->ev_end, 0) == cudaSuccess &&
          cudaStreamSynchronize(st) == cudaSuccess;
-    h->last_B = -1;        // the workspace holds the last chunk only: no bucketing of the whole batch to report
+    // the workspace holds the last chunk only: the bucketing of a small batch is made on demand from the staged leaf indices,
+    // that of a large one is not reported
+    h->last_B = B < 16384 ? B : -1;
+    h->bucketing_pending = h->pending_in_staging = true;
     return ok ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
 }
 
@@ -1954,9 +1976,14 @@ fff_status_t fff_debug_get_bucketing(fff_handle_t h, int32_t* perm, int32_t* off
     DeviceGuard g(h->device);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if (h->last_B > 0 && h->bucketing_pending) {
+        if (h->pending_in_staging) {
+            const fff_status_t gs = grow_workspace(h, h->last_B);      // (it was sized for a chunk)
+            if (gs != FFF_OK) return gs;
+            h->last_perm = h->ws_perm;
+        }
         const int saved = h->launches;
         h->launches = 0;           // an ordinary launch: nothing of this call precedes it in the stream
-        const fff_status_t bs = run_bucket(h, h->ws_leaf, (int)h->n_leaves, Coarse(), h->ws_offsets, h->last_perm, h->last_B, st,
+        const fff_status_t bs = run_bucket(h, h->pending_in_staging ? h->st_leaf : h->ws_leaf, (int)h->n_leaves, Coarse(), h->ws_offsets, h->last_perm, h->last_B, st,
                                            0, "leaf_bucketing");
         h->launches = saved;
         if (bs != FFF_OK) return bs;
