@@ -140,6 +140,7 @@ struct fff_handle_s {
     std::vector<DenseStage> gstages;   // grouped tiles: one stage of depth - 3 levels
     // the same with a first stage of up to 8 levels on the tcgen05 kernel (empty = not available)
     std::vector<DenseStage> ustages;
+    DenseStage halves;                 // the levels of ustages[0] below the root as two images (k_descent_umma, halves = 1); NP = 0: none
     int32_t* ws_pos[2] = {nullptr, nullptr};
     int *d_status = nullptr;
 
@@ -275,6 +276,7 @@ void release(fff_handle_s* h) {
     dfree(h->d_status); dfree(h->st_x); dfree(h->st_y); dfree(h->st_leaf);
     for (auto& sg : h->stages) { dfree(sg.wimg); dfree(sg.bimg); }
     for (auto& sg : h->ustages) { dfree(sg.wimg); dfree(sg.bimg); }
+    dfree(h->halves.wimg); dfree(h->halves.bimg);
     for (auto& sg : h->gstages) { dfree(sg.wimg); dfree(sg.bimg); }
     dfree(h->g_w1); dfree(h->g_b1); dfree(h->g_w2);
     dfree(h->ws_pos[0]); dfree(h->ws_pos[1]);
@@ -647,22 +649,22 @@ int64_t balanced_grid(int64_t max_ctas, int64_t units) {
 
 template <int NP>
 fff_status_t launch_descent_umma(fff_handle_s* h, const fff_handle_s::DenseStage& sg, const void* x, int32_t* pos_out,
-                                 int64_t B, cudaStream_t st) {
+                                 int64_t B, cudaStream_t st, int halves = 0) {
     using L = fff::DescentUmmaLayout<NP>;
     const int stages = std::min((int)fff::kUmmaMaxStages, (kSmemBudget - L::smem_bytes(0)) / L::kStageBytes);
     if (stages < 2) return FFF_ERR_UNSUPPORTED;
     CUtensorMap tm;
     if (!make_x_tensor_map(&tm, x, B, h->D, fff::kUM)) return FFF_ERR_CUDA;
     const int64_t n_tiles = (B + fff::kUM - 1) / fff::kUM;
-    const int64_t grid = balanced_grid(h->sm_count, n_tiles);
-    const bool ranked = !h->nslots_here && sg.k >= 4 && h->ws_rank8 && h->ws_counts8;      // also rank the tokens for the bucketing that follows
+    const int64_t grid = halves ? 2 * n_tiles : balanced_grid(h->sm_count, n_tiles);
+    const bool ranked = !halves && !h->nslots_here && sg.k >= 4 && h->ws_rank8 && h->ws_counts8;      // also rank the tokens for the bucketing that follows
     int32_t* sums = nullptr;
     if (blocksum_for_descent(h, B, ranked, st, &sums) != FFF_OK) return FFF_ERR_CUDA;
     const SlotArgs sl = slot_args(h, pos_out);
     if (launch_chain(h, fff::k_descent_umma<NP>, (unsigned)grid, fff::kUmmaThreads, (size_t)L::smem_bytes(stages), st, 1, tm,
                      (const __nv_bfloat16*)sg.wimg, (const float*)sg.bimg, pos_out, ranked ? h->ws_rank8 : (uint8_t*)nullptr,
-                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, (int)B, sg.k,
-                     stages, h->d_status) != cudaSuccess)
+                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, (int)B, sg.k + halves,
+                     stages, halves, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "tree_descent_umma");
 }
@@ -702,6 +704,14 @@ fff_status_t run_descent_umma(fff_handle_s* h, const fff_handle_s::DenseStage& s
         if (sg.NP == 128) return launch_descent_umma_pair<128>(h, sg, x, pos_out, B, st);
         if (sg.NP == 256) return launch_descent_umma_pair<256>(h, sg, x, pos_out, B, st);
     }
+    // Two CTAs per tile while they are all resident at once (where the tokens are filed, not ranked: a rank needs the whole
+    // tile).  Forwards of the 768 -> 768 layer with 256 leaves of 12, one CTA and two: 600 tokens 18.8 and 17.4 us, 3152 19.2
+    // and 18.4, 6304 20.6 and 19.9, 9472 23.9 and 23.2; 256 -> 256: 3152 tokens 13.8 and 12.5; 1024 -> 1024, leaves of 24: 9472
+    // tokens 32.5 and 31.3; 7 levels: 17.2 and 17.0 at 1024.  A second round of tiles would cost more than half an image saves.
+    if (h->halves.NP != 0 && &sg == &h->ustages[0] && (h->slots_here || h->nslots_here) &&
+        2 * ((B + fff::kUM - 1) / fff::kUM) <= h->sm_count)
+        return h->halves.NP == 64 ? launch_descent_umma<64>(h, h->halves, x, pos_out, B, st, 1)
+                                  : launch_descent_umma<128>(h, h->halves, x, pos_out, B, st, 1);
     switch (sg.NP) {
         case 32: return launch_descent_umma<32>(h, sg, x, pos_out, B, st);
         case 64: return launch_descent_umma<64>(h, sg, x, pos_out, B, st);
@@ -872,7 +882,7 @@ fff_status_t pack_stage(fff_handle_s* h, std::vector<fff_handle_s::DenseStage>& 
     plan.push_back(sg);                            // owned by the handle from here on
     if ((s = dmalloc((void**)&plan.back().bimg, groups * sg.NP * 4)) != FFF_OK) return s;
     fff::k_pack_nodes<T><<<h->sm_count * 8, 256>>>((const T*)h->node_w, (const T*)h->node_b, plan.back().wimg, plan.back().bimg,
-                                                  sg.L0, sg.k, sg.NP, h->D, h->Dp);
+                                                  sg.L0, sg.k, sg.NP, h->D, h->Dp, false);
     return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
 }
 
@@ -912,6 +922,18 @@ fff_status_t pack_node_images(fff_handle_s* h) {
             const int np = i == 0 ? std::max(32, 1 << ks[i]) : std::max(16, 1 << ks[i]);
             if ((s = pack_stage<T>(h, h->ustages, L0, ks[i], np, true)) != FFF_OK) return s;
             L0 += ks[i];
+        }
+        if (ks[0] >= 7) {
+            auto& hv = h->halves;
+            hv.L0 = 1;
+            hv.k = ks[0] - 1;
+            hv.umma = true;
+            const int np = 1 << hv.k;
+            if ((s = dmalloc((void**)&hv.wimg, (size_t)2 * np * h->Dp * 2)) != FFF_OK) return s;
+            if ((s = dmalloc((void**)&hv.bimg, (size_t)2 * np * 4)) != FFF_OK) return s;
+            fff::k_pack_nodes<T><<<h->sm_count * 8, 256>>>((const T*)h->node_w, (const T*)h->node_b, hv.wimg, hv.bimg, hv.L0, hv.k, np,
+                                                          h->D, h->Dp, true);
+            hv.NP = np;
         }
         cudaFuncSetAttribute(fff::k_descent_umma<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         cudaFuncSetAttribute(fff::k_descent_umma<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);

@@ -55,11 +55,12 @@ template <int NP> struct DescentMmaLayout {
 
 // Weight image of one stage: [group][Dp/kKS][kKS/64][NP rows][64 columns] 128-byte swizzled, rows in the
 // subtree's breadth-first order (row 2^r - 1 + p = node N_{L0+r, g*2^r + p}); unused rows zero.
-// Bias image: [group][NP] float32.
+// Bias image: [group][NP] float32.  root_last (L0 = 1): row NP - 1, which a subtree of k levels leaves free at NP = 2^k, is the
+// root of the whole tree, in both groups.
 template <typename T>
 __global__ void k_pack_nodes(const T* __restrict__ node_w, const T* __restrict__ node_b,
                              __nv_bfloat16* __restrict__ img, float* __restrict__ bimg,
-                             int L0, int k, int NP, int D, int Dp)
+                             int L0, int k, int NP, int D, int Dp, bool root_last)
 {
     const int64_t groups = (int64_t)1 << L0;
     const int64_t total = groups * NP * Dp;
@@ -69,9 +70,10 @@ __global__ void k_pack_nodes(const T* __restrict__ node_w, const T* __restrict__
         const int64_t g = i / ((int64_t)Dp * NP);
         int r = 0;
         while (((1 << (r + 1)) - 1) <= n) ++r;                 // level of local node n inside the subtree
-        const bool used = r < k;
+        const bool root = root_last && n == NP - 1;
+        const bool used = r < k || root;
         const int64_t p = n - ((1 << r) - 1);
-        const int64_t row = used ? (((int64_t)1 << (L0 + r)) - 1 + g * ((int64_t)1 << r) + p) : 0;
+        const int64_t row = used && !root ? (((int64_t)1 << (L0 + r)) - 1 + g * ((int64_t)1 << r) + p) : 0;
         const int u = kk / kKS, sb = (kk % kKS) / 64, kc = kk % 64;
         const uint32_t off = ptx::swz128((uint32_t)((sb * NP + n) * 128 + kc * 2));
         const int64_t base = (g * (Dp / kKS) + u) * (int64_t)(NP * kKS);

@@ -127,12 +127,18 @@ template <int NP> struct DescentUmmaLayout {
 // consecutive tiles are added (integer atomics: the sums do not depend on the order).
 // pos_out2 (optional): a second copy of the positions.  cursor / slots / cap (optional, instead of the ranks):
 // see slot_tokens.
+//
+// halves = 1: two CTAs per tile, each for one half of the tree below the root.  Both evaluate the root (column NP - 1) and
+// the k - 1 levels below its left (even CTA) or right (odd) child, NP = 2^(k - 1) columns, and each keeps the tokens that
+// went its way: no exchange is needed.  For batches that leave more than half of the SMs idle: the stage then is the time in
+// which one SM pulls a tile of x and the node image through L2, and half the image and half the logits are left of it.
+// Image [2][D / 64][NP][64], grid = 2 * tiles.  Measured: see run_descent_umma in fff_api.cu.
 template <int NP>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* __restrict__ wimg,
                const float* __restrict__ bimg, int32_t* __restrict__ pos_out, uint8_t* __restrict__ rank8,
                uint8_t* __restrict__ counts8, int32_t* __restrict__ block_sums, int32_t* __restrict__ pos_out2,
-               int32_t* __restrict__ cursor, int32_t* __restrict__ slots, int cap, int D, int B, int k, int kStages,
+               int32_t* __restrict__ cursor, int32_t* __restrict__ slots, int cap, int D, int B, int k, int kStages, int halves,
                int* __restrict__ status)
 {
     using L = DescentUmmaLayout<NP>;
@@ -149,6 +155,9 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles = (B + kUM - 1) / kUM;
     const int KB = D / kUKB;
+    const int half = halves ? blockIdx.x & 1 : 0, first_tile = blockIdx.x >> halves, n_ctas = gridDim.x >> halves;
+    wimg += (int64_t)half * NP * D;
+    bimg += half * NP;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -180,7 +189,7 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
         // ------------------------------------------------------------------ producer
         int stage = 0;
         uint32_t phase = 0;
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        for (int tile = first_tile; tile < n_tiles; tile += n_ctas) {
             for (int kb = 0; kb < KB; ++kb) {
                 if (!timed_out && !ptx::mbar_wait_relaxed(empty + stage, phase ^ 1)) timed_out = true;
                 if (lane == 0) {
@@ -199,7 +208,7 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
         int stage = 0;
         uint32_t phase = 0;
         int it = 0;
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+        for (int tile = first_tile; tile < n_tiles; tile += n_ctas, ++it) {
             const int a = it & 1;
             if (!timed_out && !ptx::mbar_wait(acc_empty + a, ((it >> 1) & 1) ^ 1)) timed_out = true;
             ptx::tc_fence_after_sync();
@@ -226,7 +235,7 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
         // starts with a cold instruction cache, and the first real pass took ten times as long as the later ones
         // (measured: 11.6 us against 1.1 us per tile).  Where the loads run ahead anyway (64 nodes, 1024 inputs) that
         // hid behind them; with 256 nodes on single CTAs it was exposed (first stage of a 15-level tree: 18.4 -> 17.1 us).
-        for (int it = -1, tile = blockIdx.x; tile < n_tiles; ++it, tile += it > 0 ? gridDim.x : 0) {
+        for (int it = -1, tile = first_tile; tile < n_tiles; ++it, tile += it > 0 ? n_ctas : 0) {
             const bool dry = it < 0;
             const int a = it & 1;
             if (!dry && !timed_out && !ptx::mbar_wait(acc_full + a, (it >> 1) & 1)) timed_out = true;
@@ -236,10 +245,10 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
             ptx::tc_fence_before_sync();
             if (!dry) ptx::mbar_arrive(acc_empty + a);
 
-            const int p = umma_walk<NP>(bits, k);
+            const int p = umma_walk<NP>(bits, k - halves);
             const int tok = tile * kUM + warp * 32 + lane;
-            const int key = p - ((1 << k) - 1);
-            const bool in = !dry && tok < B;
+            const int key = (half << (k - 1)) + p - ((1 << (k - halves)) - 1);
+            const bool in = !dry && tok < B && (!halves || (int)(bits[NP / 32 - 1] >> 31) == half);
             if (in) {
                 pos_out[tok] = key;
                 if (pos_out2) pos_out2[tok] = key;
