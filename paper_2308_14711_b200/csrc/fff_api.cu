@@ -24,6 +24,7 @@
 #include "kernels/descent_warp.cuh"
 #include "kernels/gemm_umma.cuh"
 #include "kernels/leaf_mma.cuh"
+#include "kernels/leaf_mma_warp.cuh"
 #include "kernels/leaf_umma.cuh"
 #include "kernels/leaf_warp.cuh"
 #include "kernels/stack.cuh"
@@ -329,6 +330,7 @@ size_t max_tiles(const fff_handle_s* h, int64_t B) { return (size_t)(B / kMinTil
 struct LeafPlan {
     int tile_rows = 0;
     bool umma = false;
+    bool resident = false;         // the tiles of all leaves run at once
 };
 
 // Tiles of tile_rows rows that B tokens spread over the leaves fill, on average (a leaf's count is about Poisson).
@@ -360,7 +362,7 @@ LeafPlan leaf_plan(const fff_handle_s* h, int64_t B) {
     // and 19.6 against 24.6 at 6144 (32-row tiles), 22.7 against 25.8 at 8192 and 25.0 against 30.1 at 12 608 (64-row tiles);
     // a second round of tiles costs more than it saves: 38.3 against 34.0 at 16 384.
     for (int rows : {32, 64})
-        if (expected_tiles(h, B, rows) <= 0.98 * leaf_mma_slots(h, rows)) return LeafPlan{rows, false};
+        if (expected_tiles(h, B, rows) <= 0.98 * leaf_mma_slots(h, rows)) return LeafPlan{rows, false, true};
     // The tcgen05 kernel works on 128-row tiles.  Measured against the mma.sync kernel it is far ahead when
     // some buckets are large (skewed routing), about level with uniformly thin buckets of 32 tokens, and is
     // left out only when buckets are thinner still (tiles of at most 64 rows are stacked in the MMA rows, so the
@@ -369,6 +371,17 @@ LeafPlan leaf_plan(const fff_handle_s* h, int64_t B) {
         return LeafPlan{fff::kLUM, true};
     }
     return LeafPlan{B / h->n_leaves <= 40 ? 32 : 64, false};
+}
+
+// Whether a forward whose descent files the tokens runs a warp per tile of up to 16 tokens (k_leaf_mma_warp) instead: thin
+// buckets, more of them than CTAs at once.  Forwards, us, with the other kernels and with it: 768 -> 768, 2048 leaves of 12:
+// 2500 tokens 53.0 and 40.0, 8192 68.1 and 55.2, 16 384 75.6 and 69.1; 1024 leaves of 16: 2500 43.9 and 32.3, 12 000 48.8 and
+// 41.5; 512 leaves of 16: 8192 42.5 and 33.9, 16 384 47.2 and 42.6; 256 -> 256, 2048 leaves of 10: 8192 42.5 and 26.4, 24 000
+// 48.4 and 36.6.  It fetches a row in pieces of 64 bytes, which tells once the rows outweigh the weights: 1024 -> 1024, 2048
+// leaves of 16: 16 384 tokens (32 MB) 91.1 and 90.2, 20 000 94.8 and 100.9; 768 -> 768, 1024 leaves of 16: 32 768 73.2 and 85.5.
+bool warp_tiles(const fff_handle_s* h, const LeafPlan& plan, int64_t B) {
+    return h->LP == 16 && !plan.resident && h->n_leaves <= kMaxListedLeaves && B < 40 * h->n_leaves &&
+           B * h->D * h->esize <= ((int64_t)32 << 20);
 }
 
 bool use_tensor_leaf(const fff_handle_s* h) {
@@ -980,6 +993,16 @@ fff_status_t launch_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm
     return launched(h, st, "grouped_leaf_ff_mma");
 }
 
+fff_status_t launch_leaf_mma_warp(fff_handle_s* h, const void* x, const int32_t* slots, void* y, int64_t B, cudaStream_t st) {
+    const int64_t n_tiles = tile_list_len(B, fff::kLWRows, (int)h->n_leaves);
+    const int64_t grid = std::min<int64_t>((int64_t)h->sm_count * 2, n_tiles);
+    if (launch_chain(h, fff::k_leaf_mma_warp, (unsigned)grid, fff::kLWThreads, sizeof(int) * (size_t)(h->n_leaves + 1), st, 1,
+                     (const __nv_bfloat16*)x, slots, (const __nv_bfloat16*)h->w1img, (const float*)h->b1img, (const unsigned char*)h->w2img,
+                     (__nv_bfloat16*)y, h->D, h->Dp, h->O, h->act, h->ws_cursor, (int)h->n_leaves, (int)h->slot_cap) != cudaSuccess)
+        return cudaGetLastError(), FFF_ERR_CUDA;
+    return launched(h, st, "grouped_leaf_ff_mma_warp");
+}
+
 template <int LP, bool kFold, bool kW8 = false>
 fff_status_t launch_leaf_umma(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, int tile_rows,
                               cudaStream_t st) {
@@ -1027,6 +1050,7 @@ fff_status_t run_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm, v
                                       : launch_leaf_umma<64, false>(h, x, perm, y, B, tile_rows, st);
         }
     }
+    if (tile_rows == fff::kLWRows) return launch_leaf_mma_warp(h, x, perm, y, B, st);
     if (tile_rows == 32) {
         switch (h->LP) {
             case 16: return launch_leaf_mma<16, 32, 6>(h, x, perm, y, B, st);
@@ -1814,7 +1838,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     if (lazy_bucketing) leaf = h->ws_leaf;
     Coarse coarse;
     DescentTail tail;
-    const LeafPlan plan = tensor_leaf ? leaf_plan(h, plan_B) : LeafPlan{};
+    LeafPlan plan = tensor_leaf ? leaf_plan(h, plan_B) : LeafPlan{};
     const int tile_rows = plan.tile_rows;
     // The descent ends with a tcgen05 stage and a tensor-core leaf kernel follows: that stage files the tokens under their
     // leaves itself and the leaf kernel follows at once, on tiles it derives from the lists' counts.
@@ -1826,7 +1850,9 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
                    (h->ustages.size() == 1 || (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> h->ustages.back().L0) >= 64) ||
                     (h->ustages.size() == 2 && h->tune[FFF_TUNE_TCGEN05_GROUPED] && h->ws_nslots && B <= h->nslot_cap &&
                      (h->nslot_cap << h->ustages[0].k) <= INT32_MAX));
-    if (tensor_leaf && plan.umma && use_group_tiles(h, B, plan_B)) {
+    const bool group_tiles = tensor_leaf && plan.umma && use_group_tiles(h, B, plan_B);
+    if (h->slots_now && !group_tiles && !h->w8 && warp_tiles(h, plan, plan_B)) plan = LeafPlan{fff::kLWRows};
+    if (group_tiles) {
         h->slots_now = false;
         s = run_forward_grouped(h, x, y, leaf, B, st);
         h->last_perm = h->ws_perm;
