@@ -141,7 +141,7 @@ struct fff_handle_s {
     std::vector<DenseStage> gstages;   // grouped tiles: one stage of depth - 3 levels
     // the same with a first stage of up to 8 levels on the tcgen05 kernel (empty = not available)
     std::vector<DenseStage> ustages;
-    DenseStage halves;                 // the levels of ustages[0] below the root as two images (k_descent_umma, halves = 1); NP = 0: none
+    DenseStage halves;                 // the levels of ustages[0] below the root as two images (k_descent_umma<NP, true>); NP = 0: none
     int32_t* ws_pos[2] = {nullptr, nullptr};
     int *d_status = nullptr;
 
@@ -660,24 +660,24 @@ int64_t balanced_grid(int64_t max_ctas, int64_t units) {
     return (units + rounds - 1) / rounds;
 }
 
-template <int NP>
+template <int NP, bool kHalves = false>
 fff_status_t launch_descent_umma(fff_handle_s* h, const fff_handle_s::DenseStage& sg, const void* x, int32_t* pos_out,
-                                 int64_t B, cudaStream_t st, int halves = 0) {
+                                 int64_t B, cudaStream_t st) {
     using L = fff::DescentUmmaLayout<NP>;
     const int stages = std::min((int)fff::kUmmaMaxStages, (kSmemBudget - L::smem_bytes(0)) / L::kStageBytes);
     if (stages < 2) return FFF_ERR_UNSUPPORTED;
     CUtensorMap tm;
     if (!make_x_tensor_map(&tm, x, B, h->D, fff::kUM)) return FFF_ERR_CUDA;
     const int64_t n_tiles = (B + fff::kUM - 1) / fff::kUM;
-    const int64_t grid = halves ? 2 * n_tiles : balanced_grid(h->sm_count, n_tiles);
-    const bool ranked = !halves && !h->nslots_here && sg.k >= 4 && h->ws_rank8 && h->ws_counts8;      // also rank the tokens for the bucketing that follows
+    const int64_t grid = kHalves ? 2 * n_tiles : balanced_grid(h->sm_count, n_tiles);
+    const bool ranked = !kHalves && !h->nslots_here && sg.k >= 4 && h->ws_rank8 && h->ws_counts8;      // also rank the tokens for the bucketing that follows
     int32_t* sums = nullptr;
     if (blocksum_for_descent(h, B, ranked, st, &sums) != FFF_OK) return FFF_ERR_CUDA;
     const SlotArgs sl = slot_args(h, pos_out);
-    if (launch_chain(h, fff::k_descent_umma<NP>, (unsigned)grid, fff::kUmmaThreads, (size_t)L::smem_bytes(stages), st, 1, tm,
+    if (launch_chain(h, fff::k_descent_umma<NP, kHalves>, (unsigned)grid, fff::kUmmaThreads, (size_t)L::smem_bytes(stages), st, 1, tm,
                      (const __nv_bfloat16*)sg.wimg, (const float*)sg.bimg, pos_out, ranked ? h->ws_rank8 : (uint8_t*)nullptr,
-                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, (int)B, sg.k + halves,
-                     stages, halves, h->d_status) != cudaSuccess)
+                     ranked ? h->ws_counts8 : (uint8_t*)nullptr, sums, sl.pos2, sl.cursor, sl.slots, sl.cap, h->Dp, (int)B, sg.k + (kHalves ? 1 : 0),
+                     stages, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "tree_descent_umma");
 }
@@ -723,8 +723,8 @@ fff_status_t run_descent_umma(fff_handle_s* h, const fff_handle_s::DenseStage& s
     // tokens 32.5 and 31.3; 7 levels: 17.2 and 17.0 at 1024.  A second round of tiles would cost more than half an image saves.
     if (h->halves.NP != 0 && &sg == &h->ustages[0] && (h->slots_here || h->nslots_here) &&
         2 * ((B + fff::kUM - 1) / fff::kUM) <= h->sm_count)
-        return h->halves.NP == 64 ? launch_descent_umma<64>(h, h->halves, x, pos_out, B, st, 1)
-                                  : launch_descent_umma<128>(h, h->halves, x, pos_out, B, st, 1);
+        return h->halves.NP == 64 ? launch_descent_umma<64, true>(h, h->halves, x, pos_out, B, st)
+                                  : launch_descent_umma<128, true>(h, h->halves, x, pos_out, B, st);
     switch (sg.NP) {
         case 32: return launch_descent_umma<32>(h, sg, x, pos_out, B, st);
         case 64: return launch_descent_umma<64>(h, sg, x, pos_out, B, st);
@@ -948,10 +948,12 @@ fff_status_t pack_node_images(fff_handle_s* h) {
                                                           h->D, h->Dp, true);
             hv.NP = np;
         }
-        cudaFuncSetAttribute(fff::k_descent_umma<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-        cudaFuncSetAttribute(fff::k_descent_umma<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-        cudaFuncSetAttribute(fff::k_descent_umma<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-        cudaFuncSetAttribute(fff::k_descent_umma<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        cudaFuncSetAttribute(fff::k_descent_umma<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        cudaFuncSetAttribute(fff::k_descent_umma<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        cudaFuncSetAttribute(fff::k_descent_umma<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        cudaFuncSetAttribute(fff::k_descent_umma<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        cudaFuncSetAttribute(fff::k_descent_umma<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        cudaFuncSetAttribute(fff::k_descent_umma<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     }
     cudaFuncSetAttribute(fff::k_descent_mma<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     cudaFuncSetAttribute(fff::k_descent_mma<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);

@@ -128,17 +128,17 @@ template <int NP> struct DescentUmmaLayout {
 // pos_out2 (optional): a second copy of the positions.  cursor / slots / cap (optional, instead of the ranks):
 // see slot_tokens.
 //
-// halves = 1: two CTAs per tile, each for one half of the tree below the root.  Both evaluate the root (column NP - 1) and
+// kHalves: two CTAs per tile, each for one half of the tree below the root.  Both evaluate the root (column NP - 1) and
 // the k - 1 levels below its left (even CTA) or right (odd) child, NP = 2^(k - 1) columns, and each keeps the tokens that
 // went its way: no exchange is needed.  For batches that leave more than half of the SMs idle: the stage then is the time in
 // which one SM pulls a tile of x and the node image through L2, and half the image and half the logits are left of it.
 // Image [2][D / 64][NP][64], grid = 2 * tiles.  Measured: see run_descent_umma in fff_api.cu.
-template <int NP>
+template <int NP, bool kHalves>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* __restrict__ wimg,
                const float* __restrict__ bimg, int32_t* __restrict__ pos_out, uint8_t* __restrict__ rank8,
                uint8_t* __restrict__ counts8, int32_t* __restrict__ block_sums, int32_t* __restrict__ pos_out2,
-               int32_t* __restrict__ cursor, int32_t* __restrict__ slots, int cap, int D, int B, int k, int kStages, int halves,
+               int32_t* __restrict__ cursor, int32_t* __restrict__ slots, int cap, int D, int B, int k, int kStages,
                int* __restrict__ status)
 {
     using L = DescentUmmaLayout<NP>;
@@ -155,9 +155,13 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles = (B + kUM - 1) / kUM;
     const int KB = D / kUKB;
-    const int half = halves ? blockIdx.x & 1 : 0, first_tile = blockIdx.x >> halves, n_ctas = gridDim.x >> halves;
-    wimg += (int64_t)half * NP * D;
-    bimg += half * NP;
+    // (a template parameter: as an argument it cost the other form 0.3 us)
+    constexpr int halves = kHalves ? 1 : 0;
+    const int half = kHalves ? blockIdx.x & 1 : 0, first_tile = blockIdx.x >> halves, n_ctas = gridDim.x >> halves;
+    if constexpr (kHalves) {
+        wimg += (int64_t)half * NP * D;
+        bimg += half * NP;
+    }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -247,8 +251,8 @@ k_descent_umma(const __grid_constant__ CUtensorMap tmap_x, const __nv_bfloat16* 
 
             const int p = umma_walk<NP>(bits, k - halves);
             const int tok = tile * kUM + warp * 32 + lane;
-            const int key = (half << (k - 1)) + p - ((1 << (k - halves)) - 1);
-            const bool in = !dry && tok < B && (!halves || (int)(bits[NP / 32 - 1] >> 31) == half);
+            const int key = p - ((1 << (k - halves)) - 1) + (kHalves ? half << (k - 1) : 0);
+            const bool in = !dry && tok < B && (!kHalves || (int)(bits[NP / 32 - 1] >> 31) == half);
             if (in) {
                 pos_out[tok] = key;
                 if (pos_out2) pos_out2[tok] = key;
