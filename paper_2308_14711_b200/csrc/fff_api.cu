@@ -1246,14 +1246,20 @@ fff_status_t run_block_forward(fff_handle_s* h, const void* x, void* y, int32_t*
 // float32 7.5 / 9.1 / 16.8 us (18 / 20 / 20).  Past that the weights fetched token by token cost more than the launches:
 // 1024 tokens 19.5 against 19.4 us, 2048 34.6 against 20.6.  Trees that the staged descent cuts in two would run five
 // launches on thin groups: 1024 -> 1024, 2048 leaves of 32: 43 against 68 us at 1024 tokens, 79 against 97 at 2048, 149
-// against 94 at 4096; 512 leaves of 8: 18.6 against 33 at 1024, level at 2048.
+// against 94 at 4096.  With leaves of up to 16 neurons those launches end in a warp per tile, and two or two and a half rounds
+// of CTAs (four per SM) are the line: 768 -> 768, 1024 leaves of 16: 23.1 against 29.9 us at 1024 tokens, 33.7 against 30.7 at
+// 1500, 43.2 against 30.9 at 2048; 2048 leaves of 12: 24.9 against 34.6, 35.1 against 35.8, 45.0 against 37.6.
 constexpr int64_t kTokenBlockMaxB = 512, kTokenBlockMaxBDeep = 2048, kTokenBlockMaxBytes = (int64_t)96 << 20;
 
 bool use_token_block(const fff_handle_s* h, int64_t B) {
     if (h->w8 || h->path != FFF_PATH_AUTO || !h->tune[FFF_TUNE_TOKEN_BLOCKS]) return false;
     if (fff::TokenBlockLayout{h->D, h->l, (int)h->esize}.total() > 100 * 1024) return false;
     const bool two_stages = use_tensor_leaf(h) && h->ustages.size() >= 2;
-    if (two_stages) return B <= std::max(kTokenBlockMaxB, std::min(kTokenBlockMaxBDeep, 2 * h->n_leaves));
+    if (two_stages) {
+        const bool thin = h->LP == 16 && h->n_leaves <= kMaxListedLeaves && h->w2uimg;
+        const int64_t most = thin ? (int64_t)h->sm_count * (h->n_leaves > 1024 ? 10 : 8) : kTokenBlockMaxBDeep;
+        return B <= std::max(kTokenBlockMaxB, std::min(most, 2 * h->n_leaves));
+    }
     const int full = h->depth / fff::kTBLevels, rest = h->depth % fff::kTBLevels;
     const int64_t nodes = (int64_t)full * ((1 << fff::kTBLevels) - 1) + ((1 << rest) - 1);
     const int64_t per_token = (nodes * h->D + (int64_t)h->l * (h->D + h->O)) * (int64_t)h->esize;

@@ -23,7 +23,7 @@ TOKEN_BLOCKS = [
     C("tb_d8_staged_twice", 256, 1030, 8, 40, "gelu", "bf16", 300, "normal"),        # 82 KB of output weights per leaf
     C("tb_d7_unaligned_w2", 72, 7, 7, 3, "gelu_tanh", "bf16", 64, "normal"),         # 42-byte output matrices
     C("tb_d15", 128, 64, 15, 1, "gelu", "bf16", 257, "normal"),
-    C("tb_d10_two_stages", 128, 64, 10, 16, "gelu", "bf16", 2000, "clusters"),
+    C("tb_d10_two_stages", 128, 64, 10, 16, "gelu", "bf16", 1184, "clusters"),           # the most tokens it is taken for on 148 SMs
     C("tb_ragged_bf16", 101, 36, 5, 7, "gelu", "bf16", 100, "normal", node_bias_std=0.2),
 ]
 BLOCKS = [
