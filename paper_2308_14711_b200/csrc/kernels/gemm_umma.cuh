@@ -509,7 +509,12 @@ template <int DEPTH> struct TrainNodesLayout {
     static constexpr int kFixed = 1024 + 512 + NP * 4 + kGEpiWarps * kWarpStage;
     static constexpr int kStages = (kGSmemMax - kFixed) / kStageBytes < kGMaxStages ? (kGSmemMax - kFixed) / kStageBytes : kGMaxStages;
     static constexpr int kSmemBytes = kFixed + kStages * kStageBytes;
-    static constexpr int kTmemCols = 2 * NP < 64 ? 64 : 2 * NP;
+    // columns that one load brings of a part (of a narrow one more than it has), and tensor memory for all that the loads of the
+    // last part of the second accumulator touch: with 2 NP columns, those of trees of 5 and 6 levels ended 12 and 8 columns past it
+    static constexpr int kLoadCols = kPart == 32 ? 32 : 16;
+    static constexpr int kTouched = NP + ((1 << T) - 1) * kPart + kLoadCols;
+    static constexpr int kTmemCols = kTouched <= 64 ? 64 : kTouched <= 128 ? 128 : kTouched <= 256 ? 256 : 512;
+    static_assert(kTouched <= kTmemCols && 2 * NP <= kTmemCols, "both accumulators and every load lie inside the allocation");
     static_assert(4 * NP * 4 <= kStages * kStageBytes, "the entropy sums take the ring's place at the end");
 };
 
@@ -612,7 +617,7 @@ k_train_nodes(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                 float z[32];
                 {
                     uint32_t v[32];
-                    if (PART == 32) ptx::tmem_ld32(tq + p * PART, v);
+                    if (L::kLoadCols == 32) ptx::tmem_ld32(tq + p * PART, v);
                     else {
                         uint32_t v16[16];
                         ptx::tmem_ld16(tq + p * PART, v16);               // (columns past the part are not used)

@@ -26,6 +26,10 @@ CASES = [
     C("train_d6_l23_wide_tiles", 128, 192, 6, 23, "gelu", "bf16", 4100, "normal", node_bias_std=0.2),
     C("train_d7_l9", 128, 64, 7, 9, "relu", "bf16", 513, "layernorm"),
     C("train_d9_l2", 64, 64, 9, 2, "gelu", "bf16", 300, "normal"),
+    # more tiles than pairs of CTAs (256 tokens each, 74 pairs): the second accumulator, whose last part is read past the tree's
+    # columns where parts are narrower than a load
+    C("train_d5_second_accumulator", 64, 32, 5, 4, "gelu", "bf16", 19300, "normal", node_bias_std=0.2),
+    C("train_d6_second_accumulator", 64, 32, 6, 4, "relu", "bf16", 19300, "normal", node_bias_std=0.2),
     C("train_d5_l7_odd_output", 128, 44, 5, 7, "gelu_tanh", "bf16", 200, "normal"),
 ]
 
