@@ -223,11 +223,18 @@ fff_status_t dmalloc(void** p, size_t bytes) {
 
 void dfree(void* p) { if (p) cudaFree(p); }
 
+// Copies of device memory and memsets go to the default stream and return before they are done; a caller's non-blocking stream
+// does not wait for that stream, so what is allocated on behalf of a call in progress is waited for here.
+fff_status_t default_stream_done(cudaError_t e) {
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    return e == cudaSuccess ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
+}
+
+// A copy of `src`, or zeroes; in place for every stream when the call returns.
 fff_status_t clone(void** dst, const void* src, size_t bytes) {
     fff_status_t s = dmalloc(dst, bytes);
     if (s != FFF_OK) return s;
-    cudaError_t e = src ? cudaMemcpy(*dst, src, bytes, cudaMemcpyDeviceToDevice) : cudaMemset(*dst, 0, bytes ? bytes : 16);
-    return e == cudaSuccess ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
+    return default_stream_done(src ? cudaMemcpy(*dst, src, bytes, cudaMemcpyDeviceToDevice) : cudaMemset(*dst, 0, bytes ? bytes : 16));
 }
 
 // Launch a kernel of the forward chain.  Every launch after the first of a call carries the
@@ -1420,8 +1427,8 @@ fff_status_t run_forward_train(fff_handle_s* h, const void* x, void* y, float* m
         if ((s = dmalloc((void**)&h->tr_hp, sizeof(__nv_bfloat16) * (size_t)B * h->tr_Kp)) != FFF_OK) return s;
         // the columns of h' past the mixture weights stay zero
         const int pad = h->tr_Kp - (int)(hidden + nl);
-        if (pad > 0 && cudaMemset2D(h->tr_hp + hidden + nl, (size_t)h->tr_Kp * 2, 0, (size_t)pad * 2, (size_t)B) != cudaSuccess)
-            return cudaGetLastError(), FFF_ERR_CUDA;
+        if (pad > 0 && (s = default_stream_done(cudaMemset2D(h->tr_hp + hidden + nl, (size_t)h->tr_Kp * 2, 0, (size_t)pad * 2, (size_t)B))) != FFF_OK)
+            return s;
         h->tr_cap_B = B;
     }
     fff_status_t s = FFF_OK;
@@ -2065,8 +2072,8 @@ fff_status_t fff_get_last_status(fff_handle_t h) {
     int word = 0;
     if (cudaMemcpy(&word, h->d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
     if (word != fff::kDevOk) {
-        cudaMemset(h->d_status, 0, sizeof(int));
-        return FFF_ERR_DEVICE_TIMEOUT;
+        const fff_status_t cs = default_stream_done(cudaMemset(h->d_status, 0, sizeof(int)));
+        return cs != FFF_OK ? cs : FFF_ERR_DEVICE_TIMEOUT;
     }
     return FFF_OK;
 }
