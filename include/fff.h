@@ -292,7 +292,9 @@ fff_status_t fff_grouped_leaf_ff(fff_handle_t h, const void *x, const int32_t *l
  * about 4 tokens per leaf, which evaluates the leaves one token at a time, and one
  * whose descent files the tokens under their leaves directly for the tensor-core
  * leaf kernel (in an order that is not the stable one).  The bucketing is then
- * computed here, from the leaf indices the forward kept in the handle's workspace. */
+ * computed here, from the leaf indices the forward kept in the handle's workspace.
+ * Once a later call (fff_reserve among them) has enlarged the buffers that held them,
+ * there is nothing to report (FFF_ERR_INVALID_ARG) until the next fff_forward_infer. */
 fff_status_t fff_debug_get_bucketing(fff_handle_t h, int32_t *perm, int32_t *offsets,
                                      void *cuda_stream);
 

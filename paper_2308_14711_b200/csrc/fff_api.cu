@@ -400,6 +400,8 @@ bool use_tensor_leaf(const fff_handle_s* h) {
 fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
     if (B <= h->cap_B) return FFF_OK;
     if (cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
+    // the last forward's permutation and leaf indices go with the buffers (a bucketing still to be made from the staging buffers stays)
+    if (!(h->pending_in_staging && h->bucketing_pending)) h->last_B = -1;
     dfree(h->ws_leaf); dfree(h->ws_perm); dfree(h->ws_perm2); dfree(h->ws_tiles); dfree(h->ws_rank); dfree(h->ws_pos[0]);
     dfree(h->ws_rank8); dfree(h->ws_counts8); dfree(h->ws_blocksum); dfree(h->ws_slots); dfree(h->ws_cursor); dfree(h->ws_nslots);
     dfree(h->ws_ncursor);
@@ -1961,6 +1963,8 @@ fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_
     DeviceGuard g(h->device);
     if (B > h->cap_host_B) {
         if (cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
+        h->last_B = -1;                     // (a bucketing made on demand would read the leaf indices that are freed here)
+        h->pending_in_staging = false;
         dfree(h->st_x); dfree(h->st_y); dfree(h->st_leaf);
         h->st_x = h->st_y = nullptr; h->st_leaf = nullptr; h->cap_host_B = 0;
         if ((s = dmalloc(&h->st_x, (size_t)B * h->D * h->esize)) != FFF_OK) return s;
@@ -2028,7 +2032,7 @@ fff_status_t fff_forward_infer_host(fff_handle_t h, const void* x_host, void* y_
          cudaStreamSynchronize(st) == cudaSuccess;
     // the workspace holds the last chunk only: the bucketing of a small batch is made on demand from the staged leaf indices,
     // that of a large one is not reported
-    h->last_B = B < 16384 ? B : -1;
+    h->last_B = ok && B < 16384 ? B : -1;
     h->bucketing_pending = h->pending_in_staging = true;
     return ok ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
 }

@@ -1,9 +1,9 @@
 """The first call of a size on a stream that does not wait for the default stream (every stream that torch makes): what the call
-allocates and clears has to be clear before the call's own kernels run."""
+allocates and clears has to be clear before the call's own kernels run.  And what such a call replaces is not read again."""
 import pytest
 import torch
 
-from paper_2308_14711_b200 import workloads as wl
+from paper_2308_14711_b200 import binding, workloads as wl
 from tests import util
 
 pytestmark = pytest.mark.gpu
@@ -61,3 +61,42 @@ def test_first_forward_infer_on_a_side_stream(cfg):
             assert torch.equal(a, b)
             assert a.dtype != torch.int32 or torch.equal(a[: cfg.B // 3], c)
         layer.close()
+
+
+@pytest.mark.parametrize("B", [100, 4000])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_no_bucketing_once_its_buffers_are_gone(dtype, B):
+    """The bucketing of the last forward is made on demand from buffers that a larger batch replaces."""
+    cfg = C("gone", 128, 64, 5, 8, "relu", dtype, B, "normal")
+    case = util.make_case(cfg, seed=1)
+    layer = util.make_layer(case)
+    x = util.to_device(case.x, dtype)
+    layer.forward_infer(x)
+    layer.reserve(20000)
+    with pytest.raises(binding.FFFError) as e:
+        layer.last_bucketing(B)
+    assert e.value.status == 1
+    _, leaf = layer.forward_infer(x)
+    _, perm = layer.last_bucketing(B)
+    assert torch.equal(perm.long(), torch.argsort(leaf.long(), stable=True))
+    layer.close()
+
+
+def test_no_bucketing_from_staging_buffers_that_are_gone():
+    """A host-buffer forward in chunks, then one whose staging buffers cannot be allocated."""
+    cfg = C("gone_staging", 1024, 1024, 3, 8, "relu", "bf16", 1200, "normal")
+    case = util.make_case(cfg, seed=1)
+    layer = util.make_layer(case)
+    xh = util.to_device(case.x, "bf16").cpu().pin_memory()
+    yh, lh = torch.empty_like(xh), torch.empty(cfg.B, dtype=torch.int32)
+    layer.forward_infer_host(xh, yh, lh)
+    too_many = 1 << 27                                     # 256 GiB of rows: the host pointers are not looked at
+    status = binding.lib().fff_forward_infer_host(layer._h, xh.data_ptr(), yh.data_ptr(), lh.data_ptr(), too_many, None)
+    assert binding.STATUS_NAMES[status] in ("FFF_ERR_ALLOC", "FFF_ERR_UNSUPPORTED")
+    with pytest.raises(binding.FFFError) as e:
+        layer.last_bucketing(cfg.B)
+    assert e.value.status == 1
+    layer.forward_infer_host(xh, yh, lh)
+    _, perm = layer.last_bucketing(cfg.B)
+    assert torch.equal(perm.cpu().long(), torch.argsort(lh.long(), stable=True))
+    layer.close()
