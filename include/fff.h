@@ -178,15 +178,18 @@ fff_status_t fff_destroy(fff_handle_t h);
 
 /* Size the workspace for batches of up to max_B tokens so that later forwards
  * allocate nothing.  Allocates and synchronises.  The workspace is a few
- * int32 per token, plus, on the tensor-core path, a table of per-leaf token
- * lists of 2^depth * max_B int32 (only while that is at most 1 GiB; larger
- * layers run a bucketing kernel instead), of which a forward touches B entries;
+ * int32 per token, plus a table of per-leaf token lists of 2^depth * max_B
+ * int32, of which a forward touches B entries: on the tensor-core path only
+ * while that is at most 1 GiB (larger layers run a bucketing kernel instead), on
+ * the one-launch kernel of float32 and odd shapes (FFF_TUNE_FUSED_SMALL) never
+ * more than 1 GiB (larger batches run it several times, with the same results);
  * trees whose descent runs as two tensor-core stages add a table of per-node
- * lists between the stages (at most 256 * max_B int32, same rule). */
+ * lists between the stages (at most 256 * max_B int32, only up to 1 GiB). */
 fff_status_t fff_reserve(fff_handle_t h, int64_t max_B);
 
 /* Pin the handle to one kernel family (FFF_PATH_*).  FFF_ERR_UNSUPPORTED if
- * the shapes of this handle cannot run on it. */
+ * the shapes of this handle cannot run on it.  May allocate: the workspace that
+ * fff_reserve has sized is completed by what the family needs. */
 fff_status_t fff_set_path(fff_handle_t h, fff_path_t path);
 
 /* Switches between kernels that compute the same thing, for A/B timing and tests.  Every switch is on (1) by

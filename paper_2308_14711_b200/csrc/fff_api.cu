@@ -397,6 +397,16 @@ bool use_tensor_leaf(const fff_handle_s* h) {
     return h->path == FFF_PATH_TENSOR || h->l >= 8;
 }
 
+// Tokens for which the leaves' lists stay within kMaxSlotBytes, and the fewest that k_block_forward is given at a time.
+int64_t listed_tokens(const fff_handle_s* h) { return (int64_t)(kMaxSlotBytes / sizeof(int32_t)) / h->n_leaves; }
+constexpr int64_t kMinListedTokens = 1024;
+
+// Whether forwards of this handle, as it is pinned now, run as the one-launch kernel on CUDA cores: the layers without a
+// tensor-core leaf path, and those pinned to it.  Shapes and the path alone decide, not what the handle has served before.
+bool runs_block_forward(const fff_handle_s* h) {
+    return h->bf_per_sm > 0 && (h->path == FFF_PATH_FUSED || (h->path == FFF_PATH_AUTO && h->LP == 0));
+}
+
 fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
     if (B <= h->cap_B) return FFF_OK;
     if (cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
@@ -431,14 +441,22 @@ fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
     }
     if ((s = dmalloc((void**)&h->ws_tiles, sizeof(fff::Tile) * max_tiles(h, B))) != FFF_OK) return s;
     // direct lists: every leaf's list can take the whole batch, so their size grows with n_leaves * B; beyond
-    // kMaxSlotBytes the forward keeps the bucketing kernel instead
+    // kMaxSlotBytes the forward keeps the bucketing kernel instead.  k_block_forward has no other way: for the layers that
+    // run it the table stops growing there, and larger batches go through it in parts.
     const bool filed_by_descent = !h->ustages.empty() && h->ustages.back().umma &&
                                   h->ustages.back().L0 + h->ustages.back().k == h->depth && (h->w2uimg || h->w2codes);
-    if ((filed_by_descent || (h->bf_per_sm > 0 && (h->LP == 0 || h->bf_pinnable))) &&
-        (size_t)h->n_leaves * (size_t)B * sizeof(int32_t) <= kMaxSlotBytes) {
-        if ((s = dmalloc((void**)&h->ws_slots, sizeof(int32_t) * (size_t)h->n_leaves * (size_t)B)) != FFF_OK) return s;
+    const int64_t most = listed_tokens(h);
+    if (runs_block_forward(h) || ((filed_by_descent || (h->bf_per_sm > 0 && h->bf_pinnable)) && B <= most)) {
+        int64_t cap = std::min(B, most);
+        s = dmalloc((void**)&h->ws_slots, sizeof(int32_t) * (size_t)h->n_leaves * (size_t)cap);
+        // (short of memory: smaller parts)
+        while (s != FFF_OK && runs_block_forward(h) && cap > kMinListedTokens) {
+            cap = std::max(cap / 4 & ~int64_t(15), kMinListedTokens);
+            s = dmalloc((void**)&h->ws_slots, sizeof(int32_t) * (size_t)h->n_leaves * (size_t)cap);
+        }
+        if (s != FFF_OK) return s;
         if ((s = clone((void**)&h->ws_cursor, nullptr, sizeof(int32_t) * (size_t)(h->n_leaves + 1))) != FFF_OK) return s;
-        h->slot_cap = B;
+        h->slot_cap = cap;
         h->cursor_dirty = false;
     }
     // node lists for trees whose descent runs as two tcgen05 stages (a forward decides: the stages it runs depend on B):
@@ -1204,20 +1222,18 @@ fff_status_t plan_block_forward(fff_handle_s* h) {
 }
 
 // Whether a forward of this handle runs as the one-launch kernel: when pinned to it, or by default for layers that have no
-// tensor-core leaf path (float32, or bf16 shapes outside it); the table of the leaves' token lists must fit.  Measured
-// against what it replaces, one warp per token (three launches) or, for small trees, a kernel that kept 32 hidden neurons
-// per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44 against 110 us; 1000 -> 992, 512 leaves
-// of 32, 8192 tokens 156 against 1148; 512 -> 512, 32 leaves of 16, 8192 tokens 32 against 429; 784 -> 10, 8 leaves of 32,
-// 2048 tokens 18 against 20.  CTAs per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
-bool use_block_forward(const fff_handle_s* h, int64_t B) {
-    if (h->bf_per_sm == 0 || !h->tune[FFF_TUNE_FUSED_SMALL] || !h->ws_slots || B > h->slot_cap) return false;
-    if (h->path == FFF_PATH_FUSED) return true;
-    return h->path == FFF_PATH_AUTO && h->LP == 0;
+// tensor-core leaf path.  Measured against what it replaces, one warp per token (three launches) or, for small trees, a kernel
+// that kept 32 hidden neurons per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44 against 110 us,
+// 50 432 tokens 289 against 646; 1000 -> 992, 512 leaves of 32, 8192 tokens 156 against 1148; 512 -> 512, 32 leaves of 16, 8192
+// tokens 32 against 429; 784 -> 10, 8 leaves of 32, 2048 tokens 18 against 20; 256 -> 64, one leaf of 16, 65 536 tokens 122
+// against 329.  CTAs per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
+bool use_block_forward(const fff_handle_s* h) {
+    return runs_block_forward(h) && h->ws_slots && h->tune[FFF_TUNE_FUSED_SMALL];
 }
 
 template <typename T>
-fff_status_t run_block_forward(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B,
-                               cudaStream_t st) {
+fff_status_t launch_block_forward(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B,
+                                  cudaStream_t st) {
     if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     h->cursor_dirty = true;
@@ -1246,6 +1262,18 @@ fff_status_t run_block_forward(fff_handle_s* h, const void* x, void* y, int32_t*
         return cudaGetLastError(), FFF_ERR_CUDA;
     const fff_status_t s = launched(h, st, "fused_forward_blocks");
     if (s == FFF_OK) h->cursor_dirty = false;
+    return s;
+}
+
+// In parts of as many tokens as the lists hold (a part's rows start on 16-byte boundaries where the batch's do: slot_cap is a
+// multiple of 16 whenever there is more than one).
+template <typename T>
+fff_status_t run_block_forward(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B,
+                               cudaStream_t st) {
+    fff_status_t s = FFF_OK;
+    for (int64_t b0 = 0; b0 < B && s == FFF_OK; b0 += h->slot_cap)
+        s = launch_block_forward<T>(h, (const T*)x + b0 * h->D, (T*)y + b0 * h->O, leaf_out + b0, leaf_out2 ? leaf_out2 + b0 : nullptr,
+                                    std::min(h->slot_cap, B - b0), st);
     return s;
 }
 
@@ -1760,6 +1788,12 @@ fff_status_t fff_set_path(fff_handle_t h, fff_path_t path) {
     if (path == FFF_PATH_FUSED && !h->bf_pinnable) return FFF_ERR_UNSUPPORTED;
     if (h->w8 && path != FFF_PATH_AUTO && path != FFF_PATH_TENSOR) return FFF_ERR_UNSUPPORTED;
     h->path = path;
+    if (runs_block_forward(h) && h->cap_B > 0 && !h->ws_slots) {      // a workspace sized without its lists
+        DeviceGuard g(h->device);
+        const int64_t B = h->cap_B;
+        h->cap_B = 0;
+        return grow_workspace(h, B);
+    }
     return FFF_OK;
 }
 
@@ -1831,7 +1865,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
         cudaEventRecord(h->prof_events[(size_t)h->prof_steps * (fff_handle_s::kMaxProfLaunches + 1)], st);
     const int64_t plan_B = std::max(B, h->plan_B);
     const bool token_blocks = use_token_block(h, plan_B);
-    if (token_blocks || use_block_forward(h, B)) {
+    if (token_blocks || use_block_forward(h)) {
         // one launch: a CTA per token; or descent, grid barrier, leaves.  The stable bucketing is made on demand from the leaf
         // indices that are left in the workspace
         s = token_blocks ? FFF_DISPATCH(h, run_token_block, h, x, y, h->ws_leaf, leaf_idx, B, st)

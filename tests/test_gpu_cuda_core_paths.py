@@ -71,3 +71,52 @@ def test_token_blocks_match_the_oracle(cfg):
 @pytest.mark.parametrize("cfg", BLOCKS, ids=lambda c: c.name)
 def test_block_forward_matches_the_oracle(cfg):
     check(cfg, "fused_small", seed=8)
+
+
+def launches_of(layer, x):
+    layer.profile_begin(1)
+    layer.forward_infer(x)
+    torch.cuda.synchronize()
+    return [n for n, _ in layer.profile_end()[0]]
+
+
+def test_the_batches_served_before_do_not_choose_the_kernel():
+    """4096 leaves: the lists of more than 65 536 tokens would pass 1 GiB."""
+    cfg = C("bf_state", 32, 24, 12, 4, "gelu", "f32", 2000, "normal")
+    case = util.make_case(cfg, seed=3)
+    layer = util.make_layer(case)
+    x = util.to_device(case.x, "f32")
+    names = launches_of(layer, x)
+    y, leaf = layer.forward_infer(x)
+    layer.reserve(70000)
+    assert launches_of(layer, x) == names == ["fused_forward_blocks"]
+    y2, leaf2 = layer.forward_infer(x)
+    assert torch.equal(y, y2) and torch.equal(leaf, leaf2)
+    layer.close()
+
+
+@pytest.mark.parametrize("pin_first", [True, False])
+def test_batches_past_the_lists_run_in_parts(pin_first):
+    cfg = C("bf_parts", 16, 24, 12, 1, "relu", "f32", 65536 + 1603, "normal", node_bias_std=0.1)
+    case = util.make_case(cfg, seed=4)
+    y_ref, leaf_ref = orc.forward_i(case.net, case.x, threads=util.ORACLE_THREADS)
+    off_ref, perm_ref = orc.bucket(leaf_ref, cfg.n_leaves)
+    layer = util.make_layer(case, path="fused" if pin_first else "auto")
+    x = util.to_device(case.x, "f32")
+    if not pin_first:
+        layer.set_path("warp")
+        layer.reserve(cfg.B)
+        layer.set_path("fused")
+    for _ in range(2):
+        y, leaf = layer.forward_infer(x)
+        torch.cuda.synchronize()
+        assert layer.last_launch_count() == 2
+        np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
+        util.check_outputs(y, y_ref, "f32")
+    off, perm = layer.last_bucketing(cfg.B)
+    np.testing.assert_array_equal(off.cpu().numpy(), off_ref)
+    np.testing.assert_array_equal(perm.cpu().numpy(), perm_ref)
+    layer.set_path("warp")                                 # one warp per token: the same sums in the same order
+    y2, leaf2 = layer.forward_infer(x)
+    assert torch.equal(y2, y) and torch.equal(leaf2, leaf)
+    layer.close()
