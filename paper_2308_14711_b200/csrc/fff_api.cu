@@ -811,7 +811,27 @@ const std::vector<fff_handle_s::DenseStage>& stage_plan(const fff_handle_s* h) {
     return h->ustages.empty() || !h->tune[FFF_TUNE_TCGEN05_DESCENT] ? h->stages : h->ustages;
 }
 
-int dense_stage_count(const fff_handle_s* h, int64_t B) {
+// Tokens that a call of B is planned for: those of the whole batch when it is one chunk of several.  Everything that chooses
+// between kernels which round differently goes by this number; only capacities go by the chunk's own.
+int64_t planned_tokens(const fff_handle_s* h, int64_t B) { return std::max(B, h->plan_B); }
+
+// Whether a later descent stage's groups fill 128-row tiles well enough.
+bool fills_grouped_tiles(const fff_handle_s* h, int64_t B, int L0) { return (planned_tokens(h, B) >> L0) >= 64; }
+
+// Whether the lists between the first and the second descent stage hold this call's tokens (and would hold the whole batch's).
+bool node_lists_fit(const fff_handle_s* h, int64_t B) {
+    const int k = h->ustages[0].k;
+    return h->ws_nslots && B <= h->nslot_cap && (h->nslot_cap << k) <= INT32_MAX &&      // (a tile's start is an int)
+           ((size_t)planned_tokens(h, B) << k) * sizeof(int32_t) <= kMaxSlotBytes;
+}
+
+// Likewise the leaves' lists.
+bool leaf_lists_fit(const fff_handle_s* h, int64_t B) {
+    return h->ws_slots && B <= h->slot_cap && h->n_leaves * h->slot_cap <= INT32_MAX && planned_tokens(h, B) <= listed_tokens(h);
+}
+
+int dense_stage_count(const fff_handle_s* h, int64_t call_B) {
+    const int64_t B = planned_tokens(h, call_B);
     const auto& plan = stage_plan(h);
     if (plan.empty() || h->path == FFF_PATH_WARP) return 0;
     if (h->path == FFF_PATH_TENSOR) return (int)plan.size();
@@ -852,8 +872,7 @@ fff_status_t run_descent(fff_handle_s* h, const void* x, int32_t* leaf_out, Coar
     const auto& plan = stage_plan(h);
     // Two tcgen05 stages and nobody downstream who would refine the node bucketing: the first stage files the tokens
     // under the nodes it reaches and the second derives its tiles from the counts; no bucketing launch in between.
-    const bool node_lists = n_dense == 2 && &plan == &h->ustages && plan[0].umma && plan[1].umma && h->ws_nslots &&
-                            B <= h->nslot_cap && (h->nslot_cap << plan[0].k) <= INT32_MAX &&      // (a tile's start is an int)
+    const bool node_lists = n_dense == 2 && &plan == &h->ustages && plan[0].umma && plan[1].umma && node_lists_fit(h, B) &&
                             h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_GROUPED] &&
                             (coarse == nullptr || defer_tail != nullptr);
     if (node_lists) {
@@ -867,7 +886,7 @@ fff_status_t run_descent(fff_handle_s* h, const void* x, int32_t* leaf_out, Coar
         const auto& sg = plan[i];
         // later stages: the tcgen05 kernel on 128-row tiles when the groups fill them reasonably, else mma.sync on 64-row tiles
         // (with node lists there is no bucketing launch that the thinner tiles would have to pay for)
-        const bool grouped_umma = i > 0 && sg.umma && h->tune[FFF_TUNE_TCGEN05_GROUPED] && (node_lists || (B >> sg.L0) >= 64);
+        const bool grouped_umma = i > 0 && sg.umma && h->tune[FFF_TUNE_TCGEN05_GROUPED] && (node_lists || fills_grouped_tiles(h, B, sg.L0));
         if (i > 0 && !node_lists) {
             // bucket by the node reached so far; buffers alternate so that the previous level stays readable
             int32_t* perm_out = (i & 1) ? h->ws_perm2 : h->ws_perm;
@@ -1148,14 +1167,14 @@ fff_status_t pack_group_images(fff_handle_s* h) {
 // per tile), which costs more than it saves unless it also replaces a second descent stage and its node bucketing:
 // so only trees that the staged descent would cut in two.  The nodes three levels above the leaves must receive
 // whole tiles on average, and the lists must fit.
-bool use_group_tiles(const fff_handle_s* h, int64_t B, int64_t plan_B) {
-    if (!h->g_w1 || !h->ws_slots || h->path == FFF_PATH_WARP || h->path == FFF_PATH_FUSED) return false;
+bool use_group_tiles(const fff_handle_s* h, int64_t B) {
+    if (!h->g_w1 || h->path == FFF_PATH_WARP || h->path == FFF_PATH_FUSED) return false;
     if (h->ustages.size() < 2) return false;
     if (!h->tune[FFF_TUNE_GROUP_TILES] || !h->tune[FFF_TUNE_TCGEN05_DESCENT] || !h->tune[FFF_TUNE_TCGEN05_LEAF] ||
         !h->tune[FFF_TUNE_DIRECT_LISTS])
         return false;
     const int64_t bins = h->n_leaves / fff::kLUGroup;
-    return B <= h->slot_cap && bins * h->slot_cap <= INT32_MAX && plan_B >= fff::kLUM * bins;
+    return leaf_lists_fit(h, B) && planned_tokens(h, B) >= fff::kLUM * bins;
 }
 
 // First stage (depth - 3 levels, files the tokens under the nodes it reaches), then the leaf kernel on grouped tiles,
@@ -1863,7 +1882,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     h->prof_active = h->prof_steps < h->prof_max_steps;
     if (h->prof_active)
         cudaEventRecord(h->prof_events[(size_t)h->prof_steps * (fff_handle_s::kMaxProfLaunches + 1)], st);
-    const int64_t plan_B = std::max(B, h->plan_B);
+    const int64_t plan_B = planned_tokens(h, B);
     const bool token_blocks = use_token_block(h, plan_B);
     if (token_blocks || use_block_forward(h)) {
         // one launch: a CTA per token; or descent, grid barrier, leaves.  The stable bucketing is made on demand from the leaf
@@ -1885,7 +1904,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     // With fewer than about 4 tokens per leaf the warp leaf kernel gains nothing from bucket order (no
     // weights to share), so the bucketing is left out of the forward and made on demand
     // (fff_debug_get_bucketing) from the leaf indices, which then also live in the workspace.
-    const bool lazy_bucketing = !tensor_leaf && B < 4 * h->n_leaves;
+    const bool lazy_bucketing = !tensor_leaf && plan_B < 4 * h->n_leaves;
     if (lazy_bucketing) leaf = h->ws_leaf;
     Coarse coarse;
     DescentTail tail;
@@ -1893,15 +1912,15 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
     const int tile_rows = plan.tile_rows;
     // The descent ends with a tcgen05 stage and a tensor-core leaf kernel follows: that stage files the tokens under their
     // leaves itself and the leaf kernel follows at once, on tiles it derives from the lists' counts.
-    h->slots_now = h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_DESCENT] && tensor_leaf && h->ws_slots && !h->ustages.empty() &&
-                   (plan.umma ? tile_rows == fff::kLUM : h->n_leaves <= kMaxListedLeaves && B <= kMaxListedTokens) && h->ustages.back().umma &&
+    h->slots_now = h->tune[FFF_TUNE_DIRECT_LISTS] && h->tune[FFF_TUNE_TCGEN05_DESCENT] && tensor_leaf && !h->ustages.empty() &&
+                   leaf_lists_fit(h, B) &&
+                   (plan.umma ? tile_rows == fff::kLUM : h->n_leaves <= kMaxListedLeaves && plan_B <= kMaxListedTokens) && h->ustages.back().umma &&
                    h->ustages.back().L0 + h->ustages.back().k == h->depth &&
-                   B <= h->slot_cap && h->n_leaves * h->slot_cap <= INT32_MAX &&
                    dense_stage_count(h, B) == (int)h->ustages.size() &&
-                   (h->ustages.size() == 1 || (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (B >> h->ustages.back().L0) >= 64) ||
-                    (h->ustages.size() == 2 && h->tune[FFF_TUNE_TCGEN05_GROUPED] && h->ws_nslots && B <= h->nslot_cap &&
-                     (h->nslot_cap << h->ustages[0].k) <= INT32_MAX));
-    const bool group_tiles = tensor_leaf && plan.umma && use_group_tiles(h, B, plan_B);
+                   (h->ustages.size() == 1 ||
+                    (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (fills_grouped_tiles(h, B, h->ustages.back().L0) ||
+                                                           (h->ustages.size() == 2 && node_lists_fit(h, B)))));
+    const bool group_tiles = tensor_leaf && plan.umma && use_group_tiles(h, B);
     if (h->slots_now && !group_tiles && !h->w8 && warp_tiles(h, plan, plan_B)) plan = LeafPlan{fff::kLWRows};
     if (group_tiles) {
         h->slots_now = false;

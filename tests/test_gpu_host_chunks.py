@@ -15,6 +15,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("D,O,depth,l,dtype,B", [
     (256, 256, 4, 12, "bf16", 3906), (256, 256, 4, 12, "bf16", 3907), (1024, 1024, 3, 8, "bf16", 1001),
     (768, 768, 9, 24, "bf16", 1400), (768, 768, 11, 1, "bf16", 3000), (256, 256, 9, 12, "bf16", 8300), (512, 512, 4, 8, "f32", 1500),
+    # chunks that alone would run fewer descent stages (12 and 14 tokens per group of the second), thin groups on other kernels,
+    # a walk through all levels
+    (768, 768, 11, 12, "bf16", 1490), (768, 768, 11, 12, "bf16", 1600), (768, 768, 10, 24, "bf16", 3000), (768, 768, 15, 1, "bf16", 12000),
 ])
 def test_small_batches_in_chunks(D, O, depth, l, dtype, B):
     cfg = wl.FFFConfig("host_small_chunks", D, O, depth, l, "gelu", dtype, B, "normal")
@@ -26,6 +29,7 @@ def test_small_batches_in_chunks(D, O, depth, l, dtype, B):
     yh = torch.zeros((B, O), dtype=td).pin_memory()
     lh = torch.full((B,), -1, dtype=torch.int32).pin_memory()
     layer.forward_infer_host(xh, yh, lh)
+    launches = layer.last_launch_count()                   # (of the last chunk)
     np.testing.assert_array_equal(lh.numpy(), leaf_ref)
     util.check_outputs(yh, y_ref, dtype)
     offsets, perm = layer.last_bucketing(B)
@@ -35,4 +39,5 @@ def test_small_batches_in_chunks(D, O, depth, l, dtype, B):
     y_dev, _ = layer.forward_infer(xh.cuda())
     torch.cuda.synchronize()
     assert torch.equal(y_dev.cpu(), yh)
+    assert layer.last_launch_count() == launches           # a chunk runs what the whole batch runs
     layer.close()
