@@ -340,11 +340,14 @@ struct LeafPlan {
     bool resident = false;         // the tiles of all leaves run at once
 };
 
-// Tiles of tile_rows rows that B tokens spread over the leaves fill, on average (a leaf's count is about Poisson).
+// Tiles of tile_rows rows that B tokens spread over the leaves fill, on average (a leaf's count is about Poisson): the sum over k
+// of the chance that a leaf has more than k tiles' worth of tokens.  Once counts spread over whole tiles (standard deviation of
+// tile_rows) the last tile of a leaf is half full on average and the sum is its mean plus a half.
 double expected_tiles(const fff_handle_s* h, int64_t B, int tile_rows) {
     const double mean = (double)B / (double)h->n_leaves, sd2 = std::sqrt(2.0 * mean);
+    if (mean >= (double)tile_rows * tile_rows) return (mean / tile_rows + 0.5) * (double)h->n_leaves;
     double per_leaf = 1.0 - std::exp(-mean);
-    for (int k = 1; k < 64 && (k * tile_rows - mean) / sd2 < 4.5; ++k) per_leaf += 0.5 * std::erfc((k * tile_rows + 0.5 - mean) / sd2);
+    for (int k = 1; (k * tile_rows - mean) / sd2 < 4.5; ++k) per_leaf += 0.5 * std::erfc((k * tile_rows + 0.5 - mean) / sd2);
     return per_leaf * (double)h->n_leaves;
 }
 
