@@ -10,6 +10,7 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 namespace {
@@ -18,7 +19,7 @@ using ForwardInfer = int (*)(void*, const void*, void*, int32_t*, int64_t, void*
 ForwardInfer g_forward = nullptr;
 
 bool matches(const at::Tensor& t, at::ScalarType type, int64_t rows, int64_t cols) {
-    if (!t.is_cuda() || t.scalar_type() != type || !t.is_contiguous()) return false;
+    if (!t.is_cuda() || t.layout() != at::kStrided || t.scalar_type() != type || !t.is_contiguous()) return false;
     if (cols < 0) return t.dim() == 1 && t.size(0) == rows;
     return t.dim() == 2 && t.size(0) == rows && t.size(1) == cols;
 }
@@ -31,7 +32,10 @@ PyObject* set_address(PyObject*, PyObject* arg) {
 
 // forward(handle, D, O, is_bf16, x, y or None, leaf_idx or None, want_leaf_idx, stream address or None)
 //   -> (status, y, leaf_idx or None), or None when the arguments are not what the call takes
+// (A tensor may answer any question about itself with an exception, a Python one from a subclass's dispatch among them: all of
+// it stands between the macros that turn C++ exceptions into Python errors, each into the type that torch raises for it.)
 PyObject* forward(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 9 || !g_forward || !THPVariable_Check(args[4])) Py_RETURN_NONE;
     void* handle = args[0] == Py_None ? nullptr : PyLong_AsVoidPtr(args[0]);
     const int64_t D = PyLong_AsLongLong(args[1]), O = PyLong_AsLongLong(args[2]);
@@ -43,42 +47,37 @@ PyObject* forward(PyObject*, PyObject* const* args, Py_ssize_t n) {
     const int64_t B = x.size(0);
     if (args[5] != Py_None && (!THPVariable_Check(args[5]) || !matches(THPVariable_Unpack(args[5]), type, B, O))) Py_RETURN_NONE;
     if (args[6] != Py_None && (!THPVariable_Check(args[6]) || !matches(THPVariable_Unpack(args[6]), at::kInt, B, -1))) Py_RETURN_NONE;
-    try {
-        at::Tensor y, leaf;
-        void* stream = nullptr;
-        if (args[8] == Py_None) stream = c10::cuda::getCurrentCUDAStream().stream();
-        else stream = PyLong_AsVoidPtr(args[8]);
-        if (PyErr_Occurred()) return nullptr;
-        if (args[5] != Py_None) y = THPVariable_Unpack(args[5]);
-        else y = at::empty({B, O}, x.options().requires_grad(false));
-        if (args[6] != Py_None) leaf = THPVariable_Unpack(args[6]);
-        else if (want_leaf) leaf = at::empty({B}, x.options().requires_grad(false).dtype(at::kInt));
-        const void* xp = x.data_ptr();
-        void* yp = y.data_ptr();
-        int32_t* lp = leaf.defined() ? static_cast<int32_t*>(leaf.data_ptr()) : nullptr;
-        int status;
-        Py_BEGIN_ALLOW_THREADS
-        status = g_forward(handle, xp, yp, lp, B, stream);
-        Py_END_ALLOW_THREADS
-        PyObject* py = args[5] != Py_None ? (Py_INCREF(args[5]), args[5]) : THPVariable_Wrap(std::move(y));
-        PyObject* pl = args[6] != Py_None   ? (Py_INCREF(args[6]), args[6])
-                       : leaf.defined()     ? THPVariable_Wrap(std::move(leaf))
-                                            : (Py_INCREF(Py_None), Py_None);
-        PyObject* ps = PyLong_FromLong(status);
-        if (!py || !pl || !ps) {
-            Py_XDECREF(py); Py_XDECREF(pl); Py_XDECREF(ps);
-            return nullptr;
-        }
-        PyObject* out = PyTuple_New(3);
-        if (!out) return nullptr;
-        PyTuple_SET_ITEM(out, 0, ps);
-        PyTuple_SET_ITEM(out, 1, py);
-        PyTuple_SET_ITEM(out, 2, pl);
-        return out;
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    at::Tensor y, leaf;
+    void* stream = nullptr;
+    if (args[8] == Py_None) stream = c10::cuda::getCurrentCUDAStream().stream();
+    else stream = PyLong_AsVoidPtr(args[8]);
+    if (PyErr_Occurred()) return nullptr;
+    if (args[5] != Py_None) y = THPVariable_Unpack(args[5]);
+    else y = at::empty({B, O}, x.options().requires_grad(false));
+    if (args[6] != Py_None) leaf = THPVariable_Unpack(args[6]);
+    else if (want_leaf) leaf = at::empty({B}, x.options().requires_grad(false).dtype(at::kInt));
+    const void* xp = x.data_ptr();
+    void* yp = y.data_ptr();
+    int32_t* lp = leaf.defined() ? static_cast<int32_t*>(leaf.data_ptr()) : nullptr;
+    int status;
+    Py_BEGIN_ALLOW_THREADS
+    status = g_forward(handle, xp, yp, lp, B, stream);
+    Py_END_ALLOW_THREADS
+    PyObject* py = args[5] != Py_None ? (Py_INCREF(args[5]), args[5]) : THPVariable_Wrap(std::move(y));
+    PyObject* pl = args[6] != Py_None   ? (Py_INCREF(args[6]), args[6])
+                   : leaf.defined()     ? THPVariable_Wrap(std::move(leaf))
+                                        : (Py_INCREF(Py_None), Py_None);
+    PyObject* ps = PyLong_FromLong(status);
+    PyObject* out = py && pl && ps ? PyTuple_New(3) : nullptr;
+    if (!out) {
+        Py_XDECREF(py); Py_XDECREF(pl); Py_XDECREF(ps);
         return nullptr;
     }
+    PyTuple_SET_ITEM(out, 0, ps);
+    PyTuple_SET_ITEM(out, 1, py);
+    PyTuple_SET_ITEM(out, 2, pl);
+    return out;
+    END_HANDLE_TH_ERRORS
 }
 
 PyMethodDef kMethods[] = {

@@ -46,6 +46,9 @@ def test_wrong_arguments_name_themselves():
     for bad in (x.cpu(), x.bfloat16(), x[:, :-1], x.t().contiguous().t(), torch.randn(4, D + 1, device="cuda")):
         with pytest.raises(ValueError, match="^x: expected"):
             layer.forward_infer(bad)
+    for bad in (x.to_sparse_csr(), x.to_sparse()):         # these raise when asked whether they are contiguous, or are not
+        with pytest.raises((RuntimeError, ValueError)):
+            layer.forward_infer(bad)
     with pytest.raises(ValueError, match="^y: expected"):
         layer.forward_infer(x, y[:3])
     with pytest.raises(ValueError, match="^leaf_idx: expected"):
