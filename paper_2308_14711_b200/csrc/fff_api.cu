@@ -223,18 +223,19 @@ fff_status_t dmalloc(void** p, size_t bytes) {
 
 void dfree(void* p) { if (p) cudaFree(p); }
 
-// Copies of device memory and memsets go to the default stream and return before they are done; a caller's non-blocking stream
-// does not wait for that stream, so what is allocated on behalf of a call in progress is waited for here.
-fff_status_t default_stream_done(cudaError_t e) {
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-    return e == cudaSuccess ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
-}
-
-// A copy of `src`, or zeroes; in place for every stream when the call returns.
+// A copy of `src`, or zeroes, made on the default stream: the call returns before they are in place (default_stream_done).
 fff_status_t clone(void** dst, const void* src, size_t bytes) {
     fff_status_t s = dmalloc(dst, bytes);
     if (s != FFF_OK) return s;
-    return default_stream_done(src ? cudaMemcpy(*dst, src, bytes, cudaMemcpyDeviceToDevice) : cudaMemset(*dst, 0, bytes ? bytes : 16));
+    cudaError_t e = src ? cudaMemcpy(*dst, src, bytes, cudaMemcpyDeviceToDevice) : cudaMemset(*dst, 0, bytes ? bytes : 16);
+    return e == cudaSuccess ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
+}
+
+// Waits for copies and memsets of device memory on the default stream, which return before they are done: a caller's
+// non-blocking stream does not wait for that stream, so whoever allocates on behalf of a call in progress does it here.
+fff_status_t default_stream_done(cudaError_t e) {
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    return e == cudaSuccess ? FFF_OK : (cudaGetLastError(), FFF_ERR_CUDA);
 }
 
 // Launch a kernel of the forward chain.  Every launch after the first of a call carries the
@@ -471,6 +472,7 @@ fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
         h->nslot_cap = B;
         h->ncursor_dirty = false;
     }
+    if ((s = default_stream_done(cudaSuccess)) != FFF_OK) return s;       // the counters are zero on every stream
     h->cap_B = B;
     return FFF_OK;
 }
