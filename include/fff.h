@@ -326,8 +326,11 @@ typedef enum {
     FFF_CAP_TCGEN05_LEAF = 8,     /* ... on tcgen05 (also O % 16 == 0) */
     FFF_CAP_FUSED_SMALL = 16,     /* the one-launch kernel (l <= 32, at most one group of 32 neurons per SM) */
     FFF_CAP_FORWARD_TRAIN = 32,   /* fff_forward_train (bf16, D % 64 == 0) */
-    FFF_CAP_PADDED = 128,         /* the tensor-core kernels run on images padded to the next multiple of 128 (D % 128 != 0, D % 8 == 0);
-                                     the bits above for them are not set then, and fff_set_path refuses FFF_PATH_TENSOR */
+    FFF_CAP_PADDED = 128,         /* the tensor-core kernels run on images padded to the next multiple of 128 (D % 128 != 0, D % 8 == 0).
+                                     The bits 1 to 8 then stay clear and fff_set_path refuses FFF_PATH_TENSOR, although the forward
+                                     does run on tensor cores: those bits promise rows taken as they are.  Hidden values enter
+                                     the second layer as sums of two bf16 values, with the float32 precision that such layers
+                                     have on CUDA cores (to 2^-18); with D % 128 == 0 they are rounded to bf16 */
     FFF_CAP_GROUP_TILES = 64      /* leaf tiles of 8 sibling leaves (FFF_TUNE_GROUP_TILES: 8 <= leaf_width < 16, 9 <= depth <= 11) */
 } fff_capability_t;
 int fff_capabilities(fff_handle_t h);

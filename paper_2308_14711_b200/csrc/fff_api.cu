@@ -51,6 +51,7 @@ struct fff_handle_s {
     int sm_count = 148;
     int D = 0, O = 0, depth = 0, l = 0;
     int Dp = 0;                   // D rounded up to the K step of the tensor-core images, which are padded with zero columns
+    bool padded() const { return D != Dp; }      // the leaf kernels then keep the hidden values' float32 precision (kSplit in leaf_umma.cuh)
     int act = 0, dtype = 0;
     size_t esize = 4;
     int64_t n_nodes = 0, n_leaves = 1;
@@ -1028,7 +1029,7 @@ fff_status_t run_leaf(fff_handle_s* h, const void* x, const int32_t* leaf_idx, c
     return launched(h, st, tail.levels > 0 ? "descent_tail+leaf_ff_warp" : "grouped_leaf_ff_warp");
 }
 
-template <int LP, int TM, int S>
+template <int LP, int TM, int S, bool kSplit>
 fff_status_t launch_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, cudaStream_t st) {
     const int n_tiles = tile_list_len(B, TM, (int)h->n_leaves);
     using L = fff::LeafMmaLayout<LP, TM, S>;
@@ -1036,35 +1037,41 @@ fff_status_t launch_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm
     int32_t* counts = h->slots_now && perm == h->ws_slots ? h->ws_cursor : nullptr;
     const int smem = L::kSmemBytes + (counts ? L::list_bytes((int)h->n_leaves) : 0);
     static bool limit_raised[kMaxDevices] = {};
-    if (!raise_smem_limit(fff::k_leaf_mma<LP, TM, S>, h->device, L::kSmemBytes + L::list_bytes(kMaxListedLeaves), limit_raised)) return FFF_ERR_CUDA;
+    if (!raise_smem_limit(fff::k_leaf_mma<LP, TM, S, kSplit>, h->device, L::kSmemBytes + L::list_bytes(kMaxListedLeaves), limit_raised)) return FFF_ERR_CUDA;
     const int per_sm = std::max(1, std::min(2, (int)((227 * 1024) / (smem + 1024))));
     const int64_t grid = std::min<int64_t>((int64_t)h->sm_count * per_sm, n_tiles);
-    if (launch_chain(h, fff::k_leaf_mma<LP, TM, S>, (unsigned)grid, L::kThreads, (size_t)smem, st, 1,
+    if (launch_chain(h, fff::k_leaf_mma<LP, TM, S, kSplit>, (unsigned)grid, L::kThreads, (size_t)smem, st, 1,
                      (const __nv_bfloat16*)x, perm, h->ws_tiles, n_tiles, h->w1img, h->b1img, h->w2img, (__nv_bfloat16*)y, h->D, h->Dp,
                      h->O, h->act, h->d_status, counts, (int)h->n_leaves, (int)h->slot_cap) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "grouped_leaf_ff_mma");
 }
 
+template <int LP, int TM, int S>
+fff_status_t launch_leaf_mma(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, cudaStream_t st) {
+    return h->padded() ? launch_leaf_mma<LP, TM, S, true>(h, x, perm, y, B, st) : launch_leaf_mma<LP, TM, S, false>(h, x, perm, y, B, st);
+}
+
 fff_status_t launch_leaf_mma_warp(fff_handle_s* h, const void* x, const int32_t* slots, void* y, int64_t B, cudaStream_t st) {
     const int64_t n_tiles = tile_list_len(B, fff::kLWRows, (int)h->n_leaves);
     const int64_t grid = std::min<int64_t>((int64_t)h->sm_count * 2, n_tiles);
-    if (launch_chain(h, fff::k_leaf_mma_warp, (unsigned)grid, fff::kLWThreads, sizeof(int) * (size_t)(h->n_leaves + 1), st, 1,
+    if (launch_chain(h, h->padded() ? fff::k_leaf_mma_warp<true> : fff::k_leaf_mma_warp<false>, (unsigned)grid, fff::kLWThreads, sizeof(int) * (size_t)(h->n_leaves + 1), st, 1,
                      (const __nv_bfloat16*)x, slots, (const __nv_bfloat16*)h->w1img, (const float*)h->b1img, (const unsigned char*)h->w2img,
                      (__nv_bfloat16*)y, h->D, h->Dp, h->O, h->act, h->ws_cursor, (int)h->n_leaves, (int)h->slot_cap) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, "grouped_leaf_ff_mma_warp");
 }
 
-template <int LP, bool kFold, bool kW8 = false>
-fff_status_t launch_leaf_umma(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, int tile_rows,
-                              cudaStream_t st) {
-    using L = fff::LeafUmmaLayout<LP, kW8>;
+template <int LP, bool kFold, bool kW8, bool kSplit>
+fff_status_t launch_leaf_umma_tiles(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, int tile_rows,
+                                    cudaStream_t st) {
+    using L = fff::LeafUmmaLayout<LP, kW8, 1, kSplit>;
+    constexpr auto kernel = fff::k_leaf_umma<LP, kFold, kW8, 1, kSplit>;
     const int n_tiles = tile_list_len(B, tile_rows, (int)h->n_leaves);
     const int stages = std::min((int)fff::kLUMaxStages, (kSmemBudget - L::smem_bytes(0)) / L::kStageBytes);
     if (stages < 2) return FFF_ERR_UNSUPPORTED;
     static bool limit_raised[kMaxDevices] = {};
-    if (!raise_smem_limit(fff::k_leaf_umma<LP, kFold, kW8>, h->device, kSmemBudget, limit_raised)) return FFF_ERR_CUDA;
+    if (!raise_smem_limit(kernel, h->device, kSmemBudget, limit_raised)) return FFF_ERR_CUDA;
     CUtensorMap tm;
     if (!make_x_tensor_map(&tm, x, B, h->D, 1)) return FFF_ERR_CUDA;       // one-row boxes: rows are gathered four at a time
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(h->sm_count, n_tiles));
@@ -1072,13 +1079,21 @@ fff_status_t launch_leaf_umma(fff_handle_s* h, const void* x, const int32_t* per
     const int passes = 1;      // two passes (full tiles first) measured slightly slower
     // direct lists: perm is the table of lists, the tiles come from its counts
     int32_t* counts = h->slots_now && perm == h->ws_slots ? h->ws_cursor : nullptr;
-    if (launch_chain(h, fff::k_leaf_umma<LP, kFold, kW8>, (unsigned)grid, fff::LeafUmmaWarps<kW8>::kThreads, (size_t)L::smem_bytes(stages), st, 1, tm, perm,
+    if (launch_chain(h, kernel, (unsigned)grid, fff::LeafUmmaWarps<kW8>::kThreads, (size_t)L::smem_bytes(stages), st, 1, tm, perm,
                      (const fff::Tile*)h->ws_tiles, n_tiles, (const __nv_bfloat16*)h->w1img, (const float*)h->b1img,
                      (const unsigned char*)(kW8 ? h->w2codes : h->w2uimg), (__nv_bfloat16*)y, h->Dp, h->O, h->l, h->act, stages, wide, passes, h->ws_sched,
                      counts, (int)h->n_leaves, (int)h->slot_cap, h->d_status, (const unsigned char*)h->w1codes, (const float*)h->scale1,
                      (const float*)h->scale2, (const float*)nullptr, (int32_t*)nullptr, (int32_t*)nullptr) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, kW8 ? "grouped_leaf_ff_umma_w8" : "grouped_leaf_ff_umma");
+}
+
+template <int LP, bool kFold, bool kW8 = false>
+fff_status_t launch_leaf_umma(fff_handle_s* h, const void* x, const int32_t* perm, void* y, int64_t B, int tile_rows,
+                              cudaStream_t st) {
+    if constexpr (!kW8)
+        if (h->padded()) return launch_leaf_umma_tiles<LP, kFold, false, true>(h, x, perm, y, B, tile_rows, st);
+    return launch_leaf_umma_tiles<LP, kFold, kW8, false>(h, x, perm, y, B, tile_rows, st);
 }
 
 // Ring depth per (LP, TM): what fits twice into an SM's shared memory (once for LP = 64).
@@ -1184,8 +1199,10 @@ bool use_group_tiles(const fff_handle_s* h, int64_t B) {
 
 // First stage (depth - 3 levels, files the tokens under the nodes it reaches), then the leaf kernel on grouped tiles,
 // which finishes the descent itself and reports the leaves.
-fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_t* leaf, int64_t B, cudaStream_t st) {
-    using L = fff::LeafUmmaLayout<16, false, fff::kLUGroup>;
+template <bool kSplit>
+fff_status_t run_forward_grouped_tiles(fff_handle_s* h, const void* x, void* y, int32_t* leaf, int64_t B, cudaStream_t st) {
+    using L = fff::LeafUmmaLayout<16, false, fff::kLUGroup, kSplit>;
+    constexpr auto kernel = fff::k_leaf_umma<16, true, false, fff::kLUGroup, kSplit>;
     const int bins = (int)(h->n_leaves / fff::kLUGroup);
     if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
@@ -1200,13 +1217,13 @@ fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_
     const int stages = std::min((int)fff::kLUMaxStages, (kSmemBudget - L::smem_bytes(0)) / L::kStageBytes);
     if (stages < 2) return FFF_ERR_UNSUPPORTED;
     static bool limit_raised[kMaxDevices] = {};
-    if (!raise_smem_limit(fff::k_leaf_umma<16, true, false, fff::kLUGroup>, h->device, kSmemBudget, limit_raised)) return FFF_ERR_CUDA;
+    if (!raise_smem_limit(kernel, h->device, kSmemBudget, limit_raised)) return FFF_ERR_CUDA;
     CUtensorMap tm;
     if (!make_x_tensor_map(&tm, x, B, h->D, 1)) return FFF_ERR_CUDA;
     const int n_tiles = tile_list_len(B, fff::kLUM, bins);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(h->sm_count, n_tiles));
     const int wide = (reinterpret_cast<uintptr_t>(y) & 31u) == 0 ? 1 : 0;
-    if (launch_chain(h, fff::k_leaf_umma<16, true, false, fff::kLUGroup>, (unsigned)grid, fff::kLUThreads, (size_t)L::smem_bytes(stages), st,
+    if (launch_chain(h, kernel, (unsigned)grid, fff::kLUThreads, (size_t)L::smem_bytes(stages), st,
                      1, tm, (const int32_t*)h->ws_slots, (const fff::Tile*)h->ws_tiles, n_tiles, (const __nv_bfloat16*)h->g_w1,
                      (const float*)h->b1img, (const unsigned char*)h->g_w2, (__nv_bfloat16*)y, h->Dp, h->O, h->l, h->act, stages, wide, 1,
                      h->ws_sched, h->ws_cursor, bins, (int)h->slot_cap, h->d_status, (const unsigned char*)nullptr,
@@ -1216,6 +1233,10 @@ fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_
     s = launched(h, st, "grouped_leaf_ff_umma_8");
     if (s == FFF_OK) h->cursor_dirty = false;
     return s;
+}
+
+fff_status_t run_forward_grouped(fff_handle_s* h, const void* x, void* y, int32_t* leaf, int64_t B, cudaStream_t st) {
+    return h->padded() ? run_forward_grouped_tiles<true>(h, x, y, leaf, B, st) : run_forward_grouped_tiles<false>(h, x, y, leaf, B, st);
 }
 
 // The one-launch kernel on CUDA cores: eligibility (at creation).

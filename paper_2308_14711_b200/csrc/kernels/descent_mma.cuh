@@ -169,7 +169,7 @@ k_descent_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ p
                                       full + stage);
                     }
                 }
-if (u * kKS + pchunk * 8 < D) {
+                if (u * kKS + pchunk * 8 < D) {
 #pragma unroll
                     for (int i = 0; i < kTM / kRowsPerPass; ++i)
                         if (src[i]) ptx::cp_async16(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, src[i] + u * kKS);

@@ -129,7 +129,7 @@ __global__ void k_pack_b1(const T* __restrict__ b1, float* __restrict__ img, int
 
 // ---- the kernel ------------------------------------------------------------------------------------
 
-template <int LP, int TM, int S>
+template <int LP, int TM, int S, bool kSplit>
 __global__ void __launch_bounds__((kLeafConsumers + kProducerWarps) * 32, LP <= 32 ? 2 : 1)
 k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm,
            const Tile* __restrict__ tiles, int n_tiles_total,
@@ -210,7 +210,7 @@ k_leaf_mma(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ perm
                     ptx::bulk_g2s(st + kTM * kXRowBytes, w1img + ((int64_t)tl.bin * U1 + u) * (LP * kKS), L::kW1StageBytes,
                                   full + stage);
                 }
-if (u * kKS + pchunk * 8 < D) {
+                if (u * kKS + pchunk * 8 < D) {
 #pragma unroll
                     for (int i = 0; i < kTM / kRowsPerPass; ++i)
                         if (src[i]) ptx::cp_async16(st + (i * kRowsPerPass + prow) * kXRowBytes + pchunk * 16, src[i] + u * kKS);
@@ -309,12 +309,20 @@ if (u * kKS + pchunk * 8 < D) {
                 }
                 asm volatile("bar.sync %0, %1;" ::"r"(1 + mi), "r"(kNSplit * 32) : "memory");
             }
-            uint32_t hA[LP / 8][2];
+            // (kSplit: as sums of two bf16 values, see leaf_umma.cuh)
+            uint32_t hA[kSplit ? 2 : 1][LP / 8][2];
 #pragma unroll
             for (int nt = 0; nt < LP / 8; ++nt) {
                 const float2 b = b1r[nt];
-                hA[nt][0] = ptx::pack_bf16(activate(act, acc1[nt][0] + b.x), activate(act, acc1[nt][1] + b.y));
-                hA[nt][1] = ptx::pack_bf16(activate(act, acc1[nt][2] + b.x), activate(act, acc1[nt][3] + b.y));
+                const float h0 = activate(act, acc1[nt][0] + b.x), h1 = activate(act, acc1[nt][1] + b.y);
+                const float h2 = activate(act, acc1[nt][2] + b.x), h3 = activate(act, acc1[nt][3] + b.y);
+                if constexpr (kSplit) {
+                    ptx::split_bf16(h0, h1, hA[0][nt][0], hA[1][nt][0]);
+                    ptx::split_bf16(h2, h3, hA[0][nt][1], hA[1][nt][1]);
+                } else {
+                    hA[0][nt][0] = ptx::pack_bf16(h0, h1);
+                    hA[0][nt][1] = ptx::pack_bf16(h2, h3);
+                }
             }
 
             // GEMM2 + bias + store, this warp's slice of the output columns of every stage
@@ -341,8 +349,12 @@ if (u * kKS + pchunk * 8 < D) {
                             for (int kk = 0; kk < LP / 16; ++kk) {
                                 uint32_t b0, b1, b2, b3;
                                 ptx::ldmatrix_x4(ws + ptx::swz128((uint32_t)(n * LP * 2 + (kk * 16 + bk) * 2)), b0, b1, b2, b3);
-                                ptx::mma_bf16(acc2[2 * np], hA[2 * kk][0], hA[2 * kk][1], hA[2 * kk + 1][0], hA[2 * kk + 1][1], b0, b1);
-                                ptx::mma_bf16(acc2[2 * np + 1], hA[2 * kk][0], hA[2 * kk][1], hA[2 * kk + 1][0], hA[2 * kk + 1][1], b2, b3);
+#pragma unroll
+                                for (int op = 0; op < (kSplit ? 2 : 1); ++op) {
+                                    const auto& a = hA[op];
+                                    ptx::mma_bf16(acc2[2 * np], a[2 * kk][0], a[2 * kk][1], a[2 * kk + 1][0], a[2 * kk + 1][1], b0, b1);
+                                    ptx::mma_bf16(acc2[2 * np + 1], a[2 * kk][0], a[2 * kk][1], a[2 * kk + 1][0], a[2 * kk + 1][1], b2, b3);
+                                }
                             }
                         }
                         // fragments -> padded staging rows (bf16), then whole 16-byte units to y

@@ -33,6 +33,8 @@ constexpr int kLWThreads = kLWWarps * 32;
 __device__ __forceinline__ int warp_tile_unit(int j, int n) { return 4 * (n >> 1) + 2 * j + (n & 1); }
 
 // x [B, D], slots [n_bins][cap] token numbers, counts [n_bins] + [1] CTAs that have finished (all zero again at the end).
+// kSplit: the hidden values as sums of two bf16 values (see leaf_umma.cuh).
+template <bool kSplit>
 __global__ void __launch_bounds__(kLWThreads, 2)
 k_leaf_mma_warp(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ slots, const __nv_bfloat16* __restrict__ w1img,
                 const float* __restrict__ b1img, const unsigned char* __restrict__ w2img, __nv_bfloat16* __restrict__ y, int D, int Dp,
@@ -100,12 +102,17 @@ k_leaf_mma_warp(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__
                     ptx::mma_bf16(acc[j], a[i][0].z, a[i][1].z, a[i][0].w, a[i][1].w, b[i][j].z, b[i][j].w);
                 }
         }
-        uint32_t h[NT][2];
+        constexpr int kOps = kSplit ? 2 : 1;
+        uint32_t h[kOps][NT][2];
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
             const float2 b1 = __ldg(reinterpret_cast<const float2*>(b1img + (int64_t)leaf * LP + warp_tile_unit(j, 2 * c)));
-            h[j][0] = ptx::pack_bf16(activate(act, acc[j][0] + b1.x), activate(act, acc[j][1] + b1.y));
-            h[j][1] = ptx::pack_bf16(activate(act, acc[j][2] + b1.x), activate(act, acc[j][3] + b1.y));
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float h0 = activate(act, acc[j][2 * r] + b1.x), h1 = activate(act, acc[j][2 * r + 1] + b1.y);
+                if constexpr (kSplit) ptx::split_bf16(h0, h1, h[0][j][r], h[1][j][r]);
+                else h[0][j][r] = ptx::pack_bf16(h0, h1);
+            }
         }
 
         // ---- GEMM2: column n of group t of a block of 32 outputs is output 8 (n / 2) + 2 t + n % 2 of the block
@@ -133,7 +140,9 @@ k_leaf_mma_warp(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                    ptx::mma_bf16(d, h[0][0], h[0][1], h[1][0], h[1][1], wv[i][t].x, wv[i][t].y);
+#pragma unroll
+                    for (int op = 0; op < kOps; ++op)
+                        ptx::mma_bf16(d, h[op][0][0], h[op][0][1], h[op][1][0], h[op][1][1], wv[i][t].x, wv[i][t].y);
                     out0[t] = ptx::pack_bf16(d[0] + bv[2 * t], d[1] + bv[2 * t + 1]);
                     out1[t] = ptx::pack_bf16(d[2] + bv[2 * t], d[3] + bv[2 * t + 1]);
                 }

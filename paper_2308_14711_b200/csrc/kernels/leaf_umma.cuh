@@ -90,8 +90,15 @@ constexpr int kLUTmemCols = 512;
 // each row's own leaf's LP columns of H and zeroes the others, and GEMM2 contracts over all 8 LP columns against the
 // 8 leaves' output weights.  The tokens' rows then cross the memory system twice in all (first stage of the descent,
 // then here) instead of being gathered once more per level group, and tiles are as full as the node's share of the batch.
-template <int LP, bool kW8 = false, int GL = 1> struct LeafUmmaLayout {
+// kSplit: the hidden values enter GEMM2 as sums of two bf16 values, in two A operands against the same weights, which keeps
+// their float32 precision to 2^-18.  For the layers whose rows are padded (D % 128 != 0): on CUDA cores their hidden values
+// are float32, and that they can be padded is no reason to round them.  Costs a second set of GEMM2's MMAs and the second operand's
+// stores, us, rounded and split: 712 -> 704, 256 leaves of 12, 50 432 tokens 61.3 and 62.5; 1000 -> 992, 2048 leaves of 32, 65 536
+// tokens 168.1 and 172.5, of 40 203 and 214; grouped tiles (which also lose a W2 slot to it) 712 -> 704, 1024 leaves of 12, 50 432
+// tokens 77.8 and 86.4.  On CUDA cores the four take 570, 4652, 2786 and 640.
+template <int LP, bool kW8 = false, int GL = 1, bool kSplit = false> struct LeafUmmaLayout {
     static_assert(LP == 16 || LP == 32 || LP == 64, "padded hidden width");
+    static_assert(!(kSplit && kW8), "8-bit weights: rows are never padded");
     static_assert(GL == 1 || (GL == 8 && LP == 16 && !kW8), "grouped tiles: 8 leaves of padded width 16, bf16 weights");
     static constexpr int kN1 = GL == 1 ? LP : GL * LP + 16;                  // columns of GEMM1
     static constexpr int kHCols = GL * LP;                                   // K of GEMM2
@@ -115,12 +122,13 @@ template <int LP, bool kW8 = false, int GL = 1> struct LeafUmmaLayout {
     static constexpr int kW2PieceBytes = (kW8 ? kW2CodeBytes : kW2Bytes) + kLUPiece * 4;    // a piece in the image: weights + biases
     static constexpr int kW2SlotStride = (kW2BiasOff + kLUPiece * 4 + 1023) & ~1023;
     static constexpr int kHBytes = kLUM * kHCols * 2;
+    static constexpr int kHOperands = kSplit ? 2 : 1;
     // W2 ring: a whole tile's pieces (O <= 1024) when they are small, so that no copy waits for an MMA just issued
-    static constexpr int kW2Slots = GL > 1 ? 3 : LP <= 16 ? 8 : LP <= 32 ? (kW8 ? 6 : 8) : 4;
+    static constexpr int kW2Slots = GL > 1 ? (kSplit ? 2 : 3) : LP <= 16 ? 8 : LP <= 32 ? (kW8 ? 6 : 8) : 4;
     static constexpr int kAcc2Col = GL > 1 ? 256 : 64;                       // first tensor-memory column of the two GEMM2 accumulators
     static constexpr int kBarrierBytes = kW8 ? 896 : 640;
     static constexpr int smem_bytes(int stages) {
-        return 1024 + stages * kStageBytes + kW2Slots * kW2SlotStride + kHBytes + kBarrierBytes;
+        return 1024 + stages * kStageBytes + kW2Slots * kW2SlotStride + kHOperands * kHBytes + kBarrierBytes;
     }
 };
 
@@ -290,7 +298,7 @@ __device__ __forceinline__ void expand_e4m3_tile(const unsigned char* __restrict
 // K-block the 8 LP + 16 rows (hidden units of the 8 leaves, the 7 nodes of the subtree breadth-first, zeros), g1bias
 // [bin][8 LP + 16] the matching biases, w2img per bin and piece the 128 x 8 LP output weights in two K-blocks (kFold:
 // every leaf's spare column carries its output bias); leaf_out / leaf_out2 (optional) receive every token's leaf.
-template <int LP, bool kFold, bool kW8 = false, int GL = 1>
+template <int LP, bool kFold, bool kW8 = false, int GL = 1, bool kSplit = false>
 __global__ void __launch_bounds__(LeafUmmaWarps<kW8>::kThreads, 1)
 k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restrict__ perm,
             const Tile* __restrict__ tiles, int n_tiles_total,
@@ -303,12 +311,12 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
 {
     static_assert(!(kW8 && kFold), "8-bit weights take their biases in the epilogue");
     static_assert(GL == 1 || kFold, "grouped tiles take the output bias through the spare hidden column");
-    using L = LeafUmmaLayout<LP, kW8, GL>;
+    using L = LeafUmmaLayout<LP, kW8, GL, kSplit>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* w2ring = ring + kStages * L::kStageBytes;
     unsigned char* hbuf = w2ring + L::kW2Slots * L::kW2SlotStride;
-    uint64_t* full = reinterpret_cast<uint64_t*>(hbuf + L::kHBytes);
+    uint64_t* full = reinterpret_cast<uint64_t*>(hbuf + L::kHOperands * L::kHBytes);
     uint64_t* empty = full + kLUMaxStages;
     uint64_t* w2_full = empty + kLUMaxStages;
     uint64_t* w2_empty = w2_full + kLUMaxW2Slots;
@@ -637,15 +645,17 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                     const uint32_t idesc = ptx::umma_idesc_bf16(kLUM, n);
                     const uint32_t ws = ptx::smem_addr(w2ring + mm_slot * L::kW2SlotStride);
 #pragma unroll
-                    for (int blk = 0; blk < L::kHBlocks; ++blk) {
-                        // (one K-block of LP columns, or with grouped tiles K-blocks of 64 columns: [128 rows][128 bytes] each)
-                        const uint64_t ad = ptx::umma_desc_rows(hs + blk * (kLUM * L::kRowBytes), L::kRowBytes);
-                        const uint64_t bd = ptx::umma_desc_rows(ws + blk * (kLUPiece * L::kRowBytes), L::kRowBytes);
+                    for (int op = 0; op < L::kHOperands; ++op)
 #pragma unroll
-                        for (int kk = 0; kk < L::kRowBytes / 32; ++kk)
-                            ptx::umma_bf16(tmem_base + L::kAcc2Col + b * kLUAccStride, ad + 2 * kk, bd + 2 * kk, idesc,
-                                           (blk | kk) != 0 ? 1u : 0u);
-                    }
+                        for (int blk = 0; blk < L::kHBlocks; ++blk) {
+                            // (one K-block of LP columns, or with grouped tiles K-blocks of 64 columns: [128 rows][128 bytes] each)
+                            const uint64_t ad = ptx::umma_desc_rows(hs + op * L::kHBytes + blk * (kLUM * L::kRowBytes), L::kRowBytes);
+                            const uint64_t bd = ptx::umma_desc_rows(ws + blk * (kLUPiece * L::kRowBytes), L::kRowBytes);
+#pragma unroll
+                            for (int kk = 0; kk < L::kRowBytes / 32; ++kk)
+                                ptx::umma_bf16(tmem_base + L::kAcc2Col + b * kLUAccStride, ad + 2 * kk, bd + 2 * kk, idesc,
+                                               (op | blk | kk) != 0 ? 1u : 0u);
+                        }
                     ptx::umma_commit(w2_empty + mm_slot);
                     ptx::umma_commit(y_full + b);
                 }
@@ -699,7 +709,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                 if (!timed_out && !ptx::mbar_wait(acc1_full, it & 1)) timed_out = true;
                 ptx::tc_fence_after_sync();
                 {
-                    uint32_t hp[HC / 2];
+                    uint32_t hp[L::kHOperands][HC / 2];
                     if (h_active) {
                         uint32_t v[32];
                         ptx::tmem_ld32(lane_base + part * HC, v);      // columns past HC are not used
@@ -712,7 +722,8 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                                 float h1 = activate_bf16(kAct, scaled(v[j + 1], s1, b1r[j + 1]));
                                 if (kFold && part * HC + j == l) h0 = 1.0f;          // the bias column
                                 if (kFold && part * HC + j + 1 == l) h1 = 1.0f;
-                                hp[j / 2] = ptx::pack_bf16(h0, h1);
+                                if constexpr (kSplit) ptx::split_bf16(h0, h1, hp[0][j / 2], hp[1][j / 2]);
+                                else hp[0][j / 2] = ptx::pack_bf16(h0, h1);
                             }
                         });
                     }
@@ -722,9 +733,12 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                         for (int cp = 0; cp < rep; ++cp) {
                             const int hrow = row + cp * (kLUM / rep);
 #pragma unroll
-                            for (int c = 0; c < HC / 8; ++c)
-                                *reinterpret_cast<uint4*>(hbuf + swz_rows((uint32_t)(hrow * L::kRowBytes + (part * HC / 8 + c) * 16), L::kRowBytes)) =
-                                    make_uint4(hp[4 * c], hp[4 * c + 1], hp[4 * c + 2], hp[4 * c + 3]);
+                            for (int op = 0; op < L::kHOperands; ++op)
+#pragma unroll
+                                for (int c = 0; c < HC / 8; ++c)
+                                    *reinterpret_cast<uint4*>(hbuf + op * L::kHBytes +
+                                                              swz_rows((uint32_t)(hrow * L::kRowBytes + (part * HC / 8 + c) * 16), L::kRowBytes)) =
+                                        make_uint4(hp[op][4 * c], hp[op][4 * c + 1], hp[op][4 * c + 2], hp[op][4 * c + 3]);
                         }
                         ptx::fence_proxy_async();
                     }
@@ -772,9 +786,11 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                 ptx::mbar_arrive(acc1_empty);
                 if (active) {
                     const bool own = (j >> 2) == part;
-                    uint32_t hp[LP / 2];
+                    uint32_t hp[L::kHOperands][LP / 2];
 #pragma unroll
-                    for (int i = 0; i < LP / 2; ++i) hp[i] = 0u;
+                    for (int op = 0; op < L::kHOperands; ++op)
+#pragma unroll
+                        for (int i = 0; i < LP / 2; ++i) hp[op][i] = 0u;
                     if (own) {
                         float b1r[LP];
 #pragma unroll
@@ -790,19 +806,23 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                                 float h1 = activate_bf16(kAct, pre[i + 1] + b1r[i + 1]);
                                 if (i == l) h0 = 1.0f;                           // the bias column
                                 if (i + 1 == l) h1 = 1.0f;
-                                hp[i / 2] = ptx::pack_bf16(h0, h1);
+                                if constexpr (kSplit) ptx::split_bf16(h0, h1, hp[0][i / 2], hp[1][i / 2]);
+                                else hp[0][i / 2] = ptx::pack_bf16(h0, h1);
                             }
                         });
                     }
                     // the row's 128 bytes of K-block `part`: the leaf's two 16-byte units, zeros elsewhere
                     const int du = own ? (j & 3) * (LP / 8) : -8;
-                    unsigned char* hb = hbuf + part * (kLUM * L::kRowBytes);
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        uint4 val = make_uint4(0u, 0u, 0u, 0u);
-                        if (u == du) val = make_uint4(hp[0], hp[1], hp[2], hp[3]);
-                        if (u == du + 1) val = make_uint4(hp[4], hp[5], hp[6], hp[7]);
-                        *reinterpret_cast<uint4*>(hb + swz_rows((uint32_t)(row * L::kRowBytes + u * 16), L::kRowBytes)) = val;
+                    for (int op = 0; op < L::kHOperands; ++op) {
+                        unsigned char* hb = hbuf + op * L::kHBytes + part * (kLUM * L::kRowBytes);
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            uint4 val = make_uint4(0u, 0u, 0u, 0u);
+                            if (u == du) val = make_uint4(hp[op][0], hp[op][1], hp[op][2], hp[op][3]);
+                            if (u == du + 1) val = make_uint4(hp[op][4], hp[op][5], hp[op][6], hp[op][7]);
+                            *reinterpret_cast<uint4*>(hb + swz_rows((uint32_t)(row * L::kRowBytes + u * 16), L::kRowBytes)) = val;
+                        }
                     }
                     ptx::fence_proxy_async();
                     if (part == 0 && tok >= 0) {

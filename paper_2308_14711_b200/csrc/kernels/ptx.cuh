@@ -125,6 +125,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// Two float32 values as sums of two bf16 values each: hi + lo is within 2^-18 of the value (a single bf16: 2^-9).  Infinities
+// stay in hi alone.
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t& hi, uint32_t& lo) {
+    hi = pack_bf16(a, b);
+    const float ah = __uint_as_float(hi << 16), bh = __uint_as_float(hi & 0xffff0000u);
+    lo = pack_bf16(isinf(ah) ? 0.0f : a - ah, isinf(bh) ? 0.0f : b - bh);
+}
+
 // Swizzle of a byte offset inside an operand tile whose rows are row_bytes (32, 64 or 128) long: the
 // 16-byte unit index inside a row is XORed with bits of the 128-byte line index, as the 32-, 64- and
 // 128-byte swizzle modes of the tensor cores and of tensor-map copies expect.
