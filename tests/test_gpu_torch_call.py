@@ -15,9 +15,18 @@ def make(dtype):
     return binding.FFFLayer(D, O, DEPTH, LW, "gelu", "bf16" if dtype == torch.bfloat16 else "f32", rnd(7, D), rnd(7), rnd(8, LW, D), rnd(8, LW), rnd(8, O, LW), rnd(8, O))
 
 
+@pytest.fixture(params=["module", "ctypes"])
+def call(request, monkeypatch):
+    """The call through the CPython module, and as it is made where that has not been built."""
+    if request.param == "ctypes":
+        monkeypatch.setattr(binding, "torch_call", lambda: None)
+    else:
+        assert binding.torch_call() is not None
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("B", [0, 1, 5])
-def test_buffers_and_results(dtype, B):
+def test_buffers_and_results(call, dtype, B):
     layer = make(dtype)
     x = torch.randn(B, D, device="cuda").to(dtype).requires_grad_(dtype == torch.float32)
     y, leaf = layer.forward_infer(x)
@@ -39,7 +48,7 @@ def test_buffers_and_results(dtype, B):
     assert torch.equal(lbuf, leaf) and torch.equal(leaf3, leaf)
 
 
-def test_wrong_arguments_name_themselves():
+def test_wrong_arguments_name_themselves(call):
     layer = make(torch.float32)
     x = torch.randn(4, D, device="cuda")
     y = torch.empty(4, O, device="cuda")
