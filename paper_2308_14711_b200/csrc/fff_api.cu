@@ -99,7 +99,7 @@ struct fff_handle_s {
     // direct lists (slot_tokens in descent_umma.cuh): when one tcgen05 stage is the whole descent and the tcgen05
     // leaf kernel follows, the descent files every token under its leaf itself and no bucketing kernel runs
     int32_t* ws_slots = nullptr;     // [n_leaves][slot_cap] token numbers
-    int32_t* ws_cursor = nullptr;    // [n_leaves] entries used (+ [1] finished CTAs of k_block_forward); zero between calls
+    int32_t* ws_cursor = nullptr;    // [n_leaves] entries used, [1] finished CTAs, [1] CTAs at k_block_forward's barrier; zero between calls
     int64_t slot_cap = 0;
     bool cursor_dirty = false;       // a descent has filled the lists and no leaf kernel has cleared the counts since
     bool slots_now = false;          // the call in progress uses the direct lists
@@ -405,6 +405,7 @@ bool use_tensor_leaf(const fff_handle_s* h) {
 // Tokens for which the leaves' lists stay within kMaxSlotBytes, and the fewest that k_block_forward is given at a time.
 int64_t listed_tokens(const fff_handle_s* h) { return (int64_t)(kMaxSlotBytes / sizeof(int32_t)) / h->n_leaves; }
 constexpr int64_t kMinListedTokens = 1024;
+size_t cursor_bytes(const fff_handle_s* h) { return sizeof(int32_t) * (size_t)(h->n_leaves + 2); }
 
 // Whether forwards of this handle, as it is pinned now, run as the one-launch kernel on CUDA cores: the layers without a
 // tensor-core leaf path, and those pinned to it.  Shapes and the path alone decide, not what the handle has served before.
@@ -460,7 +461,7 @@ fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
             s = dmalloc((void**)&h->ws_slots, sizeof(int32_t) * (size_t)h->n_leaves * (size_t)cap);
         }
         if (s != FFF_OK) return s;
-        if ((s = clone((void**)&h->ws_cursor, nullptr, sizeof(int32_t) * (size_t)(h->n_leaves + 1))) != FFF_OK) return s;
+        if ((s = clone((void**)&h->ws_cursor, nullptr, cursor_bytes(h))) != FFF_OK) return s;
         h->slot_cap = cap;
         h->cursor_dirty = false;
     }
@@ -1204,7 +1205,7 @@ fff_status_t run_forward_grouped_tiles(fff_handle_s* h, const void* x, void* y, 
     using L = fff::LeafUmmaLayout<16, false, fff::kLUGroup, kSplit>;
     constexpr auto kernel = fff::k_leaf_umma<16, true, false, fff::kLUGroup, kSplit>;
     const int bins = (int)(h->n_leaves / fff::kLUGroup);
-    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
+    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, cursor_bytes(h), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     h->cursor_dirty = true;
     h->blocksum_wanted = false;
@@ -1279,7 +1280,7 @@ bool use_block_forward(const fff_handle_s* h) {
 template <typename T>
 fff_status_t launch_block_forward(fff_handle_s* h, const void* x, void* y, int32_t* leaf_out, int32_t* leaf_out2, int64_t B,
                                   cudaStream_t st) {
-    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
+    if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, cursor_bytes(h), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     h->cursor_dirty = true;
     // (one: 2048 tokens of 768 columns keep 14 warps per SM busy instead of 3.5; four: a quarter of the node rows' traffic)
@@ -1303,7 +1304,7 @@ fff_status_t launch_block_forward(fff_handle_s* h, const void* x, void* y, int32
     if (cudaLaunchKernelEx(&cfg, single ? fff::k_block_forward<T, 1> : fff::k_block_forward<T, 4>, (const T*)x, (const T*)h->node_w,
                            (const T*)h->node_b, (const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, (T*)y, leaf_out, leaf_out2,
                            h->ws_slots, h->ws_cursor, (int)h->slot_cap, h->D, h->O, h->depth, h->l, h->act, (int)B,
-                           h->vec_ok && aligned16(x), (int)h->n_leaves, tile_rows) != cudaSuccess)
+                           h->vec_ok && aligned16(x), (int)h->n_leaves, tile_rows, h->d_status) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     const fff_status_t s = launched(h, st, "fused_forward_blocks");
     if (s == FFF_OK) h->cursor_dirty = false;
@@ -1963,7 +1964,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
         return s;
     }
     if (h->slots_now) {
-        if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, sizeof(int32_t) * (size_t)(h->n_leaves + 1), st) != cudaSuccess)
+        if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, cursor_bytes(h), st) != cudaSuccess)
             return h->slots_now = false, cudaGetLastError(), FFF_ERR_CUDA;
         h->cursor_dirty = true;
         s = run_descent(h, x, leaf, nullptr, B, st);

@@ -8,7 +8,7 @@
 //            one token per warp (batches that could not fill the GPU otherwise) the seven nodes of three levels at a time, so
 //            that a round trip to L2 decides three levels.  Each token is then filed under its leaf: one atomic add on the
 //            leaf's cursor, one store into the leaf's list;
-//   barrier  one grid-wide barrier;
+//   barrier  one grid-wide barrier (bounded, like every wait: a CTA that gives up records kDevTimeout and leaves the leaves out);
 //   phase B  leaves.  Tiles of up to tile_rows = 8 or 16 tokens of one leaf, derived by every CTA from the counts.  A warp evaluates blocks of
 //            4 tokens x 8 hidden units; the output layer runs with one output neuron per thread against the tile's tokens.
 // The dot products of a block keep all lanes along the input dimension, so that rows of x and of the weights are read as
@@ -21,8 +21,6 @@
 // float32 accumulation; a token's result depends neither on its position in a block nor on the tokens beside it (the sums
 // are added in the same tree wherever they stand), so outputs are bit-reproducible although the lists' order is not.
 #pragma once
-
-#include <cooperative_groups.h>
 
 #include "common.cuh"
 
@@ -131,17 +129,37 @@ __device__ __forceinline__ int64_t subtree_row(int m, int64_t n, int q, int leve
     return (((int64_t)1 << (m + lev)) - 1) + (n << lev) + (q - ((1 << lev) - 1));
 }
 
-// slots: [n_leaves][cap] token numbers, cursor: [n_leaves] counts + [1] CTAs that have finished; cursor is zero on entry and
-// again when the launch has ended (the last CTA clears it).  leaf_out, leaf_out2 (optional): leaf of every token.
+// Waits until all CTAs of the (cooperative) launch have arrived; `count` is zero before the launch.  What a CTA wrote before it
+// arrived is visible to all after it.  False after kGridWaitCycles: long enough for CTAs that another stream's kernel holds up.
+constexpr long long kGridWaitCycles = 1ll << 34;           // about 9 s at 1.9 GHz
+__device__ __forceinline__ bool grid_barrier(int* count) {
+    __shared__ int s_all;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(count, 1);
+        const long long t0 = clock64();
+        int seen;
+        do {
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+        } while (seen < (int)gridDim.x && clock64() - t0 < kGridWaitCycles);
+        s_all = seen >= (int)gridDim.x ? 1 : 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_all != 0;
+}
+
+// slots: [n_leaves][cap] token numbers, cursor: [n_leaves] counts + [1] CTAs that have finished + [1] CTAs at the barrier; cursor is
+// zero on entry and again when the launch has ended (the last CTA clears it).  leaf_out, leaf_out2 (optional): leaf of every token.
 template <typename T, int TPW>
 __global__ void __launch_bounds__(kBFThreads, 2)
 k_block_forward(const T* __restrict__ x, const T* __restrict__ node_w, const T* __restrict__ node_b, const T* __restrict__ w1,
                 const T* __restrict__ b1, const T* __restrict__ w2, const T* __restrict__ b2, T* __restrict__ y, int32_t* __restrict__ leaf_out,
                 int32_t* __restrict__ leaf_out2, int32_t* slots, int32_t* cursor, int cap, int D, int O, int depth, int l, int act, int B,
-                bool vec, int n_leaves, int tile_rows)
+                bool vec, int n_leaves, int tile_rows, int* __restrict__ status)
 {
     static_assert(TPW == 1 || TPW == 4, "tokens per warp in the descent");
-    namespace cg = cooperative_groups;
     extern __shared__ __align__(16) int smem_bf[];
     int* s_pre = smem_bf;                                   // [n_leaves + 1] tiles before each leaf
     float* hs = reinterpret_cast<float*>(smem_bf + ((n_leaves + 1 + 3) & ~3));      // [l][kBFTile]
@@ -263,12 +281,12 @@ k_block_forward(const T* __restrict__ x, const T* __restrict__ node_w, const T* 
             slots[leaf * cap + atomicAdd(cursor + leaf, 1)] = tok;
         }
     }
-    __threadfence();
-    cg::this_grid().sync();
+    const bool all_filed = grid_barrier(cursor + n_leaves + 1);
+    if (!all_filed && tid == 0) atomicExch(status, kDevTimeout);
 
     // ---- tiles of every leaf and their running sum, by every CTA for itself
     tiles_before_bins([&](int j) { return __ldcg(cursor + j); }, n_leaves, tile_rows, s_pre, s_wsum, kBFThreads);
-    const int n_tiles = s_pre[n_leaves];
+    const int n_tiles = all_filed ? s_pre[n_leaves] : 0;
 
     // ---- phase B
     // threads per group of outputs and tokens per thread in the output layer: narrow layers share a tile's tokens out
@@ -381,7 +399,7 @@ k_block_forward(const T* __restrict__ x, const T* __restrict__ node_w, const T* 
     }
     __syncthreads();
     if (s_last)
-        for (int j = tid; j <= n_leaves; j += kBFThreads) cursor[j] = 0;
+        for (int j = tid; j <= n_leaves + 1; j += kBFThreads) cursor[j] = 0;
 }
 
 }  // namespace fff

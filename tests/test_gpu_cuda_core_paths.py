@@ -120,3 +120,27 @@ def test_batches_past_the_lists_run_in_parts(pin_first):
     y2, leaf2 = layer.forward_infer(x)
     assert torch.equal(y2, y) and torch.equal(leaf2, leaf)
     layer.close()
+
+
+def test_two_handles_on_two_streams():
+    """Grids of all SMs with a barrier each, enqueued on two streams at the same time."""
+    cfgs = [C("bf_stream_a", 200, 70, 5, 10, "silu", "f32", 5003, "normal"), C("bf_stream_b", 784, 10, 3, 32, "relu", "f32", 4100, "normal")]
+    streams = [torch.cuda.Stream() for _ in cfgs]
+    layers, xs, refs = [], [], []
+    for i, cfg in enumerate(cfgs):
+        case = util.make_case(cfg, seed=5 + i)
+        layers.append(util.make_layer(case))
+        xs.append(util.to_device(case.x, "f32"))
+        refs.append(layers[i].forward_infer(xs[i]))
+    torch.cuda.synchronize()
+    outs = [[], []]
+    for _ in range(20):
+        for i, layer in enumerate(layers):
+            with torch.cuda.stream(streams[i]):
+                outs[i].append(layer.forward_infer(xs[i]))
+    torch.cuda.synchronize()
+    for layer, got, (y, leaf) in zip(layers, outs, refs):
+        assert layer.last_status() == 0
+        for y2, leaf2 in got:
+            assert torch.equal(y2, y) and torch.equal(leaf2, leaf)
+        layer.close()
