@@ -88,6 +88,7 @@ struct fff_handle_s {
 
     // workspace
     int64_t cap_B = 0;
+    uint64_t epoch = 0;           // counts its allocations: a recorded graph holds the addresses of one
     int32_t *ws_leaf = nullptr, *ws_perm = nullptr, *ws_offsets = nullptr;
     int32_t* ws_rank = nullptr;   // per-token rank scratch of the bucketing kernel (large batches only)
     uint8_t* ws_rank8 = nullptr;  // rank of every token inside its 128-token tile, left by the first descent stage
@@ -189,6 +190,7 @@ struct fff_stack_s {
     cudaGraphExec_t exec = nullptr;
     const void *key_x = nullptr, *key_y = nullptr, *key_leaf = nullptr, *seen_x = nullptr, *seen_y = nullptr, *seen_leaf = nullptr;
     int64_t key_B = -1, seen_B = -1;
+    uint64_t key_epoch = 0;               // sum of the layers' epochs at the recording
     cudaStream_t key_stream = nullptr, seen_stream = nullptr;
     int launches = 0;
     bool replayed = false;
@@ -418,6 +420,7 @@ fff_status_t grow_workspace(fff_handle_s* h, int64_t B) {
     if (cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
     // the last forward's permutation and leaf indices go with the buffers (a bucketing still to be made from the staging buffers stays)
     if (!(h->pending_in_staging && h->bucketing_pending)) h->last_B = -1;
+    ++h->epoch;
     dfree(h->ws_leaf); dfree(h->ws_perm); dfree(h->ws_perm2); dfree(h->ws_tiles); dfree(h->ws_rank); dfree(h->ws_pos[0]);
     dfree(h->ws_rank8); dfree(h->ws_counts8); dfree(h->ws_blocksum); dfree(h->ws_slots); dfree(h->ws_cursor); dfree(h->ws_nslots);
     dfree(h->ws_ncursor);
@@ -2402,6 +2405,14 @@ fff_status_t fff_stack_forward(fff_stack_t s, const void* x, void* y, int32_t* l
             if ((rc = grow_workspace(h, B)) != FFF_OK) return rc;
         s->cap_B = B;
     }
+    // (a layer whose workspace has been replaced since, by fff_reserve or a larger batch of its own, is no longer where the graph writes)
+    uint64_t epoch = 0;
+    for (const fff_handle_s* h : s->layers) epoch += h->epoch;
+    if (s->exec && s->key_epoch != epoch) {
+        if (cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
+        cudaGraphExecDestroy(s->exec);
+        s->exec = nullptr;
+    }
     const bool same_as_graph = s->exec && s->key_x == x && s->key_y == y && s->key_leaf == leaf_idx && s->key_B == B && s->key_stream == st;
     if (s->want_graph && same_as_graph) {
         if (cudaGraphLaunch(s->exec, st) != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
@@ -2422,6 +2433,7 @@ fff_status_t fff_stack_forward(fff_stack_t s, const void* x, void* y, int32_t* l
                 if (s->exec) cudaGraphExecDestroy(s->exec);
                 s->exec = exec;
                 s->key_x = x; s->key_y = y; s->key_leaf = leaf_idx; s->key_B = B; s->key_stream = st;
+                s->key_epoch = epoch;
                 if (cudaGraphLaunch(s->exec, st) != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
                 s->replayed = true;
                 return FFF_OK;

@@ -139,6 +139,34 @@ def test_float32_stack_replayed_from_a_graph():
         l.close()
 
 
+def test_a_graph_is_not_replayed_into_workspaces_that_are_gone():
+    """The recorded launches hold the addresses of the layers' workspaces: a layer that has grown since is recorded again."""
+    cfg = wl.FFFConfig("stack_regrown", 128, 128, 6, 16, "gelu", "bf16", 3000, "normal")
+    cases, nets, norms, x_host = build(cfg, 2, 4, True, True)
+    layers = [util.make_layer(c) for c in cases]
+    stack = FFFStack(layers, True, [util.to_device(g, "bf16") for g, _ in norms], [util.to_device(b, "bf16") for _, b in norms])
+    stack.set_graph(True)
+    x = util.to_device(x_host, "bf16")
+    y = torch.empty_like(x)
+    leaf = torch.empty((2, cfg.B), dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    replayed = []
+    for it in range(7):
+        if it == 3:
+            layers[1].reserve(4 * cfg.B)
+        stack.forward(x, y, leaf, stream=side)
+        torch.cuda.synchronize()
+        replayed.append(bool(stack.last_was_replay()))
+        if it == 0:
+            want, want_leaf = y.clone(), leaf.clone()
+        assert torch.equal(y, want) and torch.equal(leaf, want_leaf)
+    assert replayed[2] and replayed[-1]
+    stack.close()
+    for l in layers:
+        l.close()
+
+
 def test_stack_argument_errors():
     from paper_2308_14711_b200 import binding
     cfg_a = wl.FFFConfig("stack_a", 64, 64, 2, 8, "relu", "f32", 10, "normal")
