@@ -41,3 +41,22 @@ def test_small_batches_in_chunks(D, O, depth, l, dtype, B):
     assert torch.equal(y_dev.cpu(), yh)
     assert layer.last_launch_count() == launches           # a chunk runs what the whole batch runs
     layer.close()
+
+
+@pytest.mark.parametrize("pinned_x,pinned_y", [(True, True), (False, False), (True, False), (False, True)])
+def test_pageable_and_pinned_buffers_give_the_same(pinned_x, pinned_y):
+    cfg = wl.FFFConfig("host_pageable", 768, 768, 6, 12, "gelu", "bf16", 3000, "normal")
+    case = util.make_case(cfg, seed=4)
+    layer = util.make_layer(case)
+    x = util.to_device(case.x, "bf16")
+    y_dev, leaf_dev = layer.forward_infer(x)
+    xh = x.cpu()
+    yh = torch.zeros((cfg.B, cfg.O), dtype=torch.bfloat16)
+    lh = torch.full((cfg.B,), -1, dtype=torch.int32)
+    if pinned_x:
+        xh = xh.pin_memory()
+    if pinned_y:
+        yh, lh = yh.pin_memory(), lh.pin_memory()
+    layer.forward_infer_host(xh, yh, lh)
+    assert torch.equal(yh, y_dev.cpu()) and torch.equal(lh, leaf_dev.cpu())
+    layer.close()
