@@ -840,15 +840,29 @@ bool leaf_lists_fit(const fff_handle_s* h, int64_t B) {
     return h->ws_slots && B <= h->slot_cap && h->n_leaves * h->slot_cap <= INT32_MAX && planned_tokens(h, B) <= listed_tokens(h);
 }
 
+// Thin leaves that are evaluated token by token anyway, with fewer than four tokens each: whether the leaf kernel's own walk through
+// all levels beats the stages, their bucketing and the walk through the rest.  The line lies where the walk's row loads end: its
+// loop takes 256 columns at a time, and widths that fill the steps (or end in the third) are cheap.  us, walk and stages:
+//   256, 512, 768, 1024 columns and 513 to 768: 768 columns, 14 levels, 3000 tokens 20.7 and 22.8, 5409 27.6 and 35.1, 6900 33.0 and
+//   36.2, 8192 39.8 and 40.8; 12 levels, 5409 24.8 and 29.2, 8192 35.1 and 33.0;
+//   other widths below 512: 328 columns, 14 levels, 4096 tokens 22.7 and 26.8, 4800 26.8 and 26.9, 6144 31.0 and 26.9;
+//   other widths above 768: 896 columns, 12 levels, 4096 tokens 31.1 and 33.1, 5409 39.0 and 34.7, 8192 53.4 and 39.2; against a single
+//   stage (fewer than 16 tokens per group of the second) 824 columns, 14 levels, 3000 tokens 28.9 and 28.9, 3600 34.9 and 31.0; against
+//   two, 4096 35.0 and 38.8, 4800 42.9 and 39.2.
+bool walks_alone(const fff_handle_s* h, const std::vector<fff_handle_s::DenseStage>& plan, int64_t B) {
+    if (use_tensor_leaf(h) || B >= 4 * h->n_leaves) return false;
+    if (h->D % 256 == 0 || (h->D > 512 && h->D <= 768)) return B <= 7000;
+    if (h->D < 512) return B <= 5000;
+    const bool one_stage = plan.size() < 2 || (B >> plan[1].L0) < 16;
+    return B <= (one_stage ? 3072 : 4608);
+}
+
 int dense_stage_count(const fff_handle_s* h, int64_t call_B) {
     const int64_t B = planned_tokens(h, call_B);
     const auto& plan = stage_plan(h);
     if (plan.empty() || h->path == FFF_PATH_WARP) return 0;
     if (h->path == FFF_PATH_TENSOR) return (int)plan.size();
-    // Thin leaves that are evaluated token by token anyway: up to 8192 tokens the leaf kernel's own walk through all levels
-    // beats two stages, a node bucketing and the walk through the rest (600 columns, 14 levels: 18 against 21 us at 1024
-    // tokens, 21 against 36 at 4096; at 16 384 73 against 56).
-    if (!use_tensor_leaf(h) && B < 4 * h->n_leaves && B <= 8192) return 0;
+    if (walks_alone(h, plan, B)) return 0;
     int n = 0;
     for (const auto& sg : plan) {
         if ((B >> sg.L0) < 16) break;

@@ -1,4 +1,5 @@
-"""Which leaf kernel runs: trees of few leaves, where a leaf has hundreds of tiles, and the parity of what is chosen."""
+"""Which kernels run: trees of few leaves, where a leaf has hundreds of tiles; thin leaves, whose kernel can walk the whole tree; and
+the parity of what is chosen."""
 import numpy as np
 import pytest
 import torch
@@ -31,4 +32,22 @@ def test_trees_of_few_leaves(depth, l, B, kernel):
     assert names[-1] == kernel, names
     np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
     util.check_outputs(y, y_ref, "bf16")
+    layer.close()
+
+
+@pytest.mark.parametrize("D,depth,B,launches", [
+    (256, 12, 7000, 1), (256, 12, 7001, 3), (640, 13, 7000, 1), (640, 13, 7001, 3), (328, 12, 5000, 1), (328, 12, 5001, 3),
+    (896, 12, 4608, 1), (896, 12, 4609, 3), (896, 13, 3072, 1), (896, 13, 3073, 2), (896, 13, 4096, 1), (896, 13, 4609, 3),
+    (256, 10, 4095, 1), (256, 10, 4096, 5),              # (four tokens per leaf: two stages, a bucketing behind each, the leaves)
+])
+def test_thin_leaves_walk_the_tree_themselves(D, depth, B, launches):
+    cfg = C("thin", D, 64, depth, 1, "relu", "bf16", B, "normal", node_bias_std=0.1)
+    case = util.make_case(cfg, seed=2)
+    y_ref, leaf_ref = orc.forward_i(case.net, case.x, threads=util.ORACLE_THREADS)
+    layer = util.make_layer(case)
+    y, leaf = layer.forward_infer(util.to_device(case.x, "bf16"))
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
+    util.check_outputs(y, y_ref, "bf16")
+    assert layer.last_launch_count() == launches
     layer.close()
