@@ -204,7 +204,7 @@ typedef enum {
                                      that follows (0: bucketing kernels) */
     FFF_TUNE_FUSED_SMALL = 5,     /* one launch on CUDA cores: descent, grid barrier, leaves by tiles of 16 tokens (0: descent,
                                      bucketing and leaf kernels).  Taken by default by layers without a tensor-core
-                                     leaf path and at most 4096 leaves */
+                                     leaf path and at most 4096 leaves, unless thin leaves get a few tokens each */
     FFF_TUNE_GROUP_TILES = 6,     /* leaf kernel tiles of tokens that share the node three levels above the leaves: the
                                      first descent stage stops there, the leaf kernel walks the last three levels from
                                      7 extra accumulator columns and evaluates the node's 8 leaves side by side, each

@@ -1284,14 +1284,27 @@ fff_status_t plan_block_forward(fff_handle_s* h) {
     return FFF_OK;
 }
 
-// Whether a forward of this handle runs as the one-launch kernel: when pinned to it, or by default for layers that have no
-// tensor-core leaf path.  Measured against what it replaces, one warp per token (three launches) or, for small trees, a kernel
-// that kept 32 hidden neurons per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44 against 110 us,
-// 50 432 tokens 289 against 646; 1000 -> 992, 512 leaves of 32, 8192 tokens 156 against 1148; 512 -> 512, 32 leaves of 16, 8192
-// tokens 32 against 429; 784 -> 10, 8 leaves of 32, 2048 tokens 18 against 20; 256 -> 64, one leaf of 16, 65 536 tokens 122
-// against 329.  CTAs per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
-bool use_block_forward(const fff_handle_s* h) {
-    return runs_block_forward(h) && h->ws_slots && h->tune[FFF_TUNE_FUSED_SMALL];
+// Whether a forward of B tokens runs as the one-launch kernel: when pinned to it, or by default for layers that have no
+// tensor-core leaf path, where it is faster than what it replaces.  That is one warp per token (three launches) or, for small
+// trees, a kernel that kept 32 hidden neurons per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44
+// against 110 us, 50 432 tokens 289 against 646; 1000 -> 992, 512 leaves of 32, 8192 tokens 156 against 1148; 512 -> 512, 32 leaves
+// of 16, 8192 tokens 32 against 429; 784 -> 10, 8 leaves of 32, 2048 tokens 18 against 20; 256 -> 64, one leaf of 16, 65 536 tokens
+// 122 against 329.  CTAs per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
+// A tile fetches its leaf's weights once for its tokens; a leaf of a few neurons with a few tokens has little to share, while the
+// warp per token (which with fewer than four of them needs neither bucketing nor barrier) has all of its loads to itself.  One
+// launch and a warp per token, us, 768 columns, r tokens per leaf (over 1200 sizes the rule costs 1 % against the better of the two
+// each time, always taking the one launch 29 %):
+//   r < 4, float32: 512 leaves of 8, r = 2 30.0 and 31.0; 2048 leaves of 16, r = 1 106.9 and 117.9; 4096 leaves of 2, r = 1 108.5 and
+//     35.1; bf16 -> 300 (whose descent runs on tensor cores then): 2048 leaves of 16, r = 2 81.1 and 59.7;
+//   r >= 4, float32: 4096 leaves of 4, r = 4 223.9 and 146.3, r = 12 368.3 and 375.0; of 8, r = 6 314.6 and 375.9; bf16 -> 300: 4096
+//     leaves of 8, r = 4 183.9 and 107.6; of 12, r = 12 321.8 and 332.7.
+bool use_block_forward(const fff_handle_s* h, int64_t B) {
+    if (!runs_block_forward(h) || !h->ws_slots || !h->tune[FFF_TUNE_FUSED_SMALL]) return false;
+    if (h->path == FFF_PATH_FUSED) return true;
+    const bool bf16 = h->dtype == FFF_DTYPE_BF16;
+    if (B < 4 * h->n_leaves) return (int64_t)h->l * h->l * B >= h->n_leaves * (h->depth <= 9 ? 128 : 256) * (bf16 ? 2 : 1);
+    if (h->depth <= 9 || h->l >= (bf16 ? 12 : 8)) return true;
+    return !bf16 && B >= 10 * h->n_leaves && (h->l >= 4 || h->depth == 10);
 }
 
 template <typename T>
@@ -1928,7 +1941,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
         cudaEventRecord(h->prof_events[(size_t)h->prof_steps * (fff_handle_s::kMaxProfLaunches + 1)], st);
     const int64_t plan_B = planned_tokens(h, B);
     const bool token_blocks = use_token_block(h, plan_B);
-    if (token_blocks || use_block_forward(h)) {
+    if (token_blocks || use_block_forward(h, plan_B)) {
         // one launch: a CTA per token; or descent, grid barrier, leaves.  The stable bucketing is made on demand from the leaf
         // indices that are left in the workspace
         s = token_blocks ? FFF_DISPATCH(h, run_token_block, h, x, y, h->ws_leaf, leaf_idx, B, st)

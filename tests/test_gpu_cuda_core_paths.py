@@ -82,7 +82,7 @@ def launches_of(layer, x):
 
 def test_the_batches_served_before_do_not_choose_the_kernel():
     """4096 leaves: the lists of more than 65 536 tokens would pass 1 GiB."""
-    cfg = C("bf_state", 32, 24, 12, 4, "gelu", "f32", 2000, "normal")
+    cfg = C("bf_state", 32, 24, 12, 32, "gelu", "f32", 2000, "normal")
     case = util.make_case(cfg, seed=3)
     layer = util.make_layer(case)
     x = util.to_device(case.x, "f32")
@@ -144,3 +144,27 @@ def test_two_handles_on_two_streams():
         for y2, leaf2 in got:
             assert torch.equal(y2, y) and torch.equal(leaf2, leaf)
         layer.close()
+
+
+# tokens per leaf and neurons at both sides of the line; either kernel adds a token's sums in the same order
+@pytest.mark.parametrize("depth,l,B,kernel", [
+    (9, 8, 1024, "fused_forward_blocks"), (9, 8, 1023, "descent_tail+leaf_ff_warp"), (10, 16, 1024, "fused_forward_blocks"),
+    (10, 16, 1023, "descent_tail+leaf_ff_warp"), (10, 7, 4096, "grouped_leaf_ff_warp"), (10, 8, 4096, "fused_forward_blocks"),
+    (10, 3, 10240, "fused_forward_blocks"), (10, 3, 10239, "grouped_leaf_ff_warp"), (11, 3, 20480, "grouped_leaf_ff_warp"),
+    (11, 4, 20480, "fused_forward_blocks"), (8, 1, 1024, "fused_forward_blocks"), (8, 1, 1023, "descent_tail+leaf_ff_warp"),
+])
+def test_thin_leaves_with_few_tokens_keep_a_warp_per_token(depth, l, B, kernel):
+    cfg = C("bf_line", 40, 24, depth, l, "gelu", "f32", B, "normal", node_bias_std=0.1)
+    case = util.make_case(cfg, seed=3)
+    y_ref, leaf_ref = orc.forward_i(case.net, case.x, threads=util.ORACLE_THREADS)
+    layer = util.make_layer(case)
+    x = util.to_device(case.x, "f32")
+    assert launches_of(layer, x)[-1] == kernel
+    y, leaf = layer.forward_infer(x)
+    np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
+    util.check_outputs(y, y_ref, "f32")
+    layer.set_tuning("fused_small", kernel != "fused_forward_blocks")
+    if kernel == "fused_forward_blocks":
+        y2, leaf2 = layer.forward_infer(x)
+        assert launches_of(layer, x)[-1] != kernel and torch.equal(y2, y) and torch.equal(leaf2, leaf)
+    layer.close()
