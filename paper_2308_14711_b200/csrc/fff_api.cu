@@ -1031,6 +1031,13 @@ fff_status_t pack_node_images(fff_handle_s* h) {
     return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
 }
 
+// Which form of k_leaf_warp: while the warps of all tokens are resident at once with the registers that the general form wants
+// (three CTAs per SM, four where the kernel walks the last levels too), that one; beyond, the loads of six CTAs per SM outweigh the
+// few that each has in flight, as long as the leaves are narrow and rows come in vectors (769 columns, 4096 leaves of 16, 12 000 tokens
+// 460 and 508).  us, general and six CTAs: float32, 768 -> 768, 1024 leaves of 3 behind a bucketing, 3000 tokens 27.2 and 29.0, 12 000
+// 130.6 and 116.7; 512 leaves of 32, 3000 tokens 387 and 621; walking 4096 leaves of 6, 3000 tokens 60.0 and 65.1, 12 000 161 and 140; of 16, 6000 tokens 272 and 237.  Leaves of two and four neurons in vectors
+// gain at any size (768 -> 768, 4096 leaves of 2, 3000 tokens 31.3 and 28.3), leaves of one where the kernel walks (15 levels, 16 384
+// tokens 35.5 and 31.9; 12 levels behind a bucketing 35.6 and 37.2 per forward).
 template <typename T>
 fff_status_t run_leaf(fff_handle_s* h, const void* x, const int32_t* leaf_idx, const int32_t* perm, void* y,
                       int64_t B, cudaStream_t st, const DescentTail& tail = DescentTail(), int32_t* leaf_out = nullptr) {
@@ -1042,7 +1049,17 @@ fff_status_t run_leaf(fff_handle_s* h, const void* x, const int32_t* leaf_idx, c
                             h->vec_ok && aligned16(x), (const T*)h->node_w, (const T*)h->node_b, tail.level0, tail.levels, tail.pos,
                             leaf_out);
     };
-    if ((tail.levels > 0 ? launch(fff::k_leaf_warp<T, true>) : launch(fff::k_leaf_warp<T, false>)) != cudaSuccess)
+    const bool walk = tail.levels > 0, vec = h->vec_ok && aligned16(x);
+    const bool crowded = B > (int64_t)h->sm_count * fff::kLeafWarps * (walk ? 4 : 3);
+    const bool thin = vec && h->O % fff::Elem<T>::kVec == 0 && (h->l == 2 || h->l == 4 || (h->l == 1 && walk && crowded));
+    const bool dense = vec && crowded && h->l <= (walk ? 16 : 8) && (walk || h->l > 1);
+    auto kernel = [&](auto tail_form) {
+        constexpr bool kTail = decltype(tail_form)::value;
+        return thin    ? fff::k_leaf_warp<T, kTail, fff::kLeafThin>
+               : dense ? fff::k_leaf_warp<T, kTail, fff::kLeafDense>
+                       : fff::k_leaf_warp<T, kTail, fff::kLeafWide>;
+    };
+    if (launch(walk ? kernel(std::true_type{}) : kernel(std::false_type{})) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     return launched(h, st, tail.levels > 0 ? "descent_tail+leaf_ff_warp" : "grouped_leaf_ff_warp");
 }

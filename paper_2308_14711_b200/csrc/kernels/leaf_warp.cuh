@@ -46,8 +46,12 @@ __device__ __forceinline__ void copy_bytes(void* dst, const void* src) {
 
 // Dynamic shared memory: kLeafWarps * l floats (hidden activations per warp).
 // kTail: walk tail_levels levels of the descent first (a separate instantiation keeps the plain kernel lean).
-template <typename T, bool kTail>
-__global__ void __launch_bounds__(kLeafWarps * 32, 6)      // (six CTAs per SM: 35.5 -> 31.9 us on the layer named below; eight: 32.3)
+// FORM: kLeafWide the general form; kLeafDense the same at six CTAs per SM; kLeafThin for leaves of one, two or four neurons with
+// rows in 16-byte vectors, six CTAs per SM (35.5 -> 31.9 us on the layer named below; eight: 32.3) and the output weights sent for
+// early.  The line is drawn in run_leaf (fff_api.cu).
+enum : int { kLeafWide = 0, kLeafDense = 1, kLeafThin = 2 };
+template <typename T, bool kTail, int FORM>
+__global__ void __launch_bounds__(kLeafWarps * 32, FORM == kLeafWide ? 0 : 6)
 k_leaf_warp(const T* __restrict__ x, const int32_t* __restrict__ leaf_idx, const int32_t* __restrict__ perm,
             const T* __restrict__ w1, const T* __restrict__ b1, const T* __restrict__ w2, const T* __restrict__ b2,
             T* __restrict__ y, int D, int O, int l, int act, int64_t B, bool vec,
@@ -85,8 +89,10 @@ k_leaf_warp(const T* __restrict__ x, const int32_t* __restrict__ leaf_idx, const
         const T* b1j = b1 + j * (int64_t)l;
         // With about a token per leaf these weights come from DRAM: the output layer's lines are sent for now, so that they
         // arrive in L2 while the hidden layer is evaluated (15 levels, 768 columns, l = 1, 16 384 tokens: 36.8 -> 35.5 us).
-        prefetch_lines(w2 + j * (int64_t)O * l, (int64_t)O * l * (int)sizeof(T), lane);
-        prefetch_lines(b2 + j * (int64_t)O, (int64_t)O * (int)sizeof(T), lane);
+        if constexpr (FORM == kLeafThin) {
+            prefetch_lines(w2 + j * (int64_t)O * l, (int64_t)O * l * (int)sizeof(T), lane);
+            prefetch_lines(b2 + j * (int64_t)O, (int64_t)O * (int)sizeof(T), lane);
+        }
 
         // hidden layer: U neurons at a time share the loads of x
         for (int i0 = 0; i0 < l; i0 += U) {
@@ -152,12 +158,23 @@ k_leaf_warp(const T* __restrict__ x, const int32_t* __restrict__ leaf_idx, const
                 copy_bytes<N * (int)sizeof(T)>(yt + o, out);
             }
         };
-        if (vec && l == 1 && O % V == 0) {
+        if (FORM == kLeafThin && l == 1) {
             thin(std::integral_constant<int, 1>{});
-        } else if (vec && l == 2 && O % V == 0) {
+        } else if (FORM == kLeafThin && l == 2) {
             thin(std::integral_constant<int, 2>{});
-        } else if (vec && l == 4 && O % V == 0) {
+        } else if (FORM == kLeafThin && l == 4) {
             thin(std::integral_constant<int, 4>{});
+        } else if (FORM != kLeafThin && l == 1 && vec && O % V == 0) {
+            const float h0 = h[0];
+            for (int o = lane * V; o < O; o += 32 * V) {
+                float fw[V], fb[V];
+                Elem<T>::load_vec(w2j + o, fw);
+                Elem<T>::load_vec(b2j + o, fb);
+                alignas(16) T out[V];
+#pragma unroll
+                for (int e = 0; e < V; ++e) out[e] = Elem<T>::from_float(fmaf(fw[e], h0, fb[e]));
+                *reinterpret_cast<uint4*>(yt + o) = *reinterpret_cast<const uint4*>(out);
+            }
         } else {
 #pragma unroll 4
             for (int o = lane; o < O; o += 32) {

@@ -51,3 +51,23 @@ def test_thin_leaves_walk_the_tree_themselves(D, depth, B, launches):
     util.check_outputs(y, y_ref, "bf16")
     assert layer.last_launch_count() == launches
     layer.close()
+
+
+# the three forms of the warp leaf kernel at their lines (148 SMs: 3552 tokens behind a bucketing, 4736 with a walk), rows in vectors
+# and not, outputs that fill vectors and not
+@pytest.mark.parametrize("D,O,depth,l,B", [
+    (64, 48, 12, 1, 4736), (64, 48, 12, 1, 4737), (64, 46, 12, 2, 4737), (64, 48, 12, 4, 900), (64, 48, 12, 3, 4736), (64, 48, 12, 3, 4737),
+    (64, 48, 12, 16, 4737), (64, 48, 12, 17, 4737), (63, 48, 12, 3, 4737), (64, 48, 9, 1, 3553), (64, 48, 9, 4, 3553), (64, 48, 9, 8, 3552),
+    (64, 48, 9, 8, 3553), (64, 48, 9, 9, 3553), (63, 45, 9, 5, 3553),
+])
+def test_forms_of_the_warp_leaf_kernel(D, O, depth, l, B):
+    cfg = C("forms", D, O, depth, l, "silu", "f32", B, "normal", node_bias_std=0.1)
+    case = util.make_case(cfg, seed=6)
+    y_ref, leaf_ref = orc.forward_i(case.net, case.x, threads=util.ORACLE_THREADS)
+    layer = util.make_layer(case)
+    layer.set_path("warp")
+    y, leaf = layer.forward_infer(util.to_device(case.x, "f32"))
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
+    util.check_outputs(y, y_ref, "f32")
+    layer.close()
