@@ -857,12 +857,13 @@ bool walks_alone(const fff_handle_s* h, const std::vector<fff_handle_s::DenseSta
     return B <= (one_stage ? 3072 : 4608);
 }
 
-int dense_stage_count(const fff_handle_s* h, int64_t call_B) {
+// leaf_walks: a leaf kernel follows that can walk the levels left over itself.
+int dense_stage_count(const fff_handle_s* h, int64_t call_B, bool leaf_walks) {
     const int64_t B = planned_tokens(h, call_B);
     const auto& plan = stage_plan(h);
     if (plan.empty() || h->path == FFF_PATH_WARP) return 0;
     if (h->path == FFF_PATH_TENSOR) return (int)plan.size();
-    if (walks_alone(h, plan, B)) return 0;
+    if (leaf_walks && walks_alone(h, plan, B)) return 0;
     int n = 0;
     for (const auto& sg : plan) {
         if ((B >> sg.L0) < 16) break;
@@ -885,7 +886,7 @@ struct DescentTail {
 fff_status_t run_descent(fff_handle_s* h, const void* x, int32_t* leaf_out, Coarse* coarse, int64_t B, cudaStream_t st,
                          DescentTail* defer_tail = nullptr, bool leaf_bucketing_follows = false) {
     fff_status_t s = FFF_OK;
-    const int n_dense = dense_stage_count(h, B);
+    const int n_dense = dense_stage_count(h, B, defer_tail != nullptr);
     // the first stage's counts are summed per block of tiles only if the bucketing kernel that reads (and clears)
     // the sums comes next: a node bucketing before the second stage, or the caller's leaf bucketing
     h->blocksum_wanted = n_dense > 1 || (n_dense == 1 && leaf_bucketing_follows && coarse != nullptr &&
@@ -1990,7 +1991,7 @@ fff_status_t fff_forward_infer(fff_handle_t h, const void* x, void* y, int32_t* 
                    leaf_lists_fit(h, B) &&
                    (plan.umma ? tile_rows == fff::kLUM : h->n_leaves <= kMaxListedLeaves && plan_B <= kMaxListedTokens) && h->ustages.back().umma &&
                    h->ustages.back().L0 + h->ustages.back().k == h->depth &&
-                   dense_stage_count(h, B) == (int)h->ustages.size() &&
+                   dense_stage_count(h, B, false) == (int)h->ustages.size() &&
                    (h->ustages.size() == 1 ||
                     (h->tune[FFF_TUNE_TCGEN05_GROUPED] && (fills_grouped_tiles(h, B, h->ustages.back().L0) ||
                                                            (h->ustages.size() == 2 && node_lists_fit(h, B)))));

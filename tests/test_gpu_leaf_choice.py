@@ -71,3 +71,17 @@ def test_forms_of_the_warp_leaf_kernel(D, O, depth, l, B):
     np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
     util.check_outputs(y, y_ref, "f32")
     layer.close()
+
+
+def test_the_descent_alone_keeps_its_stages():
+    """The walk is the leaf kernel's: fff_tree_descent, behind which there is none, runs the stages."""
+    cfg = C("descent_alone", 256, 64, 12, 1, "relu", "bf16", 3000, "normal", node_bias_std=0.1)
+    case = util.make_case(cfg, seed=2)
+    _, leaf_ref = orc.forward_i(case.net, case.x, threads=util.ORACLE_THREADS)
+    layer = util.make_layer(case)
+    x = util.to_device(case.x, "bf16")
+    np.testing.assert_array_equal(layer.tree_descent(x).cpu().numpy(), leaf_ref)
+    assert layer.last_launch_count() == 2                  # two stages, lists between them
+    layer.forward_infer(x)
+    assert layer.last_launch_count() == 1
+    layer.close()
