@@ -128,6 +128,13 @@ fff_status_t fff_create_w8(fff_handle_t *out, int D, int O, int depth, int leaf_
  *   y         [B, O]  out
  *   leaf_idx  [B]     out, may be NULL: the region / leaf each token was routed to
  *
+ * Which kernels run follows from the shapes and B.  All accumulate in float32,
+ * in different orders, and the tensor-core kernels of layers with D % 128 == 0
+ * round hidden values to bf16 where the CUDA-core kernels (small batches, see
+ * FFF_TUNE_TOKEN_BLOCKS) keep them float32: a token's y may differ within the
+ * rounding of bf16 between two batch sizes, its leaf only if a routing logit is
+ * zero to float32 accuracy.  float32 layers give the same bits at every B.
+ *
  * B == 0 is FFF_OK and enqueues nothing.  If B exceeds what fff_reserve was
  * given, the workspace is grown first (this allocates and synchronises).
  * Otherwise the call only enqueues kernels (and at most a small memset) and
@@ -193,7 +200,8 @@ fff_status_t fff_reserve(fff_handle_t h, int64_t max_B);
 fff_status_t fff_set_path(fff_handle_t h, fff_path_t path);
 
 /* Switches between kernels that compute the same thing, for A/B timing and tests.  Every switch is on (1) by
- * default, which is the measured best; results never depend on them.  The paper describes no such choices.
+ * default, which is the measured best; results depend on them as on B (fff_forward_infer), within rounding.
+ * The paper describes no such choices.
  * FFF_ERR_INVALID_ARG for an unknown key or a value other than 0 or 1. */
 typedef enum {
     FFF_TUNE_TCGEN05_DESCENT = 0, /* first descent stage of up to 8 levels on tcgen05 (0: stages of <= 6 levels on mma.sync) */
@@ -316,15 +324,19 @@ fff_status_t fff_selftest_bounded_wait(fff_handle_t h, int64_t limit_cycles, voi
 
 /* Which kernel families the shapes of this layer admit (a bit set; -1 for a bad handle).  A bf16 layer whose
  * D is no multiple of 8, whose O is no multiple of 8 or whose leaves are wider than 64 has no tensor-core
- * kernels: its forward runs on CUDA-core kernels (the one-launch kernel when FFF_CAP_FUSED_SMALL is set, else
- * one warp per token), which is several times slower per token; float32 layers never have them.  Callers
+ * leaf kernels: it runs on CUDA-core kernels (the one-launch kernel, or one warp per token where leaves are thin
+ * and get a few tokens each), which is several times slower per token; float32 layers never have them.  Callers
  * that depend on tensor-core speed can check here instead of timing. */
 typedef enum {
     FFF_CAP_TENSOR_DESCENT = 1,   /* staged descent on tensor cores (bf16, D % 128 == 0, depth > 0) */
     FFF_CAP_TCGEN05_DESCENT = 2,  /* ... its first stage on tcgen05 */
     FFF_CAP_TENSOR_LEAF = 4,      /* grouped leaf evaluation on tensor cores (also O % 8 == 0, l <= 64) */
     FFF_CAP_TCGEN05_LEAF = 8,     /* ... on tcgen05 (also O % 16 == 0) */
-    FFF_CAP_FUSED_SMALL = 16,     /* the one-launch kernel (l <= 32, at most one group of 32 neurons per SM) */
+    FFF_CAP_FUSED_SMALL = 16,     /* FFF_PATH_FUSED may be set: small trees with thin leaves and rows that are not too wide (l <= 32;
+                                     2^depth leaves of l, rounded up to a power of two, hold at most 32 neurons per SM;
+                                     128 D' + 256 O + 32 max(D', 512) <= 225992 with D' = D rounded up to a multiple of 4).  The
+                                     kernel itself runs on more layers and is chosen by FFF_PATH_AUTO there too
+                                     (FFF_TUNE_FUSED_SMALL) */
     FFF_CAP_FORWARD_TRAIN = 32,   /* fff_forward_train (bf16, D % 64 == 0) */
     FFF_CAP_PADDED = 128,         /* the tensor-core kernels run on images padded to the next multiple of 128 (D % 128 != 0, D % 8 == 0).
                                      The bits 1 to 8 then stay clear and fff_set_path refuses FFF_PATH_TENSOR, although the forward

@@ -393,6 +393,9 @@ LeafPlan leaf_plan(const fff_handle_s* h, int64_t B) {
 // 41.5; 512 leaves of 16: 8192 42.5 and 33.9, 16 384 47.2 and 42.6; 256 -> 256, 2048 leaves of 10: 8192 42.5 and 26.4, 24 000
 // 48.4 and 36.6.  It fetches a row in pieces of 64 bytes, which tells once the rows outweigh the weights: 1024 -> 1024, 2048
 // leaves of 16: 16 384 tokens (32 MB) 91.1 and 90.2, 20 000 94.8 and 100.9; 768 -> 768, 1024 leaves of 16: 32 768 73.2 and 85.5.
+// With tokens of 16 clusters, which fill a few leaves (their weights then come from L2): 768 -> 768, 2048 leaves of 12: 16 384 tokens
+// 58.2 and 41.0; 1024 of 16: 16 384 47.4 and 37.3; 512 of 16: 8192 37.4 and 31.1, 19 968 55.5 and 48.0; 256 -> 256, 2048 of 10: 16 384
+// 44.9 and 27.6.
 bool warp_tiles(const fff_handle_s* h, const LeafPlan& plan, int64_t B) {
     return h->LP == 16 && !plan.resident && h->n_leaves <= kMaxListedLeaves && B < 40 * h->n_leaves &&
            B * h->D * h->esize <= ((int64_t)32 << 20);
@@ -1293,7 +1296,8 @@ fff_status_t plan_block_forward(fff_handle_s* h) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n4, fff::k_block_forward<T, 4>, fff::kBFThreads, smem) != cudaSuccess)
         return cudaGetLastError(), FFF_OK;
     h->bf_per_sm = std::min(2, std::min(n1, n4));
-    // layers that can be pinned to it: small trees with thin leaves
+    // The layers that may be pinned to it (FFF_PATH_FUSED, FFF_CAP_FUSED_SMALL): a promise of the interface, small trees with thin
+    // leaves and rows that are not too wide, and narrower than what the kernel takes (above).
     int lp = 1;
     while (lp < h->l) lp <<= 1;
     const int64_t Dr = (h->D + 3) & ~3, rows = std::max<int64_t>(Dr, 512);

@@ -168,3 +168,21 @@ def test_thin_leaves_with_few_tokens_keep_a_warp_per_token(depth, l, B, kernel):
         y2, leaf2 = layer.forward_infer(x)
         assert launches_of(layer, x)[-1] != kernel and torch.equal(y2, y) and torch.equal(leaf2, leaf)
     layer.close()
+
+
+@pytest.mark.parametrize("D,O,depth,l,B", [(768, 64, 5, 12, 300), (101, 37, 7, 7, 500), (64, 48, 8, 33, 200), (72, 40, 3, 1, 450)])
+def test_float32_gives_the_same_bits_on_every_kernel(D, O, depth, l, B):
+    cfg = C("same_bits", D, O, depth, l, "gelu", "f32", B, "normal", node_bias_std=0.2)
+    case = util.make_case(cfg, seed=8)
+    layer = util.make_layer(case)
+    x = util.to_device(case.x, "f32")
+    y, leaf = layer.forward_infer(x)                       # a CTA per token
+    half, _ = layer.forward_infer(x[: B // 2].contiguous())
+    assert layer.last_launch_count() == 1 and torch.equal(half, y[: B // 2])
+    for key in ("token_blocks", "fused_small"):            # the one-launch kernel, a warp per token
+        layer.set_tuning(key, False)
+        y2, leaf2 = layer.forward_infer(x)
+        assert torch.equal(y2, y) and torch.equal(leaf2, leaf)
+    big, _ = layer.forward_infer(x.repeat(13, 1))
+    assert torch.equal(big[:B], y) and torch.equal(big[-B:], y)
+    layer.close()
