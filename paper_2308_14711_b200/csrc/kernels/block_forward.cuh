@@ -15,7 +15,8 @@
 // they lie (512 bytes per load instruction, no transposition, no staging), and 4 x 8 products share 12 row loads: 128
 // multiply-adds per 12 16-byte loads.  The 32 sums of a block are then added across the lanes with 31 shuffles
 // (lane_totals) instead of 5 each.
-// Bound: L1 throughput (48 cycles of L1 per 32 cycles of multiply-adds) for large batches, latency for small ones.
+// Bound: latency, with 16 warps per SM to hide it (float32, 768 -> 768, 256 leaves of 12, 6304 tokens, by counters: issue slots 32 %
+// busy, L1 31 %, L2 9 %); a block needs 48 cycles of L1 per 32 cycles of multiply-adds, which is what would bind next.
 // Measured: see use_block_forward in fff_api.cu.
 //
 // float32 accumulation; a token's result depends neither on its position in a block nor on the tokens beside it (the sums
