@@ -66,7 +66,7 @@ struct fff_handle_s {
     float* b1img = nullptr;
     unsigned char* w2img = nullptr;
     unsigned char* w2uimg = nullptr;   // W2 pieces (+ biases) of the tcgen05 leaf kernel (nullptr = kernel not available)
-    int* ws_sched = nullptr;           // its tile counter and finished-CTA counter (zero between launches)
+    int* ws_sched = nullptr;           // its tile counter and finished-CTA counter (zero between launches); 8-bit weights: [2] has NaN codes
     // 8-bit leaf weights (fff_create_w8): code images of the tcgen05 leaf kernel and the per-leaf scales
     bool w8 = false;
     unsigned char *w1codes = nullptr, *w2codes = nullptr;
@@ -1819,7 +1819,7 @@ fff_status_t create_common(fff_handle_t* out, int D, int O, int depth, int leaf_
             // (the caller's code arrays are read directly: nothing else of the library needs a copy of them)
             fff::k_pack_leaf_codes<__nv_bfloat16><<<h->sm_count * 8, 256>>>((const unsigned char*)leaf_w1, (const unsigned char*)leaf_w2,
                                                                            (const __nv_bfloat16*)h->b2, h->w1codes, h->w2codes, (int)nl,
-                                                                           leaf_width, LP, D, O);
+                                                                           leaf_width, LP, D, O, h->ws_sched + 2);
             fff::k_pack_b1<__nv_bfloat16><<<h->sm_count * 8, 256>>>((const __nv_bfloat16*)h->b1, h->b1img, (int)nl, leaf_width, LP);
             if (cudaGetLastError() != cudaSuccess) s = FFF_ERR_CUDA;
         }
