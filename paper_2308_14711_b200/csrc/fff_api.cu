@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "kernels/block_forward.cuh"
+#include "kernels/block_tiles.cuh"
 #include "kernels/bucket.cuh"
 #include "kernels/common.cuh"
 #include "kernels/descent_mma.cuh"
@@ -118,6 +119,10 @@ struct fff_handle_s {
     // may be pinned to it (FFF_PATH_FUSED)
     int bf_per_sm = 0;
     bool bf_pinnable = false;
+    float* w2t = nullptr;         // float32: output weights as [leaf][l][O] for k_block_tiles (nullptr: shapes not eligible)
+    int64_t bt_B = -1;            // its plan for the batch size last used
+    bool bt_fits = false;
+    fff::BlockTilesLayout bt_lay = {};
 
     // FORWARD_T (fff_forward_train): transposed output weights with the output biases appended along K, and the
     // workspace of the three GEMMs (allocated on first use)
@@ -220,7 +225,7 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 fff_status_t dmalloc(void** p, size_t bytes) {
     *p = nullptr;
-    if (bytes == 0) bytes = 16;
+    bytes = std::max<size_t>((bytes + 15) & ~(size_t)15, 16);      // (whole 16-byte vectors: bulk copies read the last one)
     return cudaMalloc(p, bytes) == cudaSuccess ? FFF_OK : (cudaGetLastError(), FFF_ERR_ALLOC);
 }
 
@@ -283,6 +288,7 @@ void prof_free(fff_handle_s* h) {
 }
 
 void release(fff_handle_s* h) {
+    dfree(h->w2t);
     dfree(h->node_w); dfree(h->node_b); dfree(h->w1); dfree(h->b1); dfree(h->w2); dfree(h->b2);
     dfree(h->ws_leaf); dfree(h->ws_perm); dfree(h->ws_perm2); dfree(h->ws_offsets); dfree(h->ws_offsets2[0]); dfree(h->ws_offsets2[1]);
     dfree(h->d_status); dfree(h->st_x); dfree(h->st_y); dfree(h->st_leaf);
@@ -1306,6 +1312,49 @@ fff_status_t plan_block_forward(fff_handle_s* h) {
     return FFF_OK;
 }
 
+// float32 layers whose operands fit shared memory in pieces run it as k_block_tiles.
+fff_status_t plan_block_tiles(fff_handle_s* h) {
+    fff::BlockTilesLayout lay;
+    if (h->bf_per_sm <= 0 || h->dtype != FFF_DTYPE_F32 || h->O > fff::kBTMaxOut ||
+        !lay.plan(h->D, h->O, h->l, (int)h->n_leaves, 8, 1, kSmemBudget))
+        return FFF_OK;
+    static bool raised[kMaxDevices] = {};
+    if (!raise_smem_limit(fff::k_block_tiles, h->device, kSmemBudget, raised)) return FFF_ERR_CUDA;
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fff::k_block_tiles, fff::kBTThreads, kSmemBudget) != cudaSuccess || n < 1)
+        return cudaGetLastError(), FFF_OK;
+    if (dmalloc((void**)&h->w2t, sizeof(float) * (size_t)h->n_leaves * h->l * h->O) != FFF_OK) return FFF_OK;      // (without it: k_block_forward)
+    fff::k_pack_w2_columns<<<h->sm_count * 8, 256>>>((const float*)h->w2, h->w2t, h->n_leaves, h->l, h->O);
+    return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
+}
+
+// How k_block_tiles runs B tokens; false: not at all (k_block_forward).  Measured, us, k_block_forward and it: 768 -> 768, 256 leaves of
+// 12, 6304 tokens 57.5 and 48.0; 936 -> 928, 16 leaves of 12, 1341 tokens 24.6 and 22.5; 784 -> 10, 8 leaves of 32, 2048 tokens 20.4 and
+// 20.5 (one tile per CTA: its loads wait for the leaf either way).
+// Tokens per warp in the descent: so many that the batch is one pass.  Rows per tile: a tile costs about as much as 20 rows before its
+// first (its weights' way through the ring, the two barriers), and the launch lasts as long as the CTA with the most tiles.
+bool block_tiles_plan(fff_handle_s* h, const void* x, int64_t B, fff::BlockTilesLayout* lay) {
+    if (!h->w2t || !aligned16(x)) return false;
+    if (h->bt_B == B) return *lay = h->bt_lay, h->bt_fits;
+    const int64_t per_sm = (B + h->sm_count - 1) / h->sm_count;
+    const int tok = (int)std::min<int64_t>(fff::kBTMaxTok, (per_sm + fff::kBTWarps - 1) / fff::kBTWarps);
+    int best = 0;
+    double best_cost = 0.0;
+    for (int rows : {8, 16, 32}) {
+        fff::BlockTilesLayout l;
+        if (!l.plan(h->D, h->O, h->l, (int)h->n_leaves, rows, tok, kSmemBudget)) continue;
+        const double tiles = std::max(1.0, expected_tiles(h, B, rows));
+        const double cost = std::ceil(tiles / h->sm_count) * (20.0 + std::min<double>(rows, B / tiles));
+        if (best == 0 || cost < best_cost) {
+            best = rows;
+            best_cost = cost;
+        }
+    }
+    h->bt_B = B;
+    h->bt_fits = best != 0 && h->bt_lay.plan(h->D, h->O, h->l, (int)h->n_leaves, best, tok, kSmemBudget);
+    return *lay = h->bt_lay, h->bt_fits;
+}
+
 // Whether a forward of B tokens runs as the one-launch kernel: when pinned to it, or by default for layers that have no
 // tensor-core leaf path, where it is faster than what it replaces.  That is one warp per token (three launches) or, for small
 // trees, a kernel that kept 32 hidden neurons per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44
@@ -1335,16 +1384,7 @@ fff_status_t launch_block_forward(fff_handle_s* h, const void* x, void* y, int32
     if (h->cursor_dirty && cudaMemsetAsync(h->ws_cursor, 0, cursor_bytes(h), st) != cudaSuccess)
         return cudaGetLastError(), FFF_ERR_CUDA;
     h->cursor_dirty = true;
-    // (one: 2048 tokens of 768 columns keep 14 warps per SM busy instead of 3.5; four: a quarter of the node rows' traffic)
-    const bool single = B <= (int64_t)h->sm_count * 2 * fff::kBFWarps * 2;      // one token per warp in the descent
-    const int64_t max_ctas = (int64_t)h->sm_count * h->bf_per_sm;
-    const int64_t grid = std::min(max_ctas, std::max<int64_t>(B, 1));
-    // thinner tiles while full ones would leave CTAs without work, unless the leaves are thin themselves
-    const int tile_rows = B <= 8 * max_ctas && B >= 32 * h->n_leaves ? 8 : fff::kBFTile;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(fff::kBFThreads);
-    cfg.dynamicSmemBytes = block_forward_smem(h);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -1353,11 +1393,35 @@ fff_status_t launch_block_forward(fff_handle_s* h, const void* x, void* y, int32
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = h->pdl && !h->prof_active ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, single ? fff::k_block_forward<T, 1> : fff::k_block_forward<T, 4>, (const T*)x, (const T*)h->node_w,
-                           (const T*)h->node_b, (const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, (T*)y, leaf_out, leaf_out2,
-                           h->ws_slots, h->ws_cursor, (int)h->slot_cap, h->D, h->O, h->depth, h->l, h->act, (int)B,
-                           h->vec_ok && aligned16(x), (int)h->n_leaves, tile_rows, h->d_status) != cudaSuccess)
-        return cudaGetLastError(), FFF_ERR_CUDA;
+    cudaError_t e = cudaErrorUnknown;
+    bool staged = false;
+    if constexpr (sizeof(T) == 4) {
+        fff::BlockTilesLayout lay;
+        if (block_tiles_plan(h, x, B, &lay)) {
+            staged = true;
+            cfg.gridDim = dim3((unsigned)std::min<int64_t>(h->sm_count, B));
+            cfg.blockDim = dim3(fff::kBTThreads);
+            cfg.dynamicSmemBytes = lay.total_bytes;
+            e = cudaLaunchKernelEx(&cfg, fff::k_block_tiles, (const float*)x, (const float*)h->node_w, (const float*)h->node_b, (const float*)h->w1,
+                                   (const float*)h->b1, (const float*)h->w2t, (const float*)h->b2, (float*)y, leaf_out, leaf_out2, h->ws_slots,
+                                   h->ws_cursor, (int)h->slot_cap, h->D, h->O, h->depth, h->l, h->act, (int)B, (int)h->n_leaves, lay, h->d_status);
+        }
+    }
+    if (!staged) {
+        // (one: 2048 tokens of 768 columns keep 14 warps per SM busy instead of 3.5; four: a quarter of the node rows' traffic)
+        const bool single = B <= (int64_t)h->sm_count * 2 * fff::kBFWarps * 2;      // one token per warp in the descent
+        const int64_t max_ctas = (int64_t)h->sm_count * h->bf_per_sm;
+        // thinner tiles while full ones would leave CTAs without work, unless the leaves are thin themselves
+        const int tile_rows = B <= 8 * max_ctas && B >= 32 * h->n_leaves ? 8 : fff::kBFTile;
+        cfg.gridDim = dim3((unsigned)std::min(max_ctas, std::max<int64_t>(B, 1)));
+        cfg.blockDim = dim3(fff::kBFThreads);
+        cfg.dynamicSmemBytes = block_forward_smem(h);
+        e = cudaLaunchKernelEx(&cfg, single ? fff::k_block_forward<T, 1> : fff::k_block_forward<T, 4>, (const T*)x, (const T*)h->node_w,
+                               (const T*)h->node_b, (const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, (T*)y, leaf_out, leaf_out2,
+                               h->ws_slots, h->ws_cursor, (int)h->slot_cap, h->D, h->O, h->depth, h->l, h->act, (int)B,
+                               h->vec_ok && aligned16(x), (int)h->n_leaves, tile_rows, h->d_status);
+    }
+    if (e != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
     const fff_status_t s = launched(h, st, "fused_forward_blocks");
     if (s == FFF_OK) h->cursor_dirty = false;
     return s;
@@ -1829,6 +1893,7 @@ fff_status_t create_common(fff_handle_t* out, int D, int O, int depth, int leaf_
     }
     if (s == FFF_OK && !w8 && h->w2uimg) s = pack_group_images<__nv_bfloat16>(h);
     if (s == FFF_OK && !w8) s = FFF_DISPATCH(h, plan_block_forward, h);
+    if (s == FFF_OK) s = plan_block_tiles(h);
     if (s == FFF_OK && !w8) plan_train(h);
     if (s == FFF_OK && cudaDeviceSynchronize() != cudaSuccess) s = (cudaGetLastError(), FFF_ERR_CUDA);
     if (s != FFF_OK) { release(h); return s; }
