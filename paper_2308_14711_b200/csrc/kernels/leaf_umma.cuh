@@ -118,12 +118,13 @@ template <int LP, bool kW8 = false, int GL = 1, bool kSplit = false> struct Leaf
     // fit, x tiles first, then the W1 tiles, then their codes.  What a ring of three stages keeps in flight then no longer
     // shrinks with the rows (2048 leaves of 32, 65 536 tokens, a forward 174.0 and 171.5 us), and a tile takes fewer stages.  The MMAs read 128 rows all the same: what lies behind the last x tile is the
     // stage's own W1, and the accumulator rows of it are never looked at.  8-bit weights: always kSub, since a stage waits for the
-    // expansion of all its K-blocks (200.7 us, with more of them 206.8).
+    // expansion of all its K-blocks (200.7 us, with more of them 206.8); neither for 64 padded neurons, whose W1 leaves room for one or two
+    // (840 -> 832, 128 leaves of 38, 7781 tokens 31.0 us, with two 31.4).
     static constexpr int sub_of(int cap_rows) {
         const int n = kStageBytes / (cap_rows * kLUKB * 2 + kW1SubBytes + kW1CodeBytes);
         return n < kSub ? kSub : n;
     }
-    static constexpr int kSub32 = kW8 ? kSub : sub_of(32), kSub64 = kW8 ? kSub : sub_of(64);
+    static constexpr int kSub32 = kW8 || LP > 32 ? kSub : sub_of(32), kSub64 = kW8 || LP > 32 ? kSub : sub_of(64);
     static_assert((kSub32 - 1) * 32 * kLUKB * 2 + kXSubBytes <= kStageBytes && (kSub64 - 1) * 64 * kLUKB * 2 + kXSubBytes <= kStageBytes,
                   "an MMA reads 128 rows within the stage");
     static constexpr int kW2Bytes = kLUPiece * kHCols * 2;                   // weights of a piece (bf16 operand)
