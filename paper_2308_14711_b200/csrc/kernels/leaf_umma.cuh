@@ -77,6 +77,24 @@ template <bool kW8> struct LeafUmmaWarps {
 };
 constexpr int kLUTmemCols = 512;
 
+// Visits of the stage ring as the codes of W1 see them (8-bit weights): the stage, the warp whose turn it is to expand them, and the
+// barrier they land on.  Turns go by visits, so with an odd number of stages (three for 32 padded neurons, five for 64) a stage's visits
+// go to another warp each time.  A warp that waited on a barrier of the stage would then know nothing of the visit before its own,
+// and a parity wait passes while that one's codes are still on their way.  So every stage has a barrier per expanding warp: the owner
+// waits for each phase of its own barriers, and none can end twice without it.
+struct LeafCodeRing {
+    int stages;
+    int at = 0;                            // the barrier, of kLUExpandWarps * stages
+    uint32_t phase = 0;
+    __host__ __device__ explicit LeafCodeRing(int stages_) : stages(stages_) {}
+    __host__ __device__ int stage() const { return at >= stages ? at - stages : at; }
+    __host__ __device__ int owner() const { return at % kLUExpandWarps; }
+    __host__ __device__ void next() {
+        if (++at == kLUExpandWarps * stages) { at = 0; phase ^= 1; }
+    }
+};
+static_assert(kLUExpandWarps == 2, "LeafCodeRing::stage: two rounds of the ring");
+
 // kW8: the leaf weights are stored as 8-bit floats (e4m3 codes, one float32 scale per leaf and matrix).  The MMA wants
 // both operands as bf16, so the codes (every one is exactly a bf16 value) are expanded into the operand layout first: W1's from a
 // staging part of their ring stage, W2's in place; the scales multiply the accumulators in the epilogue.  Four warps do nothing
@@ -138,7 +156,10 @@ template <int LP, bool kW8 = false, int GL = 1, bool kSplit = false> struct Leaf
     // W2 ring: a whole tile's pieces (O <= 1024) when they are small, so that no copy waits for an MMA just issued
     static constexpr int kW2Slots = GL > 1 ? (kSplit ? 2 : 3) : LP <= 16 ? 8 : LP <= 32 ? 8 : kW8 ? 4 : 6;
     static constexpr int kAcc2Col = GL > 1 ? 256 : 64;                       // first tensor-memory column of the two GEMM2 accumulators
+    // full, empty, two per W2 slot, the queue's, seven single ones, the queue, the tensor-memory address, want; 8-bit weights: their codes'
     static constexpr int kBarrierBytes = kW8 ? 896 : 640;
+    static_assert(kBarrierBytes >= 8 * (2 * kLUMaxStages + 2 * kLUMaxW2Slots + 2 * kLUQueue + 7) + 16 * kLUQueue + 16 +
+                                       (kW8 ? 8 * (kLUExpandWarps * kLUMaxStages + kLUMaxW2Slots) : 0), "barriers");
     static constexpr int smem_bytes(int stages) {
         return 1024 + stages * kStageBytes + kW2Slots * kW2SlotStride + kHOperands * kHBytes + kBarrierBytes;
     }
@@ -371,8 +392,8 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
     Tile* queue = reinterpret_cast<Tile*>(y_empty + 2);                      // [kLUQueue]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(queue + kLUQueue);
     uint64_t* want = reinterpret_cast<uint64_t*>(tmem_slot + 2);             // the gathers have started another tile
-    uint64_t* code_full = want + 1;                                          // [kLUMaxStages] the W1 codes of a stage have landed (kW8)
-    uint64_t* w2code_full = code_full + kLUMaxStages;                        // [kLUMaxW2Slots] likewise the codes of a W2 piece
+    uint64_t* code_full = want + 1;                                          // [kLUExpandWarps * kLUMaxStages] W1 codes have landed (kW8, see LeafCodeRing)
+    uint64_t* w2code_full = code_full + kLUExpandWarps * kLUMaxStages;       // [kLUMaxW2Slots] likewise the codes of a W2 piece
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KB = D / kLUKB;                               // K-blocks of GEMM1 per tile
@@ -387,8 +408,9 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         for (int s = 0; s < kStages; ++s) {
             ptx::mbar_init(full + s, kLUGatherWarps + (kW8 ? 1 : 0));      // one arrival per gather warp (and by the warp that expands the stage)
             ptx::mbar_init(empty + s, 1);
-            if (kW8) ptx::mbar_init(code_full + s, 1);
         }
+        if (kW8)
+            for (int s = 0; s < kLUExpandWarps * kStages; ++s) ptx::mbar_init(code_full + s, 1);
         for (int s = 0; s < L::kW2Slots; ++s) {
             ptx::mbar_init(w2_full + s, 1);
             if (kW8) ptx::mbar_init(w2code_full + s, 1);
@@ -536,31 +558,30 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         // ------------------------------------------------------------------ expansion of 8-bit weights
         const int part = (warp - kLUWarps) % kLUExpandWarps;
         const bool has_nan = sched[2] != 0;                      // (written once, when the images were)
-        int mine = 0;                                            // whose turn it is: whole stages and pieces, so that the fixed costs of two overlap
+        // (turns on whole stages and pieces, so that the fixed costs of two overlap)
         if (warp < kLUWarps + kLUExpandWarps) {
             // W1: a stage's K-blocks of LP rows x 64 columns, stacked
-            int stage = 0;
-            uint32_t phase = 0;
+            LeafCodeRing codes(kStages);
             for (int it = 0; it < max_iters; ++it) {
                 const Tile tl = next_tile();
                 if (tl.rows <= 0) break;
                 const int sub = sub_blocks(tl.rows);
-                for (int k0 = 0; k0 < KB; k0 += sub, mine ^= 1) {
-                    if (mine == part) {
-                        const int n = min(sub, KB - k0);
-                        if (!timed_out && !ptx::mbar_wait(code_full + stage, phase)) timed_out = true;
+                for (int k0 = 0; k0 < KB; k0 += sub, codes.next()) {
+                    if (codes.owner() == part) {
+                        const int n = min(sub, KB - k0), stage = codes.stage();
+                        if (!timed_out && !ptx::mbar_wait(code_full + codes.at, codes.phase)) timed_out = true;
                         unsigned char* w1s = ring + stage * L::kStageBytes + n * x_sub_bytes(tl.rows);
                         expand_e4m3_tile<kLUKB>(w1s + n * L::kW1SubBytes, w1s, n * (LP * kLUKB / 16), lane, has_nan);
                         ptx::fence_proxy_async();
                         __syncwarp();
                         if (lane == 0) ptx::mbar_arrive(full + stage);
                     }
-                    if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
             }
         } else {
-            // W2: 128 output features x LP columns per piece
-            int slot = 0;
+            // W2: 128 output features x LP columns per piece (a slot's pieces are all one warp's: it sees every phase of the slot's barrier)
+            static_assert(!kW8 || L::kW2Slots % kLUExpandWarps == 0, "a slot never changes hands");
+            int slot = 0, mine = 0;
             uint32_t phase = 0;
             for (int it = 0; it < max_iters; ++it) {
                 if (next_tile().rows <= 0) break;
@@ -582,6 +603,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         const int gw = warp - kLUFirstGatherWarp;
         int stage = 0;
         uint32_t phase = 0;
+        LeafCodeRing codes(kStages);
         for (int it = 0; it < max_iters; ++it) {
             const Tile tl = next_tile();
             if (tl.rows <= 0) break;
@@ -608,8 +630,9 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                         const int64_t block = (int64_t)tl.bin * KB + k0;
                         const uint32_t w1_bytes = (uint32_t)(n * L::kW1CopyBytes);
                         if constexpr (kW8) {
-                            ptx::mbar_arrive_expect_tx(code_full + stage, w1_bytes);
-                            ptx::bulk_g2s(xs + n * (xsb + L::kW1SubBytes), w1codes + block * L::kW1CopyBytes, w1_bytes, code_full + stage);
+                            uint64_t* landed = code_full + codes.at;
+                            ptx::mbar_arrive_expect_tx(landed, w1_bytes);
+                            ptx::bulk_g2s(xs + n * (xsb + L::kW1SubBytes), w1codes + block * L::kW1CopyBytes, w1_bytes, landed);
                         } else
                             ptx::bulk_g2s(xs + n * xsb, w1img + block * (L::kW1CopyBytes / 2), w1_bytes, full + stage);
                     }
@@ -619,6 +642,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                     for (int sb = 0; sb < n; ++sb)
                         ptx::tma_gather4(xs + sb * xsb + first * 128, &tmap_x, (k0 + sb) * kLUKB, r[0], r[1], r[2], r[3], full + stage);
                 }
+                if constexpr (kW8) codes.next();
                 if (++stage == kStages) { stage = 0; phase ^= 1; }
             }
         }

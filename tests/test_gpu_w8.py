@@ -75,3 +75,25 @@ def test_w8_is_refused_where_the_tcgen05_leaf_kernel_cannot_run():
                  dev["b1"], torch.from_numpy(c2).cuda(), dev["b2"], w1_scale=torch.from_numpy(s1).cuda(),
                  w2_scale=torch.from_numpy(s2).cuda())
     assert e.value.status == 2
+
+
+# several tiles per CTA, of at most 32, at most 64 and more rows in turn (their ring stages are laid out differently), and 16 K-blocks each:
+# every stage of the rings of four, three and five is used again and again, by one expanding warp and the other
+@pytest.mark.parametrize("l", [14, 32, 64])
+def test_w8_rings_go_round_over_tiles_of_all_heights(l):
+    cfg = C("w8_rings", 1024, 256, 9, l, "gelu", "bf16", 20000, "normal", node_bias_std=0.25)
+    net, x_host, layer = make(cfg, seed=3)
+    y_ref, leaf_ref = orc.forward_i(net, x_host, threads=util.ORACLE_THREADS)
+    counts = np.bincount(leaf_ref, minlength=cfg.n_leaves)
+    last = counts[counts % 128 > 0] % 128
+    assert min((last <= 32).sum(), ((last > 32) & (last <= 64)).sum(), (last > 64).sum()) >= 40 and (counts > 0).sum() >= 400
+    x = util.to_device(x_host, "bf16")
+    y_first, _ = layer.forward_infer(x)
+    for _ in range(5):
+        y, leaf = layer.forward_infer(x)
+        torch.cuda.synchronize()
+        assert layer.last_status() == 0
+        np.testing.assert_array_equal(leaf.cpu().numpy(), leaf_ref)
+        util.check_outputs(y, y_ref, "bf16")
+        assert torch.equal(y, y_first)
+    layer.close()
