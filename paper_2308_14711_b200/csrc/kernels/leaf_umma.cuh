@@ -101,8 +101,8 @@ static_assert(kLUExpandWarps == 2, "LeafCodeRing::stage: two rounds of the ring"
 // else, two for W1 stages and two for W2 pieces, taking turns on whole stages and pieces, each starting as soon as its codes have landed.
 // What binds them is instruction fetch, with seven roles in the cache at a time: as a loop of one step of 32 units of 16 codes
 // a W2 piece of 128 x 32 takes 0.8 us, unrolled 1.9.  2048 leaves of 32, 65 536 tokens, a forward: 213 us with two warps per piece and the
-// published conversions, 208 with whole pieces per warp unrolled, 190.9 in this form.  Three or four warps per kind cost the
-// epilogue its registers.
+// published conversions, 208 with whole pieces per warp unrolled, 188.9 in this form (halves of pieces as loops 196); 896 -> 896, 256
+// leaves of 9, 8766 tokens 31.4, 32.4 and 31.3 with the first and the last.  Three or four warps per kind cost the epilogue its registers.
 // GL: leaves per tile.  1: a tile holds tokens of one leaf.  8: a tile holds tokens of one node three levels above the
 // leaves; GEMM1 then runs against the hidden units of that node's 8 leaves side by side plus the 7 nodes of its
 // subtree (N = 8 LP + 16 columns, the last 9 zero), the epilogue walks the three levels from the node logits, keeps
@@ -129,22 +129,11 @@ template <int LP, bool kW8 = false, int GL = 1, bool kSplit = false> struct Leaf
     static constexpr int kSub = GL > 1 ? 1 : LP <= 32 ? 2 : 1;
     static constexpr int kXSubBytes = kLUM * kLUKB * 2;
     static constexpr int kW1SubBytes = kN1 * kLUKB * 2;
-    static constexpr int kW1CodeBytes = kW8 ? kW1SubBytes / 2 : 0;           // staging for the codes of a W1 K-block
-    static constexpr int kW1CopyBytes = kW8 ? kW1CodeBytes : kW1SubBytes;    // what the bulk copy of a K-block brings
-    static constexpr int kStageBytes = kSub * (kXSubBytes + kW1SubBytes + kW1CodeBytes);      // a multiple of 1024
-    // Tiles of at most 64 (32) rows need half (a quarter) of a K-block's space for x: their stages hold as many more K-blocks as
-    // fit, x tiles first, then the W1 tiles, then their codes.  What a ring of three stages keeps in flight then no longer
-    // shrinks with the rows (2048 leaves of 32, 65 536 tokens, a forward 174.0 and 171.5 us), and a tile takes fewer stages.  The MMAs read 128 rows all the same: what lies behind the last x tile is the
-    // stage's own W1, and the accumulator rows of it are never looked at.  8-bit weights: always kSub, since a stage waits for the
-    // expansion of all its K-blocks (200.7 us, with more of them 206.8); neither for 64 padded neurons, whose W1 leaves room for one or two
-    // (840 -> 832, 128 leaves of 38, 7781 tokens 31.0 us, with two 31.4).
-    static constexpr int sub_of(int cap_rows) {
-        const int n = kStageBytes / (cap_rows * kLUKB * 2 + kW1SubBytes + kW1CodeBytes);
-        return n < kSub ? kSub : n;
-    }
-    static constexpr int kSub32 = kW8 || LP > 32 ? kSub : sub_of(32), kSub64 = kW8 || LP > 32 ? kSub : sub_of(64);
-    static_assert((kSub32 - 1) * 32 * kLUKB * 2 + kXSubBytes <= kStageBytes && (kSub64 - 1) * 64 * kLUKB * 2 + kXSubBytes <= kStageBytes,
-                  "an MMA reads 128 rows within the stage");
+    static constexpr int kXStageBytes = kSub * kXSubBytes;
+    static constexpr int kW1StageBytes = kSub * kW1SubBytes;
+    static constexpr int kW1CodeBytes = kW8 ? kW1StageBytes / 2 : 0;         // staging for the codes of the stage's W1 K-blocks
+    static constexpr int kW1CopyBytes = kW8 ? kW1CodeBytes : kW1StageBytes;  // what the bulk copy of a stage brings
+    static constexpr int kStageBytes = kXStageBytes + kW1StageBytes + kW1CodeBytes;      // a multiple of 1024
     static constexpr int kW2Bytes = kLUPiece * kHCols * 2;                   // weights of a piece (bf16 operand)
     static constexpr int kW2CodeBytes = kW8 ? kW2Bytes / 2 : 0;
     static constexpr int kW2BiasOff = kW2Bytes;                              // the piece's 128 float32 biases inside a slot
@@ -154,7 +143,7 @@ template <int LP, bool kW8 = false, int GL = 1, bool kSplit = false> struct Leaf
     static constexpr int kHBytes = kLUM * kHCols * 2;
     static constexpr int kHOperands = kSplit ? 2 : 1;
     // W2 ring: a whole tile's pieces (O <= 1024) when they are small, so that no copy waits for an MMA just issued
-    static constexpr int kW2Slots = GL > 1 ? (kSplit ? 2 : 3) : LP <= 16 ? 8 : LP <= 32 ? 8 : kW8 ? 4 : 6;
+    static constexpr int kW2Slots = GL > 1 ? (kSplit ? 2 : 3) : LP <= 16 ? 8 : LP <= 32 ? 8 : 4;
     static constexpr int kAcc2Col = GL > 1 ? 256 : 64;                       // first tensor-memory column of the two GEMM2 accumulators
     // full, empty, two per W2 slot, the queue's, seven single ones, the queue, the tensor-memory address, want; 8-bit weights: their codes'
     static constexpr int kBarrierBytes = kW8 ? 896 : 640;
@@ -396,12 +385,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
     uint64_t* w2code_full = code_full + kLUExpandWarps * kLUMaxStages;       // [kLUMaxW2Slots] likewise the codes of a W2 piece
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int KB = D / kLUKB;                               // K-blocks of GEMM1 per tile
-    // a tile's K-blocks per ring stage, and the bytes of x in each
-    auto sub_blocks = [](int rows) { return rows <= 32 ? L::kSub32 : rows <= 64 ? L::kSub64 : L::kSub; };
-    // how often a tile's rows are stacked in the 128 rows of GEMM2 (see the epilogue; grouped tiles are not)
-    auto stacked = [](int rows) { return GL > 1 ? 1 : rows <= 32 ? 4 : rows <= 64 ? 2 : 1; };
-    auto x_sub_bytes = [](int rows) { return (rows <= 32 ? 32 : rows <= 64 ? 64 : kLUM) * kLUKB * 2; };
+    const int KB = D / (kLUKB * L::kSub);                   // ring stages per tile
     const int P = (O + kLUPiece - 1) / kLUPiece;
 
     if (threadIdx.x == 0) {
@@ -414,7 +398,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         for (int s = 0; s < L::kW2Slots; ++s) {
             ptx::mbar_init(w2_full + s, 1);
             if (kW8) ptx::mbar_init(w2code_full + s, 1);
-            ptx::mbar_init(w2_empty + s, kFold ? 1 : 1 + kLUEpiWarps);      // the MMAs that read the weights + every reader of the biases
+            ptx::mbar_init(w2_empty + s, 1 + kLUEpiWarps);      // the MMAs that read the weights + every reader of the biases
         }
         for (int s = 0; s < kLUQueue; ++s) {
             ptx::mbar_init(q_full + s, 1);
@@ -560,18 +544,16 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         const bool has_nan = sched[2] != 0;                      // (written once, when the images were)
         // (turns on whole stages and pieces, so that the fixed costs of two overlap)
         if (warp < kLUWarps + kLUExpandWarps) {
-            // W1: a stage's K-blocks of LP rows x 64 columns, stacked
+            // W1: kSub tiles of LP rows x 64 columns per stage, stacked
             LeafCodeRing codes(kStages);
             for (int it = 0; it < max_iters; ++it) {
-                const Tile tl = next_tile();
-                if (tl.rows <= 0) break;
-                const int sub = sub_blocks(tl.rows);
-                for (int k0 = 0; k0 < KB; k0 += sub, codes.next()) {
+                if (next_tile().rows <= 0) break;
+                for (int kb = 0; kb < KB; ++kb, codes.next()) {
                     if (codes.owner() == part) {
-                        const int n = min(sub, KB - k0), stage = codes.stage();
+                        const int stage = codes.stage();
                         if (!timed_out && !ptx::mbar_wait(code_full + codes.at, codes.phase)) timed_out = true;
-                        unsigned char* w1s = ring + stage * L::kStageBytes + n * x_sub_bytes(tl.rows);
-                        expand_e4m3_tile<kLUKB>(w1s + n * L::kW1SubBytes, w1s, n * (LP * kLUKB / 16), lane, has_nan);
+                        unsigned char* w1s = ring + stage * L::kStageBytes + L::kXStageBytes;
+                        expand_e4m3_tile<kLUKB>(w1s + L::kW1StageBytes, w1s, L::kSub * LP * kLUKB / 16, lane, has_nan);
                         ptx::fence_proxy_async();
                         __syncwarp();
                         if (lane == 0) ptx::mbar_arrive(full + stage);
@@ -617,30 +599,29 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
 #pragma unroll
                 for (int i = 0; i < 4; ++i) r[i] = perm[tl.start + min(first + i, tl.rows - 1)];
             }
-            const int sub = sub_blocks(tl.rows), xsb = x_sub_bytes(tl.rows);
-            for (int k0 = 0; k0 < KB; k0 += sub) {
-                const int n = min(sub, KB - k0);
+            for (int kb = 0; kb < KB; ++kb) {
                 if (!timed_out && !ptx::mbar_wait_relaxed(empty + stage, phase ^ 1)) timed_out = true;
-                unsigned char* xs = ring + stage * L::kStageBytes;
                 if (lane == 0) {
-                    const uint32_t bytes = (uint32_t)(groups * n) * 512u + (!kW8 && gw == 0 ? (uint32_t)(n * L::kW1CopyBytes) : 0u);
+                    const uint32_t bytes = (uint32_t)groups * (512u * L::kSub) + (!kW8 && gw == 0 ? (uint32_t)L::kW1CopyBytes : 0u);
                     if (bytes > 0) ptx::mbar_arrive_expect_tx(full + stage, bytes);
                     else ptx::mbar_arrive(full + stage);
                     if (gw == 0) {
-                        const int64_t block = (int64_t)tl.bin * KB + k0;
-                        const uint32_t w1_bytes = (uint32_t)(n * L::kW1CopyBytes);
                         if constexpr (kW8) {
                             uint64_t* landed = code_full + codes.at;
-                            ptx::mbar_arrive_expect_tx(landed, w1_bytes);
-                            ptx::bulk_g2s(xs + n * (xsb + L::kW1SubBytes), w1codes + block * L::kW1CopyBytes, w1_bytes, landed);
+                            ptx::mbar_arrive_expect_tx(landed, (uint32_t)L::kW1CodeBytes);
+                            ptx::bulk_g2s(ring + stage * L::kStageBytes + L::kXStageBytes + L::kW1StageBytes,
+                                          w1codes + ((int64_t)tl.bin * KB + kb) * L::kW1CodeBytes, L::kW1CodeBytes, landed);
                         } else
-                            ptx::bulk_g2s(xs + n * xsb, w1img + block * (L::kW1CopyBytes / 2), w1_bytes, full + stage);
+                            ptx::bulk_g2s(ring + stage * L::kStageBytes + L::kXStageBytes,
+                                          w1img + ((int64_t)tl.bin * KB + kb) * (L::kW1StageBytes / 2), L::kW1StageBytes, full + stage);
                     }
                 }
                 __syncwarp();
                 if (lane < groups) {
-                    for (int sb = 0; sb < n; ++sb)
-                        ptx::tma_gather4(xs + sb * xsb + first * 128, &tmap_x, (k0 + sb) * kLUKB, r[0], r[1], r[2], r[3], full + stage);
+#pragma unroll
+                    for (int sb = 0; sb < L::kSub; ++sb)
+                        ptx::tma_gather4(ring + stage * L::kStageBytes + sb * L::kXSubBytes + first * 128, &tmap_x,
+                                         (kb * L::kSub + sb) * kLUKB, r[0], r[1], r[2], r[3], full + stage);
                 }
                 if constexpr (kW8) codes.next();
                 if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -656,22 +637,21 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             if (tl.rows <= 0) break;
             if (!timed_out && !ptx::mbar_wait(acc1_empty, (it & 1) ^ 1)) timed_out = true;
             ptx::tc_fence_after_sync();
-            const int sub = sub_blocks(tl.rows), xsb = x_sub_bytes(tl.rows);
-            for (int k0 = 0; k0 < KB; k0 += sub) {
-                const int n = min(sub, KB - k0);
+            for (int kb = 0; kb < KB; ++kb) {
                 if (!timed_out && !ptx::mbar_wait(full + stage, phase)) timed_out = true;
                 ptx::tc_fence_after_sync();
                 if (lane == 0) {
                     const uint32_t xs = ptx::smem_addr(ring + stage * L::kStageBytes);
-                    for (int sb = 0; sb < n; ++sb) {
-                        const uint64_t ad = ptx::umma_desc_k128(xs + sb * xsb);
-                        const uint64_t bd = ptx::umma_desc_k128(xs + n * xsb + sb * L::kW1SubBytes);
+#pragma unroll
+                    for (int sb = 0; sb < L::kSub; ++sb) {
+                        const uint64_t ad = ptx::umma_desc_k128(xs + sb * L::kXSubBytes);
+                        const uint64_t bd = ptx::umma_desc_k128(xs + L::kXStageBytes + sb * L::kW1SubBytes);
 #pragma unroll
                         for (int j = 0; j < kLUKB / 16; ++j)
-                            ptx::umma_bf16(tmem_base, ad + 2 * j, bd + 2 * j, idesc, (k0 | sb | j) != 0 ? 1u : 0u);
+                            ptx::umma_bf16(tmem_base, ad + 2 * j, bd + 2 * j, idesc, (kb | sb | j) != 0 ? 1u : 0u);
                     }
                     ptx::umma_commit(empty + stage);
-                    if (k0 + sub >= KB) ptx::umma_commit(acc1_full);
+                    if (kb == KB - 1) ptx::umma_commit(acc1_full);
                 }
                 __syncwarp();
                 if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -681,7 +661,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         // ------------------------------------------------------------------ W2 copies + GEMM2 issuer
         int ld_slot = 0, mm_slot = 0;
         uint32_t ld_phase = 0, mm_phase = 0;
-        int step = 0;                                            // steps issued so far (selects the accumulator)
+        int pc = 0;                                              // pieces issued so far (selects the accumulator)
         const uint32_t hs = ptx::smem_addr(hbuf);
         for (int it = 0; it < max_iters; ++it) {
             const Tile tl = next_tile();
@@ -712,47 +692,36 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             auto load_ahead = [&](int needed) {
                 while (loaded < P && load_piece(loaded <= needed)) {}
             };
-            // while the warp waits for H, slots that the tile before gives back are filled: the last pieces of a short tile are
-            // needed soon after the first
-            const long long t0 = clock64();
-            do load_ahead(-1);
-            while (loaded < P && !timed_out && !__any_sync(kFullMask, ptx::mbar_test(h_full, it & 1)) && clock64() - t0 < ptx::kWaitCycles);
+            load_ahead(-1);
             if (!timed_out && !ptx::mbar_wait(h_full, it & 1)) timed_out = true;
             ptx::tc_fence_after_sync();
-            // a step = the pieces p0 .. p0 + rep - 1, piece p0 + c into the accumulator rows of copy c
-            const int rep = stacked(tl.rows);
-            for (int p0 = 0; p0 < P; p0 += rep, ++step) {
-                const int b = step & 1, n_pieces = min(rep, P - p0);
-                load_ahead(p0 + n_pieces - 1);
-                if (!timed_out && !ptx::mbar_wait(y_empty + b, ((step >> 1) & 1) ^ 1)) timed_out = true;
-                for (int c = 0; c < n_pieces; ++c) {
-                    if (!timed_out && !ptx::mbar_wait(w2_full + mm_slot, mm_phase)) timed_out = true;
-                    ptx::tc_fence_after_sync();
-                    if (lane == 0) {
-                        const int n = min(kLUPiece, O - (p0 + c) * kLUPiece);
-                        const uint32_t idesc = ptx::umma_idesc_bf16(kLUM, n);
-                        const uint32_t ws = ptx::smem_addr(w2ring + mm_slot * L::kW2SlotStride);
-                        uint32_t skip[4];
+            for (int p = 0; p < P; ++p, ++pc) {
+                const int b = pc & 1;
+                load_ahead(p);
+                if (!timed_out && !ptx::mbar_wait(w2_full + mm_slot, mm_phase)) timed_out = true;
+                if (!timed_out && !ptx::mbar_wait(y_empty + b, ((pc >> 1) & 1) ^ 1)) timed_out = true;
+                ptx::tc_fence_after_sync();
+                if (lane == 0) {
+                    const int n = min(kLUPiece, O - p * kLUPiece);
+                    const uint32_t idesc = ptx::umma_idesc_bf16(kLUM, n);
+                    const uint32_t ws = ptx::smem_addr(w2ring + mm_slot * L::kW2SlotStride);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) skip[q] = q * rep / 4 == c ? 0u : 0xffffffffu;
+                    for (int op = 0; op < L::kHOperands; ++op)
 #pragma unroll
-                        for (int op = 0; op < L::kHOperands; ++op)
+                        for (int blk = 0; blk < L::kHBlocks; ++blk) {
+                            // (one K-block of LP columns, or with grouped tiles K-blocks of 64 columns: [128 rows][128 bytes] each)
+                            const uint64_t ad = ptx::umma_desc_rows(hs + op * L::kHBytes + blk * (kLUM * L::kRowBytes), L::kRowBytes);
+                            const uint64_t bd = ptx::umma_desc_rows(ws + blk * (kLUPiece * L::kRowBytes), L::kRowBytes);
 #pragma unroll
-                            for (int blk = 0; blk < L::kHBlocks; ++blk) {
-                                // (one K-block of LP columns, or with grouped tiles K-blocks of 64 columns: [128 rows][128 bytes] each)
-                                const uint64_t ad = ptx::umma_desc_rows(hs + op * L::kHBytes + blk * (kLUM * L::kRowBytes), L::kRowBytes);
-                                const uint64_t bd = ptx::umma_desc_rows(ws + blk * (kLUPiece * L::kRowBytes), L::kRowBytes);
-#pragma unroll
-                                for (int kk = 0; kk < L::kRowBytes / 32; ++kk)
-                                    ptx::umma_bf16_rows(tmem_base + L::kAcc2Col + b * kLUAccStride, ad + 2 * kk, bd + 2 * kk, idesc,
-                                                        (op | blk | kk) != 0 ? 1u : 0u, skip);
-                            }
-                        ptx::umma_commit(w2_empty + mm_slot);
-                        if (c == n_pieces - 1) ptx::umma_commit(y_full + b);
-                    }
-                    __syncwarp();
-                    if (++mm_slot == L::kW2Slots) { mm_slot = 0; mm_phase ^= 1; }
+                            for (int kk = 0; kk < L::kRowBytes / 32; ++kk)
+                                ptx::umma_bf16(tmem_base + L::kAcc2Col + b * kLUAccStride, ad + 2 * kk, bd + 2 * kk, idesc,
+                                               (op | blk | kk) != 0 ? 1u : 0u);
+                        }
+                    ptx::umma_commit(w2_empty + mm_slot);
+                    ptx::umma_commit(y_full + b);
                 }
+                __syncwarp();
+                if (++mm_slot == L::kW2Slots) { mm_slot = 0; mm_phase ^= 1; }
             }
         }
     } else {
@@ -760,23 +729,24 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         // A warp can only read the 32 tensor-memory lanes of its quarter, so a tile of at most 32 (64) rows would
         // leave three quarters (one half) of the epilogue warps without work and cost as much as a full tile.
         // Short tiles are therefore stacked `rep` = 4 (2) times in the 128 rows of GEMM2: H row r is written to the
-        // rows r, r + 128/rep, ... of the A operand, and a step computes `rep` pieces at once, each MMA leaving all
-        // accumulator rows but those of its copy alone.  Every warp has a half of a piece to convert and store in every
-        // step, whatever the rows; a short tile has a quarter (a half) of the steps.  (With a piece per step and the copies
-        // sharing its columns out, a step was 16 columns per thread, 0.27 us of work
-        // and 0.25 us of handshakes, and those of a tile of 32 rows took 4.2 us: now 2.3)
+        // rows r, r + 128/rep, ... of the A operand, every copy's accumulator rows then hold the same values (the
+        // rows of an MMA are independent; the extra MMA rows cost nothing), and the quarters of copy c convert and
+        // store only the c-th group of 128/rep columns of each piece.
+        // (Steps of `rep` pieces, the MMAs of piece c leaving all accumulator rows but copy c's alone, and ring stages with more
+        // K-blocks for short tiles won nothing on 2048 leaves of 32, 65 536 tokens, 168.1 and 168.0 us a forward, and lost 1 to 4 %
+        // where a CTA has few tiles: 512 -> 512, 512 leaves of 24, 12 000 tokens 38.1 and 39.5.)
         const int quarter = warp & 3, part = warp >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
         constexpr int HC = LP / kLUHParts;                       // H columns of a thread that computes H
-        int step = 0;
+        int pc = 0;
         int w2_slot = 0;
         uint32_t w2_phase = 0;
         for (int it = 0; it < max_iters; ++it) {
             const Tile tl = next_tile();
             if (tl.rows <= 0) break;
-            const int rep = stacked(tl.rows);
+            const int rep = GL > 1 ? 1 : tl.rows <= 32 ? 4 : tl.rows <= 64 ? 2 : 1;      // (grouped tiles are not stacked)
             const int qper = 4 / rep;                            // lane quarters per copy
-            const int copy = quarter / qper;                     // the copy this thread's lanes hold = its piece of every step
+            const int copy = quarter / qper;                     // the copy this thread's lanes hold = its column group
             const int row = (quarter % qper) * 32 + lane;        // the token row this thread's lane carries
             const bool active = (quarter % qper) * 32 < tl.rows; // this warp's lanes hold valid rows
             const bool h_active = active && copy == 0 && part < kLUHParts;      // the first copy's lanes hold acc1
@@ -928,64 +898,88 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
                 ptx::mbar_arrive(h_full);
             }
 
-            // Y: this thread's half of one piece of 128 columns per step
+            // Y pieces: this thread's share of the 128 columns: 64 / rep columns of column group `copy`
             __nv_bfloat16* yrow = y + (tok >= 0 ? tok : 0) * O;
-            constexpr int kCols = kLUPiece / kLUColParts;
-            for (int p0 = 0; p0 < P; p0 += rep, ++step) {
-                const int b = step & 1, n_pieces = min(rep, P - p0), p = p0 + copy;
-                if (!timed_out && !ptx::mbar_wait(y_full + b, (step >> 1) & 1)) timed_out = true;
-                const float* bias = nullptr;
-                if constexpr (!kFold) {
-                    const bool wraps = w2_slot + copy >= L::kW2Slots;
-                    const int slot = w2_slot + copy - (wraps ? L::kW2Slots : 0);
-                    if (copy < n_pieces && !timed_out && !ptx::mbar_wait(w2_full + slot, w2_phase ^ (wraps ? 1u : 0u))) timed_out = true;     // landed long ago
-                    bias = reinterpret_cast<const float*>(w2ring + slot * L::kW2SlotStride + L::kW2BiasOff);
-                }
+            const int ncw = (kLUPiece / kLUColParts) / rep;          // 64, 32 or 16
+            const int cbase = copy * (kLUPiece / rep) + part * ncw;
+            for (int p = 0; p < P; ++p, ++pc) {
+                const int b = pc & 1;
+                if (!timed_out && !ptx::mbar_wait(y_full + b, (pc >> 1) & 1)) timed_out = true;
+                if (!timed_out && !ptx::mbar_wait(w2_full + w2_slot, w2_phase)) timed_out = true;     // biases: landed long ago
                 ptx::tc_fence_after_sync();
-                const int ncols = active ? min(kLUPiece, O - p * kLUPiece) : 0;       // <= 0 past the last piece; a multiple of 16
-                for (int cc = 0; cc < kCols / 32; ++cc) {
-                    const int c0 = part * kCols + cc * 32;
-                    const int nv = min(32, ncols - c0);                  // <= 0, 16 or 32
-                    if (nv > 0) {
-                        uint32_t v[32];
-                        ptx::tmem_ld32(lane_base + L::kAcc2Col + b * kLUAccStride + c0, v);
+                const float* bias = reinterpret_cast<const float*>(w2ring + w2_slot * L::kW2SlotStride + L::kW2BiasOff);
+                const int ncols = min(kLUPiece, O - p * kLUPiece);
+                if (ncw == 16) {
+                    const int c0 = cbase;
+                    if (active && c0 < ncols) {                      // ncols is a multiple of 16
+                        uint32_t v[16];
+                        ptx::tmem_ld16(lane_base + L::kAcc2Col + b * kLUAccStride + c0, v);
                         ptx::tmem_ld_wait();
-                        const int o0 = p * kLUPiece + c0;
-                        uint32_t out[16];
-                        if (kFold) {                                     // bias already added by GEMM2
+                        uint32_t out[8];
+                        if (kFold) {
 #pragma unroll
-                            for (int e = 0; e < 16; ++e)
+                            for (int e = 0; e < 8; ++e)
                                 out[e] = ptx::pack_bf16(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
                         } else {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) {
+                            for (int e = 0; e < 4; ++e) {
                                 const float4 bb = *reinterpret_cast<const float4*>(bias + c0 + 4 * e);
                                 out[2 * e] = ptx::pack_bf16(scaled(v[4 * e], s2, bb.x), scaled(v[4 * e + 1], s2, bb.y));
                                 out[2 * e + 1] = ptx::pack_bf16(scaled(v[4 * e + 2], s2, bb.z), scaled(v[4 * e + 3], s2, bb.w));
                             }
                         }
                         if (tok >= 0) {
-                            if (wide_stores && nv == 32) {
+                            const int o0 = p * kLUPiece + c0;
+                            if (wide_stores) {
                                 ptx::st_global_v8(yrow + o0, out);
-                                ptx::st_global_v8(yrow + o0 + 16, out + 8);
+                            } else {
+                                *reinterpret_cast<uint4*>(yrow + o0) = make_uint4(out[0], out[1], out[2], out[3]);
+                                *reinterpret_cast<uint4*>(yrow + o0 + 8) = make_uint4(out[4], out[5], out[6], out[7]);
+                            }
+                        }
+                    }
+                } else {
+                    for (int cc = 0; cc * 32 < ncw; ++cc) {
+                        const int c0 = cbase + cc * 32;
+                        const int nv = min(32, ncols - c0);              // <= 0, 16 or 32
+                        if (active && nv > 0) {
+                            uint32_t v[32];
+                            ptx::tmem_ld32(lane_base + L::kAcc2Col + b * kLUAccStride + c0, v);
+                            ptx::tmem_ld_wait();
+                            const int o0 = p * kLUPiece + c0;
+                            uint32_t out[16];
+                            if (kFold) {                                 // bias already added by GEMM2
+#pragma unroll
+                                for (int e = 0; e < 16; ++e)
+                                    out[e] = ptx::pack_bf16(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
                             } else {
 #pragma unroll
-                                for (int q = 0; q < 4; ++q)
-                                    if (q * 8 < nv)
-                                        *reinterpret_cast<uint4*>(yrow + o0 + q * 8) =
-                                            make_uint4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+                                for (int e = 0; e < 8; ++e) {
+                                    const float4 bb = *reinterpret_cast<const float4*>(bias + c0 + 4 * e);
+                                    out[2 * e] = ptx::pack_bf16(scaled(v[4 * e], s2, bb.x), scaled(v[4 * e + 1], s2, bb.y));
+                                    out[2 * e + 1] = ptx::pack_bf16(scaled(v[4 * e + 2], s2, bb.z), scaled(v[4 * e + 3], s2, bb.w));
+                                }
+                            }
+                            if (tok >= 0) {
+                                if (wide_stores && nv == 32) {
+                                    ptx::st_global_v8(yrow + o0, out);
+                                    ptx::st_global_v8(yrow + o0 + 16, out + 8);
+                                } else {
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q)
+                                        if (q * 8 < nv)
+                                            *reinterpret_cast<uint4*>(yrow + o0 + q * 8) =
+                                                make_uint4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+                                }
                             }
                         }
                     }
                 }
                 ptx::tc_fence_before_sync();
                 ptx::mbar_arrive(y_empty + b);
-                if constexpr (!kFold) {
-                    __syncwarp();
-                    if (lane < n_pieces) ptx::mbar_arrive(w2_empty + (w2_slot + lane) % L::kW2Slots);
-                    w2_slot += n_pieces;
-                    if (w2_slot >= L::kW2Slots) { w2_slot -= L::kW2Slots; w2_phase ^= 1; }
-                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(w2_empty + w2_slot);
+                if (++w2_slot == L::kW2Slots) { w2_slot = 0; w2_phase ^= 1; }
             }
         }
     }

@@ -1,6 +1,6 @@
-"""The tcgen05 leaf kernel's short tiles: ring stages that hold more K-blocks for tiles of at most 64 and 32 rows, and steps that
-compute two or four output pieces at once.  Buckets of 1 to 128 rows and more, K-blocks and pieces that do not divide by those
-numbers, one piece only, pieces of 16 columns."""
+"""The tcgen05 leaf kernel's short tiles, whose rows are stacked two or four times with the copies sharing each output piece's columns
+out: buckets of 1 to 128 rows and more, numbers of K-blocks and pieces that do not divide by the copies, one piece only, pieces of 16
+columns.  And the expansion of every 8-bit code."""
 import numpy as np
 import pytest
 import torch
