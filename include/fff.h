@@ -97,7 +97,11 @@ typedef enum {
  *
  * The weights are copied (and re-laid-out for the kernels) into memory owned
  * by the handle before the call returns; the caller's buffers may be freed
- * afterwards.  The call synchronises the device.  On failure *out is NULL.
+ * afterwards.  A handle keeps each matrix in every layout that one of its
+ * kernels reads: bf16 layers with tensor-core kernels have images of all
+ * weights beside the plain ones, float32 layers with a one-launch kernel on
+ * bulk copies (most of 128 columns and more) leaf_w2 once more, transposed.
+ * The call synchronises the device.  On failure *out is NULL.
  */
 fff_status_t fff_create(fff_handle_t *out, int D, int O, int depth, int leaf_width,
                         fff_activation_t act, fff_dtype_t dtype,

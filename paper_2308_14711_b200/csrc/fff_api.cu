@@ -1312,10 +1312,20 @@ fff_status_t plan_block_forward(fff_handle_s* h) {
     return FFF_OK;
 }
 
-// float32 layers whose operands fit shared memory in pieces run it as k_block_tiles.
+// How k_block_forward runs B tokens: one token per warp in the descent or four (one: 2048 tokens of 768 columns keep 14 warps per SM
+// busy instead of 3.5; four: a quarter of the node rows' traffic), and rows per tile (thinner ones while full ones would leave CTAs
+// without work, unless the leaves are thin themselves).
+bool block_forward_single(const fff_handle_s* h, int64_t B) { return B <= (int64_t)h->sm_count * 2 * fff::kBFWarps * 2; }
+int block_forward_rows(const fff_handle_s* h, int64_t B) {
+    return B <= 8 * (int64_t)h->sm_count * h->bf_per_sm && B >= 32 * h->n_leaves ? 8 : fff::kBFTile;
+}
+
+// float32 layers whose operands fit shared memory in pieces have k_block_tiles too (block_tiles_plan says for which batches), which reads a
+// transposed copy of W2.  Rows of fewer than 128 columns and leaves of fewer than 48 neurons, or rows of more than 1500 and leaves of one, have
+// nothing for its copies to hide: of 369 random sizes of them it was faster on 19, and 1.25 times as long on average.
 fff_status_t plan_block_tiles(fff_handle_s* h) {
     fff::BlockTilesLayout lay;
-    if (h->bf_per_sm <= 0 || h->dtype != FFF_DTYPE_F32 || h->O > fff::kBTMaxOut ||
+    if (h->bf_per_sm <= 0 || h->dtype != FFF_DTYPE_F32 || h->O > fff::kBTMaxOut || (h->D < 128 && h->l < 48) || (h->l == 1 && h->D > 1500) ||
         !lay.plan(h->D, h->O, h->l, (int)h->n_leaves, 8, 1, kSmemBudget))
         return FFF_OK;
     static bool raised[kMaxDevices] = {};
@@ -1328,9 +1338,40 @@ fff_status_t plan_block_tiles(fff_handle_s* h) {
     return cudaGetLastError() == cudaSuccess ? FFF_OK : FFF_ERR_CUDA;
 }
 
-// How k_block_tiles runs B tokens; false: not at all (k_block_forward).  Measured, us, k_block_forward and it: 768 -> 768, 256 leaves of
-// 12, 6304 tokens 57.5 and 48.0; 936 -> 928, 16 leaves of 12, 1341 tokens 24.6 and 22.5; 784 -> 10, 8 leaves of 32, 2048 tokens 20.4 and
-// 20.5 (one tile per CTA: its loads wait for the leaf either way).
+// Estimates, in us, of what k_block_forward and k_block_tiles take for B tokens, less what both have in common (the launch, the barrier,
+// the rows of x and y): the passes of the descent (k steps of 128 columns for each chain of levels) and the rounds of tiles, a round being a
+// tile on every CTA.  The factors are a least-squares fit to 802 random sizes (128 to 2400 columns, 1 to 1024 outputs, 1 to
+// 4096 leaves of 2 to 80 neurons, 515 to 80 000 tokens); the whole estimates are 9 and 8 % off on average.
+double block_forward_us(const fff_handle_s* h, int64_t B) {
+    const int slots = h->sm_count * h->bf_per_sm, tile_rows = block_forward_rows(h, B);
+    const bool single = block_forward_single(h, B);
+    const double tiles = std::max(1.0, expected_tiles(h, B, tile_rows)), rounds = std::ceil(tiles / slots);
+    const double passes = std::ceil((double)B / (slots * fff::kBFWarps * (single ? 1 : 4)));
+    const int k = (h->D + 127) / 128, low = std::max(h->depth - 3, 0), chains = single ? (low + 2) / 3 : low;      // below the first three levels
+    // blocks of 4 x 8 products per warp, 2.3 times as long where rows are read value by value
+    const double blocks = std::ceil(std::ceil(std::min<double>(tile_rows, B / tiles) / 4) * ((h->l + 7) / 8) / fff::kBFWarps) * (h->vec_ok ? 1.0 : 2.3);
+    return passes * (3.7 + 0.48 * k * chains) +
+           rounds * (2.3 + 0.42 * blocks * k + 0.074 * h->l * ((h->O + 255) / 256) + 1.35e-4 * h->l * (h->D + h->O));
+}
+double block_tiles_us(const fff_handle_s* h, int64_t B, const fff::BlockTilesLayout& lay, double tiles) {
+    const double rounds = std::ceil(tiles / h->sm_count), rows = std::min<double>(lay.tile_rows, B / tiles);
+    const double passes = std::ceil((double)B / (h->sm_count * fff::kBTWarps * lay.tok));
+    const int k = (h->D + 127) / 128, low = std::max(h->depth - 3, 0), chains = lay.tok == 1 ? (low + 2) / 3 : low;
+    const int sent = (h->l + lay.w1_units - 1) / lay.w1_units + (h->l + lay.w2_units - 1) / lay.w2_units;      // ring slots per tile
+    const double blocks = std::ceil(rows / 4) * ((h->l + 7) / 8) / fff::kBTWarps;
+    return 3.4 + passes * (2.7 + chains * (0.41 + 0.085 * k * lay.tok)) + 0.012 * h->n_leaves +
+           rounds * (1.6 + 0.52 * sent + 0.39 * blocks * k + 0.047 * h->l * ((h->O + 255) / 256) * rows / 16 + 0.66e-4 * h->l * (h->D + h->O));
+}
+
+// How k_block_tiles runs B tokens; false: not at all, k_block_forward is expected to be faster.  The more rows and weights a tile has, the
+// more there is for the copies to hide; thin tiles cost their hand-overs, and one CTA per SM has no other to run meanwhile, so that a batch
+// can need two rounds of tiles where two CTAs of the other kernel need one.  Measured, us, k_block_forward and it: 768 -> 768, 256
+// leaves of 12, 6304 tokens 49.0 and 44.0, 50 432 tokens 285 and 251; 512 -> 512, 32 leaves of 16, 700 tokens 18.5 and 16.5; 1523 -> 745, 32 leaves of
+// 37, 640 tokens 76 and 33; not taken: 768 -> 768, 256 leaves of 12, 1576 tokens 26.7 and 29.9; 516 -> 780, 32 leaves of 19, 9080 tokens 51.3
+// and 67.7; 256 -> 256, 4096 leaves of 8, 16 384 tokens 135 and 175.  Over 1598 random sizes, times against the better of the two:
+// this rule 1.007 on average, always k_block_forward 1.087, it wherever it fits 1.089; more than 3 % slower than k_block_forward are 3 % of
+// the sizes with the rule and 37 % without.
+// The line is drawn 6 % past equal estimates: sizes in between are ahead as often as behind.
 // Tokens per warp in the descent: so many that the batch is one pass.  Rows per tile: a tile costs about as much as 20 rows before its
 // first (its weights' way through the ring, the two barriers), and the launch lasts as long as the CTA with the most tiles.
 bool block_tiles_plan(fff_handle_s* h, const void* x, int64_t B, fff::BlockTilesLayout* lay) {
@@ -1338,33 +1379,32 @@ bool block_tiles_plan(fff_handle_s* h, const void* x, int64_t B, fff::BlockTiles
     if (h->bt_B == B) return *lay = h->bt_lay, h->bt_fits;
     const int64_t per_sm = (B + h->sm_count - 1) / h->sm_count;
     const int tok = (int)std::min<int64_t>(fff::kBTMaxTok, (per_sm + fff::kBTWarps - 1) / fff::kBTWarps);
-    int best = 0;
-    double best_cost = 0.0;
+    double best_cost = 0.0, best_us = 0.0;
     for (int rows : {8, 16, 32}) {
         fff::BlockTilesLayout l;
         if (!l.plan(h->D, h->O, h->l, (int)h->n_leaves, rows, tok, kSmemBudget)) continue;
         const double tiles = std::max(1.0, expected_tiles(h, B, rows));
         const double cost = std::ceil(tiles / h->sm_count) * (20.0 + std::min<double>(rows, B / tiles));
-        if (best == 0 || cost < best_cost) {
-            best = rows;
+        if (best_cost == 0.0 || cost < best_cost) {
+            h->bt_lay = l;
             best_cost = cost;
+            best_us = block_tiles_us(h, B, l, tiles);
         }
     }
     h->bt_B = B;
-    h->bt_fits = best != 0 && h->bt_lay.plan(h->D, h->O, h->l, (int)h->n_leaves, best, tok, kSmemBudget);
+    h->bt_fits = best_cost > 0.0 && best_us < 1.06 * block_forward_us(h, B);
     return *lay = h->bt_lay, h->bt_fits;
 }
 
 // Whether a forward of B tokens runs as the one-launch kernel: when pinned to it, or by default for layers that have no
-// tensor-core leaf path, where it is faster than what it replaces.  That is one warp per token (three launches) or, for small
-// trees, a kernel that kept 32 hidden neurons per CTA in shared memory: float32, 768 -> 768, 256 leaves of 12, 6304 tokens 44
-// against 110 us, 50 432 tokens 289 against 646; 1000 -> 992, 512 leaves of 32, 8192 tokens 156 against 1148; 512 -> 512, 32 leaves
-// of 16, 8192 tokens 32 against 429; 784 -> 10, 8 leaves of 32, 2048 tokens 18 against 20; 256 -> 64, one leaf of 16, 65 536 tokens
-// 122 against 329.  CTAs per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
+// tensor-core leaf path, where it is faster than one warp per token (three launches): float32, 768 -> 768, 256 leaves of 12, 6304 tokens
+// 44 against 95 us, 50 432 tokens 251 against 646; 1024 -> 1024, 512 leaves of 32, 8192 tokens 141 against 1151; 512 -> 512, 32 leaves of 16,
+// 8192 tokens 35 against 174; 784 -> 10, 8 leaves of 32, 2048 tokens 21 against 44; 256 -> 64, one leaf of 16, 65 536 tokens 128 against
+// 286.  CTAs of k_block_forward per SM: two (three leave 85 registers to the 32 sums of a block: 26 against 18 us).
 // A tile fetches its leaf's weights once for its tokens; a leaf of a few neurons with a few tokens has little to share, while the
 // warp per token (which with fewer than four of them needs neither bucketing nor barrier) has all of its loads to itself.  One
-// launch and a warp per token, us, 768 columns, r tokens per leaf (over 1200 sizes the rule costs 1 % against the better of the two
-// each time, always taking the one launch 29 %):
+// launch (k_block_forward, which block_tiles_plan leaves only for less) and a warp per token, us, 768 columns, r tokens per leaf (over
+// 1200 sizes the rule costs 1 % against the better of the two each time, always taking the one launch 29 %):
 //   r < 4, float32: 512 leaves of 8, r = 2 30.0 and 31.0; 2048 leaves of 16, r = 1 106.9 and 117.9; 4096 leaves of 2, r = 1 108.5 and
 //     35.1; bf16 -> 300 (whose descent runs on tensor cores then): 2048 leaves of 16, r = 2 81.1 and 59.7;
 //   r >= 4, float32: 4096 leaves of 4, r = 4 223.9 and 146.3, r = 12 368.3 and 375.0; of 8, r = 6 314.6 and 375.9; bf16 -> 300: 4096
@@ -1408,18 +1448,13 @@ fff_status_t launch_block_forward(fff_handle_s* h, const void* x, void* y, int32
         }
     }
     if (!staged) {
-        // (one: 2048 tokens of 768 columns keep 14 warps per SM busy instead of 3.5; four: a quarter of the node rows' traffic)
-        const bool single = B <= (int64_t)h->sm_count * 2 * fff::kBFWarps * 2;      // one token per warp in the descent
-        const int64_t max_ctas = (int64_t)h->sm_count * h->bf_per_sm;
-        // thinner tiles while full ones would leave CTAs without work, unless the leaves are thin themselves
-        const int tile_rows = B <= 8 * max_ctas && B >= 32 * h->n_leaves ? 8 : fff::kBFTile;
-        cfg.gridDim = dim3((unsigned)std::min(max_ctas, std::max<int64_t>(B, 1)));
+        cfg.gridDim = dim3((unsigned)std::min((int64_t)h->sm_count * h->bf_per_sm, std::max<int64_t>(B, 1)));
         cfg.blockDim = dim3(fff::kBFThreads);
         cfg.dynamicSmemBytes = block_forward_smem(h);
-        e = cudaLaunchKernelEx(&cfg, single ? fff::k_block_forward<T, 1> : fff::k_block_forward<T, 4>, (const T*)x, (const T*)h->node_w,
+        e = cudaLaunchKernelEx(&cfg, block_forward_single(h, B) ? fff::k_block_forward<T, 1> : fff::k_block_forward<T, 4>, (const T*)x, (const T*)h->node_w,
                                (const T*)h->node_b, (const T*)h->w1, (const T*)h->b1, (const T*)h->w2, (const T*)h->b2, (T*)y, leaf_out, leaf_out2,
                                h->ws_slots, h->ws_cursor, (int)h->slot_cap, h->D, h->O, h->depth, h->l, h->act, (int)B,
-                               h->vec_ok && aligned16(x), (int)h->n_leaves, tile_rows, h->d_status);
+                               h->vec_ok && aligned16(x), (int)h->n_leaves, block_forward_rows(h, B), h->d_status);
     }
     if (e != cudaSuccess) return cudaGetLastError(), FFF_ERR_CUDA;
     const fff_status_t s = launched(h, st, "fused_forward_blocks");
