@@ -101,8 +101,8 @@ static_assert(kLUExpandWarps == 2, "LeafCodeRing::stage: two rounds of the ring"
 // else, two for W1 stages and two for W2 pieces, taking turns on whole stages and pieces, each starting as soon as its codes have landed.
 // What binds them is instruction fetch, with seven roles in the cache at a time: as a loop of one step of 32 units of 16 codes
 // a W2 piece of 128 x 32 takes 0.8 us, unrolled 1.9.  2048 leaves of 32, 65 536 tokens, a forward: 213 us with two warps per piece and the
-// published conversions, 208 with whole pieces per warp unrolled, 188.9 in this form (halves of pieces as loops 196); 896 -> 896, 256
-// leaves of 9, 8766 tokens 31.4, 32.4 and 31.3 with the first and the last.  Three or four warps per kind cost the epilogue its registers.
+// published conversions, 208 with whole pieces per warp unrolled, 187.1 in this form (halves of pieces as loops 196); 896 -> 896, 256 leaves of 9,
+// 8766 tokens 31.5 and 31.1 with the first and the last.  Three or four warps per kind cost the epilogue its registers.
 // GL: leaves per tile.  1: a tile holds tokens of one leaf.  8: a tile holds tokens of one node three levels above the
 // leaves; GEMM1 then runs against the hidden units of that node's 8 leaves side by side plus the 7 nodes of its
 // subtree (N = 8 LP + 16 columns, the last 9 zero), the epilogue walks the three levels from the node logits, keeps
@@ -132,8 +132,20 @@ template <int LP, bool kW8 = false, int GL = 1, bool kSplit = false> struct Leaf
     static constexpr int kXStageBytes = kSub * kXSubBytes;
     static constexpr int kW1StageBytes = kSub * kW1SubBytes;
     static constexpr int kW1CodeBytes = kW8 ? kW1StageBytes / 2 : 0;         // staging for the codes of the stage's W1 K-blocks
-    static constexpr int kW1CopyBytes = kW8 ? kW1CodeBytes : kW1StageBytes;  // what the bulk copy of a stage brings
+    static constexpr int kW1CopyBytes = kW8 ? kW1SubBytes / 2 : kW1SubBytes; // what the bulk copy of a stage brings, per K-block
     static constexpr int kStageBytes = kXStageBytes + kW1StageBytes + kW1CodeBytes;      // a multiple of 1024
+    // Tiles of at most 64 (32) rows need half (a quarter) of a K-block's space for x.  With 32 padded neurons their stages hold as many more
+    // K-blocks as fit, the x tiles first: what the ring keeps in flight then does not shrink with the rows (2048 leaves of 32, 65 536 tokens, a
+    // forward 167.2 and 166.0 us; 1024 leaves of 20, 40 000 tokens 96.0 and 95.1; a few per cent the other way where a CTA has full tiles:
+    // 128 leaves of 19, 34 056 tokens 43.4 and 43.9).  The MMAs read 128 rows all the same: what lies behind the last x tile is the stage's own W1, and
+    // the accumulator rows of it are never looked at.  Not with 16 padded neurons (768 -> 768, 256 leaves of 12, 20 000 tokens 39.0 and 39.4), nor with
+    // 64, whose W1 leaves no room, nor with 8-bit weights, whose stages wait for the expansion of all their K-blocks.
+    static constexpr bool kDeep = LP == 32 && !kW8;
+    static constexpr int stage_blocks(int cap_rows) {
+        return kDeep && cap_rows < kLUM ? kStageBytes / (cap_rows * kLUKB * 2 + kW1SubBytes) : kSub;
+    }
+    static_assert(!kDeep || ((stage_blocks(32) - 1) * 32 * kLUKB * 2 + kXSubBytes <= kStageBytes &&
+                             (stage_blocks(64) - 1) * 64 * kLUKB * 2 + kXSubBytes <= kStageBytes), "an MMA reads 128 rows within the stage");
     static constexpr int kW2Bytes = kLUPiece * kHCols * 2;                   // weights of a piece (bf16 operand)
     static constexpr int kW2CodeBytes = kW8 ? kW2Bytes / 2 : 0;
     static constexpr int kW2BiasOff = kW2Bytes;                              // the piece's 128 float32 biases inside a slot
@@ -385,7 +397,12 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
     uint64_t* w2code_full = code_full + kLUExpandWarps * kLUMaxStages;       // [kLUMaxW2Slots] likewise the codes of a W2 piece
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int KB = D / (kLUKB * L::kSub);                   // ring stages per tile
+    const int KB = D / kLUKB;                               // K-blocks of GEMM1 per tile (a multiple of kSub)
+    // f(rows that a stage has room for) for a tile of `rows` rows.  (The loops over a tile's stages as functions of that number: written out in
+    // place they were 0.5 to 1 % slower, 2048 leaves of 32, 65 536 tokens 166.7 against 166.0 us a forward, with 8-bit weights 189.2 against
+    // 187.1.  The instructions are the same as far as the source shows; it is the compiler's order of them.)
+    auto with_stages = [](int rows, auto f) { f(rows <= 32 ? 32 : rows <= 64 ? 64 : kLUM); };
+    constexpr int kUnroll = L::kDeep ? 1 : L::kSub;         // stages of constant length but for deep ones
     const int P = (O + kLUPiece - 1) / kLUPiece;
 
     if (threadIdx.x == 0) {
@@ -548,7 +565,7 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             LeafCodeRing codes(kStages);
             for (int it = 0; it < max_iters; ++it) {
                 if (next_tile().rows <= 0) break;
-                for (int kb = 0; kb < KB; ++kb, codes.next()) {
+                for (int kb = 0; kb < KB; kb += L::kSub, codes.next()) {
                     if (codes.owner() == part) {
                         const int stage = codes.stage();
                         if (!timed_out && !ptx::mbar_wait(code_full + codes.at, codes.phase)) timed_out = true;
@@ -599,33 +616,38 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
 #pragma unroll
                 for (int i = 0; i < 4; ++i) r[i] = perm[tl.start + min(first + i, tl.rows - 1)];
             }
-            for (int kb = 0; kb < KB; ++kb) {
-                if (!timed_out && !ptx::mbar_wait_relaxed(empty + stage, phase ^ 1)) timed_out = true;
-                if (lane == 0) {
-                    const uint32_t bytes = (uint32_t)groups * (512u * L::kSub) + (!kW8 && gw == 0 ? (uint32_t)L::kW1CopyBytes : 0u);
-                    if (bytes > 0) ptx::mbar_arrive_expect_tx(full + stage, bytes);
-                    else ptx::mbar_arrive(full + stage);
-                    if (gw == 0) {
-                        if constexpr (kW8) {
-                            uint64_t* landed = code_full + codes.at;
-                            ptx::mbar_arrive_expect_tx(landed, (uint32_t)L::kW1CodeBytes);
-                            ptx::bulk_g2s(ring + stage * L::kStageBytes + L::kXStageBytes + L::kW1StageBytes,
-                                          w1codes + ((int64_t)tl.bin * KB + kb) * L::kW1CodeBytes, L::kW1CodeBytes, landed);
-                        } else
-                            ptx::bulk_g2s(ring + stage * L::kStageBytes + L::kXStageBytes,
-                                          w1img + ((int64_t)tl.bin * KB + kb) * (L::kW1StageBytes / 2), L::kW1StageBytes, full + stage);
+            with_stages(tl.rows, [&](auto cap) {
+                const int blocks = !L::kDeep ? L::kSub : cap == 32 ? L::stage_blocks(32) : cap == 64 ? L::stage_blocks(64) : L::kSub;
+                const int x_bytes = (L::kDeep ? cap : kLUM) * kLUKB * 2;
+                for (int k0 = 0; k0 < KB; k0 += blocks) {
+                    const int n = !L::kDeep ? L::kSub : min(blocks, KB - k0);
+                    if (!timed_out && !ptx::mbar_wait_relaxed(empty + stage, phase ^ 1)) timed_out = true;
+                    unsigned char* xs = ring + stage * L::kStageBytes;
+                    if (lane == 0) {
+                        const uint32_t w1_bytes = (uint32_t)(n * L::kW1CopyBytes);
+                        const uint32_t bytes = (uint32_t)(groups * n) * 512u + (!kW8 && gw == 0 ? w1_bytes : 0u);
+                        if (bytes > 0) ptx::mbar_arrive_expect_tx(full + stage, bytes);
+                        else ptx::mbar_arrive(full + stage);
+                        if (gw == 0) {
+                            const int64_t block = (int64_t)tl.bin * KB + k0;
+                            if constexpr (kW8) {
+                                uint64_t* landed = code_full + codes.at;
+                                ptx::mbar_arrive_expect_tx(landed, w1_bytes);
+                                ptx::bulk_g2s(xs + L::kXStageBytes + L::kW1StageBytes, w1codes + block * L::kW1CopyBytes, w1_bytes, landed);
+                            } else
+                                ptx::bulk_g2s(xs + n * x_bytes, w1img + block * (L::kW1CopyBytes / 2), w1_bytes, full + stage);
+                        }
                     }
+                    __syncwarp();
+                    if (lane < groups) {
+#pragma unroll kUnroll
+                        for (int sb = 0; sb < n; ++sb)
+                            ptx::tma_gather4(xs + sb * x_bytes + first * 128, &tmap_x, (k0 + sb) * kLUKB, r[0], r[1], r[2], r[3], full + stage);
+                    }
+                    if constexpr (kW8) codes.next();
+                    if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
-                __syncwarp();
-                if (lane < groups) {
-#pragma unroll
-                    for (int sb = 0; sb < L::kSub; ++sb)
-                        ptx::tma_gather4(ring + stage * L::kStageBytes + sb * L::kXSubBytes + first * 128, &tmap_x,
-                                         (kb * L::kSub + sb) * kLUKB, r[0], r[1], r[2], r[3], full + stage);
-                }
-                if constexpr (kW8) codes.next();
-                if (++stage == kStages) { stage = 0; phase ^= 1; }
-            }
+            });
         }
     } else if (warp == kLUGemm1Warp) {
         // ------------------------------------------------------------------ GEMM1 issuer
@@ -637,25 +659,30 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             if (tl.rows <= 0) break;
             if (!timed_out && !ptx::mbar_wait(acc1_empty, (it & 1) ^ 1)) timed_out = true;
             ptx::tc_fence_after_sync();
-            for (int kb = 0; kb < KB; ++kb) {
-                if (!timed_out && !ptx::mbar_wait(full + stage, phase)) timed_out = true;
-                ptx::tc_fence_after_sync();
-                if (lane == 0) {
-                    const uint32_t xs = ptx::smem_addr(ring + stage * L::kStageBytes);
+            with_stages(tl.rows, [&](auto cap) {
+                const int blocks = !L::kDeep ? L::kSub : cap == 32 ? L::stage_blocks(32) : cap == 64 ? L::stage_blocks(64) : L::kSub;
+                const int x_bytes = (L::kDeep ? cap : kLUM) * kLUKB * 2;
+                for (int k0 = 0; k0 < KB; k0 += blocks) {
+                    const int n = !L::kDeep ? L::kSub : min(blocks, KB - k0);
+                    if (!timed_out && !ptx::mbar_wait(full + stage, phase)) timed_out = true;
+                    ptx::tc_fence_after_sync();
+                    if (lane == 0) {
+                        const uint32_t xs = ptx::smem_addr(ring + stage * L::kStageBytes);
+#pragma unroll kUnroll
+                        for (int sb = 0; sb < n; ++sb) {
+                            const uint64_t ad = ptx::umma_desc_k128(xs + sb * x_bytes);
+                            const uint64_t bd = ptx::umma_desc_k128(xs + n * x_bytes + sb * L::kW1SubBytes);
 #pragma unroll
-                    for (int sb = 0; sb < L::kSub; ++sb) {
-                        const uint64_t ad = ptx::umma_desc_k128(xs + sb * L::kXSubBytes);
-                        const uint64_t bd = ptx::umma_desc_k128(xs + L::kXStageBytes + sb * L::kW1SubBytes);
-#pragma unroll
-                        for (int j = 0; j < kLUKB / 16; ++j)
-                            ptx::umma_bf16(tmem_base, ad + 2 * j, bd + 2 * j, idesc, (kb | sb | j) != 0 ? 1u : 0u);
+                            for (int j = 0; j < kLUKB / 16; ++j)
+                                ptx::umma_bf16(tmem_base, ad + 2 * j, bd + 2 * j, idesc, (k0 | sb | j) != 0 ? 1u : 0u);
+                        }
+                        ptx::umma_commit(empty + stage);
+                        if (k0 + blocks >= KB) ptx::umma_commit(acc1_full);
                     }
-                    ptx::umma_commit(empty + stage);
-                    if (kb == KB - 1) ptx::umma_commit(acc1_full);
+                    __syncwarp();
+                    if (++stage == kStages) { stage = 0; phase ^= 1; }
                 }
-                __syncwarp();
-                if (++stage == kStages) { stage = 0; phase ^= 1; }
-            }
+            });
         }
     } else if (warp == kLUGemm2Warp) {
         // ------------------------------------------------------------------ W2 copies + GEMM2 issuer
@@ -692,7 +719,17 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
             auto load_ahead = [&](int needed) {
                 while (loaded < P && load_piece(loaded <= needed)) {}
             };
-            load_ahead(-1);
+            // While the warp waits for H, slots that the tile before gives back are filled: the last pieces of a short tile are needed soon after
+            // the first.  Only with 32 padded neurons, us a forward, without and with: 1024 -> 1024, 2048 leaves of 32, 40 000 tokens 141.3 and
+            // 139.9; 328 -> 320, 512 leaves of 18, 24 000 tokens 42.4 and 42.0; 16: 768 -> 768, 256 leaves of 12, 50 432 tokens 64.5 and 65.0; 64: 840 ->
+            // 832, 128 leaves of 38, 7781 tokens 29.7 and 30.1; 8-bit weights, 2048 leaves of 32, 65 536 tokens 188.9 and 189.3.
+            if constexpr (LP == 32 && !kW8) {
+                const long long t0 = clock64();
+                do load_ahead(-1);
+                while (loaded < P && !timed_out && !__any_sync(kFullMask, ptx::mbar_test(h_full, it & 1)) && clock64() - t0 < ptx::kWaitCycles);
+            } else {
+                load_ahead(-1);
+            }
             if (!timed_out && !ptx::mbar_wait(h_full, it & 1)) timed_out = true;
             ptx::tc_fence_after_sync();
             for (int p = 0; p < P; ++p, ++pc) {
@@ -732,9 +769,9 @@ k_leaf_umma(const __grid_constant__ CUtensorMap tmap_x, const int32_t* __restric
         // rows r, r + 128/rep, ... of the A operand, every copy's accumulator rows then hold the same values (the
         // rows of an MMA are independent; the extra MMA rows cost nothing), and the quarters of copy c convert and
         // store only the c-th group of 128/rep columns of each piece.
-        // (Steps of `rep` pieces, the MMAs of piece c leaving all accumulator rows but copy c's alone, and ring stages with more
-        // K-blocks for short tiles won nothing on 2048 leaves of 32, 65 536 tokens, 168.1 and 168.0 us a forward, and lost 1 to 4 %
-        // where a CTA has few tiles: 512 -> 512, 512 leaves of 24, 12 000 tokens 38.1 and 39.5.)
+        // (Steps of `rep` pieces, the MMAs of piece c leaving all accumulator rows but copy c's alone, won nothing on 2048 leaves of 32, 65 536
+        // tokens, 168.0 us a forward with deep stages, and lost 1 to 4 % where a CTA has few tiles: 512 -> 512, 512 leaves of 24, 12 000 tokens
+        // 38.4 and 39.4.)
         const int quarter = warp & 3, part = warp >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
         constexpr int HC = LP / kLUHParts;                       // H columns of a thread that computes H
