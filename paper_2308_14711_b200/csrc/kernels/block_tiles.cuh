@@ -5,7 +5,8 @@
 // loads of one step of 128 columns, so a block of dot products was a chain of six round trips of 1.5 us and a tile two such chains:
 // hidden layer 9.6 us, output layer 7, two tiles per CTA, of 57 us in all.  Bulk copies cost no registers: a tile's rows of x and its
 // leaf's W1 and W2, in blocks of up to a ring slot, are sent for as far ahead as the ring holds, across tiles, each by the warp that was
-// the last to read what lay there (hidden layer 3.5 to 4, output layer 4).  Measured: see block_tiles_plan in fff_api.cu.
+// the last to read what lay there (hidden layer 3.5 to 4, output layer 4).  Which batches it is taken for and what it measured: block_tiles_plan in
+// fff_api.cu.
 // Bound: in the descent the rows of the nodes below the first three levels, 130 KB per SM and level from L2 (12 us of 48); in the hidden
 // layer shared memory (48 cycles of loads per 32 of multiply-adds).  The top four levels in shared memory changed nothing.
 //   phase A  a warp takes kTok = 1 to 4 neighbouring tokens, so many that the batch is one pass where it can be, and copies
